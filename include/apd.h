@@ -79,8 +79,8 @@ typedef enum {
     APD_TC_TF32 = 2  /* the same with TF32 operands: ~3e-5 relative score error */
 } apd_precision;
 /* With APD_TC_BF16 / APD_TC_TF32, each seed preparation (the first pass of a
- * call, or of a weight solve) reads the seeds' conditioning back once (a
- * stream synchronisation): when max_i ||A_i||_F / min_i lambda_min(A_i) > 10
+ * call, or of a weight solve) reads the seeds' conditioning back once (the host
+ * waits for the records): when max_i ||A_i||_F / min_i lambda_min(A_i) > 10
  * the certificate and the candidate bounds of the tensor-core form are too
  * loose to pay, and the pass scores with the FP32 kernel instead (same labels).
  * Grids wider than the workspace's tile scratch are scored by the FP32 kernel
@@ -107,15 +107,15 @@ int apd_workspace_create(apd_workspace **ws, int32_t dim, int32_t max_n, int64_t
 void apd_workspace_destroy(apd_workspace *ws);
 
 /* Seed pruning of the scoring (default off: the dense sweep of Algorithm 1).
- * FP32: each warp skips every 32-seed group (Morton scan order) whose cost
- * lower bound over the warp's pixels,
- *     min lambda_min * dist(pixel box, seed box)^2 - (max w - w_ref),
- * exceeds the largest second-best cost among those pixels.  Tensor cores:
- * each 512-pixel tile scores only the seeds whose lower bound over the tile
- * lies below the fourth smallest upper bound lambda_max maxdist^2 - (w - w_ref);
- * the smallest bound of the seeds left out enters the certificate of every
- * label of the tile.  Either way labels and moments are the same as without
- * pruning.  Applies to every later scoring call on the workspace. */
+ * Each 512-pixel tile scores, in FP32 whatever the precision asked for, only the
+ * seeds that can be the argmin somewhere in the tile: seed i is left out when a
+ * rigorous lower bound of C_i - C_a over the tile (a quadratic in the pixel's
+ * offset; a = the seed of least cost at the tile's centre) is positive.  That
+ * leaves a few seeds per tile, too few for a tensor-core contraction.  Pixels whose
+ * two smallest values are within the rounding bound are settled in FP64.  Labels
+ * and moments are the same as without pruning.  Above 16384 seeds the FP32 kernel
+ * skips whole 32-seed groups instead.  Applies to every later scoring call on the
+ * workspace. */
 int apd_workspace_set_pruning(apd_workspace *ws, int32_t enable);
 
 /* Weight solves (Algorithm 2, and every solve inside the Lloyd, coarse-to-fine
@@ -129,7 +129,7 @@ int apd_workspace_set_pruning(apd_workspace *ws, int32_t enable);
 int apd_workspace_set_graphs(apd_workspace *ws, int32_t enable);
 
 /* Incremental evaluations inside weight solves (tensor-core scorers with
- * pruning on, one rank; default on).  The weights enter every cost
+ * pruning on, one rank), on request.  The weights enter every cost
  * C_ij = |y_j - x_i|_A^2 - w_i (eq. (2.1)) linearly: between weights w0 and w,
  * C_k - C_a changes by exactly -(D_k - D_a), D = w - w0.  A full pass at w0
  * records, per pixel, its label a, its runner-up b and certified bounds
@@ -142,9 +142,10 @@ int apd_workspace_set_graphs(apd_workspace *ws, int32_t enable);
  * changes.  The device chooses each pass's kind from the drift: it records
  * afresh when more than 8 % of the pixels have a recorded g3 within
  * max D - min D.  Labels and moments are the same as with full passes.
- * enable: 0 every pass a full one; 1 (default) incremental passes on grids of
- * at least 2^20 pixels (below that a full pass costs about as much as the
- * incremental pass's extra launches); 2 incremental passes on every grid.
+ * enable: 0 every pass a full one; 1 (default) incremental passes where they
+ * cost less than full ones, which is nowhere since full passes score from
+ * difference lists (256^3 x 1000 seeds: 108 us, against 116 us for a re-decision
+ * and 667 us for a recording); 2 incremental passes on every grid.
  * Returns APD_ERR_ARG for a null workspace or another enable value. */
 int apd_workspace_set_incremental(apd_workspace *ws, int32_t enable);
 

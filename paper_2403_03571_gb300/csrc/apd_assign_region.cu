@@ -1,0 +1,79 @@
+// The pruned scorer of the one-instance calls: one block per grid region
+// (apd_region.cuh).
+#include "apd_region.cuh"
+
+namespace apd {
+
+namespace {
+
+using namespace region;
+
+// Block b is region b of the scoring window: nx x ny (x nz) regions, the last axis
+// starting at region index `toff`.
+// Four blocks per SM (64 registers, some spills) measured 195 us per 256^3 x 1000 seed
+// dual evaluation, three 197, two (no spills) 207: the lists' two barriers and the
+// dependent loads want more warps more than they want registers.
+template <int D>
+__global__ void __launch_bounds__(kThreads, 4)
+    assign_region_kernel(const __grid_constant__ Src src, const int nx, const int ny, const int toff) {
+    __shared__ Shared<D> sm;
+    init_shared<D>(sm);
+    const int b = (int)blockIdx.x;
+    const int bx = b % nx, r = b / nx;
+    const int by = D == 3 ? r % ny : r + toff, bz = D == 3 ? r / ny + toff : 0;
+    score_region<D>(sm, src, bx, by, bz);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(src.pairs_scored, (unsigned long long)sm.pairs * (unsigned long long)kTilePix);
+        if (sm.queued) atomicAdd(&src.sc->flag_count, sm.queued);
+    }
+}
+
+template <int D>
+cudaError_t launch_t(const GridDev &g, int n, const double *x, const double *A, const double *w, Workspace &ws,
+                     int32_t *labels, unsigned long long *gmom, cudaStream_t st) {
+    using G = Geom<D>;
+    Src src;
+    src.g = g;
+    src.gf = make_gridf(g);
+    src.n = n;
+    src.n_groups = (n + kGroup - 1) / kGroup;
+    src.recs = ws.sorted ? ws.recs32s : ws.recs32;
+    src.perm = ws.sorted ? ws.perm : nullptr;
+    src.groups = ws.groups;
+    src.x = x;
+    src.A = A;
+    src.w = w;
+    src.gmom = gmom;
+    src.labels = labels;
+    src.sc = ws.sc;
+    src.pairs_scored = ws.pairs_scored;
+    constexpr int RL = D == 3 ? G::RZ : G::RY;
+    const int toff = win_lo(g) / RL;
+    const int tcount = (win_hi(g) - 1) / RL - toff + 1;
+    const int nx = (g.res[0] + G::RX - 1) / G::RX;
+    const int ny = D == 3 ? (g.res[1] + G::RY - 1) / G::RY : tcount;
+    const long long blocks = (long long)nx * ny * (D == 3 ? tcount : 1);
+    const cudaError_t ep = record_scoring_start(ws, st);
+    if (ep != cudaSuccess) return ep;
+    assign_region_kernel<D><<<(unsigned)blocks, kThreads, 0, st>>>(src, nx, ny, toff);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Needs the groups' bounds, at most two groups per lane of a region's block (the
+// Morton-sorted counts; beyond them the FP32 kernel streams the seeds) and axes
+// whose indices are exact in FP32.
+bool region_form(const GridDev &g, int n, const Workspace &ws) {
+    return ws.prune && ws.groups && (n + kGroup - 1) / kGroup <= kMaxGroups && g.res[0] < (1 << 23) &&
+           g.res[1] < (1 << 23) && g.res[2] < (1 << 23);
+}
+
+cudaError_t launch_assign_region(const GridDev &g, int n, const double *x, const double *A, const double *w,
+                                 Workspace &ws, int32_t *labels, unsigned long long *moments, cudaStream_t st) {
+    return g.dim == 3 ? launch_t<3>(g, n, x, A, w, ws, labels, moments, st)
+                      : launch_t<2>(g, n, x, A, w, ws, labels, moments, st);
+}
+
+}  // namespace apd

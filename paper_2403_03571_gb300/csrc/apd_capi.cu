@@ -64,6 +64,19 @@ void shard_range(int res, int rank, int world, int &k_begin, int &k_count) {
     k_count = (int)(e - b);
 }
 
+GridF make_gridf(const GridDev &g) {
+    GridF f;
+    for (int a = 0; a < 3; ++a) {
+        f.loh[a] = (float)g.lo[a];
+        f.lol[a] = (float)(g.lo[a] - (double)f.loh[a]);
+        f.hh[a] = (float)g.h[a];
+        f.hl[a] = (float)(g.h[a] - (double)f.hh[a]);
+        const double hi = g.lo[a] + g.h[a] * g.res[a];
+        f.ymax[a] = (float)(std::max(std::fabs(g.lo[a]), std::fabs(hi)) * (1.0 + 1e-6));
+    }
+    return f;
+}
+
 double domain_measure(const apd_grid *gr) {
     double m = 1.0;
     for (int d = 0; d < gr->dim; ++d) m *= gr->hi[d] - gr->lo[d];
@@ -130,13 +143,13 @@ void destroy_graph(EvalGraph &e) {
 // conditioning comes from the seed preparation: read back once per preparation
 // (a stream synchronisation); passes that reuse the records reuse the value.
 constexpr double kTcMaxCond = 10.0;
-bool use_tensor_cores(const GridDev &g, apd_precision prec, Workspace &ws, bool weights_only, cudaStream_t st) {
+bool use_tensor_cores(const GridDev &g, apd_precision prec, Workspace &ws, bool weights_only) {
     if (prec == APD_FP32 || tc_tile_count(g) > ws.tc_tile_cap) return false;
     if (!weights_only) {
+        // launch_seed_prep queued the copy right after the records (the Morton sort
+        // runs behind it): waiting for that copy alone keeps the stream busy
         unsigned long long bits[2] = {0ull, 0ull};  // lam_abs_bits, lam_min_bits
-        if (cudaMemcpyAsync(&ws.sc_host->lam_abs_bits, &ws.sc->lam_abs_bits, 2 * sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, st) == cudaSuccess &&
-            cudaStreamSynchronize(st) == cudaSuccess) {
+        if (cudaEventSynchronize(ws.cond_ev) == cudaSuccess) {
             bits[0] = ws.sc_host->lam_abs_bits;
             bits[1] = ws.sc_host->lam_min_bits;
         }
@@ -155,9 +168,8 @@ bool use_tensor_cores(const GridDev &g, apd_precision prec, Workspace &ws, bool 
 // need a full one (see tc_band_kernel).  The first pass of a solve records.
 constexpr int kIncNone = 0, kIncAuto = 1;
 constexpr double kIncFullMax = 0.08;
-// Below this many pixels a full pass costs about as much as the three extra
-// launches of an incremental one (apd_workspace_set_incremental mode 1).
-constexpr long long kIncMinPixels = 1ll << 20;
+// Only on request (apd_workspace_set_incremental mode 2): a full pass from region
+// lists costs less than a re-decision.
 
 // The buffers of the incremental passes, allocated on first use (never inside a
 // graph capture).
@@ -202,7 +214,7 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
                           prec != APD_FP32;
     bool tc = false, inc_on = false;
     if (weights_only) {
-        tc = !empty && use_tensor_cores(g, prec, ws, true, st);
+        tc = !empty && use_tensor_cores(g, prec, ws, true);
         inc_on = inc_form && tc;
         // one launch: moments and counters cleared, trial weights into the records
         // the first trial of a new L-BFGS direction forms p too (see Solver::iterate)
@@ -216,9 +228,14 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
         if (step) APD_TRY(cuda_ok(launch_axpy(n, step->W, step->t, step->p, const_cast<double *>(w), st)));
         APD_TRY(cuda_ok(cudaMemsetAsync(mom, 0, (size_t)n * K * sizeof(unsigned long long), st)));
         APD_TRY(cuda_ok(launch_eval_reset(ws, st, false)));  // also: no record, this pass records
-        APD_TRY(cuda_ok(launch_seed_prep(g, n, x, A, w, ws, st)));
+        ws.cond_read = !empty && prec != APD_FP32 && tc_tile_count(g) <= ws.tc_tile_cap;
+        if (ws.cond_read && !ws.cond_ev)
+            APD_TRY(cuda_ok(cudaEventCreateWithFlags(&ws.cond_ev, cudaEventDisableTiming)));
+        const cudaError_t ep = launch_seed_prep(g, n, x, A, w, ws, st);
+        ws.cond_read = false;
+        APD_TRY(cuda_ok(ep));
         APD_TRY(cuda_ok(launch_group_bounds(n, ws, st)));
-        tc = !empty && use_tensor_cores(g, prec, ws, false, st);
+        tc = !empty && use_tensor_cores(g, prec, ws, false);
         inc_on = inc_form && tc;
     }
     if (inc_on) APD_TRY(cuda_ok(launch_inc_prepare(n, mom, ws, st)));
@@ -243,10 +260,16 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
     ws.prof_e0 = e0;
     // the tensor-core tiling needs per-tile scratch; grids too thin for the
     // workspace's tile capacity are scored by the FP32 kernel (same labels)
+    // a tensor-core request brings its per-axis tile table up to date whichever scorer
+    // takes the pass (once per grid; a capture leaves it to the caller)
+    if (tc && !ws.capturing) APD_TRY(cuda_ok(launch_tc_axis(g, ws, st)));
+    const bool regions = !empty && !inc_on && region_form(g, n, ws);
     if (empty) {
-    } else if (!tc)
+    } else if (regions) {
+        APD_TRY(cuda_ok(launch_assign_region(g, n, x, A, w, ws, labels, mom, st)));
+    } else if (!tc) {
         APD_TRY(cuda_ok(launch_assign_fp32(g, n, ws, labels, mom, st)));
-    else {
+    } else {
         // an incremental pass: the pre-pass and the scorer (recording variant, the
         // labels into the record) do nothing when the device chose a re-decision
         if (inc_on) {
@@ -266,7 +289,7 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
     // the re-decision (nothing when the pass records), the rescoring in the mode
     // the device chose, and a recording's moments, weights and w_ref kept
     if (inc_on) APD_TRY(cuda_ok(launch_tc_band(g, n, ws, st)));
-    if (!empty)
+    if (!empty && !regions)
         APD_TRY(cuda_ok(launch_rescore_fp64(g, n, x, A, w, ws, labels, mom, st, inc_on ? ws.inc_labels : nullptr,
                                             inc_on ? &ws.sc->inc_go : nullptr)));
     if (inc_on) APD_TRY(cuda_ok(launch_inc_commit(n, mom, w, ws, st)));
@@ -279,7 +302,7 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
     }
     // the tensor-core launcher counts its pre-pass launches itself
     ws.kernel_launches += (weights_only ? 3 : (ws.sorted ? 6 : 4) + (ws.groups ? 1 : 0) + (step ? 1 : 0)) -
-                          (empty ? 2 : 0) +  // an empty slab launches neither scoring nor rescoring
+                          (empty ? 2 : (regions ? 1 : 0)) +  // launched: no scoring or rescoring / no rescoring
                           (inc_on ? 3 : 0);  // the incremental pass's prepare, re-decision and commit
     ws.last_pixels = win_pixels(g);
     ws.last_pairs = win_pixels(g) * (long long)n;
@@ -373,7 +396,7 @@ struct Solver {
         k.inc = inc_mode;
         k.wait_limit = ws.wait_limit;
         // the scorer the captured pass takes (the seeds' conditioning can change it between solves)
-        const bool tc = use_tensor_cores(g, prec, ws, true, st);
+        const bool tc = use_tensor_cores(g, prec, ws, true);
         k.use_tc = tc ? 1u : 0u;
         const void *ptrs[9] = {x, A, v, Wp, gf_out, pdir, step ? step->W : nullptr, step ? step->p : nullptr,
                                ws.moments};
@@ -464,8 +487,7 @@ struct Solver {
     int eval(const double *Wp, double *gf_out, const double *pdir, double &f, double &dphi,
              double &err, const TrialStep *step = nullptr) {
         inc_mode = kIncNone;
-        if (ws.incremental && ws.prune && ws.shard_world <= 1 && prec != APD_FP32 &&
-            (ws.incremental > 1 || win_pixels(g) >= kIncMinPixels)) {
+        if (ws.incremental > 1 && ws.prune && ws.shard_world <= 1 && prec != APD_FP32) {
             APD_TRY(inc_alloc(ws));  // never inside a graph capture
             inc_mode = kIncAuto;
         }
@@ -941,6 +963,7 @@ void apd_workspace_destroy(apd_workspace *ws) {
     for (cudaEvent_t e : w.ev) cudaEventDestroy(e);
     for (EvalGraph &e : w.graph_cache) destroy_graph(e);
     if (w.cap_stream) cudaStreamDestroy(w.cap_stream);
+    if (w.cond_ev) cudaEventDestroy(w.cond_ev);
     void *ptrs[] = {w.recs, w.recs32, w.recs_tmp, w.codes, w.scodes, w.perm, w.recs32s, w.tc_centre, w.tc_start, w.tc_meta, w.tc_texcl, w.tc_list, w.tc_bops, w.tc_axis, w.moments, w.flags, w.flag_gi, w.pairs_scored, w.groups, w.sc, w.part, w.grad, w.W, w.Wt, w.p, w.gf, w.gft,
                     w.Wbest, w.S, w.Y, w.gram, w.lb_part, w.lb_coef, w.rho, w.X, w.vbuf, w.wfeat, w.wpred,
                     w.S2, w.Y2, w.gram2, w.rho2, w.inc_labels, w.inc_gap, w.inc_rec, w.inc_hist, w.inc_drift, w.inc_mom0, w.inc_w0, w.inc_aux};

@@ -87,6 +87,7 @@ struct DevScalars {
     float drift_hi;                     // drift_max rounded up to a float
     int inc_go;                         // this incremental pass re-decides from the record (else records)
     int inc_valid;                      // a record of this solve exists
+    float wref_h, wref_l;               // w_ref as an FP32 pair
 };
 
 // Partial sums per block row of the L-BFGS dot-product kernels: the push's
@@ -233,6 +234,8 @@ struct Workspace {
     cudaEvent_t cap_e0 = nullptr, cap_e1 = nullptr;
     std::vector<EvalGraph> graph_cache;
     uint64_t graph_clock = 0;
+    cudaEvent_t cond_ev = nullptr;  // the seeds' conditioning has been copied to sc_host
+    bool cond_read = false;         // launch_seed_prep copies it and records cond_ev
     int64_t kernel_launches = 0;  // every kernel launched with this workspace
 };
 
@@ -251,6 +254,11 @@ struct GridDev {
     long long J;  // pixels of the full grid
     int kz0, kz1;
 };
+// The grid's axes as FP32 pairs (hi + lo), and the largest |coordinate| per axis.
+struct GridF {
+    float loh[3], lol[3], hh[3], hl[3], ymax[3];
+};
+GridF make_gridf(const GridDev &g);
 // the last axis's resolution (a select, not a dynamic index: an indexed access
 // to a kernel's by-value GridDev makes the compiler copy it to the stack)
 __host__ __device__ inline int res_last(const GridDev &g) { return g.dim == 3 ? g.res[2] : g.res[1]; }
@@ -412,6 +420,11 @@ cudaError_t launch_seed_prep(const GridDev &g, int n, const double *x, const dou
 // FP32 scoring fused with the moments; queues near ties; labels optional.
 cudaError_t launch_assign_fp32(const GridDev &g, int n, Workspace &ws, int32_t *labels,
                                unsigned long long *moments, cudaStream_t st);
+// Whether a pass is scored from candidate lists over grid regions (pruning on, the
+// seeds' group bounds at hand), and that scorer (which settles its near ties itself).
+bool region_form(const GridDev &g, int n, const Workspace &ws);
+cudaError_t launch_assign_region(const GridDev &g, int n, const double *x, const double *A, const double *w,
+                                 Workspace &ws, int32_t *labels, unsigned long long *moments, cudaStream_t st);
 // tcgen05 scoring fused with the moments (kind 0 = TF32, 1 = BF16; per-tile candidate
 // lists when ws.prune); queues the pixels it cannot certify.
 cudaError_t launch_assign_tc(const GridDev &g, int n, Workspace &ws, int32_t *labels,

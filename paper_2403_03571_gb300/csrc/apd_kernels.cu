@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(256)
     }
     if (threadIdx.x == 0) {
         sc->wref_key = dkey(wref);
+        split_f32(wref, sc->wref_h, sc->wref_l);
         sc->dual_done = 0u;
     }
 }
@@ -265,9 +266,11 @@ __global__ void __launch_bounds__(1024)
 
 template <int D>
 __global__ void group_bounds_kernel(const int n, const SeedRec *__restrict__ recs, GroupBound *__restrict__ groups,
-                                    const DevScalars *__restrict__ sc) {
+                                    DevScalars *__restrict__ sc) {
     const int grp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (grp * 32 < n) group_bound_warp<D>(recs, n, grp, groups, dkey_inv(sc->wref_key));
+    const double wref = dkey_inv(sc->wref_key);
+    if (blockIdx.x == 0 && threadIdx.x == 0) split_f32(wref, sc->wref_h, sc->wref_l);
+    if (grp * 32 < n) group_bound_warp<D>(recs, n, grp, groups, wref);
 }
 
 __global__ void gather_recs_kernel(const int n_pad, const int32_t *__restrict__ perm,
@@ -937,7 +940,14 @@ cudaError_t launch_seed_prep(const GridDev &g, int n, const double *x, const dou
     else
         seed_prep_kernel<2><<<blocks, 256, 0, st>>>(g, n, n_pad, x, A, w, dst, ws.recs32, codes, ws.sc);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !ws.sorted) return e;
+    if (e != cudaSuccess) return e;
+    if (ws.cond_read) {  // the host waits for this copy while the sort runs
+        e = cudaMemcpyAsync(&ws.sc_host->lam_abs_bits, &ws.sc->lam_abs_bits, 2 * sizeof(unsigned long long),
+                            cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaEventRecord(ws.cond_ev, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (!ws.sorted) return cudaSuccess;
     const size_t smem = (size_t)m * sizeof(unsigned long long);
     if (!(ws.attr_done & kAttrMortonSort)) {
         e = cudaFuncSetAttribute(morton_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
