@@ -681,9 +681,9 @@ int apd_points_dual_value_grad(const apd_points *pts, const apd_seeds *seeds, co
  * apd_cell_moments) feed eqs. (2.7)-(2.8) on F.  It equals the full
  * Algorithm 1 on F wherever no cell boundary passes through an interior
  * coarse pixel (always, for example, across the straight boundary of two
- * seeds with equal A away from the grid's outer layer).  Each fine pixel of a
- * boundary coarse pixel is scored against every seed (no pruning), so the
- * call only pays where few coarse pixels are boundary pixels.
+ * seeds with equal A away from the grid's outer layer).  The fine pixels
+ * of boundary coarse pixels are scored from candidate lists (factors r up to 16 and
+ * up to 16384 seeds; beyond that against every seed).
  *
  * moments: device int64 [n][1 + D + D(D+1)/2], overwritten.
  * coarse_labels: device int32 [J_G], written with H^G.

@@ -29,11 +29,29 @@ __global__ void __launch_bounds__(kThreads, 4)
     }
 }
 
+// Masked form: a persistent grid over the listed regions.
 template <int D>
-cudaError_t launch_t(const GridDev &g, int n, const double *x, const double *A, const double *w, Workspace &ws,
-                     int32_t *labels, unsigned long long *gmom, cudaStream_t st) {
-    using G = Geom<D>;
-    Src src;
+__global__ void __launch_bounds__(kThreads, 4)
+    masked_region_kernel(const __grid_constant__ Src src, const int nx, const int ny, const int32_t *__restrict__ list) {
+    __shared__ Shared<D> sm;
+    init_shared<D>(sm);
+    const int count = (int)src.sc->mask_regions;
+    unsigned queued = 0u;
+    for (int i = (int)blockIdx.x; i < count; i += (int)gridDim.x) {
+        if (threadIdx.x == 0) sm.queued = 0u;
+        const int b = list[i];
+        const int r = b / nx;
+        score_region<D, true>(sm, src, b % nx, D == 3 ? r % ny : r, D == 3 ? r / ny : 0);
+        __syncthreads();
+        if (threadIdx.x == 0) queued += sm.queued;
+    }
+    if (threadIdx.x == 0 && queued) atomicAdd(&src.sc->flag_count, queued);
+}
+
+template <int D>
+Src make_src(const GridDev &g, int n, const double *x, const double *A, const double *w, Workspace &ws,
+             int32_t *labels, unsigned long long *gmom) {
+    Src src{};
     src.g = g;
     src.gf = make_gridf(g);
     src.n = n;
@@ -48,6 +66,14 @@ cudaError_t launch_t(const GridDev &g, int n, const double *x, const double *A, 
     src.labels = labels;
     src.sc = ws.sc;
     src.pairs_scored = ws.pairs_scored;
+    return src;
+}
+
+template <int D>
+cudaError_t launch_t(const GridDev &g, int n, const double *x, const double *A, const double *w, Workspace &ws,
+                     int32_t *labels, unsigned long long *gmom, cudaStream_t st) {
+    using G = Geom<D>;
+    const Src src = make_src<D>(g, n, x, A, w, ws, labels, gmom);
     constexpr int RL = D == 3 ? G::RZ : G::RY;
     const int toff = win_lo(g) / RL;
     const int tcount = (win_hi(g) - 1) / RL - toff + 1;
@@ -65,15 +91,45 @@ cudaError_t launch_t(const GridDev &g, int n, const double *x, const double *A, 
 // Needs the groups' bounds, at most two groups per lane of a region's block (the
 // Morton-sorted counts; beyond them the FP32 kernel streams the seeds) and axes
 // whose indices are exact in FP32.
-bool region_form(const GridDev &g, int n, const Workspace &ws) {
-    return ws.prune && ws.groups && (n + kGroup - 1) / kGroup <= kMaxGroups && g.res[0] < (1 << 23) &&
-           g.res[1] < (1 << 23) && g.res[2] < (1 << 23);
+bool region_lists(const GridDev &g, int n, const Workspace &ws) {
+    return ws.groups && (n + kGroup - 1) / kGroup <= kMaxGroups && g.res[0] < (1 << 23) && g.res[1] < (1 << 23) &&
+           g.res[2] < (1 << 23);
+}
+bool region_form(const GridDev &g, int n, const Workspace &ws) { return ws.prune && region_lists(g, n, ws); }
+
+void region_dims(int dim, int (&r)[3]) {
+    r[0] = dim == 3 ? Geom<3>::RX : Geom<2>::RX;
+    r[1] = dim == 3 ? Geom<3>::RY : Geom<2>::RY;
+    r[2] = dim == 3 ? Geom<3>::RZ : 1;
 }
 
 cudaError_t launch_assign_region(const GridDev &g, int n, const double *x, const double *A, const double *w,
                                  Workspace &ws, int32_t *labels, unsigned long long *moments, cudaStream_t st) {
     return g.dim == 3 ? launch_t<3>(g, n, x, A, w, ws, labels, moments, st)
                       : launch_t<2>(g, n, x, A, w, ws, labels, moments, st);
+}
+
+template <int D>
+static cudaError_t masked_t(const GridDev &gc, const GridDev &gf, int r, int n, const double *x, const double *A,
+                            const double *w, const uint8_t *mask, const int32_t *list, Workspace &ws,
+                            unsigned long long *moments, cudaStream_t st) {
+    using G = Geom<D>;
+    Src src = make_src<D>(gf, n, x, A, w, ws, nullptr, moments);
+    src.mask = mask;
+    src.r = r;
+    for (int a = 0; a < 3; ++a) src.cres[a] = gc.res[a];
+    const int nx = (gf.res[0] + G::RX - 1) / G::RX, ny = (gf.res[1] + G::RY - 1) / G::RY;
+    const long long all = (long long)nx * ny * (D == 3 ? (gf.res[2] + G::RZ - 1) / G::RZ : 1);
+    const int blocks = (int)(all < 4ll * ws.sms ? all : 4ll * ws.sms);
+    masked_region_kernel<D><<<blocks, kThreads, 0, st>>>(src, nx, ny, list);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_masked_region(const GridDev &gc, const GridDev &gf, int r, int n, const double *x, const double *A,
+                                 const double *w, const uint8_t *mask, const int32_t *list, Workspace &ws,
+                                 unsigned long long *moments, cudaStream_t st) {
+    return gf.dim == 3 ? masked_t<3>(gc, gf, r, n, x, A, w, mask, list, ws, moments, st)
+                       : masked_t<2>(gc, gf, r, n, x, A, w, mask, list, ws, moments, st);
 }
 
 }  // namespace apd

@@ -78,7 +78,8 @@ struct DevScalars {
     unsigned int dual_done;             // block counter of the two-phase dual reduction
     int pair_ok;                        // the last pushed L-BFGS pair passed the curvature test
     long long rescored_total;
-    unsigned int mask_count;            // boundary coarse pixels listed by the masked discretisation
+    unsigned int mask_count;            // boundary coarse pixels of the masked discretisation
+    unsigned int mask_regions;          // fine regions that hold pixels of boundary coarse pixels
     unsigned int lbfgs_done;            // block counter of the L-BFGS kernels' last-block reductions
     unsigned int band_count;            // pixels re-decided by the last incremental pass
     double drift_max, drift_min;        // max and min of w - w0 (incremental passes)
@@ -425,6 +426,13 @@ cudaError_t launch_assign_fp32(const GridDev &g, int n, Workspace &ws, int32_t *
 bool region_form(const GridDev &g, int n, const Workspace &ws);
 cudaError_t launch_assign_region(const GridDev &g, int n, const double *x, const double *A, const double *w,
                                  Workspace &ws, int32_t *labels, unsigned long long *moments, cudaStream_t st);
+// The masked form's fine scoring from region lists: the regions of the fine grid gf
+// listed in `list` (sc->mask_regions of them), the pixels whose coarse pixel is marked.
+bool region_lists(const GridDev &g, int n, const Workspace &ws);
+void region_dims(int dim, int (&r)[3]);
+cudaError_t launch_masked_region(const GridDev &gc, const GridDev &gf, int r, int n, const double *x, const double *A,
+                                 const double *w, const uint8_t *mask, const int32_t *list, Workspace &ws,
+                                 unsigned long long *moments, cudaStream_t st);
 // tcgen05 scoring fused with the moments (kind 0 = TF32, 1 = BF16; per-tile candidate
 // lists when ws.prune); queues the pixels it cannot certify.
 cudaError_t launch_assign_tc(const GridDev &g, int n, Workspace &ws, int32_t *labels,

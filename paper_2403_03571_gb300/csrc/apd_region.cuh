@@ -96,6 +96,9 @@ struct Src {
     int32_t *labels;           // [J] or null
     DevScalars *sc;
     unsigned long long *pairs_scored;
+    // MASKED: only the pixels of marked coarse pixels (r pixels per axis each)
+    const uint8_t *mask;       // [product of cres]
+    int r, cres[3];
 };
 
 // A seed's cost around a point: q = d^T A d, h = A d, S (see Rounding).
@@ -428,8 +431,8 @@ __device__ __forceinline__ float group_lower(const GroupBound &gb, const float (
 }
 
 // Scores region (bx, by, bz); `s` is the same in every thread.  The caller puts a
-// barrier between the table's initialisation or the previous region and the next.
-template <int D>
+// barrier between the previous region and the next.
+template <int D, bool MASKED = false>
 __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const int bx, const int by, const int bz) {
     using G = Geom<D>;
     constexpr int K = moment_width(D);
@@ -443,6 +446,63 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
     const int rdim[3] = {G::RX, G::RY, G::RZ};
     const int rb[3] = {bx * G::RX, by * G::RY, bz * G::RZ};
     float4(&ref)[5] = sm.ref[wid];
+
+    // the warp's tile
+    const int tc[3] = {wid % (G::RX / G::TX), (wid / (G::RX / G::TX)) % (G::RY / G::TY),
+                       wid / ((G::RX / G::TX) * (G::RY / G::TY))};
+    int kb[3], lo3[3], cnt[3];
+    float toff[3] = {0.f, 0.f, 0.f}, tr[3] = {0.f, 0.f, 0.f};
+    bool empty = false, whole = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        kb[a] = rb[a] + tc[a] * tdim[a];
+        int lo = kb[a], hi = kb[a] + tdim[a];
+        if (a < D) {
+            hi = min(hi, a == D - 1 ? win_hi(g) : g.res[a]);
+            if (a == D - 1) lo = max(lo, win_lo(g));
+            toff[a] = (float)(tc[a] * tdim[a] + tdim[a] / 2 - rdim[a] / 2) * g.h32[a];
+            tr[a] = __fmul_ru(__fmul_ru(0.5f * (float)(tdim[a] - 1), g.h32[a]), 1.f + 0x1p-22f);
+        }
+        lo3[a] = lo;
+        cnt[a] = hi - lo;
+        empty = empty || cnt[a] <= 0;
+        whole = whole && cnt[a] == tdim[a];
+    }
+    const int x0 = D == 3 ? 0 : 8 * (lane & 3);  // the lane's first pixel and rows in the tile
+    const int y0 = D == 3 ? (lane & 7) : (lane >> 2), z0 = D == 3 ? (lane >> 3) : 0;
+    const int k0 = kb[0] + x0;
+    const int w0 = min(8, g.res[0] - k0);
+    const unsigned wmask = w0 >= 8 ? 0xffu : (w0 > 0 ? (1u << w0) - 1u : 0u);
+    // row r of the lane: the pixels scored
+    auto row_valid = [&](int r) -> unsigned {
+        const int k1 = kb[1] + (D == 3 ? y0 : y0 + 8 * r), kl = D == 3 ? kb[2] + z0 + 4 * r : k1;
+        return k1 < g.res[1] && kl >= win_lo(g) && kl < win_hi(g) ? wmask : 0u;
+    };
+    unsigned marked[2] = {0u, 0u};
+    if constexpr (MASKED) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const unsigned vm = row_valid(r);
+            if (!vm) continue;
+            const int k1 = kb[1] + (D == 3 ? y0 : y0 + 8 * r), k2 = D == 3 ? kb[2] + z0 + 4 * r : 0;
+            const uint8_t *row = s.mask + (size_t)s.cres[0] * ((size_t)(k1 / s.r) + (size_t)s.cres[1] * (size_t)(k2 / s.r));
+            int kx = k0 / s.r, next = (kx + 1) * s.r;
+            bool on = row[kx] != 0;
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                if (!((vm >> p) & 1u)) continue;
+                if (k0 + p == next) {
+                    on = row[++kx] != 0;
+                    next += s.r;
+                }
+                marked[r] |= on ? 1u << p : 0u;
+            }
+        }
+        whole = __all_sync(full, marked[0] == 0xffu && marked[1] == 0xffu);
+        empty = !__any_sync(full, (marked[0] | marked[1]) != 0u);
+        if (!__syncthreads_or(!empty)) return;  // no marked pixel in the region
+    }
+    auto row_mask = [&](int r) -> unsigned { return MASKED ? marked[r] : row_valid(r); };
 
     // region centre (lane a: axis a) as an FP32 pair, half-widths rounded up
     float ch[3] = {0.f, 0.f, 0.f}, cl[3] = {0.f, 0.f, 0.f};
@@ -571,27 +631,6 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
         return e < (int)total ? (int)sm.list[e] : -1;
     };
 
-    // ---- the warp's tile ----
-    const int tc[3] = {wid % (G::RX / G::TX), (wid / (G::RX / G::TX)) % (G::RY / G::TY),
-                       wid / ((G::RX / G::TX) * (G::RY / G::TY))};
-    int kb[3], lo3[3], cnt[3];
-    float toff[3] = {0.f, 0.f, 0.f}, tr[3] = {0.f, 0.f, 0.f};
-    bool empty = false, whole = true;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        kb[a] = rb[a] + tc[a] * tdim[a];
-        int lo = kb[a], hi = kb[a] + tdim[a];
-        if (a < D) {
-            hi = min(hi, a == D - 1 ? win_hi(g) : g.res[a]);
-            if (a == D - 1) lo = max(lo, win_lo(g));
-            toff[a] = (float)(tc[a] * tdim[a] + tdim[a] / 2 - rdim[a] / 2) * g.h32[a];
-            tr[a] = __fmul_ru(__fmul_ru(0.5f * (float)(tdim[a] - 1), g.h32[a]), 1.f + 0x1p-22f);
-        }
-        lo3[a] = lo;
-        cnt[a] = hi - lo;
-        empty = empty || cnt[a] <= 0;
-        whole = whole && cnt[a] == tdim[a];
-    }
     if (empty) return;
     const WordMap wm = word_map<D>();
 
@@ -679,17 +718,7 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
         }
     };
 
-    const int x0 = D == 3 ? 0 : 8 * (lane & 3);  // the lane's first pixel and rows in the tile
-    const int y0 = D == 3 ? (lane & 7) : (lane >> 2), z0 = D == 3 ? (lane >> 3) : 0;
     const long long plane = (long long)g.res[0] * (long long)g.res[1];
-    const int k0 = kb[0] + x0;
-    const int w0 = min(8, g.res[0] - k0);
-    const unsigned wmask = w0 >= 8 ? 0xffu : (w0 > 0 ? (1u << w0) - 1u : 0u);
-    // row r of the lane: its valid pixels and the id of the first
-    auto row_mask = [&](int r) -> unsigned {
-        const int k1 = kb[1] + (D == 3 ? y0 : y0 + 8 * r), kl = D == 3 ? kb[2] + z0 + 4 * r : k1;
-        return k1 < g.res[1] && kl >= win_lo(g) && kl < win_hi(g) ? wmask : 0u;
-    };
     auto row_id = [&](int r) -> long long {
         const int k1 = kb[1] + (D == 3 ? y0 : y0 + 8 * r), k2 = D == 3 ? kb[2] + z0 + 4 * r : 0;
         return (long long)k0 + (long long)g.res[0] * k1 + plane * k2;
@@ -707,8 +736,14 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
     };
 
     if (listed == 0) {  // one cell
-        const WordScale ws = word_scale(wm, lo3);
-        const unsigned long long word = box_word<D>(wm, ws, cnt);
+        unsigned long long word;
+        if (MASKED && !whole) {
+            unsigned pk[5];
+            packed_sums<D>(sm.lut, marked, (unsigned)x0, (unsigned)y0, (unsigned)z0, pk);
+            word = packed_word<D>(wm, word_scale(wm, kb), pk);
+        } else {
+            word = box_word<D>(wm, word_scale(wm, lo3), cnt);
+        }
         if (lane < K) atomicAdd(&s.gmom[(size_t)ref_id * K + lane], word);
         if (s.labels) {
             const unsigned id = (unsigned)ref_id;
