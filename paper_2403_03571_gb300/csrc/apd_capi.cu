@@ -146,7 +146,7 @@ constexpr double kTcMaxCond = 10.0;
 bool use_tensor_cores(const GridDev &g, apd_precision prec, Workspace &ws, bool weights_only) {
     if (prec == APD_FP32 || tc_tile_count(g) > ws.tc_tile_cap) return false;
     if (!weights_only) {
-        // launch_seed_prep queued the copy right after the records (the Morton sort
+        // launch_seed_prep queued the copy right after the records (the ranking
         // runs behind it): waiting for that copy alone keeps the stream busy
         unsigned long long bits[2] = {0ull, 0ull};  // lam_abs_bits, lam_min_bits
         if (cudaEventSynchronize(ws.cond_ev) == cudaSuccess) {
@@ -226,12 +226,11 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
                                           inc_on ? ws.inc_w0 : nullptr, full_max)));
     } else {
         if (step) APD_TRY(cuda_ok(launch_axpy(n, step->W, step->t, step->p, const_cast<double *>(w), st)));
-        APD_TRY(cuda_ok(cudaMemsetAsync(mom, 0, (size_t)n * K * sizeof(unsigned long long), st)));
-        APD_TRY(cuda_ok(launch_eval_reset(ws, st, false)));  // also: no record, this pass records
         ws.cond_read = !empty && prec != APD_FP32 && tc_tile_count(g) <= ws.tc_tile_cap;
         if (ws.cond_read && !ws.cond_ev)
             APD_TRY(cuda_ok(cudaEventCreateWithFlags(&ws.cond_ev, cudaEventDisableTiming)));
-        const cudaError_t ep = launch_seed_prep(g, n, x, A, w, ws, st);
+        // clears the moments and counters too (no record: this pass records)
+        const cudaError_t ep = launch_seed_prep(g, n, x, A, w, ws, mom, (long long)n * (long long)K, st);
         ws.cond_read = false;
         APD_TRY(cuda_ok(ep));
         APD_TRY(cuda_ok(launch_group_bounds(n, ws, st)));
@@ -301,7 +300,7 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
             return APD_ERR_CUDA;
     }
     // the tensor-core launcher counts its pre-pass launches itself
-    ws.kernel_launches += (weights_only ? 3 : (ws.sorted ? 6 : 4) + (ws.groups ? 1 : 0) + (step ? 1 : 0)) -
+    ws.kernel_launches += (weights_only ? 3 : (ws.sorted ? 4 : 3) + (ws.groups ? 1 : 0) + (step ? 1 : 0)) -
                           (empty ? 2 : (regions ? 1 : 0)) +  // launched: no scoring or rescoring / no rescoring
                           (inc_on ? 3 : 0);  // the incremental pass's prepare, re-decision and commit
     ws.last_pixels = win_pixels(g);
@@ -926,6 +925,13 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
     // super-tiles: at most one per tile
     w.part_rows = (int)nb;
     alloc((void **)&w.part, nb * kPartStride * sizeof(double));
+    if (w.n_pad_max <= kSortMax) {
+        // point sets: about 32 tiles a seed, room for eight polynomials a tile
+        w.pts_bytes = (size_t)std::min<long long>(32ll * std::max(max_n, 64), 1ll << 17) * (16 + 8 * 48);
+        alloc((void **)&w.pts_tiles, w.pts_bytes);
+        alloc((void **)&w.pts_geo, sizeof(PtsGeo));
+        if (ok && cudaMemset(w.pts_geo, 0, sizeof(PtsGeo)) != cudaSuccess) ok = false;
+    }
     alloc((void **)&w.grad, (size_t)max_n * sizeof(double));
     alloc((void **)&w.W, (size_t)max_n * sizeof(double));
     alloc((void **)&w.Wt, (size_t)max_n * sizeof(double));
@@ -966,7 +972,7 @@ void apd_workspace_destroy(apd_workspace *ws) {
     if (w.cond_ev) cudaEventDestroy(w.cond_ev);
     void *ptrs[] = {w.recs, w.recs32, w.recs_tmp, w.codes, w.scodes, w.perm, w.recs32s, w.tc_centre, w.tc_start, w.tc_meta, w.tc_texcl, w.tc_list, w.tc_bops, w.tc_axis, w.moments, w.flags, w.flag_gi, w.pairs_scored, w.groups, w.sc, w.part, w.grad, w.W, w.Wt, w.p, w.gf, w.gft,
                     w.Wbest, w.S, w.Y, w.gram, w.lb_part, w.lb_coef, w.rho, w.X, w.vbuf, w.wfeat, w.wpred,
-                    w.S2, w.Y2, w.gram2, w.rho2, w.inc_labels, w.inc_gap, w.inc_rec, w.inc_hist, w.inc_drift, w.inc_mom0, w.inc_w0, w.inc_aux};
+                    w.S2, w.Y2, w.gram2, w.rho2, w.inc_labels, w.inc_gap, w.inc_rec, w.inc_hist, w.inc_drift, w.inc_mom0, w.inc_w0, w.inc_aux, w.pts_tiles, w.pts_geo};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (w.sc_host) cudaFreeHost(w.sc_host);
@@ -1202,7 +1208,7 @@ int apd_points_moments(const apd_points *pts, const apd_seeds *seeds, double *mo
                        apd_workspace *ws, apd_stream_t stream) {
     APD_TRY(points_entry(pts, seeds, ws));
     if (!moments) return APD_ERR_ARG;
-    ws->w.kernel_launches += 4;
+    ws->w.kernel_launches += points_tiled(pts->count, seeds->n, ws->w) ? 6 : 3;
     return cuda_ok(launch_points_assign(pts->dim, pts->count, pts->y, pts->mass, seeds->n, seeds->x, seeds->A,
                                         seeds->w, moments, labels, ws->w, (cudaStream_t)stream));
 }
@@ -1216,7 +1222,7 @@ int apd_points_dual_value_grad(const apd_points *pts, const apd_seeds *seeds, co
     double *mom = reinterpret_cast<double *>(ws->w.moments);
     APD_TRY(cuda_ok(launch_points_assign(pts->dim, pts->count, pts->y, pts->mass, seeds->n, seeds->x, seeds->A,
                                          seeds->w, mom, nullptr, ws->w, st)));
-    ws->w.kernel_launches += 5;
+    ws->w.kernel_launches += points_tiled(pts->count, seeds->n, ws->w) ? 7 : 4;
     return cuda_ok(launch_points_dual(pts->dim, seeds->n, seeds->x, seeds->A, seeds->w, v, mom, ws->w, g_out, grad,
                                       max_rel_err, st));
 }

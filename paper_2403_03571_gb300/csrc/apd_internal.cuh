@@ -110,7 +110,7 @@ struct LbfgsCoef {
 
 // Bits of Workspace::attr_done: the dynamic shared-memory limit of these
 // kernels is raised once per workspace (a workspace lives on one device).
-constexpr unsigned kAttrFp32Score2 = 1u << 0, kAttrFp32Score3 = 1u << 1, kAttrMortonSort = 1u << 2;
+constexpr unsigned kAttrFp32Score2 = 1u << 0, kAttrFp32Score3 = 1u << 1;
 constexpr unsigned kAttrTcScore = 1u << 3;     // + 1 bit per (dimension, operand kind): 4 bits
 constexpr unsigned kAttrTcScoreRec = 1u << 7;  // the recording variant: 4 bits
 
@@ -128,6 +128,8 @@ struct EvalGraph {
     bool failed = false;  // capture refused: this key runs without a graph
     bool recorded = false;  // queued as an incremental pass (the device chooses its kind)
 };
+
+struct PtsGeo;
 
 // Workspace (host struct; device pointers inside).
 struct Workspace {
@@ -172,6 +174,9 @@ struct Workspace {
     GroupBound *groups = nullptr;       // [n_pad_max / 32] bounds of the scan-order seed groups
     DevScalars *sc = nullptr;           // device
     DevScalars *sc_host = nullptr;      // pinned host mirror
+    PtsGeo *pts_geo = nullptr;          // tiling of the last point set
+    uint8_t *pts_tiles = nullptr;       // its tiles' headers, then their polynomials (pts_bytes)
+    size_t pts_bytes = 0;
     double *part = nullptr;             // [part_rows][kPartStride] per-block partials (dual, trial weights)
     int part_rows = 0;
     double *grad = nullptr;             // [max_n] gradient of g~ of the last evaluation
@@ -260,6 +265,15 @@ struct GridF {
     float loh[3], lol[3], hh[3], hl[3], ymax[3];
 };
 GridF make_gridf(const GridDev &g);
+// Tiling of a point set's box, made on the device: tile i of axis a has its centre at
+// gf.lo + (2 i + 1) gf.h and half-width r (gf.h with slack).
+struct PtsGeo {
+    GridF gf;
+    int t[3], regions[3], n_regions;  // tiles; regions of 2 tiles per axis
+    float inv[3], r[3], ext[3];       // tiles per unit, half-widths, box extents
+    unsigned pool;                    // polynomials stored so far
+    unsigned done;                    // block counter of the box kernel
+};
 // the last axis's resolution (a select, not a dynamic index: an indexed access
 // to a kernel's by-value GridDev makes the compiler copy it to the stack)
 __host__ __device__ inline int res_last(const GridDev &g) { return g.dim == 3 ? g.res[2] : g.res[1]; }
@@ -319,6 +333,17 @@ __host__ __device__ inline uint32_t morton_code(int dim, const double *frac) {
         double f = frac[a] * 32768.0;
         q[a] = f <= 0.0 ? 0u : (f >= 32767.0 ? 32767u : (uint32_t)f);
     }
+    return spread2_15(q[0]) | (spread2_15(q[1]) << 1);
+}
+
+__host__ __device__ inline uint32_t morton_code_f(int dim, const float *frac) {
+    uint32_t q[3] = {0u, 0u, 0u};
+    const float top = dim == 3 ? 1024.f : 32768.f;
+    for (int a = 0; a < dim; ++a) {
+        const float f = frac[a] * top;
+        q[a] = !(f > 0.f) ? 0u : (f >= top - 1.f ? (uint32_t)top - 1u : (uint32_t)f);
+    }
+    if (dim == 3) return spread3_10(q[0]) | (spread3_10(q[1]) << 1) | (spread3_10(q[2]) << 2);
     return spread2_15(q[0]) | (spread2_15(q[1]) << 1);
 }
 
@@ -385,13 +410,13 @@ int warmstart_dim(const apd_mlp *net);               // dimension of a warm-star
 // ----------------------------------------------------------------------------
 constexpr int moment_width(int dim) { return 1 + dim + dim * (dim + 1) / 2; }
 
-// zero the per-evaluation counters and statistics in sc
-cudaError_t launch_eval_reset(Workspace &ws, cudaStream_t st, bool keep_geometry = false);
 // non-uniform discretisation (apd_points.cu, apd_kernels.cu): labels and FP64
 // element-measure moments of `count` points; the dual from those moments
 cudaError_t launch_points_assign(int dim, long long count, const double *y, const double *mass, int n,
                                  const double *x, const double *A, const double *w, double *mom,
                                  int32_t *labels, Workspace &ws, cudaStream_t st);
+// whether launch_points_assign takes the tiled form
+bool points_tiled(long long count, int n, const Workspace &ws);
 cudaError_t launch_points_dual(int dim, int n, const double *x, const double *A, const double *w, const double *v,
                                const double *mom_pts, Workspace &ws, double *g_out, double *grad_out,
                                double *err_out, cudaStream_t st);
@@ -415,9 +440,13 @@ cudaError_t launch_masked_refine(const GridDev &gc, const GridDev &gf, int r, in
 cudaError_t launch_eval_begin(int n, const double *W0, double t, const double *pdir, double *Wt,
                               unsigned long long *mom, Workspace &ws, cudaStream_t st, bool form_p = false,
                               const double *w0 = nullptr, unsigned full_max = 0u);
-// seed records (FP64 x, w; FP32 symmetric A) + stats (max w, max ||A||_F, min lambda bound)
+// start of an evaluation at new positions: seed records (FP64 x, w; FP32 symmetric A) in
+// scan order, their statistics (max w, max ||A||_F, min lambda bound), cleared counters
+// and, when mom is given, n_mom cleared moment words; box: the Morton codes' box, on
+// the device (null: the grid's)
 cudaError_t launch_seed_prep(const GridDev &g, int n, const double *x, const double *A,
-                             const double *w, Workspace &ws, cudaStream_t st);
+                             const double *w, Workspace &ws, unsigned long long *mom, long long n_mom,
+                             cudaStream_t st, const PtsGeo *box = nullptr);
 // FP32 scoring fused with the moments; queues near ties; labels optional.
 cudaError_t launch_assign_fp32(const GridDev &g, int n, Workspace &ws, int32_t *labels,
                                unsigned long long *moments, cudaStream_t st);

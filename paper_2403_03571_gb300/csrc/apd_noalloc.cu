@@ -30,6 +30,7 @@ struct NoAllocScratch {
     apd::SeedRec32 recs32[kMaxSeeds];
     uint32_t flags[kMaxPixels];
     apd::DevScalars sc;
+    double part[64 * apd::kPartStride];  // the seed preparation's per-block maxima (at most 16 blocks of 256)
 };
 
 static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
@@ -115,6 +116,8 @@ extern "C" int apd_cell_moments_noalloc(const apd_grid *grid, const apd_seeds *s
     ws.recs32 = s->recs32;
     ws.flags = s->flags;
     ws.sc = &s->sc;
+    ws.part = s->part;
+    ws.part_rows = 64;
 
     const int n = seeds->n;
     cudaStream_t st = (cudaStream_t)stream;
@@ -122,10 +125,8 @@ extern "C" int apd_cell_moments_noalloc(const apd_grid *grid, const apd_seeds *s
     const size_t K = (size_t)apd::moment_width(g.dim);
     // the counters, statistics and status word start at zero on every call
     if (cudaMemsetAsync(&s->sc, 0, sizeof(apd::DevScalars), st) != cudaSuccess) return APD_ERR_CUDA;
-    if (cudaMemsetAsync(mom, 0, (size_t)n * K * sizeof(unsigned long long), st) != cudaSuccess)
+    if (apd::launch_seed_prep(g, n, seeds->x, seeds->A, seeds->w, ws, mom, (long long)n * (long long)K, st) != cudaSuccess)
         return APD_ERR_CUDA;
-    if (apd::launch_eval_reset(ws, st) != cudaSuccess) return APD_ERR_CUDA;
-    if (apd::launch_seed_prep(g, n, seeds->x, seeds->A, seeds->w, ws, st) != cudaSuccess) return APD_ERR_CUDA;
     if (apd::launch_assign_fp32(g, n, ws, nullptr, mom, st) != cudaSuccess) return APD_ERR_CUDA;
     if (apd::launch_rescore_fp64(g, n, seeds->x, seeds->A, seeds->w, ws, nullptr, mom, st) != cudaSuccess)
         return APD_ERR_CUDA;

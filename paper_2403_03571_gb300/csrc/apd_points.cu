@@ -3,44 +3,471 @@
 // measure-weighted moments m_i = sum |P_j|, S1_i = sum |P_j| y_j,
 // S2_i = sum |P_j| y_j y_j^T of each cell.
 //
-// One thread per point.  The seeds stream through shared memory in chunks of
+// Tiled form.  The points' box is cut into tiles (about 32 per seed, no more than one
+// per two points), every tile gets its candidate list as the grid's tiles do
+// (apd_region.cuh: the difference of two costs over the tile's box), stored as
+// polynomials; a thread per point finds its tile, evaluates the few polynomials there
+// and settles near ties in FP64 itself.  The points need no order.
+//   points_box_kernel    the box and the tiling, on the device (high words of the
+//                        coordinates: 20 bits are enough for a box)
+//   points_lists_kernel  a block per 2 x 2 (x 2) tiles, eight warps listing, a warp
+//                        per tile storing
+//   points_score_kernel  labels and moments
+// Bounds: the scoring kernel reads 32 (2D: 24) bytes a point from memory, a 16-byte
+// header and about three 48-byte polynomials a point from L2, issues nine FP64
+// products a point (16 clocks of an SM per warp each) and ten FP64 reductions.
+// 1000 seeds, 4 M random points in 3D: 13.6 ms for the direct form below -> MEASURED.
+//
+// Direct form (few seeds or points, or more seeds than region lists take): the seeds
+// stream through shared memory in chunks of
 // 256 FP32 direct-form records (coordinates and weights split into FP32 high
 // and low parts).  Pass 1 takes the smallest FP32 cost plus its rounding bound
 // over all seeds as a threshold; pass 2 recomputes every seed whose FP32 cost
 // minus its bound lies below it in FP64 with the reference operation order, and
 // the smallest FP64 cost wins (lowest index on ties): the label equals the
-// FP64 argmin over all seeds (the rescoring argument of the grid path).  The
+// FP64 argmin over all seeds (the rescoring argument of the grid path).  Points whose
+// tile's list did not fit its store, or that are not finite, take the same two passes a
+// warp at a time.  The
 // moments are FP64 sums accumulated with atomics (their rounding depends on
 // the order of the additions).
 #include <algorithm>
 
 #include "apd_common.cuh"
 #include "apd_cost.cuh"
+#include "apd_region.cuh"
 
 namespace apd {
 
 namespace {
 
-constexpr int kPtThreads = 256;
+using namespace region;
 
-// FP32 direct-form records and the reference weight of the seeds.
+constexpr int kPtThreads = 256;
+constexpr int kMaxTiles = 1024;  // per axis
+
+// One tile: 2 max E of its list, the reference seed (natural index; -1: no list, the
+// points are searched in full), where its polynomials start and how many there are.
+struct TileHead {
+    float gap;
+    int ref;
+    unsigned first, count;
+};
+
+// Adds one point to its cell's moments.
 template <int D>
-__global__ void points_prep_kernel(const int n, const double *__restrict__ x, const double *__restrict__ A,
-                                   const double *__restrict__ w, SeedRec32 *__restrict__ r32,
-                                   DevScalars *__restrict__ sc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    SeedRec r;
-    SeedRec32 q;
-    double wkey, frob, lam;
-    int bad;
-    build_seed<D>(i, n, x, A, w, r, q, wkey, frob, lam, bad);
-    if (i < n) {
-        r32[i] = q;
-        if (bad) atomicOr(&sc->status, bad);
+__device__ __forceinline__ void add_point(double *__restrict__ mom, int label, double mj, const double (&yy)[D]) {
+    double *o = mom + (size_t)label * moment_width(D);
+    atomicAdd(&o[0], mj);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const double m = mj * yy[a];
+        atomicAdd(&o[1 + a], m);
+        int e = 1 + D;
+#pragma unroll
+        for (int c = 0; c < a; ++c) e += D - c;
+#pragma unroll
+        for (int b = a; b < D; ++b) atomicAdd(&o[e + b - a], m * yy[b]);
     }
-    const double wmax = warp_max(i < n ? wkey : -DBL_MAX);
-    const bool any = __any_sync(0xffffffffu, i < n);
-    if ((threadIdx.x & 31) == 0 && any) atomicMax(&sc->wref_key, dkey(wmax));
+}
+
+// High and low FP32 parts of a double by integer operations (the FP64 pipe converts a
+// warp in 16 clocks of the SM): hi is v truncated to 24 bits, lo the rounded remainder,
+// |v - hi - lo| <= 2^-47 |v|.  Values beyond FP32's normal range give 0 or infinity.
+__device__ __forceinline__ void split_trunc(double v, float &hi, float &lo) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned h = (unsigned)(b >> 32), l = (unsigned)b;
+    const int e = (int)((h >> 20) & 0x7ffu) - 1023 + 127;  // FP32 exponent
+    const unsigned sign = h & 0x80000000u;
+    if (e <= 30 || e >= 255) {
+        hi = e >= 255 ? __uint_as_float(sign | 0x7f800000u) : 0.f;
+        lo = 0.f;
+        return;
+    }
+    hi = __uint_as_float(sign | ((unsigned)e << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
+    const float r = (float)(l & 0x1fffffffu);  // units of 2^(e - 127 - 52)
+    const float scale = __uint_as_float((unsigned)(e - 29) << 23) * 0x1p-23f;
+    lo = __uint_as_float(__float_as_uint(r * scale) | sign);
+}
+
+// The points' box from the high words of their coordinates, then (last block) the
+// tiling: about `want` tiles of near-cubic shape.
+template <int D>
+__global__ void __launch_bounds__(kPtThreads)
+    points_box_kernel(const long long count, const double *__restrict__ y, const long long want,
+                      unsigned *__restrict__ part, PtsGeo *__restrict__ geo) {
+    __shared__ unsigned smn[D], smx[D];
+    __shared__ bool last;
+    if (threadIdx.x < D) {
+        smn[threadIdx.x] = 0xffffffffu;
+        smx[threadIdx.x] = 0u;
+    }
+    __syncthreads();
+    unsigned mn[D], mx[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        mn[a] = 0xffffffffu;
+        mx[a] = 0u;
+    }
+    const uint2 *y2 = reinterpret_cast<const uint2 *>(y);
+#pragma unroll 4
+    for (long long j = (long long)blockIdx.x * kPtThreads + threadIdx.x; j < count; j += (long long)gridDim.x * kPtThreads)
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const unsigned h = y2[j * D + a].y;
+            if ((h & 0x7ff00000u) == 0x7ff00000u) continue;  // not finite
+            const unsigned k = h ^ ((h >> 31) ? 0xffffffffu : 0x80000000u);
+            mn[a] = min(mn[a], k);
+            mx[a] = max(mx[a], k);
+        }
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        mn[a] = __reduce_min_sync(0xffffffffu, mn[a]);
+        mx[a] = __reduce_max_sync(0xffffffffu, mx[a]);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&smn[a], mn[a]);
+            atomicMax(&smx[a], mx[a]);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            part[(size_t)blockIdx.x * 6 + a] = smn[a];
+            part[(size_t)blockIdx.x * 6 + 3 + a] = smx[a];
+        }
+        __threadfence();
+        last = atomicAdd(&geo->done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    float lo[3] = {0.f, 0.f, 0.f}, ext[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        unsigned m = 0xffffffffu, x = 0u;
+        for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) {
+            m = min(m, *(volatile unsigned *)&part[(size_t)b * 6 + a]);
+            x = max(x, *(volatile unsigned *)&part[(size_t)b * 6 + 3 + a]);
+        }
+        m = __reduce_min_sync(0xffffffffu, m);
+        x = __reduce_max_sync(0xffffffffu, x);
+        // outward: the dropped low words all zeros or all ones
+        const unsigned hm = (m >> 31) ? m ^ 0x80000000u : ~m, hx = (x >> 31) ? x ^ 0x80000000u : ~x;
+        const double dl = __longlong_as_double((long long)(((unsigned long long)hm << 32) | ((hm >> 31) ? 0xffffffffull : 0ull)));
+        const double dh = __longlong_as_double((long long)(((unsigned long long)hx << 32) | ((hx >> 31) ? 0ull : 0xffffffffull)));
+        const bool some = m <= x;
+        lo[a] = some ? __double2float_rd(dl) : 0.f;
+        ext[a] = some ? __fsub_ru(__double2float_ru(dh), lo[a]) : 1.f;
+    }
+    if (threadIdx.x != 0) return;
+    float big = 1e-30f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) big = fmaxf(big, ext[a]);
+    float vol = 1.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        ext[a] = fmaxf(ext[a], 1e-4f * big);
+        vol *= ext[a] / big;
+    }
+    float side = D == 3 ? cbrtf(vol / (float)want) : sqrtf(vol / (float)want);  // in units of big
+    int t[3] = {1, 1, 1};
+    for (int it = 0; it < 64; ++it) {  // shrink until the product fits
+        long long n = 1;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            t[a] = max(1, min(kMaxTiles, (int)(ext[a] / big / side + 0.5f)));
+            n *= t[a];
+        }
+        if (n <= want) break;
+        side *= 1.03f;
+    }
+    long long n = 1;
+    for (int a = 0; a < D; ++a) n *= t[a];
+    if (n > want) t[0] = t[1] = t[2] = 1;
+    geo->n_regions = 1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const bool ax = a < D;
+        const float h = ax ? __fmul_ru(__fdiv_ru(0.5f * ext[a], (float)t[a]), 1.f + 0x1p-20f) : 1.f;
+        geo->gf.loh[a] = ax ? lo[a] : 0.f;
+        geo->gf.lol[a] = 0.f;
+        geo->gf.hh[a] = h;
+        geo->gf.hl[a] = 0.f;
+        geo->gf.ymax[a] = ax ? fmaxf(fabsf(lo[a]), fabsf(lo[a]) + ext[a]) * (1.f + 1e-6f) : 0.f;
+        geo->t[a] = t[a];
+        geo->regions[a] = (t[a] + 1) / 2;
+        geo->n_regions *= geo->regions[a];
+        geo->inv[a] = 0.5f / h;
+        geo->r[a] = h * (1.f + 0x1p-9f);
+        geo->ext[a] = ext[a];
+    }
+    geo->pool = 0u;
+    geo->done = 0u;
+}
+
+// Candidate lists of the tiles, stored.
+template <int D>
+__global__ void __launch_bounds__(kThreads, 4)
+    points_lists_kernel(const __grid_constant__ Src src, PtsGeo *__restrict__ geo, TileHead *__restrict__ heads,
+                        float4 *__restrict__ polys, const unsigned pool_cap) {
+    using G = Geom<D>;
+    constexpr int NP = G::NP;
+    constexpr int PV = D == 3 ? 3 : 2;  // float4s of a polynomial
+    __shared__ Shared<D> sm;
+    __shared__ Src s;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned full = 0xffffffffu;
+    for (int i = tid; i < (int)(sizeof(Src) / 4); i += kThreads)
+        reinterpret_cast<int *>(&s)[i] = reinterpret_cast<const int *>(&src)[i];
+    __syncthreads();
+    if (tid == 0) s.gf = geo->gf;
+    __syncthreads();
+    const int nr = geo->n_regions;
+    const float hh[3] = {s.gf.hh[0], s.gf.hh[1], s.gf.hh[2]};
+    float tr[3], rr[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        tr[a] = a < D ? geo->r[a] : 0.f;
+        rr[a] = a < D ? hh[a] + tr[a] : 0.f;
+    }
+    for (int reg = (int)blockIdx.x; reg < nr; reg += (int)gridDim.x) {
+        const int q = reg / geo->regions[0];
+        const int rb[3] = {reg % geo->regions[0], D == 3 ? q % geo->regions[1] : q, D == 3 ? q / geo->regions[1] : 0};
+        float ch[3] = {0.f, 0.f, 0.f}, cl[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int a = 0; a < D; ++a) axis_point(s.gf, a, 4 * rb[a] + 2, ch[a], cl[a]);
+        float r0h, r0l;
+        const unsigned total = region_list<D>(sm, s, ch, cl, rr, r0h, r0l);
+        const int tc[3] = {wid & 1, (wid >> 1) & 1, wid >> 2};
+        int ti[3];
+        float toff[3] = {0.f, 0.f, 0.f};
+        bool real = D == 3 || wid < 4;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            ti[a] = a < D ? 2 * rb[a] + tc[a] : 0;
+            if (a < D) toff[a] = tc[a] ? hh[a] : -hh[a];
+            real = real && ti[a] < geo->t[a];
+        }
+        if (real) {
+            const bool scan = total > (unsigned)kListCap;
+            const int n_src = scan ? s.n_groups : (int)((total + 31u) / 32u);
+            auto source = [&](int c) -> int {
+                const int e = c * 32 + lane;
+                if (scan) return e < s.n ? e : -1;
+                return e < (int)total ? (int)sm.list[e] : -1;
+            };
+            unsigned best = 0xffffffffu;
+            int best_pos = 0x7fffffff;
+            Local<D> L;
+            for (int c = 0; c < n_src; ++c) {
+                const int p = source(c);
+                unsigned ck = 0xffffffffu;
+                if (p >= 0) {
+                    local_terms<D>(s.recs[p], ch, cl, toff, tr, s.gf, L);
+                    ck = min(okey(L.q - ((L.wh - r0h) + (L.wl - r0l))), 0xfffffffeu);
+                }
+                const unsigned cm = __reduce_min_sync(full, ck);
+                const int who = (int)__reduce_min_sync(full, ck == cm && p >= 0 ? (unsigned)p : 0x7fffffffu);
+                if (cm < best || (cm == best && who < best_pos)) {
+                    best = cm;
+                    best_pos = who;
+                    if (p == who && p >= 0) store_local<D>(sm.ref[wid], L, s.perm ? s.perm[p] : p);
+                }
+            }
+            __syncwarp();
+            Local<D> R;
+            int ref_id = 0;
+            if (best != 0xffffffffu) load_local<D>(sm.ref[wid], R, ref_id);
+            // counted first (the pool is taken in one piece), then stored
+            auto test = [&](int c, Diff<D> &F) -> bool {
+                const int p = source(c);
+                if (p < 0 || p == best_pos) return false;
+                local_terms<D>(s.recs[p], ch, cl, toff, tr, s.gf, L);
+                difference<D>(L, R, F);
+                return can_win<D>(F, tr);
+            };
+            unsigned keep_bits = 0u;  // of the first 32 chunks
+            unsigned count = 0u;
+            float Emax = 0.f;
+            for (int c = 0; c < n_src; ++c) {
+                Diff<D> F;
+                const bool keep = test(c, F);
+                if (keep) Emax = fmaxf(Emax, F.E);
+                if (keep && c < 32) keep_bits |= 1u << c;
+                count += (unsigned)__popc(__ballot_sync(full, keep));
+            }
+            Emax = __uint_as_float(__reduce_max_sync(full, __float_as_uint(Emax)));
+            unsigned first = 0u;
+            if (lane == 0 && count) first = atomicAdd(&geo->pool, count);
+            first = __shfl_sync(full, first, 0);
+            const bool fits = best != 0xffffffffu && first <= pool_cap && count <= pool_cap - first;
+            if (lane == 0) {
+                TileHead h;
+                h.gap = 2.f * Emax;
+                h.ref = fits ? ref_id : -1;
+                h.first = first;
+                h.count = count;
+                heads[(size_t)ti[0] + (size_t)geo->t[0] * ((size_t)ti[1] + (size_t)geo->t[1] * (size_t)ti[2])] = h;
+            }
+            if (fits && count) {
+                unsigned at = first;
+                for (int c = 0; c < n_src; ++c) {
+                    const bool maybe = c >= 32 || ((keep_bits >> c) & 1u);
+                    if (!__any_sync(full, maybe)) continue;
+                    Diff<D> F;
+                    const bool keep = maybe && test(c, F);
+                    const unsigned km = __ballot_sync(full, keep);
+                    if (keep) {
+                        const int p = source(c);
+                        const int id = s.perm ? s.perm[p] : p;
+                        float4 *o = polys + (size_t)(at + (unsigned)__popc(km & ((1u << lane) - 1u))) * PV;
+                        o[0] = make_float4(F.d0, F.g[0], F.g[1], D == 3 ? F.g[D - 1] : __int_as_float(id));
+                        if (D == 3) {
+                            o[1] = make_float4(F.a[0], 2.f * F.a[1], 2.f * F.a[2], F.a[NP - 3]);
+                            o[2] = make_float4(2.f * F.a[NP - 2], F.a[NP - 1], __int_as_float(id), 0.f);
+                        } else {
+                            o[1] = make_float4(F.a[0], 2.f * F.a[1], F.a[2], 0.f);
+                        }
+                    }
+                    at += (unsigned)__popc(km);
+                }
+            }
+        }
+        __syncthreads();  // the list is read until here
+    }
+}
+
+// Labels and moments from the tiles' lists.
+template <int D>
+__global__ void __launch_bounds__(kPtThreads)
+    points_score_kernel(const long long count, const double *__restrict__ y, const double *__restrict__ mass,
+                        const int n, const double *__restrict__ x, const double *__restrict__ A,
+                        const double *__restrict__ w, const SeedRec32 *__restrict__ r32, const PtsGeo *__restrict__ geo,
+                        const TileHead *__restrict__ heads, const float4 *__restrict__ polys,
+                        DevScalars *__restrict__ sc, double *__restrict__ mom, int32_t *__restrict__ labels) {
+    constexpr int PV = D == 3 ? 3 : 2;
+    __shared__ PtsGeo ge;
+    for (int i = threadIdx.x; i < (int)(sizeof(PtsGeo) / 4); i += kPtThreads)
+        reinterpret_cast<int *>(&ge)[i] = reinterpret_cast<const int *>(geo)[i];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const float finf = __int_as_float(0x7f800000);
+    for (long long j0 = (long long)blockIdx.x * kPtThreads; j0 < count; j0 += (long long)gridDim.x * kPtThreads) {
+        const long long j = j0 + threadIdx.x;
+        const bool active = j < count;
+        double yy[D];
+        float yh[3] = {0.f, 0.f, 0.f}, yl[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
+        size_t tile = 0;
+        bool inside = active;
+#pragma unroll
+        for (int a = D - 1; a >= 0; --a) {
+            yy[a] = active ? y[j * D + a] : 0.0;
+            split_trunc(yy[a], yh[a], yl[a]);
+            const float d = (yh[a] - ge.gf.loh[a]) + yl[a];
+            const int t = min(max((int)(d * ge.inv[a]), 0), ge.t[a] - 1);
+            float ch, cl;
+            axis_point(ge.gf, a, 2 * t + 1, ch, cl);
+            e[a] = (yh[a] - ch) + (yl[a] - cl);
+            inside = inside && fabsf(e[a]) <= ge.r[a];  // false for a NaN
+            tile = tile * (size_t)ge.t[a] + (size_t)t;
+        }
+        const double mj = active ? mass[j] : 0.0;
+        TileHead h{0.f, -1, 0u, 0u};
+        if (inside) h = heads[tile];
+        const bool listed = h.ref >= 0;
+        auto value = [&](unsigned k, int &id) -> float {
+            const float4 *o = polys + (size_t)(h.first + k) * PV;
+            const float4 v0 = o[0], v1 = o[1];
+            if (D == 3) {
+                const float4 v2 = o[2];
+                id = __float_as_int(v2.z);
+                const float b = fmaf(v1.z, e[2], fmaf(v1.y, e[1], v0.y));
+                const float t1 = fmaf(v2.x, e[2], fmaf(v1.w, e[1], v0.z));
+                const float t2 = fmaf(v2.y, e[2], v0.w);
+                return fmaf(fmaf(v1.x, e[0], b), e[0], fmaf(e[2], t2, fmaf(e[1], t1, v0.x)));
+            }
+            id = __float_as_int(v0.w);
+            return fmaf(fmaf(v1.x, e[0], fmaf(v1.y, e[1], v0.y)), e[0], fmaf(e[1], fmaf(v1.z, e[1], v0.z), v0.x));
+        };
+        int bi = h.ref;
+        if (listed) {
+            float v1 = 0.f, v2 = finf;
+            for (unsigned k = 0; k < h.count; ++k) {
+                int id;
+                const float v = value(k, id);
+                v2 = fminf(v2, fmaxf(v1, v));
+                bi = v < v1 ? id : bi;
+                v1 = fminf(v1, v);
+            }
+            const float thr = v1 + h.gap;
+            if (!(v2 > thr)) {  // near tie: FP64 among the seeds within the gap
+                double best = __longlong_as_double(0x7ff0000000000000ll);
+                bi = 0x7fffffff;
+                for (int k = -1; k < (int)h.count; ++k) {
+                    int id = h.ref;
+                    const float v = k < 0 ? 0.f : value((unsigned)k, id);
+                    if (v > thr) continue;
+                    const double c = cost64<D>(yy, x + (size_t)id * D, A + (size_t)id * D * D, w[id]);
+                    if (c < best || (c == best && id < bi)) {
+                        best = c;
+                        bi = id;
+                    }
+                }
+            }
+        }
+        // points without a list, a warp per point: both passes over every seed
+        unsigned todo = __ballot_sync(full, active && !listed);
+        while (todo) {
+            const int p = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            double py[D];
+            float ph[3] = {0.f, 0.f, 0.f}, pl[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                py[a] = __shfl_sync(full, yy[a], p);
+                split_f32(py[a], ph[a], pl[a]);
+            }
+            const float wrh = sc->wref_h, wrl = sc->wref_l;
+            float thr = finf;
+            for (int s = lane; s < n; s += 32) {
+                float c, E;
+                cost32_bound<D>(r32[s], ph, pl, wrh, wrl, c, E);
+                thr = fminf(thr, c + E);
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) thr = fminf(thr, __shfl_xor_sync(full, thr, off));
+            double best = __longlong_as_double(0x7ff0000000000000ll);
+            int ib = 0x7fffffff;
+            for (int s = lane; s < n; s += 32) {
+                float c, E;
+                cost32_bound<D>(r32[s], ph, pl, wrh, wrl, c, E);
+                if (!(c - E <= thr)) continue;
+                const double c64 = cost64<D>(py, x + (size_t)s * D, A + (size_t)s * D * D, w[s]);
+                if (c64 < best) {
+                    best = c64;
+                    ib = s;
+                }
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                const double ob = __shfl_xor_sync(full, best, off);
+                const int oi = __shfl_xor_sync(full, ib, off);
+                if (ob < best || (ob == best && oi < ib)) {
+                    best = ob;
+                    ib = oi;
+                }
+            }
+            if (lane == p) bi = ib;
+        }
+        if (!active) continue;
+        if (bi < 0 || bi >= n) {
+            atomicOr(&sc->status, ST_BAD_LABEL);
+            continue;
+        }
+        if (labels) labels[j] = bi;
+        add_point<D>(mom, bi, mj, yy);
+    }
 }
 
 template <int D>
@@ -104,42 +531,74 @@ __global__ void __launch_bounds__(kPtThreads)
             continue;
         }
         if (labels) labels[j] = bi;
-        const double mj = mass[j];
-        double *o = mom + (size_t)bi * K;
-        atomicAdd(&o[0], mj);
-#pragma unroll
-        for (int a = 0; a < D; ++a) atomicAdd(&o[1 + a], mj * yy[a]);
-        int e = 1 + D;
-#pragma unroll
-        for (int a = 0; a < D; ++a)
-#pragma unroll
-            for (int b = a; b < D; ++b) atomicAdd(&o[e++], mj * yy[a] * yy[b]);
+        add_point<D>(mom, bi, mass[j], yy);
     }
+}
+
+template <int D>
+cudaError_t launch_t(long long count, const double *y, const double *mass, int n, const double *x, const double *A,
+                     const double *w, double *mom, int32_t *labels, Workspace &ws, cudaStream_t st) {
+    const long long n_mom = (long long)n * moment_width(D);
+    unsigned long long *m64 = reinterpret_cast<unsigned long long *>(mom);
+    GridDev none{};
+    none.dim = D;
+    none.res[0] = none.res[1] = none.res[2] = 1;
+    none.h32[0] = none.h32[1] = none.h32[2] = 1.f;
+    const bool tiled = points_tiled(count, n, ws);
+    const long long want_blocks = (count + kPtThreads - 1) / kPtThreads;
+    if (tiled) {
+        const int blocks = (int)std::min<long long>(want_blocks, (long long)ws.sms * 8);
+        // about 32 tiles a seed, no more than one per two points or the store holds
+        const long long cap = (long long)(ws.pts_bytes / (sizeof(TileHead) + 8 * 48));
+        const long long tiles = std::max<long long>(1, std::min<long long>(std::min<long long>(32ll * n, count / 2), cap));
+        // the blocks' boxes (24 bytes each) go where the tiles' headers follow
+        points_box_kernel<D><<<blocks, kPtThreads, 0, st>>>(count, y, tiles, reinterpret_cast<unsigned *>(ws.pts_tiles),
+                                                            ws.pts_geo);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        e = launch_seed_prep(none, n, x, A, w, ws, m64, n_mom, st, ws.pts_geo);
+        if (e != cudaSuccess) return e;
+        e = launch_group_bounds(n, ws, st);
+        if (e != cudaSuccess) return e;
+        Src src{};
+        src.n = n;
+        src.n_groups = (n + kGroup - 1) / kGroup;
+        src.recs = ws.sorted ? ws.recs32s : ws.recs32;
+        src.perm = ws.sorted ? ws.perm : nullptr;
+        src.groups = ws.groups;
+        src.sc = ws.sc;
+        TileHead *heads = reinterpret_cast<TileHead *>(ws.pts_tiles);
+        float4 *polys = reinterpret_cast<float4 *>(ws.pts_tiles + ((size_t)tiles * sizeof(TileHead) + 255) / 256 * 256);
+        const size_t rest = ws.pts_bytes - ((size_t)tiles * sizeof(TileHead) + 255) / 256 * 256;
+        const unsigned pool = (unsigned)std::min<size_t>(rest / ((D == 3 ? 3 : 2) * sizeof(float4)), 0x7fffffffu);
+        const int lb = (int)std::min<long long>(4ll * ws.sms, tiles);
+        points_lists_kernel<D><<<lb, kThreads, 0, st>>>(src, ws.pts_geo, heads, polys, pool);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        const int sb = (int)std::min<long long>(want_blocks, (long long)ws.sms * 8);
+        points_score_kernel<D><<<sb, kPtThreads, 0, st>>>(count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, polys,
+                                                          ws.sc, mom, labels);
+        return cudaGetLastError();
+    }
+    cudaError_t e = launch_seed_prep(none, n, x, A, w, ws, m64, n_mom, st);
+    if (e != cudaSuccess) return e;
+    const int blocks = (int)std::min<long long>(want_blocks, (long long)ws.sms * 8);
+    points_assign_kernel<D><<<blocks, kPtThreads, 0, st>>>(count, y, mass, n, x, A, w, ws.recs32, ws.sc, mom, labels);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
+// The tiled form's six launches and lists against two passes over all seeds a point.
+bool points_tiled(long long count, int n, const Workspace &ws) {
+    return ws.groups && ws.pts_tiles && (n + kGroup - 1) / kGroup <= kMaxGroups && count >= 256 && n >= 8;
+}
+
 cudaError_t launch_points_assign(int dim, long long count, const double *y, const double *mass, int n,
                                  const double *x, const double *A, const double *w, double *mom,
                                  int32_t *labels, Workspace &ws, cudaStream_t st) {
-    const int K = moment_width(dim);
-    cudaError_t e = cudaMemsetAsync(mom, 0, (size_t)n * K * sizeof(double), st);
-    if (e != cudaSuccess) return e;
-    e = launch_eval_reset(ws, st, false);
-    if (e != cudaSuccess) return e;
-    const int pb = (n + 255) / 256;
-    if (dim == 3) points_prep_kernel<3><<<pb, 256, 0, st>>>(n, x, A, w, ws.recs32, ws.sc);
-    else points_prep_kernel<2><<<pb, 256, 0, st>>>(n, x, A, w, ws.recs32, ws.sc);
-    const int sms = ws.sms;
-    const long long want = (count + kPtThreads - 1) / kPtThreads;
-    const int blocks = (int)std::min<long long>(want, (long long)sms * 8);
-    if (dim == 3)
-        points_assign_kernel<3><<<blocks, kPtThreads, 0, st>>>(count, y, mass, n, x, A, w, ws.recs32, ws.sc, mom,
-                                                               labels);
-    else
-        points_assign_kernel<2><<<blocks, kPtThreads, 0, st>>>(count, y, mass, n, x, A, w, ws.recs32, ws.sc, mom,
-                                                               labels);
-    return cudaGetLastError();
+    return dim == 3 ? launch_t<3>(count, y, mass, n, x, A, w, mom, labels, ws, st)
+                    : launch_t<2>(count, y, mass, n, x, A, w, mom, labels, ws, st);
 }
 
 }  // namespace apd

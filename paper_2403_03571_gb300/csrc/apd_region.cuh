@@ -430,6 +430,120 @@ __device__ __forceinline__ float group_lower(const GroupBound &gb, const float (
     return __fadd_rd(__fmul_rd(__fmul_rd(gb.lam, d2), 1.f - 1e-5f), gb.wgap);
 }
 
+// The seeds that can be the argmin somewhere in the box of half-widths rr around ch + cl,
+// listed in sm.list by the whole block (two barriers; none follows the last entry's
+// write but the second).  Returns their number, which may exceed kListCap (the list is
+// then incomplete); r0h + r0l is the reference seed's weight.
+template <int D>
+__device__ __forceinline__ unsigned region_list(Shared<D> &sm, const Src &s, const float (&ch)[3], const float (&cl)[3],
+                                                const float (&rr)[3], float &r0h, float &r0l) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned full = 0xffffffffu;
+    const float finf = __int_as_float(0x7f800000);
+    const int n = s.n;
+    float4(&ref)[5] = sm.ref[wid];
+    const float zero3[3] = {0.f, 0.f, 0.f};
+    const float wrh = s.sc->wref_h, wrl = s.sc->wref_l;
+
+    // the groups' lower bounds: warp w takes the groups w, w + 8, ... (one per lane and
+    // round, so that near groups, adjacent in scan order, go to different warps)
+    float glb[2] = {finf, finf};
+    {
+        float alo[3] = {0.f, 0.f, 0.f}, ahi[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            alo[a] = __fsub_rd(ch[a], __fadd_ru(rr[a], fabsf(cl[a])));
+            ahi[a] = __fadd_ru(ch[a], __fadd_ru(rr[a], fabsf(cl[a])));
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            if (s.n_groups <= t * kThreads) break;
+            const int grp = wid + kWarps * (lane + 32 * t);
+            if (grp < s.n_groups) glb[t] = group_lower<D>(s.groups[grp], alo, ahi);
+        }
+    }
+    // each warp's group of least bound, and in it the seed of least cost at the centre
+    // with an upper bound U of its cost over the region (relative to w_ref)
+    {
+        const unsigned k0 = okey(fminf(glb[0], glb[1]));
+        const unsigned kmin = __reduce_min_sync(full, k0);
+        const int src = __ffs(__ballot_sync(full, k0 == kmin)) - 1;
+        const int t = glb[0] <= glb[1] ? 0 : 1;
+        const int grp = wid + kWarps * (src + 32 * __shfl_sync(full, t, src));
+        unsigned ck = 0xffffffffu;
+        const int p = grp * 32 + lane;
+        Local<D> L;
+        float wn = 0.f;
+        const bool have = grp < s.n_groups && p < n;
+        if (have) {
+            local_terms<D>(s.recs[p], ch, cl, zero3, rr, s.gf, L);
+            wn = -((L.wh - wrh) + (L.wl - wrl));
+            ck = min(okey(L.q + wn), 0xfffffffeu);
+        }
+        const unsigned cm = __reduce_min_sync(full, ck);
+        const int who = __ffs(__ballot_sync(full, ck == cm)) - 1;
+        if (lane == who) {
+            sm.key[wid] = cm;
+            sm.pos[wid] = have ? p : 0;
+            if (have) {
+                float v = L.q + 1e-5f * (L.S + fabsf(wn)) + 1e-30f;
+#pragma unroll
+                for (int a = 0; a < D; ++a) {
+                    v += 2.f * fabsf(L.h[a]) * rr[a];
+#pragma unroll
+                    for (int b = 0; b < D; ++b) v += fabsf(L.a[tri<D>(a < b ? a : b, a < b ? b : a)]) * rr[a] * rr[b];
+                }
+                store_local<D>(ref, L, p);
+                ref[4].x = v + wn + 1e-5f * (fabsf(v) + fabsf(wn)) + 1e-13f * fabsf(L.wh);
+            }
+        }
+    }
+    if (tid == 0) {
+        sm.count = 0u;
+    }
+    __syncthreads();
+    Local<D> R;
+    int a0;
+    float U;
+    {
+        const unsigned k = lane < kWarps ? sm.key[lane] : 0xffffffffu;
+        const unsigned km = __reduce_min_sync(full, k);
+        const int w = __ffs(__ballot_sync(full, lane < kWarps && k == km)) - 1;
+        load_local<D>(sm.ref[w], R, a0);
+        U = sm.ref[w][4].x;
+    }
+    r0h = R.wh;
+    r0l = R.wl;
+    // the seeds that can win somewhere in the region against a0
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        if (s.n_groups <= t * kThreads) break;
+        unsigned m = __ballot_sync(full, !(glb[t] > U) && wid + kWarps * (lane + 32 * t) < s.n_groups);
+        while (m) {
+            const int gl = __ffs(m) - 1;
+            m &= m - 1u;
+            const int p = (wid + kWarps * (gl + 32 * t)) * 32 + lane;
+            bool keep = false;
+            if (p < n) {
+                Local<D> L;
+                Diff<D> F;
+                local_terms<D>(s.recs[p], ch, cl, zero3, rr, s.gf, L);
+                difference<D>(L, R, F);
+                keep = p == a0 || can_win<D>(F, rr);
+            }
+            const unsigned km = __ballot_sync(full, keep);
+            if (km) {
+                unsigned at = 0u;
+                if (lane == 0) at = atomicAdd(&sm.count, (unsigned)__popc(km));
+                at = __shfl_sync(full, at, 0) + (unsigned)__popc(km & ((1u << lane) - 1u));
+                if (keep && at < (unsigned)kListCap) sm.list[at] = (uint16_t)p;
+            }
+        }
+    }
+    __syncthreads();
+    return sm.count;
+}
+
 // Scores region (bx, by, bz); `s` is the same in every thread.  The caller puts a
 // barrier between the previous region and the next.
 template <int D, bool MASKED = false>
@@ -518,111 +632,16 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
             cl[a] = __shfl_sync(full, l, a);
         }
     }
-    const float zero3[3] = {0.f, 0.f, 0.f};
     float rr[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int a = 0; a < D; ++a)
         rr[a] = __fmul_ru(__fmul_ru(0.5f * (float)(rdim[a] - 1), g.h32[a]), 1.f + 0x1p-22f);
-    const float wrh = s.sc->wref_h, wrl = s.sc->wref_l;
-
-    // the groups' lower bounds: warp w takes the groups w, w + 8, ... (one per lane and
-    // round, so that near groups, adjacent in scan order, go to different warps)
-    float glb[2] = {finf, finf};
-    {
-        float alo[3] = {0.f, 0.f, 0.f}, ahi[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            alo[a] = __fsub_rd(ch[a], __fadd_ru(rr[a], fabsf(cl[a])));
-            ahi[a] = __fadd_ru(ch[a], __fadd_ru(rr[a], fabsf(cl[a])));
-        }
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            if (s.n_groups <= t * kThreads) break;
-            const int grp = wid + kWarps * (lane + 32 * t);
-            if (grp < s.n_groups) glb[t] = group_lower<D>(s.groups[grp], alo, ahi);
-        }
-    }
-    // each warp's group of least bound, and in it the seed of least cost at the centre
-    // with an upper bound U of its cost over the region (relative to w_ref)
-    {
-        const unsigned k0 = okey(fminf(glb[0], glb[1]));
-        const unsigned kmin = __reduce_min_sync(full, k0);
-        const int src = __ffs(__ballot_sync(full, k0 == kmin)) - 1;
-        const int t = glb[0] <= glb[1] ? 0 : 1;
-        const int grp = wid + kWarps * (src + 32 * __shfl_sync(full, t, src));
-        unsigned ck = 0xffffffffu;
-        const int p = grp * 32 + lane;
-        Local<D> L;
-        float wn = 0.f;
-        const bool have = grp < s.n_groups && p < n;
-        if (have) {
-            local_terms<D>(s.recs[p], ch, cl, zero3, rr, s.gf, L);
-            wn = -((L.wh - wrh) + (L.wl - wrl));
-            ck = min(okey(L.q + wn), 0xfffffffeu);
-        }
-        const unsigned cm = __reduce_min_sync(full, ck);
-        const int who = __ffs(__ballot_sync(full, ck == cm)) - 1;
-        if (lane == who) {
-            sm.key[wid] = cm;
-            sm.pos[wid] = have ? p : 0;
-            if (have) {
-                float v = L.q + 1e-5f * (L.S + fabsf(wn)) + 1e-30f;
-#pragma unroll
-                for (int a = 0; a < D; ++a) {
-                    v += 2.f * fabsf(L.h[a]) * rr[a];
-#pragma unroll
-                    for (int b = 0; b < D; ++b) v += fabsf(L.a[tri<D>(a < b ? a : b, a < b ? b : a)]) * rr[a] * rr[b];
-                }
-                store_local<D>(ref, L, p);
-                ref[4].x = v + wn + 1e-5f * (fabsf(v) + fabsf(wn)) + 1e-13f * fabsf(L.wh);
-            }
-        }
-    }
     if (tid == 0) {
-        sm.count = 0u;
         sm.pairs = 0u;
         sm.queued = 0u;
     }
-    __syncthreads();
-    Local<D> R;  // the region's reference, later the tile's
-    int a0;
-    float U;
-    {
-        const unsigned k = lane < kWarps ? sm.key[lane] : 0xffffffffu;
-        const unsigned km = __reduce_min_sync(full, k);
-        const int w = __ffs(__ballot_sync(full, lane < kWarps && k == km)) - 1;
-        load_local<D>(sm.ref[w], R, a0);
-        U = sm.ref[w][4].x;
-    }
-    const float r0h = R.wh, r0l = R.wl;
-    // the seeds that can win somewhere in the region against a0
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        if (s.n_groups <= t * kThreads) break;
-        unsigned m = __ballot_sync(full, !(glb[t] > U) && wid + kWarps * (lane + 32 * t) < s.n_groups);
-        while (m) {
-            const int gl = __ffs(m) - 1;
-            m &= m - 1u;
-            const int p = (wid + kWarps * (gl + 32 * t)) * 32 + lane;
-            bool keep = false;
-            if (p < n) {
-                Local<D> L;
-                Diff<D> F;
-                local_terms<D>(s.recs[p], ch, cl, zero3, rr, s.gf, L);
-                difference<D>(L, R, F);
-                keep = p == a0 || can_win<D>(F, rr);
-            }
-            const unsigned km = __ballot_sync(full, keep);
-            if (km) {
-                unsigned at = 0u;
-                if (lane == 0) at = atomicAdd(&sm.count, (unsigned)__popc(km));
-                at = __shfl_sync(full, at, 0) + (unsigned)__popc(km & ((1u << lane) - 1u));
-                if (keep && at < (unsigned)kListCap) sm.list[at] = (uint16_t)p;
-            }
-        }
-    }
-    __syncthreads();
-    const unsigned total = sm.count;
+    float r0h, r0l;
+    const unsigned total = region_list<D>(sm, s, ch, cl, rr, r0h, r0l);
     const bool scan = total > (unsigned)kListCap;  // too many: the tiles take every group
     const int n_src = scan ? s.n_groups : (int)((total + 31u) / 32u);
     auto source = [&](int c) -> int {  // scan position of candidate `lane` of chunk c (-1: none)
@@ -659,6 +678,7 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
         return;
     }
     __syncwarp();
+    Local<D> R;
     int ref_id;
     load_local<D>(ref, R, ref_id);
 
