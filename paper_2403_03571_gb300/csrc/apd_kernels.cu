@@ -290,23 +290,32 @@ __global__ void seed_prep_kernel(const GridDev g, const int n, const int n_pad,
 // all SMs instead of a sort in one block (10^4 seeds: 190 us with the gather -> 12 us;
 // 1000 seeds: 17 -> 4 us); the order is the same, by (code, index).
 constexpr int kRankThreads = 256;
+constexpr int kRankPiece = 4096;
 __global__ void __launch_bounds__(kRankThreads)
     rank_kernel(const int n, const uint32_t *__restrict__ codes, uint32_t *__restrict__ scodes,
                 int32_t *__restrict__ perm, const SeedRec *__restrict__ src, SeedRec *__restrict__ dst,
                 const SeedRec32 *__restrict__ src32, SeedRec32 *__restrict__ dst32, const int n_pad) {
+    __shared__ uint4 piece[kRankPiece / 4];
     __shared__ int part[kRankThreads / 32][32];
     __shared__ int rank[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 32, i = i0 + lane;
     const uint32_t ci = codes[i];
-    const int len = n_pad / (kRankThreads / 32);  // a multiple of 32
+    // the codes in pieces of 4096 through shared memory; warp w counts an eighth of each
     int below = 0;
-    if (i0 < n) {
-        const int j1 = min((wid + 1) * len, n);
-        const uint4 *c4 = reinterpret_cast<const uint4 *>(codes);
+    for (int base = 0; base < n; base += kRankPiece) {
+        const int m = min(kRankPiece, n_pad - base);  // a multiple of 256
+        __syncthreads();
+        for (int e = threadIdx.x; e < m / 4; e += kRankThreads)
+            piece[e] = reinterpret_cast<const uint4 *>(codes + base)[e];
+        __syncthreads();
+        if (i0 >= n) continue;
+        const int len = m / (kRankThreads / 32);
+        int j = base + wid * len;
+        const uint4 *c4 = piece + (wid * len >> 2);
 #pragma unroll 4
-        for (int j = wid * len; j < j1; j += 4) {  // padding codes count for no seed
-            const uint4 c = c4[j >> 2];
+        for (int e = 0; e < len / 4; ++e, j += 4) {  // padding codes count for no seed
+            const uint4 c = c4[e];
             if (j + 4 <= i0) {
                 below += (c.x <= ci) + (c.y <= ci) + (c.z <= ci) + (c.w <= ci);
             } else if (j >= i0 + 32) {

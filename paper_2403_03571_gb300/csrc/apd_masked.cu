@@ -107,7 +107,7 @@ __device__ __forceinline__ void block_moments(const int (&K)[3], unsigned long l
 }
 
 // Mask for the region scorer, a warp per run of 32 coarse pixels of a row: the
-// boundary pixels' bytes, the fine regions they reach (each listed once, by its bit),
+// boundary pixels' bytes, the fine regions they reach (each listed once, by its word),
 // and the interior pixels' fine moments.  A run's label sums need one packed reduction
 // (sum x, sum x^2 of 0 .. 31; the count is a ballot), and lane v forms word v: with
 // coarse sums N, X_a, X_ab of U the fine words are r^D N, r^(D+1) X_a and
@@ -156,17 +156,22 @@ __global__ void __launch_bounds__(kMaskThreads)
         if (act && !valid) atomicOr(&sc->status, ST_BAD_LABEL);
         const bool boundary = valid && differs;
         if (act) mask[j] = boundary ? 1 : 0;
-        const unsigned bm = __ballot_sync(full, boundary);
+        const unsigned bm = __ballot_sync(full, boundary);  // mark, list, count
         boundary_count += (unsigned)__popc(bm);
-        if (boundary) {  // the fine regions of its r^D pixels
-            const int f[3] = {x * r, kb[1] * r, kb[2] * r};
+        // the fine regions of its r^D pixels; a lane whose left neighbour reaches the same
+        // ones leaves them to it (all boundary lanes at once on the same few words cost
+        // 150 us at 128^3)
+        const int f[3] = {x * r, kb[1] * r, kb[2] * r};
+        const int xa = f[0] / rdim.x, xz = (f[0] + r - 1) / rdim.x;
+        const int pa = __shfl_up_sync(full, xa, 1), pz = __shfl_up_sync(full, xz, 1);
+        const bool same = lane > 0 && pa == xa && pz == xz && ((bm >> ((lane + 31) & 31)) & 1u);
+        if (boundary && !same) {
             for (int z = D == 3 ? f[2] / rdim.z : 0; z <= (D == 3 ? (f[2] + r - 1) / rdim.z : 0); ++z)
                 for (int y = f[1] / rdim.y; y <= (f[1] + r - 1) / rdim.y; ++y)
-                    for (int a = f[0] / rdim.x; a <= (f[0] + r - 1) / rdim.x; ++a) {
-                        const unsigned id = (unsigned)a + (unsigned)regions.x * ((unsigned)y + (unsigned)regions.y * (unsigned)z);
-                        const unsigned bit = 1u << (id & 31u);
-                        if (*(volatile unsigned *)&seen[id >> 5] & bit) continue;
-                        if (!(atomicOr(&seen[id >> 5], bit) & bit)) list[atomicAdd(&sc->mask_regions, 1u)] = (int32_t)id;
+                    for (int c = xa; c <= xz; ++c) {
+                        const int id = c + regions.x * (y + regions.y * z);
+                        if (*(volatile unsigned *)&seen[id]) continue;
+                        if (!atomicExch(&seen[id], 1u)) list[atomicAdd(&sc->mask_regions, 1u)] = id;
                     }
         }
         unsigned todo = __ballot_sync(full, valid && !differs);
@@ -342,10 +347,8 @@ cudaError_t launch_masked_refine(const GridDev &gc, const GridDev &gf, int r, in
     e = cudaMemsetAsync(&ws.sc->mask_count, 0, 2 * sizeof(unsigned int), st);
     if (e != cudaSuccess) return e;
     const int sms = ws.sms;
-    // Region lists on the fine grid: the mask bytes and the listed regions' bits take the
-    // pixel queue's first 5 J / 4 + 4 bytes (of 4 J), the list the hints' buffer.  A coarse pixel
-    // reaches at most two regions per axis while r <= 16, and the regions are no more than the
-    // coarse pixels.
+    // Region lists on the fine grid: the mask bytes and a word per region take the pixel
+    // queue's buffer (J words for the J coarse pixels), the list of regions the hints'.
     int rd[3];
     region_dims(gc.dim, rd);
     long long regions = 1;
@@ -354,10 +357,10 @@ cudaError_t launch_masked_refine(const GridDev &gc, const GridDev &gf, int r, in
     nr.y = (gf.res[1] + rd[1] - 1) / rd[1];
     if (gc.dim == 3) nr.z = (gf.res[2] + rd[2] - 1) / rd[2];
     regions = (long long)nr.x * nr.y * nr.z;
-    if (region_lists(gf, n, ws) && r <= 16 && regions <= gc.J && ws.flag_gi && gc.J >= 64) {
+    if (region_lists(gf, n, ws) && r <= 16 && regions <= gc.J / 2 && ws.flag_gi && gc.J >= 64) {
         uint8_t *mask = reinterpret_cast<uint8_t *>(ws.flags);
         unsigned *seen = ws.flags + (gc.J + 3) / 4;
-        e = cudaMemsetAsync(seen, 0, (size_t)((regions + 31) / 32) * sizeof(unsigned), st);
+        e = cudaMemsetAsync(seen, 0, (size_t)regions * sizeof(unsigned), st);
         if (e != cudaSuccess) return e;
         const int nx = (gc.res[0] + 31) / 32;
         const long long runs = (long long)nx * gc.res[1] * gc.res[2];

@@ -15,8 +15,11 @@
 //   points_score_kernel  labels and moments
 // Bounds: the scoring kernel reads 32 (2D: 24) bytes a point from memory, a 16-byte
 // header and about three 48-byte polynomials a point from L2, issues nine FP64
-// products a point (16 clocks of an SM per warp each) and ten FP64 reductions.
-// 1000 seeds, 4 M random points in 3D: 13.6 ms for the direct form below -> MEASURED.
+// products a point (16 clocks of an SM per warp each) and ten FP64 additions to the
+// cell's words, which are what it waits for (in shared memory 275 us per 4 M points, as
+// global reductions 610 us).  1000 seeds, 4 M random points in 3D: the call took
+// 13.6 ms with the direct form below and takes 0.41 ms (box 26, preparation 21, lists
+// 81, scoring 275 us).
 //
 // Direct form (few seeds or points, or more seeds than region lists take): the seeds
 // stream through shared memory in chunks of
@@ -44,6 +47,7 @@ using namespace region;
 
 constexpr int kPtThreads = 256;
 constexpr int kMaxTiles = 1024;  // per axis
+constexpr size_t kPtShared = 200 * 1024;  // block sums of the moments
 
 // One tile: 2 max E of its list, the reference seed (natural index; -1: no list, the
 // points are searched in full), where its polynomials start and how many there are.
@@ -53,21 +57,25 @@ struct TileHead {
     unsigned first, count;
 };
 
-// Adds one point to its cell's moments.
+// The moment words of one point, and their addition to its cell.
 template <int D>
-__device__ __forceinline__ void add_point(double *__restrict__ mom, int label, double mj, const double (&yy)[D]) {
-    double *o = mom + (size_t)label * moment_width(D);
-    atomicAdd(&o[0], mj);
+__device__ __forceinline__ void point_words(double mj, const double (&yy)[D], double (&v)[moment_width(D)]) {
+    v[0] = mj;
+    int e = 1 + D;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        const double m = mj * yy[a];
-        atomicAdd(&o[1 + a], m);
-        int e = 1 + D;
+        v[1 + a] = mj * yy[a];
 #pragma unroll
-        for (int c = 0; c < a; ++c) e += D - c;
-#pragma unroll
-        for (int b = a; b < D; ++b) atomicAdd(&o[e + b - a], m * yy[b]);
+        for (int b = a; b < D; ++b) v[e++] = v[1 + a] * yy[b];
     }
+}
+template <int D>
+__device__ __forceinline__ void add_point(double *mom, int label, double mj, const double (&yy)[D]) {
+    double v[moment_width(D)];
+    point_words<D>(mj, yy, v);
+    double *o = mom + (size_t)label * moment_width(D);
+#pragma unroll
+    for (int k = 0; k < moment_width(D); ++k) atomicAdd(&o[k], v[k]);
 }
 
 // High and low FP32 parts of a double by integer operations (the FP64 pipe converts a
@@ -337,23 +345,29 @@ __global__ void __launch_bounds__(kThreads, 4)
     }
 }
 
-// Labels and moments from the tiles' lists.
-template <int D>
-__global__ void __launch_bounds__(kPtThreads)
+// Labels and moments from the tiles' lists.  SHARED: the block sums its moments in
+// shared memory (n K doubles) and adds them to the global ones at the end; a warp whose
+// points lie in one cell sums them first.
+template <int D, bool SHARED, int T>
+__global__ void __launch_bounds__(T)
     points_score_kernel(const long long count, const double *__restrict__ y, const double *__restrict__ mass,
                         const int n, const double *__restrict__ x, const double *__restrict__ A,
                         const double *__restrict__ w, const SeedRec32 *__restrict__ r32, const PtsGeo *__restrict__ geo,
                         const TileHead *__restrict__ heads, const float4 *__restrict__ polys,
                         DevScalars *__restrict__ sc, double *__restrict__ mom, int32_t *__restrict__ labels) {
     constexpr int PV = D == 3 ? 3 : 2;
+    constexpr int K = moment_width(D);
     __shared__ PtsGeo ge;
-    for (int i = threadIdx.x; i < (int)(sizeof(PtsGeo) / 4); i += kPtThreads)
+    extern __shared__ double acc[];
+    for (int i = threadIdx.x; i < (int)(sizeof(PtsGeo) / 4); i += T)
         reinterpret_cast<int *>(&ge)[i] = reinterpret_cast<const int *>(geo)[i];
+    if (SHARED)
+        for (int i = threadIdx.x; i < n * K; i += T) acc[i] = 0.0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
     const float finf = __int_as_float(0x7f800000);
-    for (long long j0 = (long long)blockIdx.x * kPtThreads; j0 < count; j0 += (long long)gridDim.x * kPtThreads) {
+    for (long long j0 = (long long)blockIdx.x * T; j0 < count; j0 += (long long)gridDim.x * T) {
         const long long j = j0 + threadIdx.x;
         const bool active = j < count;
         double yy[D];
@@ -460,13 +474,28 @@ __global__ void __launch_bounds__(kPtThreads)
             }
             if (lane == p) bi = ib;
         }
-        if (!active) continue;
-        if (bi < 0 || bi >= n) {
-            atomicOr(&sc->status, ST_BAD_LABEL);
-            continue;
+        const bool good = active && bi >= 0 && bi < n;
+        if (active && !good) atomicOr(&sc->status, ST_BAD_LABEL);
+        if (good && labels) labels[j] = bi;
+        if (SHARED) {
+            const int b0 = __shfl_sync(full, bi, 0);
+            if (__all_sync(full, good && bi == b0)) {  // points in spatial order: one cell
+                double v[K];
+                point_words<D>(mj, yy, v);
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const double t = warp_sum(v[k]);
+                    if (lane == 0) atomicAdd(&acc[(size_t)b0 * K + k], t);
+                }
+                continue;
+            }
         }
-        if (labels) labels[j] = bi;
-        add_point<D>(mom, bi, mj, yy);
+        if (good) add_point<D>(SHARED ? acc : mom, bi, mj, yy);
+    }
+    if (SHARED) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < n * K; i += T)
+            if (acc[i] != 0.0) atomicAdd(&mom[i], acc[i]);
     }
 }
 
@@ -575,9 +604,26 @@ cudaError_t launch_t(long long count, const double *y, const double *mass, int n
         points_lists_kernel<D><<<lb, kThreads, 0, st>>>(src, ws.pts_geo, heads, polys, pool);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        const int sb = (int)std::min<long long>(want_blocks, (long long)ws.sms * 8);
-        points_score_kernel<D><<<sb, kPtThreads, 0, st>>>(count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, polys,
-                                                          ws.sc, mom, labels);
+        // block sums where n K doubles fit (one block of 1024 per SM) and a block gets
+        // several points per word it then adds to the global moments
+        const size_t smem = (size_t)n_mom * sizeof(double);
+        if (smem <= kPtShared && count >= 4ll * ws.sms * n) {
+            constexpr int T = 1024;
+            constexpr unsigned bit = D == 3 ? kAttrPoints3 : kAttrPoints2;
+            if (!(ws.attr_done & bit)) {
+                e = cudaFuncSetAttribute(points_score_kernel<D, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kPtShared);
+                if (e != cudaSuccess) return e;
+                ws.attr_done |= bit;
+            }
+            const int per_sm = smem <= kPtShared / 2 ? 2 : 1;
+            points_score_kernel<D, true, T><<<per_sm * ws.sms, T, smem, st>>>(
+                count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, polys, ws.sc, mom, labels);
+        } else {
+            const int sb = (int)std::min<long long>(want_blocks, (long long)ws.sms * 8);
+            points_score_kernel<D, false, kPtThreads><<<sb, kPtThreads, 0, st>>>(
+                count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, polys, ws.sc, mom, labels);
+        }
         return cudaGetLastError();
     }
     cudaError_t e = launch_seed_prep(none, n, x, A, w, ws, m64, n_mom, st);
