@@ -414,10 +414,11 @@ void apd_batch_destroy(apd_batch *batch);
 int apd_batch_tile_info(apd_batch *batch, int32_t *tile, int32_t *n_variants, double *ms,
                         int32_t *shape);
 
-/* Seed-group pruning of the batch's FP32 scoring, as apd_workspace_set_pruning. */
+/* Seed pruning of the batch's scoring, as apd_workspace_set_pruning (with it no tile
+ * shape is timed or used while every instance has at most 16384 seeds). */
 int apd_batch_set_pruning(apd_batch *batch, int32_t enable);
 
-/* Kernels this batch has launched (graph replays count their six kernels). */
+/* Kernels this batch has launched (graph replays count theirs). */
 int64_t apd_batch_kernel_launches(apd_batch *batch);
 
 /* One evaluation of every instance at weights w: moments int64 device

@@ -2,17 +2,22 @@
 // dimension, each with its own grid and seed count, solved together.
 //
 // One iteration evaluates the dual of every unconverged instance and advances
-// its solver by one step, with six launches whatever the instance count:
+// its solver by one step, with a few launches whatever the instance count:
 //   schedule  (1 CTA)        list the active instances, prefix-sum their tiles
-//   prep      (CTA/instance) seed records at the trial weights, Morton sort
+//   regions   (persistent)   pruning on: (instance, region) items scored from candidate
+//                            lists (apd_region.cuh), near ties included; or
 //   assign    (persistent)   one CTA per SM slot pulls (instance, tile) items
 //                            from a shared queue, heaviest instances first, and
 //                            scores each tile with the FP32 tile routine of the
-//                            one-instance path (Algorithm 1 fused with moments)
-//   rescore   (CTAs/instance) FP64 near-tie rescoring
-//   dual      (CTA/instance) eqs. (2.7)-(2.8) from the integer moments
-//   lbfgs     (CTA/instance) one transition of the L-BFGS / strong-Wolfe state
-//                            machine of Algorithm 2, writing the next trial point
+//                            one-instance path (Algorithm 1 fused with moments), then
+//   rescore   (persistent)   FP64 near-tie rescoring
+//   cells     (thread/cell)  the per-cell terms of eqs. (2.7)-(2.8) from the moments
+//   lbfgs     (CTA/instance) their sums, one transition of the L-BFGS / strong-Wolfe
+//                            state machine of Algorithm 2, the next trial point and its
+//                            weights in the seed records
+// The records' positions and matrices are made by one prep launch (CTA/instance) before
+// a solve's first iteration; rebuilding them every iteration took 94 of about 900 us
+// (48 diagrams, mean 530 seeds), the terms a CTA per instance 40 us.
 // The iteration is captured once in a CUDA graph and replayed until no
 // instance is active.  The tile shape of the persistent kernel is picked per
 // batch by timing every compiled variant on the batch itself (autotune).
@@ -27,6 +32,7 @@
 #include "apd_common.cuh"
 #include "apd_cost.cuh"
 #include "apd_fp32_tile.cuh"
+#include "apd_region.cuh"
 
 namespace apd {
 namespace {
@@ -116,6 +122,9 @@ struct BArgs {             // everything the per-iteration kernels touch
     unsigned long long *mom;  // [total_n][K]
     uint32_t *flags;
     int32_t *flag_gi;            // FP32 best seed of each queued pixel
+    const int32_t *inst_of;      // [total_n] instance of each seed row
+    double *Q, *err;             // [total_n] per-cell terms of the last evaluation
+    const region::Src *srcs;     // [count] region form: the instances' scoring problems
 };
 
 __device__ __forceinline__ int map_bits_dev(int bits) {
@@ -238,6 +247,7 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __grid_c
         }
         sc->flag_count = 0u;
         sc->wref_key = dkey(shw[0]);
+        split_f32(shw[0], sc->wref_h, sc->wref_l);
         sc->lam_abs_bits = (unsigned long long)__double_as_longlong(shf[0]);
         sc->lam_min_bits = (unsigned long long)__double_as_longlong(shl[0]);
     }
@@ -318,6 +328,37 @@ __global__ void __launch_bounds__(TX *TY *TZ, MINB) batch_assign_kernel(const __
     }
 }
 
+// Pruned form: regions of all active instances, item by item, from candidate lists.
+template <int D>
+__global__ void __launch_bounds__(region::kThreads, 4) batch_region_kernel(const __grid_constant__ BArgs a) {
+    __shared__ region::Shared<D> sm;
+    __shared__ region::Src cur;
+    region::init_shared<D>(sm);
+    const unsigned total = a.sched->total_items;
+    const int n_act = a.sched->n_active;
+    for (unsigned item = blockIdx.x; item < total; item += gridDim.x) {
+        int lo = 0, hi = n_act - 1;  // last k with act_start[k] <= item
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.act_start[mid] <= item) lo = mid;
+            else hi = mid - 1;
+        }
+        const int b = a.act_list[lo];
+        const int *src = reinterpret_cast<const int *>(a.srcs + b);
+        for (int i = threadIdx.x; i < (int)(sizeof(region::Src) / 4); i += region::kThreads)
+            reinterpret_cast<int *>(&cur)[i] = src[i];
+        const BInst &I = a.inst[b];
+        const unsigned local = item - a.act_start[lo];
+        const int bx = (int)(local % (unsigned)I.tiles_x);
+        const unsigned rest = local / (unsigned)I.tiles_x;
+        const int by = (int)(rest % (unsigned)I.tiles_y), bz = (int)(rest / (unsigned)I.tiles_y);
+        __syncthreads();
+        region::score_region<D>(sm, cur, bx, by, bz);
+        __syncthreads();
+        if (threadIdx.x == 0 && sm.queued) atomicAdd(&cur.sc->flag_count, sm.queued);
+    }
+}
+
 // Near-tie rescoring of the queued pixels of all active instances: every warp
 // pulls pixels (4 at a time) from one queue over the concatenated per-instance
 // queues, so an instance with many queued pixels is spread over the whole GPU.
@@ -364,56 +405,26 @@ __global__ void __launch_bounds__(256) batch_rescore_kernel(const __grid_constan
     }
 }
 
-// eqs. (2.7)-(2.8) per instance; writes grad f = -(v - m|P|) into gft and the
-// scalars (g~, max relative error, <grad f, p>, sum v, min v) into the
-// instance's DevScalars.  Fixed reduction tree: deterministic.
+// The terms of eqs. (2.7)-(2.8) of every cell of the active instances, a thread per cell:
+// grad f_i = -(v_i - m_i |P|) into gft, Q_i and |grad_i| / v_i.  About a hundred FP64
+// operations a cell (the pipe takes a warp's in 16 clocks of an SM), so the cells are
+// spread over all SMs; the sums, in a fixed order, are the lbfgs kernel's.
+constexpr int kCellThreads = 64;
 template <int D>
-__global__ void __launch_bounds__(kSolveThreads) batch_dual_kernel(const __grid_constant__ BArgs a) {
+__global__ void __launch_bounds__(kCellThreads) batch_cells_kernel(const __grid_constant__ BArgs a) {
     constexpr int K = moment_width(D);
-    __shared__ double sh[33];
-    const int b = blockIdx.x;
+    const long long i = (long long)blockIdx.x * kCellThreads + threadIdx.x;
+    if (i >= a.total_n) return;
+    const int b = a.inst_of[i];
     const BSolve &s = a.sol[b];
     if (!s.active || s.phase == PH_EVAL_ONLY) return;
-    const bool with_p = in_line_search(s.phase);
-    const BInst &I = a.inst[b];
-    const long long off = I.seed_off;
-    double gsum = 0.0, emax = 0.0, gp = 0.0, sv = 0.0, vmin = DBL_MAX;
-    for (int i = threadIdx.x; i < I.n; i += blockDim.x) {
-        const double vi = a.v[off + i], wi = a.Wt[off + i];
-        if (!(vi > 0.0) || !isfinite(vi)) atomicOr(&a.scs[b].status, ST_BAD_VOLUME);
-        double gr, Q;
-        dual_terms<D>(I.g, a.mom + (off + i) * K, vi, a.x + (off + i) * D, a.A + (off + i) * D * D, gr, Q);
-        gsum += gr * wi + I.g.cell * Q;
-        emax = fmax(emax, __ddiv_rn(fabs(gr), vi));
-        a.gft[off + i] = -gr;
-        if (with_p) gp += -gr * a.p[off + i];
-        sv += vi;
-        vmin = fmin(vmin, vi);
-    }
-    const double G = block_sum(gsum, sh);
-    const double GP = block_sum(gp, sh);
-    const double SV = block_sum(sv, sh);
-    __shared__ double shm[kSolveThreads / 32], shn[kSolveThreads / 32];
-    const double em = warp_max(emax), vm = warp_min(vmin);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        shm[wid] = em;
-        shn[wid] = vm;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double mx = 0.0, mn = DBL_MAX;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-            mx = fmax(mx, shm[k]);
-            mn = fmin(mn, shn[k]);
-        }
-        DevScalars *sc = a.scs + b;
-        sc->g = G;
-        sc->max_rel_err = mx;
-        sc->dot_gp = GP;
-        sc->sum_v = SV;
-        sc->min_v = mn;
-    }
+    const double vi = a.v[i];
+    if (!(vi > 0.0) || !isfinite(vi)) atomicOr(&a.scs[b].status, ST_BAD_VOLUME);
+    double gr, Q;
+    dual_terms<D>(a.inst[b].g, a.mom + i * K, vi, a.x + i * D, a.A + i * D * D, gr, Q);
+    a.gft[i] = -gr;
+    a.Q[i] = Q;
+    a.err[i] = __ddiv_rn(fabs(gr), vi);
 }
 
 // ---------------------------------------------------------------------------
@@ -426,14 +437,16 @@ __global__ void __launch_bounds__(kSolveThreads) batch_dual_kernel(const __grid_
 // path: strong-Wolfe line search (c1 = 1e-4, c2 = 0.9, expansion x4, cubic
 // zoom with safeguards) on f = -g~, two-loop recursion, curvature-pair skip,
 // best-iterate fallback, stop at the first evaluation with max rel err < eps.
+constexpr int kOwn = 8;  // seeds a thread keeps in registers
 struct SolveCtx {
     const BArgs &a;
     const BInst &I;
     BSolve &s;
-    double *sh;
+    double *sh;        // [16]
     int b, n, history;
     long long off;
     double *W, *Wt, *p, *gf, *gft, *Wbest, *Wout, *rho;
+    unsigned turn;
 
     __device__ void copy(double *dst, const double *src) {
         for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
@@ -449,8 +462,80 @@ struct SolveCtx {
         s.phase = PH_DONE;
         s.active = 0;
     }
-    // p = -H gf (two-loop recursion, H0 = gamma I); returns <gf, p>
+    // Deterministic block sum (block_sum's order: lanes by a butterfly, then the eight
+    // warps), one barrier: two buffers in turn.
+    __device__ double sum(double d) {
+        d = warp_sum(d);
+        double *buf = sh + 8 * (turn & 1);
+        ++turn;
+        if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = d;
+        __syncthreads();
+        double r = buf[threadIdx.x & 7];
+        r += __shfl_xor_sync(0xffffffffu, r, 4);
+        r += __shfl_xor_sync(0xffffffffu, r, 2);
+        r += __shfl_xor_sync(0xffffffffu, r, 1);
+        return r;
+    }
+    // p = -H gf (two-loop recursion, H0 = gamma I); returns <gf, p>.  Up to kOwn seeds a
+    // thread keep p in registers, with the next pair's rows loaded ahead of the sums
+    // (through memory a step took 5 us, 21 steps a direction); the roundings are written
+    // out, so that both forms give the same bits.
     __device__ double direction() {
+        return n <= kOwn * kSolveThreads ? direction_own() : direction_any();
+    }
+    __device__ double direction_own() {
+        double al[kBHist], pr[kOwn], u[kOwn], v[kOwn];
+        const int t = threadIdx.x;
+        const int hist = s.hist;
+        auto row = [&](const double *base, int idx) { return base + (size_t)idx * a.total_n + off; };
+        auto slot = [&](int k) { return (s.newest - k + kBHist) % kBHist; };
+        auto load = [&](const double *r, double (&d)[kOwn]) {
+#pragma unroll
+            for (int e = 0; e < kOwn; ++e) d[e] = t + e * kSolveThreads < n ? r[t + e * kSolveThreads] : 0.0;
+        };
+        load(gf, pr);
+        if (hist > 0) load(row(a.S, slot(0)), u);
+        for (int k = 0; k < hist; ++k) {
+            const int idx = slot(k);
+            load(row(a.Y, idx), v);
+            double d = 0.0;
+#pragma unroll
+            for (int e = 0; e < kOwn; ++e)
+                if (t + e * kSolveThreads < n) d = __fma_rn(u[e], pr[e], d);
+            if (k + 1 < hist) load(row(a.S, slot(k + 1)), u);
+            al[idx] = __dmul_rn(rho[idx], sum(d));
+#pragma unroll
+            for (int e = 0; e < kOwn; ++e)
+                if (t + e * kSolveThreads < n) pr[e] = __fma_rn(-al[idx], v[e], pr[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < kOwn; ++e) pr[e] = __dmul_rn(pr[e], s.gamma);
+        if (hist > 0) load(row(a.Y, slot(hist - 1)), v);
+        for (int k = hist - 1; k >= 0; --k) {
+            const int idx = slot(k);
+            load(row(a.S, idx), u);
+            double d = 0.0;
+#pragma unroll
+            for (int e = 0; e < kOwn; ++e)
+                if (t + e * kSolveThreads < n) d = __fma_rn(v[e], pr[e], d);
+            if (k > 0) load(row(a.Y, slot(k - 1)), v);
+            const double c = __fma_rn(-rho[idx], sum(d), al[idx]);
+#pragma unroll
+            for (int e = 0; e < kOwn; ++e)
+                if (t + e * kSolveThreads < n) pr[e] = __fma_rn(u[e], c, pr[e]);
+        }
+        double d = 0.0;
+        load(gf, u);
+#pragma unroll
+        for (int e = 0; e < kOwn; ++e)
+            if (t + e * kSolveThreads < n) {
+                pr[e] = -pr[e];
+                p[t + e * kSolveThreads] = pr[e];
+                d = __fma_rn(u[e], pr[e], d);
+            }
+        return sum(d);
+    }
+    __device__ double direction_any() {
         double al[kBHist];
         for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = gf[i];
         for (int k = 0; k < s.hist; ++k) {
@@ -459,8 +544,8 @@ struct SolveCtx {
             const double *yk = a.Y + (size_t)idx * a.total_n + off;
             double d = 0.0;
             for (int i = threadIdx.x; i < n; i += blockDim.x) d += sk[i] * p[i];
-            al[idx] = rho[idx] * block_sum(d, sh);
-            for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] -= al[idx] * yk[i];
+            al[idx] = __dmul_rn(rho[idx], sum(d));
+            for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = __fma_rn(-al[idx], yk[i], p[i]);
         }
         for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] *= s.gamma;
         for (int k = s.hist - 1; k >= 0; --k) {
@@ -469,15 +554,15 @@ struct SolveCtx {
             const double *yk = a.Y + (size_t)idx * a.total_n + off;
             double d = 0.0;
             for (int i = threadIdx.x; i < n; i += blockDim.x) d += yk[i] * p[i];
-            const double bta = rho[idx] * block_sum(d, sh);
-            for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] += sk[i] * (al[idx] - bta);
+            const double c = __fma_rn(-rho[idx], sum(d), al[idx]);
+            for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = __fma_rn(sk[i], c, p[i]);
         }
         double d = 0.0;
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
             p[i] = -p[i];
             d += gf[i] * p[i];
         }
-        return block_sum(d, sh);
+        return sum(d);
     }
     // store s = Wt - W, y = gft - gf in the next slot; returns whether it was kept
     __device__ void push_pair() {
@@ -494,9 +579,9 @@ struct SolveCtx {
             yy += yi * yi;
             ss += si * si;
         }
-        sy = block_sum(sy, sh);
-        yy = block_sum(yy, sh);
-        ss = block_sum(ss, sh);
+        sy = sum(sy);
+        yy = sum(yy);
+        ss = sum(ss);
         if (threadIdx.x == 0) rho[slot] = sy != 0.0 ? 1.0 / sy : 0.0;
         __syncthreads();
         if (sy > 1e-12 * sqrt(ss * yy) && yy > 0.0) {
@@ -505,12 +590,60 @@ struct SolveCtx {
             s.gamma = sy / yy;
         }
     }
+    // The next evaluation's start: the trial weights in the scan-order and natural
+    // records, the reference weight, the groups' weight gaps, cleared moments and queue.
+    // Maxima by ordered keys (no FP64 comparisons).
+    __device__ void publish(DevScalars *sc, unsigned long long *skey) {
+        __syncthreads();  // Wt is written
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        unsigned long long wmax = 0ull;
+        const int K = moment_width(I.g.dim);
+        unsigned long long *mom = a.mom + I.seed_off * K;
+        for (int e = threadIdx.x; e < n * K; e += blockDim.x) mom[e] = 0ull;
+        SeedRec *recs = a.recs + I.rec_off;
+        SeedRec32 *r32 = a.recs32 + I.rec_off, *r32s = a.recs32s + I.rec_off;
+        GroupBound *groups = a.groups + I.rec_off / 32;
+        int bad = 0;
+        for (int p0 = wid * 32; p0 < n; p0 += kSolveThreads) {
+            const int q = p0 + lane;
+            unsigned long long key = 0ull;
+            if (q < n) {
+                const int src = I.sorted ? a.perm[I.rec_off + q] : q;
+                const double wi = Wt[src];
+                float wh, wl;
+                split_f32(wi, wh, wl);
+                recs[q].w = wi;
+                r32s[q].wh = wh;
+                r32s[q].wl = wl;
+                r32[src].wh = wh;
+                r32[src].wl = wl;
+                if (isfinite(wi)) key = dkey(wi);
+                else bad = 1;
+            }
+            const unsigned long long top = warp_max_key(key);
+            if (lane == 0) groups[p0 >> 5].wmax = dkey_inv(top ? top : dkey(-DBL_MAX));
+            wmax = top > wmax ? top : wmax;
+        }
+        if (bad) atomicOr(&sc->status, ST_NONFINITE);
+        if (threadIdx.x == 0) *skey = 0ull;
+        __syncthreads();
+        if (lane == 0) atomicMax(skey, wmax);
+        __syncthreads();
+        const double wref = dkey_inv(*skey ? *skey : dkey(-DBL_MAX));
+        for (int g = threadIdx.x; g * 32 < n; g += blockDim.x) groups[g].wgap = __double2float_rd(wref - groups[g].wmax);
+        if (threadIdx.x == 0) {
+            sc->flag_count = 0u;
+            sc->wref_key = dkey(wref);
+            split_f32(wref, sc->wref_h, sc->wref_l);
+        }
+    }
 };
 
 enum : int { NX_NONE = 0, NX_NEWDIR, NX_ACCEPT, NX_LSEND, NX_FAIL, NX_ZOOM, NX_GIVEUP };
 
 __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid_constant__ BArgs a) {
-    __shared__ double sh[33];
+    __shared__ double sh[16];
+    __shared__ unsigned long long skey, sk_err, sk_min;
     const int b = blockIdx.x;
     BSolve s = a.sol[b];
     if (!s.active) return;
@@ -520,13 +653,49 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
     const long long off = I.seed_off;
     SolveCtx c{a,          I,           s,           sh,          b,          I.n,  prm.history,
                off,        a.W + off,   a.Wt + off,  a.p + off,   a.gf + off, a.gft + off,
-               a.Wbest + off, a.Wout + off, a.rho + (size_t)b * kBHist};
+               a.Wbest + off, a.Wout + off, a.rho + (size_t)b * kBHist, 0u};
     const double c1 = 1e-4, c2 = 0.9;
     const int dim = I.g.dim;
 
     const int bits = sc->status;
-    const double gval = sc->g, err = sc->max_rel_err;
-    const double phi = -gval, dphi = sc->dot_gp;
+    // the evaluation's sums from the cells' terms: g~, <grad f, p>, the largest relative
+    // volume error; at a solve's first evaluation also sum v and min v
+    double gval = 0.0, dot_gp = 0.0, err = 0.0, sum_v = 0.0, min_v = 0.0;
+    if (s.phase != PH_EVAL_ONLY) {
+        const bool with_p = in_line_search(s.phase), with_v = s.phase == PH_INIT || s.phase == PH_INIT_PRED;
+        if (threadIdx.x == 0) {
+            sk_err = 0ull;
+            sk_min = ~0ull;
+        }
+        double gsum = 0.0, gp = 0.0, sv = 0.0;
+        unsigned long long emax = 0ull, vmin = ~0ull;
+        for (int i = threadIdx.x; i < c.n; i += blockDim.x) {
+            const double gr = -c.gft[i], wi = c.Wt[i], Q = a.Q[off + i];
+            gsum = __dadd_rn(gsum, __fma_rn(gr, wi, __dmul_rn(I.g.cell, Q)));
+            if (with_p) gp += -gr * c.p[i];
+            const unsigned long long e = (unsigned long long)__double_as_longlong(a.err[off + i]);
+            emax = e > emax ? e : emax;
+            if (with_v) {
+                const double vi = a.v[off + i];
+                sv += vi;
+                const unsigned long long k = dkey(vi);
+                vmin = k < vmin ? k : vmin;
+            }
+        }
+        __syncthreads();
+        emax = warp_max_key(emax);
+        vmin = ~warp_max_key(~vmin);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&sk_err, emax);
+            if (with_v) atomicMin(&sk_min, vmin);
+        }
+        gval = c.sum(gsum);
+        dot_gp = with_p ? c.sum(gp) : 0.0;
+        sum_v = with_v ? c.sum(sv) : 0.0;
+        err = __longlong_as_double((long long)sk_err);
+        min_v = with_v ? dkey_inv(sk_min) : 0.0;
+    }
+    const double phi = -gval, dphi = dot_gp;
     s.rescored += sc->flag_count;
     __syncthreads();
     int next = NX_NONE;
@@ -545,9 +714,9 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
         s.last_g = gval;
         s.last_err = err;
         const bool first = s.phase == PH_INIT || s.phase == PH_INIT_PRED;
-        if (first) s.min_v = sc->min_v;
+        if (first) s.min_v = min_v;
         const bool bad_volumes = first && prm.check_volumes &&
-                                 (!(sc->min_v > 0.0) || fabs(sc->sum_v - I.measure) > 1e-9 * I.measure);
+                                 (!(min_v > 0.0) || fabs(sum_v - I.measure) > 1e-9 * I.measure);
         if (err < s.best_err) {
             s.best_err = err;
             s.best_g = gval;
@@ -737,6 +906,7 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
     }
     if (next != NX_NONE) c.finish(APD_NOT_CONVERGED, c.Wbest);  // guard exhausted (not expected)
     __syncthreads();
+    if (s.active) c.publish(sc, &skey);
     if (threadIdx.x == 0) {
         a.sol[b] = s;
         if (s.active) atomicAdd(&a.sched->next_active, 1);
@@ -793,6 +963,7 @@ struct apd_batch {
     std::vector<double> measure;
     std::vector<int> order;
     int variant = -1;                  // chosen tile variant (-1: autotune pending)
+    int table_variant = -1;            // the variant d_inst is laid out for
     std::vector<double> variant_ms;    // autotune timings
     int grid_blocks = 0, rescore_blocks = 0;
     size_t smem_assign = 0, smem_prep = 0, smem_sched = 0;
@@ -802,13 +973,16 @@ struct apd_batch {
     BSched *h_sched = nullptr;         // pinned
     BParams *h_prm = nullptr;          // pinned
     double *d_w0 = nullptr;
-    void *blocks[32] = {};
+    region::Src *d_srcs = nullptr;
+    int sms = 152;
+    bool can_region = false;           // every instance suits the region form
+    void *blocks[40] = {};
     int nblocks = 0;
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int graph_variant = -1;
-    long long launches = 0;
+    long long launches = 0, graph_launches = 0;
 };
 
 namespace {
@@ -821,8 +995,17 @@ int cuda_rc(cudaError_t e) { return e == cudaSuccess ? APD_OK : APD_ERR_CUDA; }
         if (_rc != APD_OK) return _rc; \
     } while (0)
 
+// Variant index of the region form (pruning on).
+constexpr int kRegionVariant = 1000;
+
+// The variant an evaluation uses: the region form when pruning is on, else the chosen tile.
+int active_variant(const apd_batch &bt) { return bt.args.prune && bt.can_region ? kRegionVariant : bt.variant; }
+
 std::vector<BInst> instance_table(const apd_batch &bt, int vi) {
-    const Variant &V = variants(bt.dim)[vi];
+    int rd[3];
+    region_dims(bt.dim, rd);
+    const Variant V = vi == kRegionVariant ? Variant{1, rd[0], rd[1], rd[2], region::kThreads, nullptr, nullptr}
+                                           : variants(bt.dim)[vi];
     std::vector<BInst> t(bt.count);
     for (int b = 0; b < bt.count; ++b) {
         BInst &I = t[b];
@@ -848,10 +1031,17 @@ std::vector<BInst> instance_table(const apd_batch &bt, int vi) {
 }
 
 int use_variant(apd_batch &bt, int vi, cudaStream_t st) {
-    const Variant &V = variants(bt.dim)[vi];
     const std::vector<BInst> t = instance_table(bt, vi);
     BTRY(cuda_rc(cudaMemcpyAsync(bt.d_inst, t.data(), t.size() * sizeof(BInst), cudaMemcpyHostToDevice, st)));
     BTRY(cuda_rc(cudaStreamSynchronize(st)));
+    bt.table_variant = vi;
+    if (vi == kRegionVariant) {
+        long long regions = 0;
+        for (const BInst &I : t) regions += I.ntiles;
+        bt.grid_blocks = (int)std::min<long long>(regions, 4ll * bt.sms);
+        return APD_OK;
+    }
+    const Variant &V = variants(bt.dim)[vi];
     const size_t smem = bt.dim == 3 ? sizeof(fp32::SharedLayout<3>) : sizeof(fp32::SharedLayout<2>);
     BTRY(cuda_rc(cudaFuncSetAttribute(V.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)));
     int per_sm = 0, sms = 0;
@@ -862,21 +1052,33 @@ int use_variant(apd_batch &bt, int vi, cudaStream_t st) {
     return APD_OK;
 }
 
-// The per-iteration launches (also the body of the captured graph).
+int enqueue_prep(apd_batch &bt, cudaStream_t st) {
+    if (bt.dim == 3) batch_prep_kernel<3><<<bt.count, kPrepThreads, bt.smem_prep, st>>>(bt.args);
+    else batch_prep_kernel<2><<<bt.count, kPrepThreads, bt.smem_prep, st>>>(bt.args);
+    bt.launches += 1;
+    return cuda_rc(cudaGetLastError());
+}
+
+// The per-iteration launches (also the body of the captured graph); the records are
+// ready (batch_prep_kernel, then the lbfgs kernel's weights).
 int enqueue_iteration(apd_batch &bt, int vi, bool solve_steps, cudaStream_t st) {
-    const Variant &V = variants(bt.dim)[vi];
     const BArgs &a = bt.args;
     batch_schedule_kernel<<<1, 1024, bt.smem_sched, st>>>(a);
-    if (bt.dim == 3) batch_prep_kernel<3><<<bt.count, kPrepThreads, bt.smem_prep, st>>>(a);
-    else batch_prep_kernel<2><<<bt.count, kPrepThreads, bt.smem_prep, st>>>(a);
+    bt.launches += 2;
+    if (vi == kRegionVariant) {
+        if (bt.dim == 3) batch_region_kernel<3><<<bt.grid_blocks, region::kThreads, 0, st>>>(a);
+        else batch_region_kernel<2><<<bt.grid_blocks, region::kThreads, 0, st>>>(a);
+    } else {
+        BTRY(cuda_rc(variants(bt.dim)[vi].launch(a, bt.grid_blocks, bt.smem_assign, st)));
+        if (bt.dim == 3) batch_rescore_kernel<3><<<bt.rescore_blocks, 256, bt.smem_sched + 4, st>>>(a);
+        else batch_rescore_kernel<2><<<bt.rescore_blocks, 256, bt.smem_sched + 4, st>>>(a);
+        bt.launches += 1;
+    }
     BTRY(cuda_rc(cudaGetLastError()));
-    BTRY(cuda_rc(V.launch(a, bt.grid_blocks, bt.smem_assign, st)));
-    if (bt.dim == 3) batch_rescore_kernel<3><<<bt.rescore_blocks, 256, bt.smem_sched + 4, st>>>(a);
-    else batch_rescore_kernel<2><<<bt.rescore_blocks, 256, bt.smem_sched + 4, st>>>(a);
-    bt.launches += 4;
     if (solve_steps) {
-        if (bt.dim == 3) batch_dual_kernel<3><<<bt.count, kSolveThreads, 0, st>>>(a);
-        else batch_dual_kernel<2><<<bt.count, kSolveThreads, 0, st>>>(a);
+        const unsigned cells = (unsigned)((bt.total_n + kCellThreads - 1) / kCellThreads);
+        if (bt.dim == 3) batch_cells_kernel<3><<<cells, kCellThreads, 0, st>>>(a);
+        else batch_cells_kernel<2><<<cells, kCellThreads, 0, st>>>(a);
         batch_lbfgs_kernel<<<bt.count, kSolveThreads, 0, st>>>(a);
         bt.launches += 2;
     }
@@ -914,15 +1116,14 @@ int autotune(apd_batch &bt, cudaStream_t st) {
         for (int rep = 0; rep < 3; ++rep) {
             BTRY(init_solves(bt, true, st));
             batch_schedule_kernel<<<1, 1024, bt.smem_sched, st>>>(bt.args);
-            if (bt.dim == 3) batch_prep_kernel<3><<<bt.count, kPrepThreads, bt.smem_prep, st>>>(bt.args);
-            else batch_prep_kernel<2><<<bt.count, kPrepThreads, bt.smem_prep, st>>>(bt.args);
+            BTRY(enqueue_prep(bt, st));
             BTRY(cuda_rc(cudaEventRecord(e0, st)));
             BTRY(cuda_rc(vs[vi].launch(bt.args, bt.grid_blocks, bt.smem_assign, st)));
             BTRY(cuda_rc(cudaEventRecord(e1, st)));
             BTRY(cuda_rc(cudaEventSynchronize(e1)));
             float ms = 0.f;
             BTRY(cuda_rc(cudaEventElapsedTime(&ms, e0, e1)));
-            bt.launches += 4;
+            bt.launches += 2;
             if (rep > 0) best_ms = std::min(best_ms, ms);
         }
         bt.variant_ms[vi] = best_ms;
@@ -934,15 +1135,16 @@ int autotune(apd_batch &bt, cudaStream_t st) {
     return use_variant(bt, best, st);
 }
 
-int capture_graph(apd_batch &bt) {
-    if (bt.exec && bt.graph_variant == bt.variant) return APD_OK;
+int capture_graph(apd_batch &bt, int vi) {
+    if (bt.exec && bt.graph_variant == vi) return APD_OK;
     if (bt.exec) cudaGraphExecDestroy(bt.exec);
     if (bt.graph) cudaGraphDestroy(bt.graph);
     bt.exec = nullptr;
     bt.graph = nullptr;
     BTRY(cuda_rc(cudaStreamBeginCapture(bt.cap, cudaStreamCaptureModeThreadLocal)));
     const long long before = bt.launches;
-    const int rc = enqueue_iteration(bt, bt.variant, true, bt.cap);
+    const int rc = enqueue_iteration(bt, vi, true, bt.cap);
+    bt.graph_launches = bt.launches - before;
     bt.launches = before;
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(bt.cap, &g);
@@ -953,12 +1155,14 @@ int capture_graph(apd_batch &bt) {
     BTRY(cuda_rc(e));
     bt.graph = g;
     BTRY(cuda_rc(cudaGraphInstantiate(&bt.exec, bt.graph, 0)));
-    bt.graph_variant = bt.variant;
+    bt.graph_variant = vi;
     return APD_OK;
 }
 
 int prepare(apd_batch &bt, cudaStream_t st) {
-    if (bt.variant < 0) BTRY(autotune(bt, st));
+    const int vi = active_variant(bt);
+    if (vi < 0) BTRY(autotune(bt, st));
+    else if (bt.table_variant != vi) BTRY(use_variant(bt, vi, st));
     return APD_OK;
 }
 
@@ -1057,6 +1261,39 @@ int apd_batch_create(apd_batch **out, int32_t dim, int32_t count, const apd_grid
     alloc((void **)&a.mom, N * K * sizeof(unsigned long long));
     alloc((void **)&a.flags, (size_t)fo * sizeof(uint32_t));
     alloc((void **)&a.flag_gi, (size_t)fo * sizeof(int32_t));
+    alloc((void **)&a.inst_of, N * sizeof(int32_t));
+    alloc((void **)&a.Q, N * sizeof(double));
+    alloc((void **)&a.err, N * sizeof(double));
+    alloc((void **)&bt->d_srcs, count * sizeof(region::Src));
+    a.srcs = bt->d_srcs;
+    bt->can_region = true;
+    if (ok) {
+        std::vector<int32_t> inst_of(N);
+        std::vector<region::Src> srcs(count);
+        for (int b = 0; b < count; ++b) {
+            const GridDev &g = bt->grids[b];
+            const int nb = bt->n[b];
+            std::fill(inst_of.begin() + bt->seed_off[b], inst_of.begin() + bt->seed_off[b] + nb, b);
+            region::Src &src = srcs[b];
+            std::memset((void *)&src, 0, sizeof src);
+            src.g = g;
+            src.gf = make_gridf(g);
+            src.n = nb;
+            src.n_groups = (nb + kGroup - 1) / kGroup;
+            src.recs = a.recs32s + bt->rec_off[b];
+            src.perm = (nb + kChunk - 1) / kChunk * kChunk <= kBSortMax ? a.perm + bt->rec_off[b] : nullptr;
+            src.groups = a.groups + bt->rec_off[b] / 32;
+            src.x = a.x + bt->seed_off[b] * D;
+            src.A = a.A + bt->seed_off[b] * D * D;
+            src.w = a.Wt + bt->seed_off[b];
+            src.gmom = a.mom + bt->seed_off[b] * K;
+            src.sc = a.scs + b;
+            bt->can_region = bt->can_region && src.n_groups <= region::kMaxGroups && g.res[0] < (1 << 23) &&
+                             g.res[1] < (1 << 23) && g.res[2] < (1 << 23);
+        }
+        ok = cudaMemcpy((void *)a.inst_of, inst_of.data(), N * sizeof(int32_t), cudaMemcpyHostToDevice) == cudaSuccess &&
+             cudaMemcpy(bt->d_srcs, srcs.data(), count * sizeof(region::Src), cudaMemcpyHostToDevice) == cudaSuccess;
+    }
     if (ok && cudaMallocHost((void **)&bt->h_sol, count * sizeof(BSolve)) != cudaSuccess) ok = false;
     if (ok && cudaMallocHost((void **)&bt->h_sched, sizeof(BSched)) != cudaSuccess) ok = false;
     if (ok && cudaMallocHost((void **)&bt->h_prm, sizeof(BParams)) != cudaSuccess) ok = false;
@@ -1083,6 +1320,7 @@ int apd_batch_create(apd_batch **out, int32_t dim, int32_t count, const apd_grid
     int sms = 0;
     if (ok && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device) != cudaSuccess) ok = false;
     bt->rescore_blocks = std::max(1, sms) * kRescoreBlocksPerSM;
+    bt->sms = std::max(1, sms);
     if (ok && tile >= 0) {
         bt->variant = tile;
         if (use_variant(*bt, tile, nullptr) != APD_OK) ok = false;
@@ -1150,7 +1388,8 @@ int apd_batch_cell_moments(apd_batch *bt, const double *x, const double *A, cons
     BTRY(load_inputs(*bt, x, A, w, nullptr, st));
     BTRY(prepare(*bt, st));
     BTRY(init_solves(*bt, true, st));
-    BTRY(enqueue_iteration(*bt, bt->variant, false, st));
+    BTRY(enqueue_prep(*bt, st));
+    BTRY(enqueue_iteration(*bt, active_variant(*bt), false, st));
     const size_t K = (size_t)moment_width(bt->dim);
     BTRY(cuda_rc(cudaMemcpyAsync(moments, bt->args.mom, (size_t)bt->total_n * K * sizeof(int64_t),
                                  cudaMemcpyDeviceToDevice, st)));
@@ -1184,17 +1423,18 @@ static int batch_solve(apd_batch *bt, const double *x, const double *A, const do
     bt->h_prm->check_volumes = o.check_volumes != 0;
     BTRY(cuda_rc(cudaMemcpyAsync((void *)bt->args.prm, bt->h_prm, sizeof(BParams), cudaMemcpyHostToDevice, st)));
     BTRY(prepare(*bt, st));
-    BTRY(capture_graph(*bt));
+    BTRY(capture_graph(*bt, active_variant(*bt)));
     BTRY(init_solves(*bt, false, st, judge));
+    BTRY(enqueue_prep(*bt, st));
     // Each replay is one evaluation of every active instance; a finished batch
-    // replays as six near-empty launches, so the host polls every few replays.
+    // replays as a few near-empty launches, so the host polls every few replays.
     const int max_iters = o.max_evals + 8;
     int iters = 0;
     for (;;) {
         const int burst = iters < 8 ? 2 : 8;
         for (int r = 0; r < burst; ++r) {
             BTRY(cuda_rc(cudaGraphLaunch(bt->exec, st)));
-            bt->launches += 6;
+            bt->launches += bt->graph_launches;
         }
         iters += burst;
         BTRY(cuda_rc(cudaMemcpyAsync(bt->h_sched, bt->args.sched, sizeof(BSched), cudaMemcpyDeviceToHost, st)));

@@ -203,13 +203,6 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Largest of 64-bit keys over the warp, by two 32-bit reductions.
-__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k) {
-    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
-    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
-    return ((unsigned long long)hi << 32) | lo;
-}
-
 // Seed records at new positions, one seed per thread, with the scalars of the pass: the
 // blocks' maxima (w, ||A||_F, -lambda bound as ordered keys: no FP64 comparisons) go to
 // `part`, the last block to finish reduces them and clears the pass's counters; mom's
