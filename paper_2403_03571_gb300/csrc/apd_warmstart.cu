@@ -25,6 +25,7 @@
 // step (forward, backward by hand, per-CTA gradient partials summed in a fixed
 // order by the Adam kernel), and the input statistics.  All FP32 except the
 // neighbour distances (FP64) and the statistic sums (FP64).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -37,7 +38,6 @@ namespace {
 
 constexpr int kH = 64;       // hidden width
 constexpr int kNN = 8;       // neighbours per seed
-constexpr int kTrainB = 128; // samples (threads) per CTA of the network kernels
 
 constexpr int kRadii = 3;    // neighbourhood radii 2, 4, 8 (mean spacings)
 __host__ __device__ constexpr int feat_dim(int D) { return 1 + D * (D + 1) / 2 + 2 * kNN + D + 2 * kRadii; }
@@ -196,79 +196,118 @@ __global__ void __launch_bounds__(256)
 }
 
 // ---------------------------------------------------------------------------
-// network evaluation (one sample per thread; weights and the thread's
-// activation rows in shared memory, rows padded to avoid bank conflicts)
+// network evaluation: a block takes kTile samples, layer by layer as small matrix
+// products in FP32 registers: a thread owns 4 outputs x 2 samples, the weights lie
+// transposed in shared memory ([input][output], one 16-byte broadcast a step), the
+// activations as [unit][sample].  One thread per sample (128 a block, 47 blocks for
+// 6000 samples) ran a sample's 10^4 multiply-adds in one thread: a training step on 6000
+// 3D samples took 349 us, so 56 us (188 blocks, 1.2 a SM).  Its 0.4 GFLOP in FP32 would
+// take 6 us: the chain of nine layers between barriers and four launches bounds it.
 // ---------------------------------------------------------------------------
-constexpr int kRow = kH + 1;
+constexpr int kTile = 32;      // samples per block
+constexpr int kNet = 256;      // threads per block
+constexpr int kWS = kH + 4;    // row stride of a transposed weight matrix
+constexpr int kAS = kTile + 4; // row stride of the activations
+constexpr int kMaxParts = 608;  // gradient partials: four blocks per SM bounds their memory to 25 MB at any batch
+static_assert(kNet == (kH / 4) * (kTile / 2), "thread tiles");
 
 template <int F>
-struct Rows {
-    float x[kTrainB][F + 1];
-    float h1[kTrainB][kRow];
-    float h2[kTrainB][kRow];
-    float h3[kTrainB][kRow];
-    float d[kTrainB][kRow];   // delta of the layer being back-propagated
-    float dy[kTrainB];
-    float loss[kTrainB];
+struct NetShared {
+    alignas(16) float w1[F][kWS], w2[kH][kWS], w3[kH][kWS];  // transposed: [input][output]
+    float b[3][kH], w4[kH], norm[2 * F], b4;
+    alignas(16) float x[F][kAS];
+    alignas(16) float h1[kH][kAS], h2[kH][kAS], h3[kH][kAS];
+};
+template <int F>
+struct GradShared {
+    NetShared<F> n;
+    alignas(16) float d[kH][kAS];
+    float dy[kTile], loss[kTile];
 };
 
 template <int F>
-constexpr size_t rows_offset() {  // floats before the rows: parameters, then mean / inverse std
-    return ((size_t)param_count(F) + 2 * F + 3) & ~(size_t)3;
-}
-template <int F>
-constexpr size_t net_smem() {
-    return rows_offset<F>() * sizeof(float) + sizeof(Rows<F>);
-}
-
-template <int F>
-__device__ __forceinline__ void load_net(float *sp, const float *__restrict__ params, const float *__restrict__ norm) {
-    constexpr int P = param_count(F);
-    for (int k = threadIdx.x; k < P; k += blockDim.x) sp[k] = params[k];
-    for (int k = threadIdx.x; k < 2 * F; k += blockDim.x) sp[P + k] = norm[k];
-}
-
-// out[j] = relu(b[j] + sum_k W[j][k] in[k]) for the calling thread's rows
-__device__ __forceinline__ void dense_relu(const float *sp, int w, int bo, int in_dim, const float *in, float *out) {
-    for (int j = 0; j < kH; ++j) {
-        float acc = sp[bo + j];
-        const float *wr = sp + w + j * in_dim;
-#pragma unroll 8
-        for (int k = 0; k < in_dim; ++k) acc = fmaf(wr[k], in[k], acc);
-        out[j] = fmaxf(acc, 0.f);
-    }
-}
-
-// standardised input of sample s into the thread's x row, then the forward pass
-template <int F>
-__device__ __forceinline__ float forward(const float *sp, Rows<F> &R, int t, const float *__restrict__ feat,
-                                         long long s) {
+__device__ __forceinline__ void load_net(NetShared<F> &S, const float *__restrict__ params,
+                                         const float *__restrict__ norm) {
     constexpr Layout L(F);
-    const float *mean = sp + L.P, *istd = sp + L.P + F;
+    for (int e = threadIdx.x; e < kH * F; e += kNet) S.w1[e % F][e / F] = params[L.w1 + e];
+    for (int e = threadIdx.x; e < kH * kH; e += kNet) {
+        S.w2[e % kH][e / kH] = params[L.w2 + e];
+        S.w3[e % kH][e / kH] = params[L.w3 + e];
+    }
+    for (int e = threadIdx.x; e < kH; e += kNet) {
+        S.b[0][e] = params[L.b1 + e];
+        S.b[1][e] = params[L.b2 + e];
+        S.b[2][e] = params[L.b3 + e];
+        S.w4[e] = params[L.w4 + e];
+    }
+    for (int e = threadIdx.x; e < 2 * F; e += kNet) S.norm[e] = norm[e];
+    if (threadIdx.x == 0) S.b4 = params[L.b4];
+}
+
+// out[j][s] = relu(b[j] + sum_k w[k][j] in[k][s])
+__device__ __forceinline__ void layer(const float (*w)[kWS], const float *b, int in_dim, const float (*in)[kAS],
+                                      float (*out)[kAS]) {
+    const int s0 = (threadIdx.x & 15) * 2, j0 = (threadIdx.x >> 4) * 4;
+    float acc[4][2];
 #pragma unroll
-    for (int k = 0; k < F; ++k) R.x[t][k] = (feat[s * F + k] - mean[k]) * istd[k];
-    dense_relu(sp, L.w1, L.b1, F, R.x[t], R.h1[t]);
-    dense_relu(sp, L.w2, L.b2, kH, R.h1[t], R.h2[t]);
-    dense_relu(sp, L.w3, L.b3, kH, R.h2[t], R.h3[t]);
-    float y = sp[L.b4];
-    for (int k = 0; k < kH; ++k) y = fmaf(sp[L.w4 + k], R.h3[t][k], y);
+    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = b[j0 + i];
+#pragma unroll 8
+    for (int k = 0; k < in_dim; ++k) {
+        const float4 v = *reinterpret_cast<const float4 *>(&w[k][j0]);
+        const float2 a = *reinterpret_cast<const float2 *>(&in[k][s0]);
+        const float wv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            acc[i][0] = fmaf(wv[i], a.x, acc[i][0]);
+            acc[i][1] = fmaf(wv[i], a.y, acc[i][1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float2 *>(&out[j0 + i][s0]) = make_float2(fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f));
+}
+
+// Forward pass of samples rows[0 .. nvalid) (absent ones: zero inputs); returns the
+// output of sample threadIdx.x in threads 0 .. kTile - 1.  Activations stay in S.
+template <int F, class Row>
+__device__ __forceinline__ float forward(NetShared<F> &S, const float *__restrict__ feat, int nvalid, Row row) {
+    for (int e = threadIdx.x; e < F * kTile; e += kNet) {
+        const int s = e / F, k = e % F;
+        S.x[k][s] = s < nvalid ? (feat[row(s) * F + k] - S.norm[k]) * S.norm[F + k] : 0.f;
+    }
+    __syncthreads();
+    layer(S.w1, S.b[0], F, S.x, S.h1);
+    __syncthreads();
+    layer(S.w2, S.b[1], kH, S.h1, S.h2);
+    __syncthreads();
+    layer(S.w3, S.b[2], kH, S.h2, S.h3);
+    __syncthreads();
+    // The sums run over the inputs in order, in every layer: a solve started from the
+    // predicted weights follows their last bit.
+    float y = S.b4;
+    if (threadIdx.x < kTile) {
+#pragma unroll 16
+        for (int j = 0; j < kH; ++j) y = fmaf(S.w4[j], S.h3[j][threadIdx.x], y);
+    }
     return y;
 }
 
 // W_pred of every seed: y_i s^(-2/D), s = n_b / |O_b|
 template <int D>
-__global__ void __launch_bounds__(kTrainB)
+__global__ void __launch_bounds__(kNet, 2)
     predict_kernel(const int count, const long long *__restrict__ offs, const double *__restrict__ box,
                    const float *__restrict__ params, const float *__restrict__ norm, const float *__restrict__ feat,
                    double *__restrict__ w_out) {
     constexpr int F = feat_dim(D);
-    extern __shared__ float sp[];
-    Rows<F> &R = *reinterpret_cast<Rows<F> *>(sp + rows_offset<F>());
-    load_net<F>(sp, params, norm);
+    extern __shared__ __align__(16) unsigned char net_raw[];
+    NetShared<F> &S = *reinterpret_cast<NetShared<F> *>(net_raw);
+    load_net<F>(S, params, norm);
     __syncthreads();
-    const long long total = offs[count];
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= total) return;
+    const long long total = offs[count], s0 = (long long)blockIdx.x * kTile;
+    const int nvalid = (int)min((long long)kTile, total - s0);
+    const float y = forward<F>(S, feat, nvalid, [&](int s) { return s0 + s; });
+    if ((int)threadIdx.x >= nvalid) return;
+    const long long s = s0 + threadIdx.x;
     int lo = 0, hi = count - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -279,123 +318,181 @@ __global__ void __launch_bounds__(kTrainB)
     double meas = 1.0;
 #pragma unroll
     for (int a = 0; a < D; ++a) meas *= box[(size_t)lo * 6 + 3 + a] - box[(size_t)lo * 6 + a];
-    const float y = forward<F>(sp, R, threadIdx.x, feat, s);
     w_out[s] = (double)y * pow((double)n / meas, -2.0 / D);
 }
 
 // ---------------------------------------------------------------------------
 // training: loss = (1/B) sum_s (y_s - t_s)^2 over the batch idx[0 .. B)
 // ---------------------------------------------------------------------------
-// One CTA = kTrainB samples, forward as above, then backward layer by layer:
+// One block = kTile samples, forward as above, then backward layer by layer:
 //   dy = 2 (y - t) / B;  gW4 = sum dy h3, gb4 = sum dy
 //   d3 = dy W4 . [h3 > 0];  gW3 = sum d3 h2^T, gb3 = sum d3
 //   d2 = W3^T d3 . [h2 > 0];  gW2 = sum d2 h1^T, gb2 = sum d2
 //   d1 = W2^T d2 . [h1 > 0];  gW1 = sum d1 x^T,  gb1 = sum d1
-// The CTA's gradient goes to part[blockIdx.x][P]; the Adam kernel sums the
-// partials in CTA order (deterministic).
-__device__ __forceinline__ void grad_outer(const float (*dl)[kRow], const float *hin, int hstride, int in_dim,
-                                           int nvalid, float *gw, float *gb) {
-    // gW[j][k] = sum_s d[s][j] hin[s][k]; thread t takes entries t, t + blockDim, ...
-    for (int e = threadIdx.x; e < kH * in_dim; e += blockDim.x) {
-        const int j = e / in_dim, k = e % in_dim;
-        float acc = 0.f;
-        for (int s = 0; s < nvalid; ++s) acc = fmaf(dl[s][j], hin[s * hstride + k], acc);
-        gw[e] = acc;
+// The block's gradient goes to part[blockIdx.x][P] (a batch of more than kMaxParts tiles:
+// summed over the block's tiles there); the Adam kernel sums the partials in a fixed order.
+
+// A gradient entry of this block: its first tile writes it, later tiles add.
+__device__ __forceinline__ void put(float *g, float v, bool add) { *g = add ? *g + v : v; }
+
+// gW[j][k] = sum_s d[j][s] hin[k][s] (row-major [64][in_dim]) and gb[j] = sum_s d[j][s]; a
+// thread takes j = jt + 16 i, k = kt + 16 c, four samples a step.
+template <int KC>
+__device__ __forceinline__ void grad_outer(const float (*d)[kAS], const float (*hin)[kAS], int in_dim, float *gw,
+                                           float *gb, bool add) {
+    const int kt = threadIdx.x & 15, jt = threadIdx.x >> 4;
+    float acc[4][KC], bs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < KC; ++c) acc[i][c] = 0.f;
+#pragma unroll 2
+    for (int s = 0; s < kTile; s += 4) {
+        float4 dv[4], hv[KC];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dv[i] = *reinterpret_cast<const float4 *>(&d[jt + 16 * i][s]);
+#pragma unroll
+        for (int c = 0; c < KC; ++c) {
+            const int k = kt + 16 * c;
+            hv[c] = k < in_dim ? *reinterpret_cast<const float4 *>(&hin[k][s]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+            for (int c = 0; c < KC; ++c)
+                acc[i][c] = fmaf(dv[i].w, hv[c].w, fmaf(dv[i].z, hv[c].z, fmaf(dv[i].y, hv[c].y, fmaf(dv[i].x, hv[c].x, acc[i][c]))));
+            bs[i] += (dv[i].x + dv[i].y) + (dv[i].z + dv[i].w);
+        }
     }
-    for (int j = threadIdx.x; j < kH; j += blockDim.x) {
-        float acc = 0.f;
-        for (int s = 0; s < nvalid; ++s) acc += dl[s][j];
-        gb[j] = acc;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int c = 0; c < KC; ++c)
+            if (kt + 16 * c < in_dim) put(gw + (jt + 16 * i) * in_dim + kt + 16 * c, acc[i][c], add);
+        if (kt == 0) put(gb + jt + 16 * i, bs[i], add);
     }
 }
 
-// d_new[k] = [h[k] > 0] sum_j W[j][k] d[j] for the calling thread's row (W [64][64])
-__device__ __forceinline__ void back_hidden(const float *sp, int w, const float *h, float *d) {
-    float nd[kH];
-    for (int k = 0; k < kH; ++k) {
-        float acc = 0.f;
-#pragma unroll 8
-        for (int j = 0; j < kH; ++j) acc = fmaf(sp[w + j * kH + k], d[j], acc);
-        nd[k] = h[k] > 0.f ? acc : 0.f;
+// out[k][s] = [h[k][s] > 0] sum_j W[j][k] d[j][s], w transposed ([k][j])
+__device__ __forceinline__ void back_hidden(const float (*w)[kWS], const float (*d)[kAS], const float (*h)[kAS],
+                                            float (*out)[kAS]) {
+    const int s0 = (threadIdx.x & 15) * 2, k0 = (threadIdx.x >> 4) * 4;
+    float acc[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0.f;
+#pragma unroll 4
+    for (int j = 0; j < kH; j += 4) {
+        float4 wv[4];
+        float2 a[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) wv[i] = *reinterpret_cast<const float4 *>(&w[k0 + i][j]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a[e] = *reinterpret_cast<const float2 *>(&d[j + e][s0]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float q[4] = {wv[i].x, wv[i].y, wv[i].z, wv[i].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                acc[i][0] = fmaf(q[e], a[e].x, acc[i][0]);
+                acc[i][1] = fmaf(q[e], a[e].y, acc[i][1]);
+            }
+        }
     }
 #pragma unroll
-    for (int k = 0; k < kH; ++k) d[k] = nd[k];
+    for (int i = 0; i < 4; ++i) {
+        const float2 hv = *reinterpret_cast<const float2 *>(&h[k0 + i][s0]);
+        *reinterpret_cast<float2 *>(&out[k0 + i][s0]) =
+            make_float2(hv.x > 0.f ? acc[i][0] : 0.f, hv.y > 0.f ? acc[i][1] : 0.f);
+    }
 }
 
 template <int F>
-__global__ void __launch_bounds__(kTrainB)
+__global__ void __launch_bounds__(kNet, 2)
     train_grad_kernel(const int B, const int *__restrict__ idx, const float *__restrict__ params,
                       const float *__restrict__ norm, const float *__restrict__ feat, const float *__restrict__ target,
                       const float *__restrict__ dy_in, float *__restrict__ part, float *__restrict__ loss_part) {
     constexpr Layout L(F);
-    extern __shared__ float sp[];
-    Rows<F> &R = *reinterpret_cast<Rows<F> *>(sp + rows_offset<F>());
-    load_net<F>(sp, params, norm);
+    extern __shared__ __align__(16) unsigned char net_raw[];
+    GradShared<F> &G = *reinterpret_cast<GradShared<F> *>(net_raw);
+    NetShared<F> &S = G.n;
+    load_net<F>(S, params, norm);
     __syncthreads();
     const int t = threadIdx.x;
-    const int s0 = blockIdx.x * kTrainB;
-    const int nvalid = min(kTrainB, B - s0);
     float *gp = part + (size_t)blockIdx.x * L.P;
-    if (t < nvalid) {
-        const long long s = idx[s0 + t];
-        const float y = forward<F>(sp, R, t, feat, s);
-        if (dy_in) {  // loss gradient supplied (neighbour-difference loss)
-            R.dy[t] = dy_in[s];
-            R.loss[t] = 0.f;
-        } else {
-            const float r = y - target[s];
-            R.dy[t] = 2.f * r / (float)B;
-            R.loss[t] = r * r;
+    const int tiles = (B - 1) / kTile + 1;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const bool add = tile != (int)blockIdx.x;
+        const int s0 = tile * kTile;
+        const int nvalid = min(kTile, B - s0);
+        const float y = forward<F>(S, feat, nvalid, [&](int s) { return (long long)idx[s0 + s]; });
+        if (t < kTile) {
+            float dy = 0.f, l = 0.f;  // absent samples contribute nothing
+            if (t < nvalid) {
+                const long long s = idx[s0 + t];
+                if (dy_in) {  // loss gradient supplied (neighbour-difference loss)
+                    dy = dy_in[s];
+                } else {
+                    const float r = y - target[s];
+                    dy = 2.f * r / (float)B;
+                    l = r * r;
+                }
+            }
+            G.dy[t] = dy;
+            G.loss[t] = l;
         }
-    } else {  // rows of absent samples contribute nothing
-        for (int k = 0; k <= F; ++k) R.x[t][k] = 0.f;
-        for (int k = 0; k < kRow; ++k) R.h1[t][k] = R.h2[t][k] = R.h3[t][k] = 0.f;
-        R.dy[t] = 0.f;
-        R.loss[t] = 0.f;
-    }
-    // d3 = dy W4 . [h3 > 0]
-    for (int j = 0; j < kH; ++j) R.d[t][j] = R.h3[t][j] > 0.f ? R.dy[t] * sp[L.w4 + j] : 0.f;
-    __syncthreads();
-    for (int k = t; k < kH; k += blockDim.x) {
-        float acc = 0.f;
-        for (int s = 0; s < nvalid; ++s) acc = fmaf(R.dy[s], R.h3[s][k], acc);
-        gp[L.w4 + k] = acc;
-    }
-    if (t == 0) {
-        float acc = 0.f, la = 0.f;
-        for (int s = 0; s < nvalid; ++s) {
-            acc += R.dy[s];
-            la += R.loss[s];
+        __syncthreads();
+        // gW4, gb4 and the loss; d3 = dy W4 . [h3 > 0] into d
+        if (t < kH) {
+            float acc = 0.f;
+#pragma unroll 8
+            for (int s = 0; s < kTile; ++s) acc = fmaf(G.dy[s], S.h3[t][s], acc);
+            put(gp + L.w4 + t, acc, add);
+        } else if (t < kH + 32) {
+            float acc = G.dy[t - kH], la = G.loss[t - kH];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                la += __shfl_xor_sync(0xffffffffu, la, off);
+            }
+            if (t == kH) {
+                put(gp + L.b4, acc, add);
+                put(loss_part + blockIdx.x, la, add);
+            }
         }
-        gp[L.b4] = acc;
-        loss_part[blockIdx.x] = la;
+        for (int e = t; e < kH * kTile; e += kNet) {
+            const int j = e / kTile, s = e % kTile;
+            G.d[j][s] = S.h3[j][s] > 0.f ? G.dy[s] * S.w4[j] : 0.f;
+        }
+        __syncthreads();
+        grad_outer<4>(G.d, S.h2, kH, gp + L.w3, gp + L.b3, add);
+        back_hidden(S.w3, G.d, S.h2, S.h3);  // d2 in h3's place
+        __syncthreads();
+        grad_outer<4>(S.h3, S.h1, kH, gp + L.w2, gp + L.b2, add);
+        back_hidden(S.w2, S.h3, S.h1, G.d);  // d1
+        __syncthreads();
+        grad_outer<2>(G.d, S.x, F, gp + L.w1, gp + L.b1, add);
+        __syncthreads();
     }
-    grad_outer(R.d, &R.h2[0][0], kRow, kH, nvalid, gp + L.w3, gp + L.b3);
-    __syncthreads();
-    back_hidden(sp, L.w3, R.h2[t], R.d[t]);
-    __syncthreads();
-    grad_outer(R.d, &R.h1[0][0], kRow, kH, nvalid, gp + L.w2, gp + L.b2);
-    __syncthreads();
-    back_hidden(sp, L.w2, R.h1[t], R.d[t]);
-    __syncthreads();
-    grad_outer(R.d, &R.x[0][0], F + 1, F, nvalid, gp + L.w1, gp + L.b1);
 }
 
-// Network outputs of the batch samples into y[s] (global sample index), and a
-// zeroed loss gradient dy[s] for the pair kernel.
+// Network outputs of the batch samples into y[s] (global sample index), a zeroed loss
+// gradient dy[s] and loss for the pair kernel.
 template <int F>
-__global__ void __launch_bounds__(kTrainB)
+__global__ void __launch_bounds__(kNet, 2)
     forward_batch_kernel(const int B, const int *__restrict__ idx, const float *__restrict__ params,
                          const float *__restrict__ norm, const float *__restrict__ feat, float *__restrict__ y,
-                         float *__restrict__ dy) {
-    extern __shared__ float sp[];
-    Rows<F> &R = *reinterpret_cast<Rows<F> *>(sp + rows_offset<F>());
-    load_net<F>(sp, params, norm);
+                         float *__restrict__ dy, float *__restrict__ loss) {
+    extern __shared__ __align__(16) unsigned char net_raw[];
+    NetShared<F> &S = *reinterpret_cast<NetShared<F> *>(net_raw);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *loss = 0.f;
+    load_net<F>(S, params, norm);
     __syncthreads();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const long long s = idx[b];
-    y[s] = forward<F>(sp, R, threadIdx.x, feat, s);
+    const int s0 = blockIdx.x * kTile;
+    const int nvalid = min(kTile, B - s0);
+    const float v = forward<F>(S, feat, nvalid, [&](int s) { return (long long)idx[s0 + s]; });
+    if ((int)threadIdx.x >= nvalid) return;
+    const long long s = idx[s0 + threadIdx.x];
+    y[s] = v;
     dy[s] = 0.f;
 }
 
@@ -439,22 +536,36 @@ __global__ void pair_loss_kernel(const int B, const int *__restrict__ idx, const
     }
 }
 
-// Sum of the CTA partials (fixed order) -> grad (optional) and an Adam step
-// (optional, lr > 0): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
-// p -= lr (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + 1e-8).
-__global__ void adam_kernel(const int P, const int nparts, const float *__restrict__ part,
-                            const float *__restrict__ loss_part, float *__restrict__ params, float *__restrict__ m,
-                            float *__restrict__ v, const float lr, const float bc1, const float bc2,
-                            float *__restrict__ grad_out, float *__restrict__ loss_out) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0 && loss_out) {
+// Sum of the block partials (a fixed order: eight strided sums, then those) -> grad
+// (optional) and an Adam step (optional, lr > 0): m = b1 m + (1-b1) g, v = b2 v + (1-b2)
+// g^2, p -= lr (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + 1e-8).  A block takes 32
+// parameters: one warp per strided sum, so a parameter's partials are not one chain.
+constexpr int kAdam = 256;
+__global__ void __launch_bounds__(kAdam)
+    adam_kernel(const int P, const int nparts, const float *__restrict__ part,
+                const float *__restrict__ loss_part, float *__restrict__ params, float *__restrict__ m,
+                float *__restrict__ v, const float lr, const float bc1, const float bc2,
+                float *__restrict__ grad_out, float *__restrict__ loss_out) {
+    __shared__ float sums[kAdam / 32][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    if (blockIdx.x == 0 && wid == 0 && loss_out) {
         double l = 0.0;
-        for (int b = 0; b < nparts; ++b) l += (double)loss_part[b];
-        *loss_out = (float)l;
+        for (int b = lane; b < nparts; b += 32) l += (double)loss_part[b];
+        l = warp_sum(l);
+        if (lane == 0) *loss_out = (float)l;
     }
-    if (p >= P) return;
     float g = 0.f;
-    for (int b = 0; b < nparts; ++b) g += part[(size_t)b * P + p];
+    if (p < P) {
+#pragma unroll 8
+        for (int b = wid; b < nparts; b += kAdam / 32) g += part[(size_t)b * P + p];
+    }
+    sums[wid][lane] = g;
+    __syncthreads();
+    if (wid != 0 || p >= P) return;
+    g = 0.f;
+#pragma unroll
+    for (int k = 0; k < kAdam / 32; ++k) g += sums[k][lane];
     if (grad_out) grad_out[p] = g;
     if (lr > 0.f) {
         const float mm = 0.9f * m[p] + 0.1f * g;
@@ -572,18 +683,18 @@ int apd_warmstart_create(apd_mlp **out, int32_t dim, const float *params, const 
          cudaMemset(net->v, 0, P * sizeof(float)) == cudaSuccess;
     if (ok && dim == 2)
         ok = cudaFuncSetAttribute(predict_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)net_smem<F2>()) == cudaSuccess &&
+                                  (int)sizeof(NetShared<F2>)) == cudaSuccess &&
              cudaFuncSetAttribute(forward_batch_kernel<F2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)net_smem<F2>()) == cudaSuccess &&
+                                  (int)sizeof(NetShared<F2>)) == cudaSuccess &&
              cudaFuncSetAttribute(train_grad_kernel<F2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)net_smem<F2>()) == cudaSuccess;
+                                  (int)sizeof(GradShared<F2>)) == cudaSuccess;
     if (ok && dim == 3)
         ok = cudaFuncSetAttribute(predict_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)net_smem<F3>()) == cudaSuccess &&
+                                  (int)sizeof(NetShared<F3>)) == cudaSuccess &&
              cudaFuncSetAttribute(forward_batch_kernel<F3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)net_smem<F3>()) == cudaSuccess &&
+                                  (int)sizeof(NetShared<F3>)) == cudaSuccess &&
              cudaFuncSetAttribute(train_grad_kernel<F3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)net_smem<F3>()) == cudaSuccess;
+                                  (int)sizeof(GradShared<F3>)) == cudaSuccess;
     if (!ok) {
         apd_warmstart_destroy(net);
         return APD_ERR_CUDA;
@@ -650,20 +761,20 @@ int apd_warmstart_predict(apd_mlp *net, int32_t count, const int64_t *offsets, c
     rc = ensure_instances(net, count, offsets, box, st);
     if (rc != APD_OK) return rc;
     const long long total = offsets[count];
-    const int blocks = (int)((total + kTrainB - 1) / kTrainB);
+    const int blocks = (int)((total + kTile - 1) / kTile);
     if (net->dim == 2)
-        predict_kernel<2><<<blocks, kTrainB, net_smem<F2>(), st>>>(count, net->offs, net->box, net->params,
-                                                                    net->norm, features, w_out);
+        predict_kernel<2><<<blocks, kNet, sizeof(NetShared<F2>), st>>>(count, net->offs, net->box, net->params,
+                                                                       net->norm, features, w_out);
     else
-        predict_kernel<3><<<blocks, kTrainB, net_smem<F3>(), st>>>(count, net->offs, net->box, net->params,
-                                                                    net->norm, features, w_out);
+        predict_kernel<3><<<blocks, kNet, sizeof(NetShared<F3>), st>>>(count, net->offs, net->box, net->params,
+                                                                       net->norm, features, w_out);
     return ws_rc(cudaGetLastError());
 }
 
 static int train_step_impl(apd_mlp *net, int32_t batch, const int32_t *idx, const float *features,
                            const float *targets, const float *dy_in, float lr, float *grad_out, float *loss_out,
                            cudaStream_t st) {
-    const int nparts = (batch + kTrainB - 1) / kTrainB;
+    const int nparts = std::min((batch - 1) / kTile + 1, kMaxParts);
     if (nparts > net->part_cap) {
         if (net->part) cudaFree(net->part);
         if (net->loss_part) cudaFree(net->loss_part);
@@ -675,20 +786,19 @@ static int train_step_impl(apd_mlp *net, int32_t batch, const int32_t *idx, cons
             return APD_ERR_CUDA;
         net->part_cap = nparts;
     }
-    const size_t smem = net->F == F2 ? net_smem<F2>() : net_smem<F3>();
     if (net->F == F2)
-        train_grad_kernel<F2><<<nparts, kTrainB, smem, st>>>(batch, idx, net->params, net->norm, features, targets,
-                                                             dy_in, net->part, net->loss_part);
+        train_grad_kernel<F2><<<nparts, kNet, sizeof(GradShared<F2>), st>>>(
+            batch, idx, net->params, net->norm, features, targets, dy_in, net->part, net->loss_part);
     else
-        train_grad_kernel<F3><<<nparts, kTrainB, smem, st>>>(batch, idx, net->params, net->norm, features, targets,
-                                                             dy_in, net->part, net->loss_part);
+        train_grad_kernel<F3><<<nparts, kNet, sizeof(GradShared<F3>), st>>>(
+            batch, idx, net->params, net->norm, features, targets, dy_in, net->part, net->loss_part);
     float bc1 = 1.f, bc2 = 1.f;
     if (lr > 0.f) {
         net->step += 1;
         bc1 = 1.f - powf(0.9f, (float)net->step);
         bc2 = 1.f - powf(0.999f, (float)net->step);
     }
-    adam_kernel<<<(net->P + 255) / 256, 256, 0, st>>>(net->P, nparts, net->part, net->loss_part, net->params, net->m,
+    adam_kernel<<<(net->P + 31) / 32, kAdam, 0, st>>>(net->P, nparts, net->part, net->loss_part, net->params, net->m,
                                                       net->v, lr, bc1, bc2, grad_out, loss_out);
     return ws_rc(cudaGetLastError());
 }
@@ -706,18 +816,18 @@ int apd_warmstart_train_step_pairs(apd_mlp *net, int32_t batch, const int32_t *i
         !(mu >= 0.f))
         return APD_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    const int blocks = (batch + kTrainB - 1) / kTrainB;
-    if (net->F == F2)
-        forward_batch_kernel<F2><<<blocks, kTrainB, net_smem<F2>(), st>>>(batch, idx, net->params, net->norm,
-                                                                           features, y_buf, dy_buf);
-    else
-        forward_batch_kernel<F3><<<blocks, kTrainB, net_smem<F3>(), st>>>(batch, idx, net->params, net->norm,
-                                                                           features, y_buf, dy_buf);
-    if (loss_out && cudaMemsetAsync(loss_out, 0, sizeof(float), st) != cudaSuccess) return APD_ERR_CUDA;
     if (!net->pair_loss && cudaMalloc((void **)&net->pair_loss, sizeof(float)) != cudaSuccess) return APD_ERR_CUDA;
+    float *loss = loss_out ? loss_out : net->pair_loss;
+    const int blocks = (batch - 1) / kTile + 1;
+    if (net->F == F2)
+        forward_batch_kernel<F2><<<blocks, kNet, sizeof(NetShared<F2>), st>>>(batch, idx, net->params, net->norm,
+                                                                              features, y_buf, dy_buf, loss);
+    else
+        forward_batch_kernel<F3><<<blocks, kNet, sizeof(NetShared<F3>), st>>>(batch, idx, net->params, net->norm,
+                                                                              features, y_buf, dy_buf, loss);
     pair_loss_kernel<<<(batch + 255) / 256, 256, 0, st>>>(batch, idx, knn, y_buf, targets,
                                                           1.f / ((float)batch * (float)kNN), mu, dy_buf,
-                                                          loss_out ? loss_out : net->pair_loss);
+                                                          loss);
     const int rc = ws_rc(cudaGetLastError());
     if (rc != APD_OK) return rc;
     return train_step_impl(net, batch, idx, features, targets, dy_buf, lr, grad_out, nullptr, st);
