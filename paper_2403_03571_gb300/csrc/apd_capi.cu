@@ -3,6 +3,7 @@
 // moments + eqs. (2.7)-(2.8)), the L-BFGS weight solve of Algorithm 2 and the
 // Lloyd loop of Algorithm 3.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -122,6 +123,7 @@ struct TrialStep {
     const double *W;
     double t;
     const double *p;
+    const PushState *push;  // the history the trial's push follows
 };
 
 constexpr size_t kGraphCap = 16;  // evaluation graphs kept per workspace
@@ -223,7 +225,7 @@ int enqueue_assign(const GridDev &g_in, int n, const double *x, const double *A,
         const unsigned full_max = (unsigned)(kIncFullMax * (double)win_pixels(g));
         APD_TRY(cuda_ok(launch_eval_begin(n, step ? step->W : w, step ? step->t : 0.0, step ? step->p : nullptr,
                                           const_cast<double *>(w), mom, ws, st, form_p,
-                                          inc_on ? ws.inc_w0 : nullptr, full_max)));
+                                          inc_on ? ws.inc_w0 : nullptr, full_max, step ? step->push : nullptr)));
     } else {
         if (step) APD_TRY(cuda_ok(launch_axpy(n, step->W, step->t, step->p, const_cast<double *>(w), st)));
         ws.cond_read = !empty && prec != APD_FP32 && tc_tile_count(g) <= ws.tc_tile_cap;
@@ -358,9 +360,35 @@ struct Solver {
         // the records' positions and matrices are built once per solve
         APD_TRY(enqueue_assign(g, n, x, A, Wp, prec, ws, nullptr, ws.moments, s, geometry_ready, step, inc_mode));
         APD_TRY(cuda_ok(launch_dual(g, n, x, A, Wp, v, pdir, ws.moments, ws, nullptr, ws.grad, gf_out,
-                                    nullptr, s)));
+                                    nullptr, s, ws.sc_host)));
         ws.kernel_launches += 1;
-        return cuda_ok(cudaMemcpyAsync(ws.sc_host, ws.sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
+        if (step) {  // the pair of this trial, before its value is known
+            APD_TRY(cuda_ok(launch_lbfgs_push(n, kHistCap, history, ws.push_state, true, ws.Wbest, ws, s)));
+            ws.kernel_launches += 1;
+        }
+        return APD_OK;
+    }
+
+    // Waits for the evaluation's scalars: its last kernel writes them, then their number,
+    // into the pinned host copy, while the trial's push runs on.  (With a copy node, a stream
+    // synchronisation and the push launched after it a trial at n = 20 took 55 us, so 38 us.)
+    // The stream is asked now and then, for errors.
+    int wait_scalars() {
+        const unsigned want = ws.sc_seq + 1u;
+        const volatile unsigned *seq = &ws.sc_host->seq;
+        for (unsigned spin = 1; *seq != want; ++spin) {
+            if (spin & 0x3fffu) continue;
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e == cudaErrorNotReady) {
+                cudaGetLastError();
+                continue;
+            }
+            if (e != cudaSuccess) return cuda_ok(e);
+            if (*seq != want) return APD_ERR_CUDA;  // the stream has run dry without them
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        ws.sc_seq = want;
+        return APD_OK;
     }
 
     // A weights-only evaluation replayed from a captured graph (captured on
@@ -370,10 +398,10 @@ struct Solver {
         eg = nullptr;
         if (!ws.graphs || !geometry_ready || ws.shard_world > 1) return APD_OK;
         struct Key {
-            int dim, res[3], kz0, kz1, n, prec, prune, sorted, profiling, has_step, form_p, inc;
+            int dim, res[3], kz0, kz1, n, prec, prune, sorted, profiling, has_step, form_p, inc, history;
             uint32_t wait_limit, use_tc;
             double lo[3], h[3];
-            const void *ptr[9];
+            const void *ptr[14];
         } k;
         std::memset(&k, 0, sizeof k);
         k.dim = g.dim;
@@ -393,12 +421,13 @@ struct Solver {
         const bool form_p = ws.p_pending && step && step->p == ws.p;  // as enqueue_assign decides it
         k.form_p = form_p ? 1 : 0;
         k.inc = inc_mode;
+        k.history = step ? history : 0;
         k.wait_limit = ws.wait_limit;
         // the scorer the captured pass takes (the seeds' conditioning can change it between solves)
         const bool tc = use_tensor_cores(g, prec, ws, true);
         k.use_tc = tc ? 1u : 0u;
-        const void *ptrs[9] = {x, A, v, Wp, gf_out, pdir, step ? step->W : nullptr, step ? step->p : nullptr,
-                               ws.moments};
+        const void *ptrs[14] = {x, A, v, Wp, gf_out, pdir, step ? step->W : nullptr, step ? step->p : nullptr,
+                                ws.moments, ws.gf, ws.S, ws.Y, ws.rho, ws.gram};
         std::memcpy(k.ptr, ptrs, sizeof ptrs);
         const unsigned char *kb = reinterpret_cast<const unsigned char *>(&k);
         for (EvalGraph &e : ws.graph_cache)
@@ -474,7 +503,7 @@ struct Solver {
             APD_TRY(cuda_ok(set_eval_begin_node(eg->exec, eg->begin, n, step->W, step->t, step->p,
                                                 const_cast<double *>(Wp), ws.moments, ws, form_p,
                                                 eg->recorded ? ws.inc_w0 : nullptr,
-                                                (unsigned)(kIncFullMax * (double)win_pixels(g)))));
+                                                (unsigned)(kIncFullMax * (double)win_pixels(g)), step->push)));
         APD_TRY(cuda_ok(cudaGraphLaunch(eg->exec, st)));
         ws.kernel_launches += eg->launches;
         ws.last_pixels = eg->pixels;
@@ -494,7 +523,7 @@ struct Solver {
         APD_TRY(graph_eval(Wp, gf_out, pdir, step, eg));
         if (!eg) APD_TRY(enqueue_eval(Wp, gf_out, pdir, step, st));
         geometry_ready = true;
-        APD_TRY(cuda_ok(cudaStreamSynchronize(st)));
+        APD_TRY(wait_scalars());
         // a re-decision ran no scoring kernel: its (empty) launch is not timed
         const bool redecided = ws.inc_recorded && ws.sc_host->inc_go;
         if (redecided) {
@@ -506,6 +535,7 @@ struct Solver {
         }
         if (eg && eg->e0 && ws.profiling && !redecided) {
             float ms = 0.f;
+            APD_TRY(cuda_ok(cudaEventSynchronize(eg->e1)));
             APD_TRY(cuda_ok(cudaEventElapsedTime(&ms, eg->e0, eg->e1)));
             ws.prof_ms_graph += ms;
             ws.prof_n_graph += 1;
@@ -536,8 +566,9 @@ struct Solver {
         if (err < best_err) {
             best_err = err;
             best_g = h.g;
-            APD_TRY(cuda_ok(cudaMemcpyAsync(ws.Wbest, Wp, (size_t)n * sizeof(double),
-                                            cudaMemcpyDeviceToDevice, st)));
+            if (!step)  // a trial's push has copied it
+                APD_TRY(cuda_ok(cudaMemcpyAsync(ws.Wbest, Wp, (size_t)n * sizeof(double),
+                                                cudaMemcpyDeviceToDevice, st)));
             last_is_best = true;
         }
         return APD_OK;
@@ -550,7 +581,9 @@ struct Solver {
     // evaluation's scalars, so the direction needs no read of its own; a
     // direction that is not a descent direction ends the search (LS_NOT_DESCENT)
     // unless that first point has already converged.
-    int line_search(double f0, double t_init, LsResult &res, double &f_acc) {
+    // Each trial's push is queued behind it (the accepted point is the last one evaluated);
+    // a pair still undecided at the first trial is settled in ps by its scalars.
+    int line_search(double f0, double t_init, PushState &ps, LsResult &res, double &f_acc) {
         const double c1 = 1e-4, c2 = 0.9;
         double dphi0 = 0.0;
         double t_prev = 0.0, phi_prev = f0, dphi_prev = 0.0;
@@ -558,8 +591,18 @@ struct Solver {
         double best_t = 0.0, best_phi = f0;
         double cur_t = -1.0;  // t at which Wt/gft were last evaluated
         auto evaluate = [&](double tt, double &phi, double &dphi, double &err) -> int {
-            const TrialStep step{ws.W, tt, ws.p};  // Wt = W + tt p, formed by the evaluation's first kernel
+            const TrialStep step{ws.W, tt, ws.p, &ps};  // Wt = W + tt p, formed by the evaluation's first kernel
+            ps.eps = eps;
+            ps.best_err = best_err;
             APD_TRY(eval(ws.Wt, ws.gft, ws.p, phi, dphi, err, &step));
+            if (ps.pend) {
+                if (ws.sc_host->pair_ok) {
+                    ps.newest = ps.p_slot;
+                    ps.hist = ps.hist_acc;
+                    ps.gamma = ws.sc_host->sy / ws.sc_host->yy;
+                }
+                ps.pend = 0;
+            }
             cur_t = tt;
             return APD_OK;
         };
@@ -714,37 +757,36 @@ struct Solver {
     // and read once; a pair pushed after an accepted step is taken or dropped by
     // the device (its curvature test) and the host learns which at that read.
     int iterate(double f0, double *out, bool &converged) {
-        int hist = 0, newest = kHistCap - 1;
-        double gamma = 1.0;
+        PushState ps{};
+        ps.newest = kHistCap - 1;
+        ps.gamma = 1.0;
+        ps.history = history;
         if (ws.carry_on && ws.carry.valid) {  // continue the history of the previous solve
-            hist = std::min(ws.carry.hist, history);
-            newest = ws.carry.newest;
-            gamma = ws.carry.gamma;
+            ps.hist = std::min(ws.carry.hist, history);
+            ps.newest = ws.carry.newest;
+            ps.gamma = ws.carry.gamma;
         }
         auto keep = [&]() {
             if (!ws.carry_on) return;
-            ws.carry.hist = hist;
-            ws.carry.newest = newest;
-            ws.carry.gamma = gamma;
+            ws.carry.hist = ps.hist;
+            ws.carry.newest = ps.newest;
+            ws.carry.gamma = ps.gamma;
             ws.carry.valid = true;
         };
         int fails = 0;
-        bool pending = false;  // a pushed pair whose test result is not read yet
-        int p_slot = 0;
         bool dir_ready = false;  // the last push also formed this direction's coefficients
         while (evals < max_evals && !(stall_evals > 0 && evals - last_gain >= stall_evals)) {
-            const int hist_acc = std::min(hist + 1, history);
             // the coefficients of p come from the last push or from the dots kernel;
             // the first trial's eval_begin forms p from them (and <grad f, p>)
             if (!dir_ready) {
-                APD_TRY(cuda_ok(launch_lbfgs_coefficients(n, hist, newest, kHistCap, gamma, pending, hist_acc,
-                                                          p_slot, ws, st)));
+                APD_TRY(cuda_ok(launch_lbfgs_coefficients(n, ps.hist, ps.newest, kHistCap, ps.gamma, false, ps.hist,
+                                                          ps.newest, ws, st)));
                 ws.kernel_launches += 1;
             }
             ws.p_pending = true;
             dir_ready = false;
             double t0 = 1.0;
-            if (!pending && hist == 0) {
+            if (!ps.pend && ps.hist == 0) {
                 // first step (or after a reset): p = -grad f; take t0 ~ 1 / H_ii with the
                 // cell-volume sensitivity H_ii ~ D V^(1 - 2/D) of a cell of volume V = |Omega| / n
                 const double V = measure / (double)n;
@@ -752,20 +794,11 @@ struct Solver {
             }
             LsResult res;
             double f_acc = f0;
-            const int evals_before = evals;
-            APD_TRY(line_search(f0, t0, res, f_acc));
-            if (pending && evals > evals_before) {
-                if (ws.sc_host->pair_ok) {
-                    newest = p_slot;
-                    hist = hist_acc;
-                    gamma = ws.sc_host->sy / ws.sc_host->yy;
-                }
-                pending = false;
-            }
+            APD_TRY(line_search(f0, t0, ps, res, f_acc));
             if (res == LS_NOT_DESCENT) {
-                if (hist == 0) break;
-                hist = 0;
-                gamma = 1.0;
+                if (ps.hist == 0) break;
+                ps.hist = 0;
+                ps.gamma = 1.0;
                 continue;
             }
             if (res == LS_CONVERGED) {
@@ -776,22 +809,20 @@ struct Solver {
             }
             if (res == LS_BUDGET) break;
             if (res == LS_FAIL) {
-                if (hist == 0 || ++fails > 3) break;
-                hist = 0;
-                gamma = 1.0;
+                if (ps.hist == 0 || ++fails > 3) break;
+                ps.hist = 0;
+                ps.gamma = 1.0;
                 continue;
             }
             fails = 0;
             ++iters;
-            const int slot = (newest + 1) % kHistCap;
-            // Gram entries with the pairs kept beside it if it is accepted, and the
-            // next direction's coefficients for either outcome of its curvature test
-            const int next_acc = std::min(hist + 1, history);
-            APD_TRY(cuda_ok(launch_lbfgs_push(n, slot, kHistCap, next_acc - 1, true, hist, next_acc, gamma, ws, st)));
-            ws.kernel_launches += 1;
+            // the accepted trial's push has stored its pair in the next slot, the Gram entries with
+            // the pairs kept beside it and the next direction's coefficients, for either outcome of
+            // its curvature test
+            ps.p_slot = (ps.newest + 1) % kHistCap;
+            ps.hist_acc = std::min(ps.hist + 1, history);
+            ps.pend = 1;
             dir_ready = true;
-            pending = true;
-            p_slot = slot;
             std::swap(ws.W, ws.Wt);
             std::swap(ws.gf, ws.gft);
             f0 = f_acc;
@@ -924,7 +955,8 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
     alloc((void **)&w.tc_axis, (size_t)3 * w.tc_tile_cap * sizeof(float4));
     // super-tiles: at most one per tile
     w.part_rows = (int)nb;
-    alloc((void **)&w.part, nb * kPartStride * sizeof(double));
+    // one row per warp of an evaluation's first kernel (part_rows: the blocks the sums are made in)
+    alloc((void **)&w.part, std::max(nb, (size_t)w.n_pad_max / 32) * kPartStride * sizeof(double));
     if (w.n_pad_max <= kSortMax) {
         // point sets: about 32 tiles a seed, room for eight polynomials a tile
         w.pts_bytes = (size_t)std::min<long long>(32ll * std::max(max_n, 64), 1ll << 17) * (16 + 8 * 48);
@@ -945,12 +977,14 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
     w.lb_rows = w.sms;
     alloc((void **)&w.lb_part, (size_t)w.lb_rows * kLbfgsDots * sizeof(double));
     alloc((void **)&w.lb_coef, sizeof(LbfgsCoef));
+    alloc((void **)&w.push_state, sizeof(PushState));
     alloc((void **)&w.rho, kHistCap * sizeof(double));
     alloc((void **)&w.X, (size_t)max_n * dim * sizeof(double));
     alloc((void **)&w.vbuf, (size_t)max_n * sizeof(double));
     alloc((void **)&w.wfeat, (size_t)max_n * kWarmFeatMax * sizeof(float));
     alloc((void **)&w.wpred, (size_t)max_n * sizeof(double));
     if (ok && cudaMallocHost((void **)&w.sc_host, sizeof(DevScalars)) != cudaSuccess) ok = false;
+    if (ok) std::memset(w.sc_host, 0, sizeof(DevScalars));
     if (ok && cudaMemset(w.sc, 0, sizeof(DevScalars)) != cudaSuccess) ok = false;
     if (ok && cudaMemset(w.pairs_scored, 0, sizeof(unsigned long long)) != cudaSuccess) ok = false;
     if (ok && cudaMemset(w.recs, 0, (size_t)w.n_pad_max * sizeof(SeedRec)) != cudaSuccess) ok = false;
@@ -971,7 +1005,7 @@ void apd_workspace_destroy(apd_workspace *ws) {
     if (w.cap_stream) cudaStreamDestroy(w.cap_stream);
     if (w.cond_ev) cudaEventDestroy(w.cond_ev);
     void *ptrs[] = {w.recs, w.recs32, w.recs_tmp, w.codes, w.scodes, w.perm, w.recs32s, w.tc_centre, w.tc_start, w.tc_meta, w.tc_texcl, w.tc_list, w.tc_bops, w.tc_axis, w.moments, w.flags, w.flag_gi, w.pairs_scored, w.groups, w.sc, w.part, w.grad, w.W, w.Wt, w.p, w.gf, w.gft,
-                    w.Wbest, w.S, w.Y, w.gram, w.lb_part, w.lb_coef, w.rho, w.X, w.vbuf, w.wfeat, w.wpred,
+                    w.Wbest, w.S, w.Y, w.gram, w.lb_part, w.lb_coef, w.push_state, w.rho, w.X, w.vbuf, w.wfeat, w.wpred,
                     w.S2, w.Y2, w.gram2, w.rho2, w.inc_labels, w.inc_gap, w.inc_rec, w.inc_hist, w.inc_drift, w.inc_mom0, w.inc_w0, w.inc_aux, w.pts_tiles, w.pts_geo};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -1082,16 +1116,22 @@ int apd_lbfgs_check(int32_t n, int32_t hist, const double *S, const double *Y, c
     w.lb_rows = w.sms;
     alloc((void **)&w.lb_part, (size_t)w.lb_rows * kLbfgsDots * sizeof(double));
     alloc((void **)&w.lb_coef, sizeof(LbfgsCoef));
+    alloc((void **)&w.push_state, sizeof(PushState));
     alloc((void **)&w.sc, sizeof(DevScalars));
     cudaStream_t st = 0;
     // pair k enters as W = 0, Wt = s_k, gf = 0, gft = y_k in slot k
     if (ok) ok = cudaMemset(w.W, 0, nb) == cudaSuccess && cudaMemset(w.gf, 0, nb) == cudaSuccess &&
                  cudaMemset(w.sc, 0, sizeof(DevScalars)) == cudaSuccess;
+    auto push = [&](int k, bool dir) {  // pair k behind the k pairs before it
+        const PushState ps{k, (k - 1 + kHistCap) % kHistCap, 1.0, kHistCap - 1, 0, 0, 0, 0.0, 0.0};
+        return cudaMemcpy(w.push_state, &ps, sizeof ps, cudaMemcpyHostToDevice) == cudaSuccess &&
+               launch_lbfgs_push(n, kHistCap, kHistCap - 1, w.push_state, dir, nullptr, w, st) == cudaSuccess;
+    };
     const int plain = fused ? hist - 1 : hist;
     for (int k = 0; ok && k < plain; ++k) {
         ok = cudaMemcpy(w.Wt, S + (size_t)k * n, nb, cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(w.gft, Y + (size_t)k * n, nb, cudaMemcpyHostToDevice) == cudaSuccess &&
-             launch_lbfgs_push(n, k, kHistCap, k, false, 0, 0, 1.0, w, st) == cudaSuccess;
+             push(k, false);
     }
     if (ok && !fused) {
         // the newest pair is the pending one, taken by the direction kernels if it passed
@@ -1105,7 +1145,7 @@ int apd_lbfgs_check(int32_t n, int32_t hist, const double *S, const double *Y, c
              cudaMemcpy(w.gft, g, nb, cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(w.p, Y + (size_t)(hist - 1) * n, nb, cudaMemcpyHostToDevice) == cudaSuccess &&
              launch_axpy(n, w.gft, -1.0, w.p, w.gf, st) == cudaSuccess &&
-             launch_lbfgs_push(n, hist - 1, kHistCap, hist - 1, true, hist - 1, hist, 1.0, w, st) == cudaSuccess;
+             push(hist - 1, true);
         std::swap(w.gf, w.gft);
         if (ok) ok = launch_lbfgs_pdir(n, w, st) == cudaSuccess;
     }

@@ -89,6 +89,7 @@ struct DevScalars {
     int inc_go;                         // this incremental pass re-decides from the record (else records)
     int inc_valid;                      // a record of this solve exists
     float wref_h, wref_l;               // w_ref as an FP32 pair
+    unsigned int seq;                   // solver evaluations finished (their scalars are in the host's copy)
 };
 
 // Partial sums per block row of the L-BFGS dot-product kernels: the push's
@@ -98,6 +99,15 @@ constexpr int kPartStride = 6;  // doubles per block row of Workspace::part
 // Bins of the incremental record's margin histogram: a positive float margin
 // falls in bin (its bits >> 21), four bins per octave (bin 0: no margin).
 constexpr int kIncBins = 1024;
+
+// State of the L-BFGS history at a push (see lbfgs_push_kernel).
+struct PushState {
+    int hist, newest;      // pairs in use, newest slot
+    double gamma;
+    int history;           // pairs kept at most
+    int pend, hist_acc, p_slot;  // an undecided pair in p_slot, and the pairs in use if it was taken
+    double eps, best_err;
+};
 
 // Coefficients of an L-BFGS direction p = -gamma g + sum_k (cy_k y_k + cs_k s_k)
 // over the pairs in slot[0..hist) (device; written by the direction's first kernel).
@@ -174,7 +184,8 @@ struct Workspace {
     int32_t *flag_gi = nullptr;         // [max_j] FP32 best seed of each queued pixel (-1: none)
     GroupBound *groups = nullptr;       // [n_pad_max / 32] bounds of the scan-order seed groups
     DevScalars *sc = nullptr;           // device
-    DevScalars *sc_host = nullptr;      // pinned host mirror
+    DevScalars *sc_host = nullptr;      // pinned host mirror, written by a solver evaluation's last kernel
+    unsigned int sc_seq = 0;            // number of the last evaluation the host has read
     PtsGeo *pts_geo = nullptr;          // tiling of the last point set
     uint8_t *pts_tiles = nullptr;       // its tiles' headers, then their polynomials (pts_bytes)
     size_t pts_bytes = 0;
@@ -190,6 +201,7 @@ struct Workspace {
     double *lb_part = nullptr;          // [lb_rows][kLbfgsDots] per-block partial sums of the L-BFGS kernels
     int lb_rows = 0;
     LbfgsCoef *lb_coef = nullptr;       // the last direction's coefficients
+    PushState *push_state = nullptr;    // the push's state of the trial in flight (device)
     bool p_pending = false;             // lb_coef holds a direction that ws.p does not yet hold
     // incremental evaluation (weight solves with the pruned tensor-core scorer): a
     // full pass records each pixel's label, runner-up and certified cost margins,
@@ -440,7 +452,8 @@ cudaError_t launch_masked_refine(const GridDev &gc, const GridDev &gf, int r, in
 // recorded pixels have a g3 margin within the drift (sc->inc_go), else record.
 cudaError_t launch_eval_begin(int n, const double *W0, double t, const double *pdir, double *Wt,
                               unsigned long long *mom, Workspace &ws, cudaStream_t st, bool form_p = false,
-                              const double *w0 = nullptr, unsigned full_max = 0u);
+                              const double *w0 = nullptr, unsigned full_max = 0u,
+                              const PushState *push = nullptr);
 // start of an evaluation at new positions: seed records (FP64 x, w; FP32 symmetric A) in
 // scan order, their statistics (max w, max ||A||_F, min lambda bound), cleared counters
 // and, when mom is given, n_mom cleared moment words; box: the Morton codes' box, on
@@ -487,7 +500,7 @@ cudaError_t launch_tie_gap(const GridDev &g, int n, const double *x, const doubl
 cudaError_t launch_dual(const GridDev &g, int n, const double *x, const double *A, const double *w,
                         const double *v, const double *p_dir, const unsigned long long *moments,
                         Workspace &ws, double *g_out, double *grad_out, double *gf_out,
-                        double *err_out, cudaStream_t st);
+                        double *err_out, cudaStream_t st, DevScalars *host = nullptr);
 // discrete centroids from the moments (empty cells keep x)
 cudaError_t launch_centroids(const GridDev &g, int n, const double *x,
                              const unsigned long long *moments, double *x_out, cudaStream_t st);
@@ -502,7 +515,7 @@ cudaError_t launch_lbfgs_direction(int n, int hist, int newest, int cap, double 
 // for the gradient gft (taken with the pair if it passes the curvature test:
 // hist_acc pairs; else the hist pairs before it and gamma).  launch_lbfgs_pdir
 // then forms p from the last coefficients and the gradient ws.gf.
-cudaError_t launch_lbfgs_push(int n, int slot, int cap, int nprev, bool dir, int hist, int hist_acc, double gamma,
+cudaError_t launch_lbfgs_push(int n, int cap, int history, const PushState *state, bool dir, double *Wbest,
                               Workspace &ws, cudaStream_t st);
 cudaError_t launch_lbfgs_pdir(int n, Workspace &ws, cudaStream_t st);
 // Records the pending profiling start event (if any) on st: called by the
@@ -519,7 +532,8 @@ inline cudaError_t record_scoring_start(Workspace &ws, cudaStream_t st) {
 const void *eval_begin_kernel_fn();
 cudaError_t set_eval_begin_node(cudaGraphExec_t exec, cudaGraphNode_t node, int n, const double *W0, double t,
                                 const double *pdir, double *Wt, unsigned long long *mom, Workspace &ws,
-                                bool form_p, const double *w0, unsigned full_max);
+                                bool form_p, const double *w0, unsigned full_max,
+                              const PushState *push = nullptr);
 // the direction's coefficients only (p is then formed by the next trial's eval_begin)
 cudaError_t launch_lbfgs_coefficients(int n, int hist, int newest, int cap, double gamma, bool use_pair,
                                       int hist_acc, int newest_acc, Workspace &ws, cudaStream_t st);

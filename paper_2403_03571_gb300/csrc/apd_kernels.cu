@@ -2,7 +2,11 @@
 // moments, the discrete centroids of Algorithm 3, and the vector kernels of
 // the L-BFGS weight solve (Algorithm 2).
 #include <float.h>
+#include <math.h>
+#include <stddef.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "apd_common.cuh"
 
@@ -10,7 +14,16 @@ namespace apd {
 
 namespace {
 
-constexpr int kRedThreads = 1024;
+// Counts a block in: the caller's earlier writes (and those a barrier made visible to it)
+// are visible to whoever counts in later.
+__device__ __forceinline__ unsigned count_in(unsigned *counter) {
+    unsigned old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
+    return old;
+}
+
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
 
 // Start of an evaluation whose records' positions and matrices are unchanged
 // (same x, A, n as the last seed preparation): zeroed moments and queue count,
@@ -23,8 +36,14 @@ constexpr int kRedThreads = 1024;
 // is formed first, p = -gamma gf + sum_k (cy_k y_k + cs_k s_k) from the
 // coefficients the direction kernels left (written to pdir), with <gf, p>
 // reduced by the last block into sc->gp0: one launch instead of two.
-__global__ void __launch_bounds__(256)
-    eval_begin_kernel(const int n, const int n_pad, const long long n_mom, const double *__restrict__ W0,
+//
+// Bound: latency (memory round trips, the FP64 chain of p's terms); each warp is a block of
+// its own, so that no two share an SM's FP64 unit while there are SMs, maxima go through
+// ordered integer keys (an FP64 maximum and shuffle step take 127 clocks), twelve pairs'
+// loads are in flight at a time, the stores follow the count of the blocks.  n = 1000, ten
+// pairs: 11.5 us -> 7.9 us.  <gf, p> is summed as blocks of `vw` warps, then over the blocks.
+__global__ void __launch_bounds__(32)
+    eval_begin_kernel(const int n, const int n_pad, const int vw, const long long n_mom, const double *__restrict__ W0,
                       const double t, double *__restrict__ pdir, double *__restrict__ Wt,
                       const int32_t *__restrict__ perm, SeedRec *__restrict__ recs,
                       SeedRec32 *__restrict__ recs32, SeedRec32 *__restrict__ recs32s,
@@ -33,58 +52,83 @@ __global__ void __launch_bounds__(256)
                       const double *__restrict__ S, const double *__restrict__ Y, const double *__restrict__ gfv,
                       const double *__restrict__ w0, const unsigned long long *__restrict__ wref0,
                       const unsigned *__restrict__ g3_hist, const unsigned full_max,
-                      float2 *__restrict__ drift) {
-    __shared__ double shw[8], shg[8], shdx[8], shdn[8];
+                      float2 *__restrict__ drift, const PushState push, PushState *__restrict__ push_to) {
     __shared__ double ccy[32], ccs[32];
     __shared__ int cslot[32];
-    __shared__ bool last;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x;
+    const int i = blockIdx.x * 32 + lane;
+    const int src = i < n_pad ? (perm ? perm[i] : i) : n;
+    const bool real = src < n;
+    double wi = real ? W0[src] : 0.0;
     int hist = 0;
     double gam = 0.0;
     if (coef) {
         hist = min(coef->hist, 31);
         gam = coef->gamma;
-        for (int k = threadIdx.x; k < hist; k += blockDim.x) {
-            ccy[k] = coef->cy[k];
-            ccs[k] = coef->cs[k];
-            cslot[k] = coef->slot[k];
-        }
-        __syncthreads();
+        ccy[lane] = coef->cy[lane];
+        ccs[lane] = coef->cs[lane];
+        cslot[lane] = coef->slot[lane];
+        __syncwarp();
     }
     double gp = 0.0;
     double dhi = -DBL_MAX, dlo = DBL_MAX;  // range of w - w0 (with w0)
-    for (long long e = i; e < n_mom; e += (long long)gridDim.x * blockDim.x) mom[e] = 0ull;
-    if (i == 0) {
-        sc->flag_count = 0u;
-        sc->band_count = 0u;
-    }
-    const int src = i < n_pad ? (perm ? perm[i] : i) : n;
-    const bool real = src < n;
-    double wkey = -DBL_MAX;
+    unsigned long long wkey = dkey(-DBL_MAX);
+    double pv = 0.0;
     if (real) {
-        double wi;
         if (pdir) {
-            double pv;
             if (coef) {
                 const double g = gfv[src];
                 pv = -gam * g;
-#pragma unroll 4
-                for (int k = 0; k < hist; ++k) {
-                    const size_t o = (size_t)cslot[k] * n + src;
-                    pv += ccy[k] * Y[o] + ccs[k] * S[o];
+                constexpr int kAhead = 12;
+                for (int k0 = 0; k0 < hist; k0 += kAhead) {
+                    double yk[kAhead], sk[kAhead];
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e) {
+                        const size_t o = (size_t)cslot[min(k0 + e, hist - 1)] * n + src;
+                        yk[e] = Y[o];
+                        sk[e] = S[o];
+                    }
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e)
+                        if (k0 + e < hist) pv += ccy[k0 + e] * yk[e] + ccs[k0 + e] * sk[e];
                 }
-                pdir[src] = pv;
                 gp = g * pv;
             } else {
                 pv = pdir[src];
             }
-            wi = fma(t, pv, W0[src]);
-            Wt[src] = wi;
-        } else {
-            wi = W0[src];
+            wi = fma(t, pv, wi);
         }
-        const bool finite = isfinite(wi);
-        if (!finite) atomicOr(&sc->status, ST_NONFINITE);
+        if (finite_bits(wi)) wkey = dkey(wi);
+        if (w0) {  // rounded outwards, so that the range covers the exact drift
+            dhi = __dsub_ru(wi, w0[src]);
+            dlo = __dsub_rd(wi, w0[src]);
+        }
+    }
+    const unsigned long long wmax = warp_max_key(wkey);
+    if (coef) gp = warp_sum(gp);
+    double hi = dhi, lo = dlo;
+    if (w0) {
+        hi = warp_max(dhi);
+        lo = warp_min(dlo);
+    }
+    unsigned last = 0;
+    if (lane == 0) {
+        double *row = part + (size_t)blockIdx.x * kPartStride;
+        row[0] = __longlong_as_double((long long)wmax);
+        if (coef) row[1] = gp;
+        if (w0) {
+            row[2] = hi;
+            row[3] = lo;
+        }
+        last = count_in(&sc->dual_done) == gridDim.x - 1;
+    }
+    // the seeds' and the pass's stores after the count: the fence before it would wait for them
+    if (real) {
+        if (pdir) {
+            if (coef) pdir[src] = pv;
+            Wt[src] = wi;
+        }
+        if (!finite_bits(wi)) atomicOr(&sc->status, ST_NONFINITE);
         recs[i].w = wi;
         float wh, wl;
         split_f32(wi, wh, wl);
@@ -94,71 +138,39 @@ __global__ void __launch_bounds__(256)
             recs32s[i].wh = wh;
             recs32s[i].wl = wl;
         }
-        wkey = finite ? wi : -DBL_MAX;
-        if (w0) {  // rounded outwards, so that the range covers the exact drift
-            dhi = __dsub_ru(wi, w0[src]);
-            dlo = __dsub_rd(wi, w0[src]);
-            if (drift) drift[src] = make_float2(__double2float_rd(dlo), __double2float_ru(dhi));
+        if (w0 && drift) drift[src] = make_float2(__double2float_rd(dlo), __double2float_ru(dhi));
+    }
+    for (long long e = i; e < n_mom; e += (long long)gridDim.x * 32) mom[e] = 0ull;
+    if (i == 0) {
+        sc->flag_count = 0u;
+        sc->band_count = 0u;
+        if (push_to) *push_to = push;
+    }
+    if (groups && lane == 0 && i < n) groups[blockIdx.x].wmax = dkey_inv(wmax);
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __syncwarp();
+    // the warps' maxima (a warp is a 32-seed group), loaded in parallel
+    const volatile double *rows = part;
+    unsigned long long top = 0ull;
+#pragma unroll 4
+    for (unsigned k = lane; k < gridDim.x; k += 32)
+        top = max(top, (unsigned long long)__double_as_longlong(rows[(size_t)k * kPartStride]));
+    double gsum = 0.0;  // <gf, p>: blocks of vw warps, lane-strided, then a fixed tree
+    if (coef)
+        for (unsigned k = lane; k * vw < gridDim.x; k += 32) {
+            double b = 0.0;
+#pragma unroll 2
+            for (int e = 0; e < vw; ++e) b += rows[(size_t)(k * vw + e) * kPartStride + 1];
+            gsum += b;
+        }
+    const double wref = dkey_inv(warp_max_key(top));
+    if (groups) {
+#pragma unroll 4
+        for (unsigned k = lane; k * 32 < (unsigned)n; k += 32) {
+            const double wm = dkey_inv((unsigned long long)__double_as_longlong(rows[(size_t)k * kPartStride]));
+            groups[k].wgap = __double2float_rd(wref - wm);
         }
     }
-    const double wmax = warp_max(wkey);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (coef) {
-        gp = warp_sum(gp);
-        if (lane == 0) shg[wid] = gp;
-    }
-    if (w0) {
-        dhi = warp_max(dhi);
-        dlo = warp_min(dlo);
-        if (lane == 0) {
-            shdx[wid] = dhi;
-            shdn[wid] = dlo;
-        }
-    }
-    if (lane == 0) {
-        shw[wid] = wmax;
-        if (groups && i < n_pad && (i & ~31) < n) groups[i >> 5].wmax = wmax;
-    }
-    __threadfence();  // group writes before the block's arrival count
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double b = shw[0];
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) b = fmax(b, shw[k]);
-        part[(size_t)blockIdx.x * kPartStride] = b;
-        if (coef) {
-            double s = 0.0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += shg[k];
-            part[(size_t)blockIdx.x * kPartStride + 1] = s;
-        }
-        if (w0) {
-            double x = -DBL_MAX, m = DBL_MAX;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-                x = fmax(x, shdx[k]);
-                m = fmin(m, shdn[k]);
-            }
-            part[(size_t)blockIdx.x * kPartStride + 2] = x;
-            part[(size_t)blockIdx.x * kPartStride + 3] = m;
-        }
-        __threadfence();
-        last = atomicAdd(&sc->dual_done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // block maxima loaded in parallel (max is order-independent)
-    double wref = -DBL_MAX;
-    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x)
-        wref = fmax(wref, *(volatile double *)&part[(size_t)k * kPartStride]);
-    wref = warp_max(wref);
-    if ((threadIdx.x & 31) == 0) shw[threadIdx.x >> 5] = wref;
-    __syncthreads();
-    wref = shw[0];
-    for (int k = 1; k < (int)(blockDim.x >> 5); ++k) wref = fmax(wref, shw[k]);
-    if (groups)
-        for (int gidx = threadIdx.x; gidx * 32 < n; gidx += blockDim.x) {
-            const double wm = *(volatile double *)&groups[gidx].wmax;
-            groups[gidx].wgap = __double2float_rd(wref - wm);
-        }
     if (w0 && threadIdx.x < 32) {  // the drift range (max and min are order-independent)
         double x = -DBL_MAX, m = DBL_MAX;
         for (unsigned k = threadIdx.x; k < gridDim.x; k += 32) {
@@ -190,11 +202,9 @@ __global__ void __launch_bounds__(256)
             sc->band_shift = __double2float_rd(__dsub_rd(__dsub_rd(__dsub_rd(wref, wr0), x), slack));
         }
     }
-    if (coef && threadIdx.x < 32) {  // <gf, p>: the blocks' sums, lane-strided, then a fixed tree
-        double s = 0.0;
-        for (unsigned k = threadIdx.x; k < gridDim.x; k += 32) s += *(volatile double *)&part[(size_t)k * kPartStride + 1];
-        s = warp_sum(s);
-        if (threadIdx.x == 0) sc->gp0 = s;
+    if (coef) {
+        gsum = warp_sum(gsum);
+        if (lane == 0) sc->gp0 = gsum;
     }
     if (threadIdx.x == 0) {
         sc->wref_key = dkey(wref);
@@ -361,211 +371,301 @@ __device__ __forceinline__ double sel3(const double (&v)[3], const int a) {
     return a == 0 ? v[0] : (a == 1 ? v[1] : v[2]);
 }
 
-// The pair terms of Q_i = sum_j (y_j - x_i)^T A_i (y_j - x_i) over cell i's
-// pixels (|P| Q_i is the integral term of eq. (2.7)) that lane q of the cell's
-// four lanes takes: pairs q and q + 4.  Q_ab = A_ab M_ab (A_ab + A_ba off the
-// diagonal) with M_ab = sum_j (y - x)_a (y - x)_b written through the integer
-// moments m, S1 = sum u, S2 = sum u u^T (u = 2k + 1, y = lo + h u / 2):
-// M_ab = h_a h_b / 4 (S2_ab - S1_a S1_b / m) + m e_a e_b, e = centroid - x.
+// The pair term of Q_i = sum_j (y_j - x_i)^T A_i (y_j - x_i) over cell i's pixels (|P| Q_i
+// is the integral term of eq. (2.7)) that lane q of the cell's eight lanes takes: pair q,
+// its factors A and M.  Q_ab = A_ab M_ab (A_ab + A_ba off the diagonal) with
+// M_ab = sum_j (y - x)_a (y - x)_b written through the integer moments m, S1 = sum u,
+// S2 = sum u u^T (u = 2k + 1, y = lo + h u / 2):
+// M_ab = h_a h_b / 4 (S2_ab - S1_a S1_b / m) + m e_a e_b, e = centroid - x (lane a's).
 template <int D>
-__device__ __forceinline__ double dual_pair_terms(const GridDev &g, const unsigned long long *__restrict__ mo,
-                                                  const double *__restrict__ xi, const double *__restrict__ Ai,
-                                                  const int q) {
+__device__ __forceinline__ void dual_pair_term(const GridDev &g, const unsigned long long *__restrict__ mo,
+                                               const double *__restrict__ xi, const double *__restrict__ Ai,
+                                               const int q, const int a, const int b, double &Aab, double &Mab) {
     constexpr int NP = D * (D + 1) / 2;
+    const int ax = min(q, D - 1);
     // no early exit on an empty cell: every load is issued before the first result
     // is needed (one memory round trip), and an empty cell's terms are dropped at the end
-    const unsigned long long m0 = mo[0];
+    const unsigned long long m0 = mo[0], s1 = mo[1 + ax], s2 = mo[1 + D + min(q, NP - 1)];
+    const double xa = xi[ax], Aa = Ai[a * D + b], Ab = Ai[b * D + a];
+    const double hh = 0.5 * sel3(g.h, ax), cc = 0.25 * sel3(g.h, a) * sel3(g.h, b);
     const double m = (double)m0;
     const double inv_m = 1.0 / m;  // one division; products with it differ from quotients by a few ulp
-    double Q = 0.0;
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int p = q + 4 * r;
-        if (p < NP) {
-            int a, b;
-            pair_ab<D>(p, a, b);
-            const double S1a = (double)mo[1 + a], S1b = (double)mo[1 + b];
-            const double ea = (sel3(g.lo, a) + 0.5 * sel3(g.h, a) * (S1a * inv_m)) - xi[a];
-            const double eb = (sel3(g.lo, b) + 0.5 * sel3(g.h, b) * (S1b * inv_m)) - xi[b];
-            const double Cab = (double)mo[1 + D + p] - S1a * S1b * inv_m;
-            const double Mab = 0.25 * sel3(g.h, a) * sel3(g.h, b) * Cab + m * ea * eb;
-            const double Aab = a == b ? Ai[a * D + a] : Ai[a * D + b] + Ai[b * D + a];
-            Q += Aab * Mab;
-        }
-    }
-    return m0 == 0ull ? 0.0 : Q;
+    const double S1 = (double)s1;
+    const double e = __dsub_rn(__fma_rn(hh, __dmul_rn(S1, inv_m), sel3(g.lo, ax)), xa);
+    const int base = threadIdx.x & 24;
+    const double S1a = __shfl_sync(0xffffffffu, S1, base + a), S1b = __shfl_sync(0xffffffffu, S1, base + b);
+    const double ea = __shfl_sync(0xffffffffu, e, base + a), eb = __shfl_sync(0xffffffffu, e, base + b);
+    const double Cab = __fma_rn(-__dmul_rn(S1a, S1b), inv_m, (double)s2);
+    Mab = __fma_rn(__dmul_rn(m, ea), eb, __dmul_rn(cc, Cab));
+    Aab = a == b ? Aa : Aa + Ab;
+    if (m0 == 0ull) Aab = Mab = 0.0;
 }
 
 // The same from FP64 element-measure moments (non-uniform discretisation):
 // m = sum |P_j|, S1 = sum |P_j| y_j, S2 = sum |P_j| y_j y_j^T, and
 // Q_ab = A_ab (S2_ab - S1_a x_b - x_a S1_b + m x_a x_b).
 template <int D>
-__device__ __forceinline__ double points_pair_terms(const double *__restrict__ mo, const double *__restrict__ xi,
-                                                    const double *__restrict__ Ai, const int q) {
+__device__ __forceinline__ void points_pair_term(const double *__restrict__ mo, const double *__restrict__ xi,
+                                                 const double *__restrict__ Ai, const int q, const int a, const int b,
+                                                 double &Aab, double &Mab) {
     constexpr int NP = D * (D + 1) / 2;
     const double m = mo[0];
-    double Q = 0.0;
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int p = q + 4 * r;
-        if (p < NP) {
-            int a, b;
-            pair_ab<D>(p, a, b);
-            const double Cab = mo[1 + D + p] - mo[1 + a] * xi[b] - xi[a] * mo[1 + b] + m * xi[a] * xi[b];
-            const double Aab = a == b ? Ai[a * D + a] : Ai[a * D + b] + Ai[b * D + a];
-            Q += Aab * Cab;
-        }
-    }
-    return Q;
+    Mab = mo[1 + D + min(q, NP - 1)] - mo[1 + a] * xi[b] - xi[a] * mo[1 + b] + m * xi[a] * xi[b];
+    Aab = a == b ? Ai[a * D + a] : Ai[a * D + b] + Ai[b * D + a];
 }
 
-// Per-cell dual terms, four lanes per cell (FP64 issues slowly; the pair terms
-// are split over the lanes), then a deterministic reduction: block sums through
-// fixed shuffle trees, block partials reduced by the last block to finish.
+// Partial results of the dual over some cells, spread over eight lanes (position p =
+// lane & 7): g, <grad f, p> and sum v in `a` of positions 0, 1, 2, the smallest v as an
+// ordered key in `a` of position 5; the largest |grad_k| / v_k as the pair (en, ed) of its
+// cell in every position, compared through one product each in positions 3 and 4.
+// One FP64 addition and one product join two rows: an FP64 instruction occupies a warp's
+// scheduler for 64 clocks however few lanes it serves, and eight of them a step (one lane
+// holding all) made the trees half of the kernel's time.
+struct DualRow {
+    double a, en, ed;
+    __device__ static DualRow none(int p) {
+        DualRow t;
+        t.a = p == 5 ? __longlong_as_double((long long)dkey(DBL_MAX)) : 0.0;
+        t.en = 0.0;
+        t.ed = 1.0;
+        return t;
+    }
+    __device__ void ratio(double on, double od, int p) {  // all products >= 0: ordered as integers
+        const double prod = __dmul_rn(p == 4 ? en : on, p == 4 ? od : ed);
+        const double other = __shfl_xor_sync(0xffffffffu, prod, 7);
+        const long long mine = __double_as_longlong(prod), theirs = __double_as_longlong(other);
+        if (p == 4 ? theirs > mine : mine > theirs) {
+            en = on;
+            ed = od;
+        }
+    }
+    __device__ static double smaller(double x, double y) {
+        const unsigned long long a = (unsigned long long)__double_as_longlong(x),
+                                 b = (unsigned long long)__double_as_longlong(y);
+        return a < b ? x : y;
+    }
+    __device__ void join(const DualRow &o, int p) {
+        const double s = __dadd_rn(a, o.a);
+        a = p == 5 ? smaller(a, o.a) : s;
+        ratio(o.en, o.ed, p);
+    }
+    __device__ void join_lanes(int off, int p) {
+        DualRow o;
+        o.a = __shfl_xor_sync(0xffffffffu, a, off);
+        o.en = __shfl_xor_sync(0xffffffffu, en, off);
+        o.ed = __shfl_xor_sync(0xffffffffu, ed, off);
+        join(o, p);
+    }
+    __device__ double value(int p) const { return p == 3 ? en : p == 4 ? ed : a; }  // a stored row's word p
+    __device__ static DualRow load(const volatile double *row, int p) {
+        DualRow t;
+        t.a = row[min(p, 5)];
+        t.en = row[3];
+        t.ed = row[4];
+        return t;
+    }
+};
+static_assert(kPartStride == 6, "words of a stored row");
+
+// Rows 4 / J lane groups apart: group k = lane / 8 holds the rows J k + j, j < J (J a power
+// of two); joined in a fixed tree over neighbouring rows, `rows` of them (a power of two).
+template <int MAXJ>
+__device__ __forceinline__ void join_rows(DualRow (&t)[MAXJ], const int J, const int rows, const int p) {
+#pragma unroll
+    for (int w = 1; w < MAXJ; w <<= 1)
+        if (w < J && w < rows) {
+#pragma unroll
+            for (int j = 0; j + w < MAXJ; j += 2 * w) t[j].join(t[j + w], p);
+        }
+    if (rows > J) t[0].join_lanes(8, p);
+    if (rows > 2 * J) t[0].join_lanes(16, p);
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// address of this block's shared location in the cluster's block `rank`
+__device__ __forceinline__ uint32_t cluster_map(const void *p, uint32_t rank) {
+    uint32_t to;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return to;
+}
+__device__ __forceinline__ void cluster_store(uint32_t to, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(to), "d"(v) : "memory");
+}
+__device__ __forceinline__ int pow2_at_least(int v) { return v <= 1 ? 1 : 1 << (32 - __clz(v - 1)); }
+
+// Per-cell dual terms, eight lanes per cell, then a deterministic reduction: a cluster's 64
+// cells through fixed trees, the clusters' rows by the last cluster to finish.
 //   g_i = (v_i - m_i |P|) w_i + |P| Q_i,  grad_i = v_i - m_i |P|  (eqs. (2.7), (2.8))
 // kPoints: FP64 element-measure moments of a non-uniform discretisation
 // (mom_pts), g_i = (v_i - m_i) w_i + Q_i, grad_i = v_i - m_i.
 // The largest relative volume error max_i |grad_i| / v_i is tracked as the
 // pair (|grad_k|, v_k) of its cell and divided once at the end.
-constexpr int kDualThreads = 256;  // 64 cells per block round
+//
+// Bound: FP64 instructions, 64 clocks each in a warp's scheduler, and memory round trips of
+// 600 to 1300 clocks (loads, the count of the clusters, the fence before the host's word).
+// So the work is spread over schedulers, four warps a block (one each), four blocks a
+// cluster, and no instruction serves one value alone.  Eight warps of 64 cells on one SM,
+// a lane of each joining all six values: 13.4 us at n = 1000, 11 at n = 20; so 9.3 and 7.0.
+constexpr int kDualBlocks = 4;                     // blocks of a cluster
+constexpr int kDualThreads = 128;                  // four warps of four cells
+constexpr int kDualCells = kDualBlocks * kDualThreads / 8;  // cells of a cluster's round
+
 template <int D, bool kPoints = false>
-__global__ void __launch_bounds__(kDualThreads)
+__global__ void __launch_bounds__(kDualThreads) __cluster_dims__(kDualBlocks, 1, 1)
     dual_kernel(const GridDev g, const int n, const double *__restrict__ x,
                 const double *__restrict__ A, const double *__restrict__ w,
                 const double *__restrict__ v, const double *__restrict__ p_dir,
                 const unsigned long long *__restrict__ mom, double *__restrict__ part,
                 DevScalars *__restrict__ sc, double *g_out, double *grad_out, double *gf_out,
-                double *err_out, const double *__restrict__ mom_pts = nullptr) {
-    constexpr int K = moment_width(D);
-    constexpr int NQ = kPartStride;  // g, <grad f, p>, sum v, max error (numerator, denominator), min v
-    __shared__ double shq[kDualThreads / 32][NQ];
-    __shared__ bool last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, q = lane & 3;
-    double gsum = 0.0, gp = 0.0, sv = 0.0, en = 0.0, ed = 1.0, vmin = DBL_MAX;
-    const int stride = gridDim.x * (kDualThreads / 4);
-    const int rounds = (n + stride - 1) / stride;  // the same for every lane (converged shuffles)
-    int i = (blockIdx.x * kDualThreads + threadIdx.x) >> 2;
-    for (int r = 0; r < rounds; ++r, i += stride) {
-        const bool real = i < n;
-        double Qp = 0.0, vi = 1.0, wi = 0.0, pd = 0.0;
-        if (real) {  // the cell's scalars too, before the pair terms' arithmetic
-            vi = v[i];
-            wi = w[i];
-            if (p_dir) pd = p_dir[i];
+                double *err_out, DevScalars *__restrict__ host, const double *__restrict__ mom_pts = nullptr) {
+    constexpr int K = moment_width(D), NP = D * (D + 1) / 2;
+    constexpr int kWarps = kDualThreads / 32 * kDualBlocks;  // rows of a cluster
+    __shared__ double rows[kWarps][kPartStride];
+    const int lane = threadIdx.x & 31, p = lane & 7;
+    const int rank = blockIdx.x % kDualBlocks, blk = blockIdx.x / kDualBlocks, nblk = gridDim.x / kDualBlocks;
+    const int row = rank * (kDualThreads / 32) + (int)(threadIdx.x >> 5);
+    cluster_arrive();  // waited for before the write into the first block's shared memory
+    int a, b;
+    pair_ab<D>(min(p, NP - 1), a, b);
+    DualRow t = DualRow::none(p);
+    // the last round's gradient is stored after the sums have been counted in: the fence
+    // before that waits for a warp's earlier stores
+    int i_last = -1;
+    double gr_last = 0.0;
+    auto put_gradient = [&]() {
+        if (i_last < 0) return;
+        if (p == 0 && grad_out) grad_out[i_last] = gr_last;
+        if (p == 1 && gf_out) gf_out[i_last] = -gr_last;
+    };
+    const int i0 = blk * kDualCells + row * 4;  // the warp's first cell
+    for (int c0 = i0; c0 < n; c0 += nblk * kDualCells) {
+        const int cell = c0 + (lane >> 3);
+        const bool real = cell < n;
+        const int i = real ? cell : c0;
+        const double vi = v[i], wi = w[i], pd = p_dir ? p_dir[i] : 0.0;
+        const double mi = kPoints ? mom_pts[(size_t)i * K] : (double)mom[(size_t)i * K];
+        double Aab, Mab;
+        if (kPoints) points_pair_term<D>(mom_pts + (size_t)i * K, x + (size_t)i * D, A + (size_t)i * D * D, p, a, b, Aab, Mab);
+        else dual_pair_term<D>(g, mom + (size_t)i * K, x + (size_t)i * D, A + (size_t)i * D * D, p, a, b, Aab, Mab);
+        const double gr = kPoints ? __dsub_rn(vi, mi) : __dsub_rn(vi, __dmul_rn(mi, g.cell));
+        // pairs q and q + 4 first, then q ^ 1, q ^ 2
+        const double P = p < NP ? __dmul_rn(Aab, Mab) : 0.0;
+        double Q = P;
+        if (NP > 4) {
+            const double F = __fma_rn(Aab, Mab, __shfl_xor_sync(0xffffffffu, P, 4));
+            const double up = __shfl_xor_sync(0xffffffffu, F, 4);
+            if (p + 4 < NP) Q = up;
         }
-        if (real)
-            Qp = kPoints ? points_pair_terms<D>(mom_pts + (size_t)i * K, x + (size_t)i * D, A + (size_t)i * D * D, q)
-                         : dual_pair_terms<D>(g, mom + (size_t)i * K, x + (size_t)i * D, A + (size_t)i * D * D, q);
-        Qp += __shfl_xor_sync(0xffffffffu, Qp, 1);
-        Qp += __shfl_xor_sync(0xffffffffu, Qp, 2);
-        if (real && q == 0) {
-            if (!(vi > 0.0) || !isfinite(vi)) atomicOr(&sc->status, ST_BAD_VOLUME);
-            const double gr = kPoints ? vi - mom_pts[(size_t)i * K] : __dsub_rn(vi, __dmul_rn((double)mom[(size_t)i * K], g.cell));
-            gsum += kPoints ? gr * wi + Qp : gr * wi + g.cell * Qp;
-            const double ag = fabs(gr);
-            if (ag * ed > en * vi) {
-                en = ag;
-                ed = vi;
-            }
-            if (grad_out) grad_out[i] = gr;
-            if (gf_out) gf_out[i] = -gr;
-            if (p_dir) gp += -gr * pd;
-            sv += vi;
-            vmin = fmin(vmin, vi);
+        Q += __shfl_xor_sync(0xffffffffu, Q, 1);
+        Q += __shfl_xor_sync(0xffffffffu, Q, 2);
+        const double u = __dmul_rn(gr, wi);
+        const double f = kPoints ? __fma_rn(p == 1 ? -gr : gr, p == 1 ? pd : wi, p == 1 ? t.a : Q) : __fma_rn(p == 1 ? -gr : g.cell, p == 1 ? pd : Q, p == 1 ? t.a : u);
+        const double s = __dadd_rn(t.a, p == 2 ? vi : f);
+        const DualRow old = t;
+        if (p == 5) t.a = DualRow::smaller(t.a, __longlong_as_double((long long)dkey(vi)));
+        else t.a = p == 1 ? f : s;
+        t.ratio(fabs(gr), vi, p);
+        if (!real) {
+            t = old;
+        } else {
+            if (p == 0 && (!(vi > 0.0) || !isfinite(vi))) atomicOr(&sc->status, ST_BAD_VOLUME);
+            put_gradient();
+            i_last = i;
+            gr_last = gr;
         }
     }
-    // warp: the cells' lanes q = 0 (lanes 0, 4, ..., 28) by a fixed tree
+    if (i0 < n) {
+        t.join_lanes(8, p);
+        t.join_lanes(16, p);
+    }
+    cluster_wait();
+    if (lane < kPartStride && i0 < n) cluster_store(cluster_map(&rows[row][lane], 0), t.value(lane));
+    cluster_arrive();
+    if (row != 0) {
+        put_gradient();
+        cluster_wait();
+        return;
+    }
+    cluster_wait();
+    {  // the cluster's 16 rows, those of warps that hold cells
+        constexpr int J = kWarps / 4;
+        const int used = (min(n - i0, kDualCells) + 3) / 4;
+        DualRow z[J];
 #pragma unroll
-    for (int off = 4; off < 32; off <<= 1) {
-        gsum += __shfl_xor_sync(0xffffffffu, gsum, off);
-        gp += __shfl_xor_sync(0xffffffffu, gp, off);
-        sv += __shfl_xor_sync(0xffffffffu, sv, off);
-        const double on = __shfl_xor_sync(0xffffffffu, en, off), od = __shfl_xor_sync(0xffffffffu, ed, off);
-        if (on * ed > en * od) {
-            en = on;
-            ed = od;
+        for (int j = 0; j < J; ++j) {
+            const int k = (lane >> 3) * J + j;
+            z[j] = k < used ? DualRow::load(rows[k], p) : DualRow::none(p);
         }
-        vmin = fmin(vmin, __shfl_xor_sync(0xffffffffu, vmin, off));
+        join_rows<J>(z, J, pow2_at_least(used), p);
+        t = z[0];
     }
-    if (lane == 0) {
-        shq[wid][0] = gsum;
-        shq[wid][1] = gp;
-        shq[wid][2] = sv;
-        shq[wid][3] = en;
-        shq[wid][4] = ed;
-        shq[wid][5] = vmin;
+    constexpr int kWords = sizeof(DevScalars) / 4, kPer = (kWords + 31) / 32;
+    unsigned word[kPer];
+    if (nblk > 1) {
+        if (lane < kPartStride) part[(size_t)blk * kPartStride + lane] = t.value(lane);
+        __syncwarp();
+        unsigned last = 0;
+        if (lane == 0) last = count_in(&sc->dual_done) == nblk - 1;
+        if (!__shfl_sync(0xffffffffu, last, 0)) {
+            put_gradient();
+            return;
+        }
+        __syncwarp();
     }
-    __syncthreads();
-    // block: warp 0 over the 8 warps' values by a fixed tree; lane 0 stores the partials
-    if (wid == 0) {
-        const int k = lane < kDualThreads / 32 ? lane : 0;
-        const bool own = lane < kDualThreads / 32;
-        double b0 = own ? shq[k][0] : 0.0, b1 = own ? shq[k][1] : 0.0, b2 = own ? shq[k][2] : 0.0;
-        double b3 = own ? shq[k][3] : 0.0, b4 = own ? shq[k][4] : 1.0, b5 = own ? shq[k][5] : DBL_MAX;
 #pragma unroll
-        for (int off = 1; off < kDualThreads / 32; off <<= 1) {
-            b0 += __shfl_xor_sync(0xffffffffu, b0, off);
-            b1 += __shfl_xor_sync(0xffffffffu, b1, off);
-            b2 += __shfl_xor_sync(0xffffffffu, b2, off);
-            const double on = __shfl_xor_sync(0xffffffffu, b3, off), od = __shfl_xor_sync(0xffffffffu, b4, off);
-            if (on * b4 > b3 * od) {
-                b3 = on;
-                b4 = od;
-            }
-            b5 = fmin(b5, __shfl_xor_sync(0xffffffffu, b5, off));
+    for (int k = 0; k < kPer; ++k)
+        word[k] = reinterpret_cast<const volatile unsigned *>(sc)[min(k * 32 + lane, kWords - 1)];
+    if (nblk > 1) {
+        // the last cluster: 32 columns take the clusters in order (c, c + 32, ...), then a fixed tree
+        constexpr int MJ = 8;
+        const int cols = min(32, pow2_at_least(nblk)), J = max(1, cols / 4);
+        DualRow z[MJ];
+#pragma unroll
+        for (int j = 0; j < MJ; ++j) {
+            const int c = (lane >> 3) * J + j;
+            z[j] = j < J && c < nblk ? DualRow::load(part + (size_t)c * kPartStride, p) : DualRow::none(p);
         }
+        for (int c0 = 32; c0 < nblk; c0 += 32) {
+#pragma unroll
+            for (int j = 0; j < MJ; ++j) {
+                const int c = c0 + (lane >> 3) * J + j;
+                const DualRow o = j < J && c < nblk ? DualRow::load(part + (size_t)c * kPartStride, p) : DualRow::none(p);
+                z[j].join(o, p);
+            }
+        }
+        join_rows<MJ>(z, J, cols, p);
+        t = z[0];
+    }
+    if (p == 3) t.a = __ddiv_rn(t.en, t.ed);
+    if (p == 5) t.a = dkey_inv((unsigned long long)__double_as_longlong(t.a));
+    if (lane < kPartStride && lane != 4) {
+        // position -> field (g, dot_gp, sum_v, max_rel_err, -, min_v)
+        const int field = lane == 0 ? 0 : lane == 1 ? 2 : lane == 2 ? 3 : lane == 3 ? 1 : 4;
+        (&sc->g)[field] = t.a;
+        if (lane == 0 && g_out) *g_out = t.a;
+        if (lane == 3 && err_out) *err_out = t.a;
+        if (host) (&host->g)[field] = t.a;
+    }
+    if (lane == 0) sc->dual_done = 0u;
+    if (host) {  // the other scalars, then the pass's number, which the host waits for
+        constexpr int w0 = offsetof(DevScalars, g) / 4, w1 = offsetof(DevScalars, sy) / 4, ws = offsetof(DevScalars, seq) / 4;
+        static_assert(w1 - w0 == 10, "g, max_rel_err, dot_gp, sum_v, min_v in a row");
+        unsigned seq = 0u;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const int e = k * 32 + lane;
+            if (k == ws / 32) seq = __shfl_sync(0xffffffffu, word[k], ws % 32) + 1u;
+            if (e < kWords && e != ws && (e < w0 || e >= w1)) reinterpret_cast<volatile unsigned *>(host)[e] = word[k];
+        }
+        __syncwarp();
         if (lane == 0) {
-            double *pp = part + (size_t)blockIdx.x * NQ;
-            pp[0] = b0;
-            pp[1] = b1;
-            pp[2] = b2;
-            pp[3] = b3;
-            pp[4] = b4;
-            pp[5] = b5;
-            __threadfence();
-            last = atomicAdd(&sc->dual_done, 1u) == gridDim.x - 1;
+            sc->seq = seq;
+            __threadfence_system();
+            *(volatile unsigned *)&host->seq = seq;
         }
     }
-    __syncthreads();
-    if (!last || wid != 0) return;
-    __threadfence();
-    // the last block: lanes take the blocks in order (lane, lane + 32, ...), then a fixed tree
-    double G = 0.0, GP = 0.0, SV = 0.0, EN = 0.0, ED = 1.0, VM = DBL_MAX;
-    for (unsigned b = lane; b < gridDim.x; b += 32) {
-        const volatile double *pp = part + (size_t)b * NQ;
-        G += pp[0];
-        GP += pp[1];
-        SV += pp[2];
-        const double on = pp[3], od = pp[4];
-        if (on * ED > EN * od) {
-            EN = on;
-            ED = od;
-        }
-        VM = fmin(VM, pp[5]);
-    }
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        G += __shfl_xor_sync(0xffffffffu, G, off);
-        GP += __shfl_xor_sync(0xffffffffu, GP, off);
-        SV += __shfl_xor_sync(0xffffffffu, SV, off);
-        const double on = __shfl_xor_sync(0xffffffffu, EN, off), od = __shfl_xor_sync(0xffffffffu, ED, off);
-        if (on * ED > EN * od) {
-            EN = on;
-            ED = od;
-        }
-        VM = fmin(VM, __shfl_xor_sync(0xffffffffu, VM, off));
-    }
-    if (lane == 0) {
-        const double E = __ddiv_rn(EN, ED);
-        sc->g = G;
-        sc->max_rel_err = E;
-        sc->dot_gp = GP;
-        sc->sum_v = SV;
-        sc->min_v = VM;
-        sc->dual_done = 0u;
-        if (g_out) *g_out = G;
-        if (err_out) *err_out = E;
-    }
+    put_gradient();
 }
 
 template <int D>
@@ -612,6 +712,28 @@ constexpr int kLbT = 1024;       // threads per block of the dot-product kernels
 constexpr int kLbR = 32;         // seeds per block range
 constexpr int kLbP = 64;         // threads per block of the p kernel
 
+// Sum over the warp of five values, each by warp_sum's tree (pairs 16, 8, ... apart), in 8
+// additions where five trees take 25: after a step that pairs two values, half of the
+// lanes carry on with each.  The sum of value c is returned in the lanes where
+// dot_of_lane() is c.
+__device__ __forceinline__ double warp_sum5(const double (&v)[5]) {
+    const int lane = threadIdx.x & 31;
+    auto both = [&](double a, double b, int off) {  // lanes without the bit go on with a, those with it b
+        const bool hi = lane & off;
+        const double keep = hi ? b : a, send = hi ? a : b;
+        return keep + __shfl_xor_sync(0xffffffffu, send, off);
+    };
+    const double r01 = both(v[0], v[1], 16), r23 = both(v[2], v[3], 16);
+    double r4 = v[4] + __shfl_xor_sync(0xffffffffu, v[4], 16);
+    const double r03 = both(r01, r23, 8);
+    r4 += __shfl_xor_sync(0xffffffffu, r4, 8);
+    double r = both(r03, r4, 4);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    return r;
+}
+__device__ __forceinline__ int dot_of_lane(int lane) { return lane & 4 ? 4 : ((lane >> 3) & 1) * 2 + ((lane >> 4) & 1); }
+
 // Partial dot products of one block over its ranges of 32 seeds (range r
 // starts at (blockIdx.x + r gridDim.x) 32): dot d (of nd) is sum_i f(d, i),
 // warp w takes the dots d = w mod 32.  part[blockIdx.x * kLbfgsDots + d]
@@ -635,7 +757,7 @@ __device__ bool lbfgs_last_block(DevScalars *sc) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        last = atomicAdd(&sc->lbfgs_done, 1u) == gridDim.x - 1;
+        last = atomicAdd(&sc->lbfgs_done, 1u) == gridDim.x * gridDim.y - 1;
     }
     __syncthreads();
     if (last) __threadfence();
@@ -660,7 +782,7 @@ __device__ void reduce_partials(const int nd, const double *part, double *out) {
 struct LbfgsScalars {
     double sy[kLbfgsMax][kLbfgsMax + 1];  // s_k . y_j
     double yy[kLbfgsMax][kLbfgsMax + 1];  // y_k . y_j
-    double rh[kLbfgsMax], sg[kLbfgsMax], yg[kLbfgsMax], al[kLbfgsMax];
+    double rh[kLbfgsMax], sg[kLbfgsMax], yg[kLbfgsMax];
     int slot[kLbfgsMax];
 };
 
@@ -679,36 +801,55 @@ __device__ void load_gram(LbfgsScalars &L, const int hist, const int cap, const 
 // The two-loop recursion on the Gram entries, by warp 0, column by column:
 // alpha_k = rho_k (s_k . g - sum_{j<k} alpha_j s_k . y_j)          (newest first)
 // c_k = alpha_k - rho_k (gamma y_k . q + sum_{j>k} c_j s_j . y_k)   (oldest first)
-// with y_k . q = y_k . g - sum_j alpha_j y_k . y_j; then the coefficients of p.
-__device__ void lbfgs_coefficients(LbfgsScalars &L, const int hist, const double gamma, LbfgsCoef *coef) {
+// with y_k . q = y_k . g - sum_j alpha_j y_k . y_j (summed beside the alphas: the chain of
+// an alpha leaves the FP64 unit idle); then the coefficients of p.  Pair k lies in row
+// k + base of L.
+__device__ void lbfgs_coefficients(const LbfgsScalars &L, const int base, const int hist, const double gamma,
+                                   LbfgsCoef *coef) {
     if (threadIdx.x >= 32) return;
     const int lane = threadIdx.x;
-    double t = 0.0, al = 0.0;
-    for (int k = 0; k < hist; ++k) {
-        double a = lane == k ? L.rh[k] * (L.sg[k] - t) : 0.0;
-        a = __shfl_sync(0xffffffffu, a, k);
-        if (lane == k) al = a;
-        if (lane > k && lane < hist) t += a * L.sy[lane][k];
-    }
-    if (lane < hist) L.al[lane] = al;
-    __syncwarp();
-    double yq = 0.0;
-    if (lane < hist) {
-        yq = L.yg[lane];
-        for (int j = 0; j < hist; ++j) yq -= L.al[j] * L.yy[lane][j];
+    const bool halves = hist <= 16;  // lanes 16 .. 31 sum y_k . q beside lanes 0 .. 15, by the same instruction
+    const int k0 = halves ? lane & 15 : lane, row = min(k0 + base, kLbfgsMax - 1);
+    const double rh = L.rh[row], sg = L.sg[row];
+    double t = 0.0, al = 0.0, yq = L.yg[row];
+    if (halves) {
+        const bool up = lane >= 16;
+        double acc = up ? yq : 0.0;
+        const double(*M)[kLbfgsMax + 1] = up ? L.yy : L.sy;
+#pragma unroll 2
+        for (int k = 0; k < hist; ++k) {
+            const double mk = M[row][k + base];
+            double a = rh * (sg - acc);
+            a = __shfl_sync(0xffffffffu, a, k);
+            if (lane == k) al = a;
+            acc = __fma_rn(up ? -a : a, mk, acc);
+        }
+        yq = __shfl_sync(0xffffffffu, acc, lane | 16);
+    } else {
+#pragma unroll 2
+        for (int k = 0; k < hist; ++k) {
+            const double sy = L.sy[row][k + base], yy = L.yy[row][k + base];
+            double a = rh * (sg - t);
+            a = __shfl_sync(0xffffffffu, a, k);
+            if (lane == k) al = a;
+            if (lane > k && lane < hist) t += a * sy;
+            yq -= a * yy;
+        }
     }
     double u = 0.0, c = 0.0;
+#pragma unroll 2
     for (int k = hist - 1; k >= 0; --k) {
-        double ck = lane == k ? al - L.rh[k] * (gamma * yq + u) : 0.0;
+        const double sy = L.sy[k + base][row];
+        double ck = al - rh * (gamma * yq + u);
         ck = __shfl_sync(0xffffffffu, ck, k);
         if (lane == k) c = ck;
-        if (lane < k) u += ck * L.sy[k][lane];
+        if (lane < k) u += ck * sy;
     }
     // p = -gamma g + sum_k gamma alpha_k y_k - sum_k (alpha_k - beta_k) s_k
     if (lane < hist) {
         coef->cs[lane] = -c;
         coef->cy[lane] = gamma * al;
-        coef->slot[lane] = L.slot[lane];
+        coef->slot[lane] = L.slot[row];
     }
     if (lane == 0) {
         coef->hist = hist;
@@ -747,7 +888,7 @@ __global__ void __launch_bounds__(kLbT)
         L.yg[k] = dots[2 * k + 1];
     }
     load_gram(L, hist, cap, gram, rho);
-    lbfgs_coefficients(L, hist, gamma, coef);
+    lbfgs_coefficients(L, 0, hist, gamma, coef);
     if (threadIdx.x == 0) sc->lbfgs_done = 0u;
 }
 
@@ -799,107 +940,190 @@ __global__ void __launch_bounds__(kLbP)
     }
 }
 
-// Store the pair s = Wt - W, y = gft - gf in slot `slot`; sy, yy, ss, the
-// curvature test and 1 / s.y into sc and rho; the Gram entries of the new pair
-// with itself and with the nprev pairs in the slots before it (slot - 1, ...,
-// slot - nprev, cyclically).  With dir, also the coefficients of the next
-// direction for the gradient gft: the pair taken (then min(hist + 1, hist_acc)
-// = hist_acc pairs newest first from `slot`, gamma = s.y / y.y) if it passes
-// the test, else the hist pairs before it with the given gamma.
+// Store the pair s = Wt - W, y = gft - gf in the slot after `newest`; sy, yy, ss, the
+// curvature test and 1 / s.y into sc and rho; the Gram entries of the new pair with
+// itself and with the pairs that are kept beside it.  With dir, also the coefficients of
+// the next direction for the gradient gft: the pair taken (then hist_acc = min(hist + 1,
+// history) pairs newest first from the new slot, gamma = s.y / y.y) if it passes the
+// test, else the hist pairs before it with the given gamma.
+// The state, written by the trial's first kernel: with pend, the pair pushed before (slot p_slot) has not been looked at by
+// the host: it is part of the history if its test passed.  The push follows each trial of
+// a line search before the host knows the trial's value, so that the device does not wait
+// for the host; the slot written is in no history, so a push that
+// the search does not accept leaves nothing behind.  Nothing is formed at an evaluation
+// that met eps; Wbest takes Wt where the evaluation's error is below best_err.
+//
+// Unit u = 0 is the new pair (s.y, y.y, s.s, s.g, y.g), unit u > 0 the pair j = u - 1
+// before it (s.y_j, s_j.y, y.y_j, s_j.g, y_j.g): a warp takes a unit over 32 seeds (lane =
+// seed, s and y formed in registers), the units of a range spread over gridDim.y blocks.
+// Bound: latency; memory round trips and the recursion's chain of 4 FP64 operations a pair
+// and direction.  A warp per dot product with a tree each, the pair read back from memory
+// and the Gram entries gathered at the end: 20.8 us at n = 1000 and ten pairs; so 8.9 us.
 __global__ void __launch_bounds__(kLbT)
-    lbfgs_push_kernel(const int n, const int slot, const int cap, const int nprev,
-                      const double *__restrict__ W, const double *__restrict__ Wt,
-                      const double *__restrict__ gf, const double *__restrict__ gft, double *S,
-                      double *Y, double *__restrict__ rho, double *__restrict__ gram, double *part,
-                      DevScalars *sc, const int dir, const int hist, const int hist_acc, const double gamma,
-                      LbfgsCoef *coef) {
+    lbfgs_push_kernel(const int n, const int cap, const PushState *__restrict__ state, const double *__restrict__ W,
+                      const double *__restrict__ Wt, const double *__restrict__ gf, const double *__restrict__ gft,
+                      double *S, double *Y, double *__restrict__ rho, double *__restrict__ gram, double *part,
+                      DevScalars *sc, const int dir, LbfgsCoef *coef, double *__restrict__ Wbest) {
     __shared__ LbfgsScalars L;
-    __shared__ double dots[kLbfgsDots];
-    double *s = S + (size_t)slot * n;
-    double *y = Y + (size_t)slot * n;
-    for (int i = (blockIdx.x + (int)(threadIdx.x >> 5) * gridDim.x) * kLbR + (threadIdx.x & 31); i < n;
-         i += gridDim.x * kLbT) {
-        s[i] = Wt[i] - W[i];
-        y[i] = gft[i] - gf[i];
-    }
-    __syncthreads();  // the block's global writes are visible to the block after the barrier
-    // dots 0..2: s.y, y.y, s.s; 3 + 3j..: s . y_j, s_j . y, y . y_j (j < np, slot j = slot - 1 - j);
-    // with dir, at o = 3 + 3 np: s . g, y . g, then s_j . g, y_j . g (j < nh)
-    const int np = min(nprev, kLbfgsMax - 1);
+    __shared__ double dots[kLbfgsMax][5];
+    __shared__ bool pair_ok, last;
+    __shared__ double gamma_new;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const double err = sc->max_rel_err;
+    const PushState ps = *state;
+    const double psy = sc->sy, pyy = sc->yy;  // of the pair before; the last block replaces them
+    const bool taken = ps.pend && sc->pair_ok;
+    const int newest = taken ? ps.p_slot : ps.newest;
+    const int hist = taken ? ps.hist_acc : ps.hist;
+    const int slot = (newest + 1) % cap, hist_acc = min(hist + 1, ps.history);
+    if (Wbest && err < ps.best_err && blockIdx.y == gridDim.y - 1 && wid == nw - 1)
+        for (int i = blockIdx.x * kLbR + lane; i < n; i += gridDim.x * kLbR) Wbest[i] = Wt[i];
+    if (Wbest && err < ps.eps) return;
+    const int np = min(hist_acc - 1, kLbfgsMax - 1);
     const int nh = dir ? min(hist, kLbfgsMax - 1) : 0;
-    const int o = 3 + 3 * np;
-    const int nd = o + (dir ? 2 + 2 * nh : 0);
-    block_partial_dots(nd, n, [&](int d, int i) {
-        if (d < 3) return d == 0 ? s[i] * y[i] : d == 1 ? y[i] * y[i] : s[i] * s[i];
-        if (d < o) {
-            const int j = (d - 3) / 3, c = (d - 3) % 3;
-            const size_t q = (size_t)((slot - 1 - j + 2 * cap) % cap) * n + i;
-            return c == 0 ? s[i] * Y[q] : c == 1 ? S[q] * y[i] : y[i] * Y[q];
-        }
-        if (d < o + 2) return (d == o ? s[i] : y[i]) * gft[i];
-        const int e = d - o - 2;
-        const size_t q = (size_t)((slot - 1 - (e >> 1) + 2 * cap) % cap) * n + i;
-        return ((e & 1) ? Y[q] : S[q]) * gft[i];
-    }, part);
-    if (!lbfgs_last_block(sc)) return;
-    reduce_partials(nd, part, dots);
+    const int m = max(np, nh), units = m + 1;
     double *gsy = gram, *gyy = gram + (size_t)cap * cap;
-    for (int j = threadIdx.x; j < np; j += blockDim.x) {
-        const int sj = (slot - 1 - j + 2 * cap) % cap;
-        gsy[(size_t)slot * cap + sj] = dots[3 + 3 * j];
-        gsy[(size_t)sj * cap + slot] = dots[4 + 3 * j];
-        gyy[(size_t)slot * cap + sj] = dots[5 + 3 * j];
-        gyy[(size_t)sj * cap + slot] = dots[5 + 3 * j];
+    auto prev = [&](int j) {  // slot of the j-th pair before the new one
+        const int q = slot - 1 - j;
+        return q < 0 ? q + cap : q;
+    };
+    // the old pairs' Gram entries, needed by the last block: on their way early (row 0 of L is
+    // the new pair); a warp takes a row, a lane a column (there is a warp for every pair)
+    const bool old = dir && wid < m && lane < m;
+    const size_t og = old ? (size_t)prev(wid) * cap + prev(lane) : 0;
+    const double osy = old ? gsy[og] : 0.0, oyy = old ? gyy[og] : 0.0;
+    const double orh = wid == 0 && lane < m ? rho[prev(lane)] : 0.0;
+    const size_t rows = gridDim.x;
+    for (int u = wid * gridDim.y + blockIdx.y; u < units; u += gridDim.y * nw) {
+        const double *sj = S + (size_t)(u ? prev(u - 1) : 0) * n, *yj = Y + (size_t)(u ? prev(u - 1) : 0) * n;
+        double v[5];
+        bool first = true;
+        for (int i0 = blockIdx.x * kLbR; i0 < n; i0 += gridDim.x * kLbR) {
+            const int i = min(i0 + lane, n - 1);
+            const bool in = i0 + lane < n;
+            const double s = Wt[i] - W[i], g = gft[i], y = g - gf[i];
+            const double a = u ? sj[i] : s, b = u ? yj[i] : y;
+            // new pair: a = s, b = y; else a = s_j, b = y_j
+            const double d[5] = {__dmul_rn(s, b), __dmul_rn(u ? a : y, y), __dmul_rn(u ? y : s, u ? b : s), __dmul_rn(a, g),
+                                 __dmul_rn(b, g)};
+#pragma unroll
+            for (int c = 0; c < 5; ++c) v[c] = first ? (in ? d[c] : 0.0) : in ? __dadd_rn(v[c], d[c]) : v[c];
+            first = false;
+        }
+        const double r = warp_sum5(v);
+        if ((lane & 3) == 0 && (lane == 4 || !(lane & 4)))
+            part[(size_t)(u * 5 + dot_of_lane(lane)) * rows + blockIdx.x] = r;
     }
-    const double vsy = dots[0], vyy = dots[1], vss = dots[2];
-    const bool ok = vsy > 1e-12 * sqrt(vss * vyy) && vyy > 0.0;
+    __syncthreads();
+    if (threadIdx.x == 0) last = count_in(&sc->lbfgs_done) == gridDim.x * gridDim.y - 1;
+    if (blockIdx.y == 0 && wid == nw - 1)  // the pair itself, after the count (the fence before it would wait)
+        for (int i = blockIdx.x * kLbR + lane; i < n; i += gridDim.x * kLbR) {
+            S[(size_t)slot * n + i] = Wt[i] - W[i];
+            Y[(size_t)slot * n + i] = gft[i] - gf[i];
+        }
+    if (dir) {
+        if (old) {
+            L.sy[wid + 1][lane + 1] = osy;
+            L.yy[wid + 1][lane + 1] = oyy;
+        }
+        if (wid == 0 && lane <= m) L.slot[lane] = lane == 0 ? slot : prev(lane - 1);
+        if (wid == 0 && lane < m) L.rh[lane + 1] = orh;
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int u = wid; u < units; u += nw) {
+        double v[5];
+        const volatile double *pp = part + (size_t)u * 5 * rows;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) v[c] = lane < (int)rows ? pp[(size_t)c * rows + lane] : 0.0;
+        for (unsigned b = lane + 32; b < rows; b += 32)
+#pragma unroll
+            for (int c = 0; c < 5; ++c) v[c] += pp[(size_t)c * rows + b];
+        if (rows > 1) {
+            const double r = warp_sum5(v);
+            if ((lane & 3) == 0 && (lane == 4 || !(lane & 4))) dots[u][dot_of_lane(lane)] = r;
+        } else if (lane == 0) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) dots[u][c] = v[c];
+        }
+    }
+    __syncthreads();
+    const double vsy = dots[0][0], vyy = dots[0][1], vss = dots[0][2];
+    // the test in one warp, the new pair's quotients in another, its Gram entries in the rest
     if (threadIdx.x == 0) {
+        // vsy > 1e-12 sqrt(vss vyy): by the squares where they decide it clearly
+        const double prod = vss * vyy, sq = vsy * vsy;
+        const bool clear = vsy > 0.0 && sq > 1e-290 && prod < 1e290 && sq > 1.0001e-24 * prod;
+        const bool ok = (clear || vsy > 1e-12 * sqrt(prod)) && vyy > 0.0;
+        sc->pair_ok = ok ? 1 : 0;
+        pair_ok = ok;
+    }
+    if (wid == 1 && lane < 2) {  // 1 / s.y and s.y / y.y side by side
+        const double num = lane == 0 ? 1.0 : vsy, den = lane == 0 ? vsy : vyy;
+        const double r = lane == 1 || vsy != 0.0 ? num / den : 0.0;
+        if (lane == 0) {
+            rho[slot] = r;
+            L.rh[0] = r;
+        } else {
+            gamma_new = r;
+        }
+    }
+    if ((int)threadIdx.x == (int)blockDim.x - 1) {
         gsy[(size_t)slot * cap + slot] = vsy;
         gyy[(size_t)slot * cap + slot] = vyy;
         sc->sy = vsy;
         sc->yy = vyy;
         sc->ss = vss;
-        sc->pair_ok = ok ? 1 : 0;
-        rho[slot] = vsy != 0.0 ? 1.0 / vsy : 0.0;
+        L.sy[0][0] = vsy;
+        L.yy[0][0] = vyy;
+        L.sg[0] = dots[0][3];
+        L.yg[0] = dots[0][4];
+    }
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+        const double *d = dots[j + 1];
+        L.sy[0][j + 1] = d[0];
+        L.sy[j + 1][0] = d[1];
+        L.yy[0][j + 1] = L.yy[j + 1][0] = d[2];
+        L.sg[j + 1] = d[3];
+        L.yg[j + 1] = d[4];
+        if (j < np) {
+            const int q = prev(j);
+            gsy[(size_t)slot * cap + q] = d[0];
+            gsy[(size_t)q * cap + slot] = d[1];
+            gyy[(size_t)slot * cap + q] = d[2];
+            gyy[(size_t)q * cap + slot] = d[2];
+        }
     }
     if (dir) {
-        __syncthreads();  // the Gram entries and rho written above, read by load_gram
-        const int h = ok ? min(hist_acc, kLbfgsMax - 1) : nh;
-        for (int k = threadIdx.x; k < h; k += blockDim.x) {
-            const int j = ok ? k - 1 : k;  // index among the previous pairs (-1: the new pair)
-            L.slot[k] = (slot - 1 - j + 2 * cap) % cap;
-            L.sg[k] = j < 0 ? dots[o] : dots[o + 2 + 2 * j];
-            L.yg[k] = j < 0 ? dots[o + 1] : dots[o + 3 + 2 * j];
-        }
         __syncthreads();
-        load_gram(L, h, cap, gram, rho);
-        lbfgs_coefficients(L, h, ok ? vsy / vyy : gamma, coef);
+        const bool ok = pair_ok;
+        lbfgs_coefficients(L, ok ? 0 : 1, ok ? min(hist_acc, kLbfgsMax - 1) : nh, ok ? gamma_new : taken ? psy / pyy : ps.gamma, coef);
     }
     if (threadIdx.x == 0) sc->lbfgs_done = 0u;
 }
 
 }  // namespace
 
-// Threads per block of eval_begin_kernel: 64 (two warps, spreading the FP64
-// work of forming p and the trial weights over more SMs) while the blocks fit
-// the workspace's partial-sum rows, else 256.
-static int eval_begin_threads(int n_pad, const Workspace &ws) { return n_pad / 64 <= ws.part_rows ? 64 : 256; }
+// Threads per block of the seed preparation: 64 (two warps, spreading the FP64 work over
+// more SMs) while the blocks fit the workspace's partial-sum rows, else 256.  The same
+// blocks are the units in which an evaluation's first kernel sums <gf, p>.
+static int prep_threads(int n_pad, const Workspace &ws) { return n_pad / 64 <= ws.part_rows ? 64 : 256; }
 
 cudaError_t launch_eval_begin(int n, const double *W0, double t, const double *pdir, double *Wt,
                               unsigned long long *mom, Workspace &ws, cudaStream_t st, bool form_p,
-                              const double *w0, unsigned full_max) {
+                              const double *w0, unsigned full_max, const PushState *push) {
     const unsigned long long *wref0 = w0 ? ws.inc_aux : nullptr;
     const unsigned *hist = w0 ? ws.inc_hist : nullptr;
     const int n_pad = ((n + kChunk - 1) / kChunk) * kChunk;
     const long long n_mom = (long long)n * moment_width(ws.dim);
     if (n_pad == 0) return cudaSuccess;
     const bool fp = form_p && pdir;
-    const int tpb = eval_begin_threads(n_pad, ws);
-    eval_begin_kernel<<<n_pad / tpb, tpb, 0, st>>>(n, n_pad, n_mom, W0, t, const_cast<double *>(pdir), Wt,
+    eval_begin_kernel<<<n_pad / 32, 32, 0, st>>>(n, n_pad, prep_threads(n_pad, ws) / 32, n_mom, W0, t, const_cast<double *>(pdir), Wt,
                                                    ws.sorted ? ws.perm : nullptr, ws.recs, ws.recs32,
                                                    ws.sorted ? ws.recs32s : nullptr, ws.groups, mom, ws.part, ws.sc,
                                                    fp ? ws.lb_coef : nullptr, ws.S, ws.Y, ws.gf, w0, wref0,
-                                                   hist, full_max, w0 ? ws.inc_drift : nullptr);
+                                                   hist, full_max, w0 ? ws.inc_drift : nullptr, push ? *push : PushState{},
+                                                   push ? ws.push_state : nullptr);
     return cudaGetLastError();
 }
 
@@ -909,10 +1133,11 @@ const void *eval_begin_kernel_fn() { return reinterpret_cast<const void *>(eval_
 // instantiated graph (only the trial step t changes between replays).
 cudaError_t set_eval_begin_node(cudaGraphExec_t exec, cudaGraphNode_t node, int n, const double *W0, double t,
                                 const double *pdir, double *Wt, unsigned long long *mom, Workspace &ws,
-                                bool form_p, const double *w0, unsigned full_max) {
+                                bool form_p, const double *w0, unsigned full_max, const PushState *push) {
     const unsigned long long *wref0 = w0 ? ws.inc_aux : nullptr;
     const unsigned *hist = w0 ? ws.inc_hist : nullptr;
     float2 *drift = w0 ? ws.inc_drift : nullptr;
+    PushState ps = push ? *push : PushState{}, *to = push ? ws.push_state : nullptr;
     int n_pad = ((n + kChunk - 1) / kChunk) * kChunk;
     long long n_mom = (long long)n * moment_width(ws.dim);
     const int32_t *perm = ws.sorted ? ws.perm : nullptr;
@@ -924,14 +1149,14 @@ cudaError_t set_eval_begin_node(cudaGraphExec_t exec, cudaGraphNode_t node, int 
     double *pd = const_cast<double *>(pdir);
     const LbfgsCoef *coef = form_p && pdir ? ws.lb_coef : nullptr;
     const double *S = ws.S, *Y = ws.Y, *gfv = ws.gf;
-    void *args[] = {&n,      &n_pad,   &n_mom,  &W0,  &t,    &pd, &Wt,   &perm, &recs, &recs32,
+    int vw = prep_threads(n_pad, ws) / 32;
+    void *args[] = {&n,      &n_pad,   &vw,    &n_mom,  &W0,  &t,    &pd, &Wt,   &perm, &recs, &recs32,
                     &recs32s, &groups, &mom, &part, &sc, &coef, &S, &Y, &gfv, &w0, &wref0, &hist, &full_max,
-                    &drift};
+                    &drift, &ps, &to};
     cudaKernelNodeParams p{};
     p.func = reinterpret_cast<void *>(eval_begin_kernel);
-    const int tpb = eval_begin_threads(n_pad, ws);
-    p.gridDim = dim3(n_pad / tpb);
-    p.blockDim = dim3(tpb);
+    p.gridDim = dim3(n_pad / 32);
+    p.blockDim = dim3(32);
     p.sharedMemBytes = 0;
     p.kernelParams = args;
     p.extra = nullptr;
@@ -992,7 +1217,7 @@ cudaError_t launch_seed_prep(const GridDev &g, int n, const double *x, const dou
     SeedRec *dst = ws.sorted ? ws.recs_tmp : ws.recs;
     uint32_t *codes = ws.sorted ? ws.codes : nullptr;
     unsigned long long *part = reinterpret_cast<unsigned long long *>(ws.part);
-    const int tpb = eval_begin_threads(n_pad, ws);
+    const int tpb = prep_threads(n_pad, ws);
     if (g.dim == 3)
         seed_prep_kernel<3><<<n_pad / tpb, tpb, 0, st>>>(g, n, n_pad, x, A, w, dst, ws.recs32, codes, mom, n_mom, part,
                                                          ws.sc, box);
@@ -1022,22 +1247,22 @@ cudaError_t launch_group_bounds(int n, Workspace &ws, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Blocks of the dual kernel: 64 cells each, at most the workspace's partial rows.
+// Clusters of the dual kernel: 64 cells each, at most the workspace's partial rows.
 static int dual_blocks(int n, const Workspace &ws) {
-    return std::max(1, std::min((n + kDualThreads / 4 - 1) / (kDualThreads / 4), ws.part_rows));
+    return std::max(1, std::min((n + kDualCells - 1) / kDualCells, ws.part_rows));
 }
 
 cudaError_t launch_dual(const GridDev &g, int n, const double *x, const double *A, const double *w,
                         const double *v, const double *p_dir, const unsigned long long *moments,
                         Workspace &ws, double *g_out, double *grad_out, double *gf_out,
-                        double *err_out, cudaStream_t st) {
+                        double *err_out, cudaStream_t st, DevScalars *host) {
     const int blocks = dual_blocks(n, ws);
     if (g.dim == 3)
-        dual_kernel<3><<<blocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, p_dir, moments, ws.part, ws.sc, g_out,
-                                                   grad_out, gf_out, err_out);
+        dual_kernel<3><<<blocks * kDualBlocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, p_dir, moments, ws.part, ws.sc, g_out,
+                                                   grad_out, gf_out, err_out, host);
     else
-        dual_kernel<2><<<blocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, p_dir, moments, ws.part, ws.sc, g_out,
-                                                   grad_out, gf_out, err_out);
+        dual_kernel<2><<<blocks * kDualBlocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, p_dir, moments, ws.part, ws.sc, g_out,
+                                                   grad_out, gf_out, err_out, host);
     return cudaGetLastError();
 }
 
@@ -1049,11 +1274,11 @@ cudaError_t launch_points_dual(int dim, int n, const double *x, const double *A,
     memset(&g, 0, sizeof g);
     g.dim = dim;
     if (dim == 3)
-        dual_kernel<3, true><<<blocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, nullptr, nullptr, ws.part, ws.sc, g_out,
-                                                         grad_out, nullptr, err_out, mom_pts);
+        dual_kernel<3, true><<<blocks * kDualBlocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, nullptr, nullptr, ws.part, ws.sc, g_out,
+                                                         grad_out, nullptr, err_out, nullptr, mom_pts);
     else
-        dual_kernel<2, true><<<blocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, nullptr, nullptr, ws.part, ws.sc, g_out,
-                                                         grad_out, nullptr, err_out, mom_pts);
+        dual_kernel<2, true><<<blocks * kDualBlocks, kDualThreads, 0, st>>>(g, n, x, A, w, v, nullptr, nullptr, ws.part, ws.sc, g_out,
+                                                         grad_out, nullptr, err_out, nullptr, mom_pts);
     return cudaGetLastError();
 }
 
@@ -1104,14 +1329,17 @@ cudaError_t launch_lbfgs_pdir(int n, Workspace &ws, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_lbfgs_push(int n, int slot, int cap, int nprev, bool dir, int hist, int hist_acc, double gamma,
+cudaError_t launch_lbfgs_push(int n, int cap, int history, const PushState *state, bool dir, double *Wbest,
                               Workspace &ws, cudaStream_t st) {
-    if (cap > kLbfgsMax || nprev >= cap || hist >= cap || hist_acc >= cap || !ws.lb_part || !ws.lb_coef ||
-        !ws.gram || ws.lb_rows < 1)
+    if (cap > kLbfgsMax || history >= cap || history < 1 || !state || !ws.lb_part || !ws.lb_coef || !ws.gram ||
+        ws.lb_rows < 1)
         return cudaErrorInvalidValue;
-    lbfgs_push_kernel<<<lbfgs_blocks(n, kLbR, ws), kLbT, 0, st>>>(n, slot, cap, nprev, ws.W, ws.Wt, ws.gf, ws.gft,
-                                                                  ws.S, ws.Y, ws.rho, ws.gram, ws.lb_part, ws.sc,
-                                                                  dir ? 1 : 0, hist, hist_acc, gamma, ws.lb_coef);
+    // a warp per pair and the new one; the pairs of one range over up to four SMs
+    const int ranges = lbfgs_blocks(n, kLbR, ws), warps = std::max(2, std::min(kLbT / 32, history + 1));
+    const int split = std::max(1, std::min({4, ws.lb_rows / ranges, (history + 2) / 2}));
+    lbfgs_push_kernel<<<dim3(ranges, split), warps * 32, 0, st>>>(n, cap, state, ws.W, ws.Wt, ws.gf, ws.gft, ws.S, ws.Y,
+                                                                  ws.rho, ws.gram, ws.lb_part, ws.sc, dir ? 1 : 0,
+                                                                  ws.lb_coef, Wbest);
     return cudaGetLastError();
 }
 
