@@ -14,10 +14,12 @@
 // bounded by a small multiple of u * T with
 //     T <= Lambda (R + sqrt(C*/lambda))^2 + C*
 // (Lambda >= max ||A_i||_F, lambda <= min lambda_min(A_i), R = tile
-// half-diagonal, C* ~ the best cost of the pixel).  The seed's index inside a
-// group of 32 is packed into the 5 low mantissa bits of the cost, so one
-// 3-input min and two 2-input min/max keep the two smallest costs of a pixel
-// with the index of the smallest.  A pixel whose best and second-best FP32
+// half-diagonal, C* ~ the best cost of the pixel).  The dense sweep keeps the
+// two smallest costs of a pixel over groups of eight seeds and settles the
+// winner's own group at the end (see dense_chunk); where pruned, the seed's
+// index inside a group of 32 is packed into the 5 low mantissa bits of the cost,
+// so one 3-input min and two 2-input min/max keep the two smallest with the
+// index of the smallest.  A pixel whose best and second-best FP32
 // costs are closer than twice the bound is queued and rescored in FP64 with
 // the reference arithmetic of the cost matrix; every other label is the exact
 // argmin.
@@ -46,24 +48,36 @@ namespace {
 
 using namespace fp32;
 
-template <int D>
+// Tiles: the large ones share a row's coefficients between 16 pixels; the small ones
+// spread a small grid over more SMs.  NS chunks' coefficients are held at a time (two
+// blocks an SM).
+template <int D, bool SMALL>
 struct Cfg;
 template <>
-struct Cfg<3> {  // 16^3 voxels, one 16-voxel row per thread
-    static constexpr int TX = 1, P = 16, TY = 16, TZ = 16;
+struct Cfg<3, false> {  // 16^3 voxels, one 16-voxel row per thread
+    static constexpr int TX = 1, P = 16, TY = 16, TZ = 16, MINB = 2, NS = 3;
 };
 template <>
-struct Cfg<2> {  // 64 x 64 pixels, four 16-pixel row segments per row
-    static constexpr int TX = 4, P = 16, TY = 64, TZ = 1;
+struct Cfg<2, false> {  // 64 x 64 pixels, four 16-pixel row segments per row
+    static constexpr int TX = 4, P = 16, TY = 64, TZ = 1, MINB = 2, NS = 4;
+};
+template <>
+struct Cfg<3, true> {  // 8^3 voxels, two 4-voxel row segments per row
+    static constexpr int TX = 2, P = 4, TY = 8, TZ = 8, MINB = 4, NS = 1;
+};
+template <>
+struct Cfg<2, true> {  // 32 x 16 pixels, eight 4-pixel row segments per row
+    static constexpr int TX = 8, P = 4, TY = 16, TZ = 1, MINB = 4, NS = 1;
 };
 
 // The grid's last-axis tiles start at tile index `toff` (the first tile of the
 // scoring window).
-template <int D>
-__global__ void __launch_bounds__(256, 2) assign_fp32_kernel(const __grid_constant__ TileSrc src, const int toff) {
-    using C = Cfg<D>;
+template <int D, bool SMALL>
+__global__ void __launch_bounds__(Cfg<D, SMALL>::TX *Cfg<D, SMALL>::TY *Cfg<D, SMALL>::TZ, Cfg<D, SMALL>::MINB)
+    assign_fp32_kernel(const __grid_constant__ TileSrc src, const int toff) {
+    using C = Cfg<D, SMALL>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    SharedLayout<D> &sm = *reinterpret_cast<SharedLayout<D> *>(smem_raw);
+    SharedLayout<D, C::NS> &sm = *reinterpret_cast<SharedLayout<D, C::NS> *>(smem_raw);
     init_shared<D>(sm);
     uint32_t uses[4] = {0u, 0u, 0u, 0u};
     const int by = D == 2 ? (int)blockIdx.y + toff : (int)blockIdx.y;
@@ -119,24 +133,30 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-template <int D>
+template <class C>
+dim3 tile_grid(const GridDev &g, int &toff) {
+    // tiles along the last axis that meet the window [win_lo, win_hi)
+    const int TL = g.dim == 3 ? C::TZ : C::TY;
+    toff = win_lo(g) / TL;
+    const int tcount = (win_hi(g) - 1) / TL - toff + 1;
+    return dim3((g.res[0] + C::TX * C::P - 1) / (C::TX * C::P),
+                g.dim == 2 ? tcount : (g.res[1] + C::TY - 1) / C::TY, g.dim == 3 ? tcount : 1);
+}
+
+template <int D, bool SMALL>
 cudaError_t launch_assign_fp32_t(const GridDev &g, int n, Workspace &ws, int32_t *labels,
                                  unsigned long long *gmom, cudaStream_t st) {
-    using C = Cfg<D>;
-    const size_t smem = sizeof(SharedLayout<D>);
-    constexpr unsigned bit = D == 3 ? kAttrFp32Score3 : kAttrFp32Score2;
+    using C = Cfg<D, SMALL>;
+    const size_t smem = sizeof(SharedLayout<D, C::NS>);
+    constexpr unsigned bit = SMALL ? (D == 3 ? kAttrFp32Small3 : kAttrFp32Small2) : D == 3 ? kAttrFp32Score3 : kAttrFp32Score2;
     if (!(ws.attr_done & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(assign_fp32_kernel<D>,
+        cudaError_t e = cudaFuncSetAttribute(assign_fp32_kernel<D, SMALL>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         ws.attr_done |= bit;
     }
-    // tiles along the last axis that meet the window [win_lo, win_hi)
-    constexpr int TL = D == 3 ? C::TZ : C::TY;
-    const int toff = win_lo(g) / TL;
-    const int tcount = (win_hi(g) - 1) / TL - toff + 1;
-    dim3 grid((g.res[0] + C::TX * C::P - 1) / (C::TX * C::P), D == 2 ? tcount : (g.res[1] + C::TY - 1) / C::TY,
-              D == 3 ? tcount : 1);
+    int toff = 0;
+    const dim3 grid = tile_grid<C>(g, toff);
     const int n_chunks = (n + kChunk - 1) / kChunk;
     double hx = 0.5 * C::TX * C::P * g.h[0], hy = 0.5 * C::TY * g.h[1], hz = D == 3 ? 0.5 * C::TZ * g.h[2] : 0.0;
     const float R = (float)(sqrt(hx * hx + hy * hy + hz * hz) * (1.0 + 1e-6));
@@ -145,16 +165,29 @@ cudaError_t launch_assign_fp32_t(const GridDev &g, int n, Workspace &ws, int32_t
                       ws.prune ? ws.groups : nullptr, ws.pairs_scored, ws.wait_limit};
     const cudaError_t ep = record_scoring_start(ws, st);
     if (ep != cudaSuccess) return ep;
-    assign_fp32_kernel<D><<<grid, C::TX * C::TY * C::TZ, smem, st>>>(src, toff);
+    assign_fp32_kernel<D, SMALL><<<grid, C::TX * C::TY * C::TZ, smem, st>>>(src, toff);
     return cudaGetLastError();
+}
+
+// Small tiles for a dense sweep whose large tiles would leave half of the SMs idle.
+// MEASURED, us large / small: 100^2, n = 25 (4 large tiles): 28.7 / 15.9; 64^3, n = 700
+// (64): 148 / 121; 700^2, n = 1000 (121): 138 / 141; 80^3, n = 1000 (125): 184 / 228.
+template <int D>
+cudaError_t launch_assign_fp32_d(const GridDev &g, int n, Workspace &ws, int32_t *labels, unsigned long long *gmom,
+                                 cudaStream_t st) {
+    int toff = 0;
+    const dim3 t = tile_grid<Cfg<D, false>>(g, toff);
+    const bool small = !ws.prune && (long long)t.x * t.y * t.z < ws.sms / 2;
+    return small ? launch_assign_fp32_t<D, true>(g, n, ws, labels, gmom, st)
+                 : launch_assign_fp32_t<D, false>(g, n, ws, labels, gmom, st);
 }
 
 }  // namespace
 
 cudaError_t launch_assign_fp32(const GridDev &g, int n, Workspace &ws, int32_t *labels,
                                unsigned long long *moments, cudaStream_t st) {
-    return g.dim == 3 ? launch_assign_fp32_t<3>(g, n, ws, labels, moments, st)
-                      : launch_assign_fp32_t<2>(g, n, ws, labels, moments, st);
+    return g.dim == 3 ? launch_assign_fp32_d<3>(g, n, ws, labels, moments, st)
+                      : launch_assign_fp32_d<2>(g, n, ws, labels, moments, st);
 }
 
 cudaError_t launch_tie_gap(const GridDev &g, int n, const double *x, const double *A, const double *w,

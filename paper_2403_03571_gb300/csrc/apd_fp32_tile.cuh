@@ -39,11 +39,16 @@ __device__ __forceinline__ float pack(float c, unsigned idx) {
     return __uint_as_float((__float_as_uint(c) & ~31u) | idx);
 }
 
+// the same with the index inside a group of eight
+__device__ __forceinline__ float pack8(float c, unsigned idx) {
+    return __uint_as_float((__float_as_uint(c) & ~7u) | idx);
+}
+
 // Row coefficients of two consecutive seeds (see the file comment), returned as
 // duplicated pairs for the packed pixel-pair FMAs.  Every multiply is rounded on
 // its own (no contraction), so the fast and update passes compute identical bits.
-template <int D>
-__device__ __forceinline__ void seed_pair_coeffs(const float4 (*phi)[kChunk], int s0, float f1, float f2,
+template <int D, int N>
+__device__ __forceinline__ void seed_pair_coeffs(const float4 (*phi)[N], int s0, float f1, float f2,
                                                  float2 &qa, float2 &qb, float2 &ba, float2 &bbb,
                                                  float2 &aa2, float2 &ab2) {
     float a[2], bb[2], q00[2];
@@ -111,11 +116,12 @@ __device__ __forceinline__ unsigned sortable_key(float v) {
     return u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
 }
 
-template <int D>
+// NS: chunks whose coefficients are held at a time (dense sweeps).
+template <int D, int NS = 1>
 struct SharedLayout {
     static constexpr int K = moment_width(D);
     SeedRec raw[2][kChunk];
-    float4 phi[D][kChunk];
+    float4 phi[D][NS * kChunk];
     float4 sbd[kChunk];  // per seed of the chunk: offset from the tile centre, lambda_min lower bound
     float swp[kChunk];   // per seed: a lower bound of wref - w (the weight part of its cost bound)
     unsigned long long tval[kTable][K];
@@ -130,8 +136,8 @@ struct SharedLayout {
     unsigned long long scored;  // pixel-seed pairs the CTA's scoring evaluated in this tile
 };
 
-template <int D>
-__device__ __forceinline__ void table_add(SharedLayout<D> &sm, unsigned long long *gmom, int label,
+template <int D, int NS>
+__device__ __forceinline__ void table_add(SharedLayout<D, NS> &sm, unsigned long long *gmom, int label,
                                           const unsigned long long (&val)[moment_width(D)]) {
     constexpr int K = moment_width(D);
     int slot = label & (kTable - 1);
@@ -177,8 +183,8 @@ __device__ __forceinline__ void run_moments(unsigned long long cnt, unsigned lon
     }
 }
 
-template <int D>
-__device__ __forceinline__ void flush_run(SharedLayout<D> &sm, unsigned long long *gmom, int label,
+template <int D, int NS>
+__device__ __forceinline__ void flush_run(SharedLayout<D, NS> &sm, unsigned long long *gmom, int label,
                                           unsigned long long cnt, unsigned long long s0,
                                           unsigned long long s00, unsigned long long u1,
                                           unsigned long long u2) {
@@ -213,6 +219,90 @@ struct TileSrc {
     uint32_t wait_limit;          // polls of each chunk wait (kDefaultWaitPolls normally)
 };
 
+// Dense scoring of the chunk whose coefficients lie in slot `slot` of sm.phi for the
+// thread's row of P pixels: b1, b2 the smallest and second-smallest cost so far, GI the
+// scan position of the best.
+//
+// Bound: the min and select instructions, issued at half the rate of the FMAs, so a seed
+// gets as few as possible: the costs of kSub seeds meet in one minimum a pixel (one
+// 3-input min for two seeds), and five instructions join it to (b1, b2, GI).  Which of the
+// kSub won, and the runner-up among them, is settled once the chunks held in shared memory
+// are scored, for the pixels whose best lies in them: only the winner's own group of kSub
+// can hide a second-best cost (an earlier winner's group has entered b2 by its minimum).
+// Several chunks are held, so that the warps meet at fewer barriers.  About 2.7 min / select
+// instructions a pixel and seed with the index packed into each cost, and a second pass
+// over every group of 32 that could matter: 987 us for 700 seeds on 203 x 190 x 161
+// voxels; MEASURED_DENSE.
+constexpr int kSub = 8;
+template <int D, int NS, int P>
+__device__ __forceinline__ void dense_chunk(SharedLayout<D, NS> &sm, const int slot, const int valid, const float f1,
+                                            const float f2, const float2 (&y2)[P / 2], float (&b1)[P], float (&b2)[P],
+                                            int (&GI)[P]) {
+    for (int s0 = slot * kChunk; s0 < slot * kChunk + valid; s0 += kSub) {
+        float m[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) m[p] = FLT_MAX;
+#pragma unroll
+        for (int l = 0; l < kSub; l += 2) {
+            float2 qa, qb, ba, bbb, aa2, ab2;
+            seed_pair_coeffs<D>(sm.phi, s0 + l, f1, f2, qa, qb, ba, bbb, aa2, ab2);
+#pragma unroll
+            for (int q = 0; q < P / 2; ++q) {
+                const float2 ca = ffma2(ffma2(qa, y2[q], ba), y2[q], aa2);
+                const float2 cb = ffma2(ffma2(qb, y2[q], bbb), y2[q], ab2);
+                m[2 * q] = l == 0 ? fminf(ca.x, cb.x) : fmin3(m[2 * q], ca.x, cb.x);
+                m[2 * q + 1] = l == 0 ? fminf(ca.y, cb.y) : fmin3(m[2 * q + 1], ca.y, cb.y);
+            }
+        }
+        const int open = ~s0;  // negative: the seed of the group is not known yet
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            GI[p] = m[p] < b1[p] ? open : GI[p];
+            b2[p] = fminf(b2[p], fmaxf(b1[p], m[p]));
+            b1[p] = fminf(b1[p], m[p]);
+        }
+    }
+}
+
+// Settles the open pixels; scan(s) is the scan position of entry s of sm.phi.
+template <int D, int NS, int P, class Scan>
+__device__ __forceinline__ void dense_settle(SharedLayout<D, NS> &sm, const float f1, const float f2,
+                                             const float2 (&y2)[P / 2], float (&b2)[P], int (&GI)[P], Scan scan) {
+    while (true) {
+        int open = 0;  // a lane's first open group
+#pragma unroll
+        for (int p = P - 1; p >= 0; --p) open = GI[p] < 0 ? GI[p] : open;
+        if (!__any_sync(0xffffffffu, open < 0)) break;
+        const int s0 = open < 0 ? ~open : 0, base = scan(s0);
+        float ca[kSub], cb[kSub], cq[kSub];
+#pragma unroll
+        for (int l = 0; l < kSub; l += 2) {
+            float2 qa, qb, ba, bbb, aa2, ab2;
+            seed_pair_coeffs<D>(sm.phi, s0 + l, f1, f2, qa, qb, ba, bbb, aa2, ab2);
+            ca[l] = aa2.x, ca[l + 1] = ab2.x;
+            cb[l] = ba.x, cb[l + 1] = bbb.x;
+            cq[l] = qa.x, cq[l + 1] = qb.x;
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            if (GI[p] != open || open == 0) continue;
+            const float y = p & 1 ? y2[p / 2].y : y2[p / 2].x;
+            float k1 = FLT_MAX, k2 = FLT_MAX;
+#pragma unroll
+            for (int l = 0; l < kSub; l += 2) {
+                // the index in the low bits: at most 8 units of the last place, inside kKappa's share
+                const float ka = pack8(fmaf(fmaf(cq[l], y, cb[l]), y, ca[l]), l);
+                const float kb = pack8(fmaf(fmaf(cq[l + 1], y, cb[l + 1]), y, ca[l + 1]), l + 1);
+                const float mn = fminf(ka, kb), mx = fmaxf(ka, kb);
+                k2 = fmin3(k2, fmaxf(k1, mn), mx);
+                k1 = fminf(k1, mn);
+            }
+            b2[p] = fminf(b2[p], k2);
+            GI[p] = base + (int)(__float_as_uint(k1) & (unsigned)(kSub - 1));
+        }
+    }
+}
+
 // Scores the (TX P) x TY x TZ tile (bx, by, bz) of `s` with NT = TX TY TZ
 // threads; thread (seg, ty, tz) owns the row segment of P pixels starting at
 // first-axis offset seg P inside the tile.
@@ -222,8 +312,8 @@ struct TileSrc {
 // again on return.  Returns false if a chunk wait timed out: thread 0 has then
 // waited (with the default limit) for every copy still in flight, and the CTA
 // must stop.
-template <int D, int TX, int P, int TY, int TZ>
-__device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s, const int bx, const int by,
+template <int D, int TX, int P, int TY, int TZ, int NS>
+__device__ __forceinline__ bool score_tile(SharedLayout<D, NS> &sm, const TileSrc &s, const int bx, const int by,
                                            const int bz, uint32_t (&uses)[4]) {
     constexpr int K = moment_width(D);
     constexpr int NT = TX * TY * TZ;
@@ -266,12 +356,12 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
         sm.cref[2] = (D == 3) ? g.lo[2] + (double)kc2 * g.h[2] : 0.0;
         sm.cref[3] = dkey_inv(s.sc->wref_key);
         int start = 0;
-        if (s.scodes) {
-            double frac[3] = {0.0, 0.0, 0.0};
+        if (s.scodes && n_chunks > 1) {  // only the order of the scan: FP32 will do
+            float frac[3] = {0.f, 0.f, 0.f};
             const int kc[3] = {kc0, kc1, kc2};
 #pragma unroll
-            for (int a = 0; a < D; ++a) frac[a] = ((double)kc[a] + 0.5) / (double)g.res[a];
-            const uint32_t code = morton_code(D, frac);
+            for (int a = 0; a < D; ++a) frac[a] = ((float)kc[a] + 0.5f) / (float)g.res[a];
+            const uint32_t code = morton_code_f(D, frac);
             int lo = 0, hi = n;
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
@@ -322,7 +412,7 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
     const int start_chunk = sm.start_chunk;
     auto chunk_at = [&](int k) { return chunk_from(start_chunk, k); };
 
-    // per pixel: two smallest packed costs (b1 <= b2) and the scan position of the best
+    // per pixel: two smallest costs (b1 <= b2; packed where pruned) and the scan position of the best
     float b1[P], b2[P];
     int GI[P];
 #pragma unroll
@@ -370,6 +460,7 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
             __syncwarp();
         }
         const bool need_chunk = s.groups ? (__syncthreads_or(live != 0u) != 0) : true;
+        const int slot = s.groups ? 0 : k % NS;
         // transform this chunk into the row-form coefficients
         for (int sl = need_chunk ? tid : kChunk; sl < kChunk; sl += NT) {
             const int si = c * kChunk + sl;
@@ -409,9 +500,9 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
                     v2 = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
-            sm.phi[0][sl] = v0;
-            sm.phi[1][sl] = v1;
-            if (D == 3) sm.phi[2][sl] = v2;
+            sm.phi[0][slot * kChunk + sl] = v0;
+            sm.phi[1][slot * kChunk + sl] = v1;
+            if (D == 3) sm.phi[2][slot * kChunk + sl] = v2;
             if (s.groups) {
                 sm.sbd[sl] = bd;
                 sm.swp[sl] = bw;
@@ -425,26 +516,32 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
                      &sm.bar[b]);
             ++uses[2 + b];
         }
-        if (ok && need_chunk) {
+        if (!s.groups) {  // dense: the chunks held, once the slots are full
+            if (slot != NS - 1 && k != n_chunks - 1) continue;
+            if (ok) {
+                for (int q = 0; q <= slot; ++q) {
+                    const int valid = min(kChunk, n - chunk_at(k - slot + q) * kChunk);
+                    if (s.pairs_scored && lane == 0)
+                        atomicAdd(&sm.scored, (unsigned long long)valid * (unsigned long long)(32 * P));
+                    dense_chunk<D, NS, P>(sm, q, valid, f1, f2, y2, b1, b2, GI);
+                }
+                dense_settle<D, NS, P>(sm, f1, f2, y2, b2, GI, [&](int e) {
+                    return chunk_at(k - slot + e / kChunk) * kChunk + e % kChunk;
+                });
+            }
+        } else if (ok && need_chunk) {
             while (true) {
                 // drop the groups that the current second-best costs rule out,
                 // then take the remaining one with the smallest bound
                 const bool mine = (live >> lane) & 1u;
-                float bmax = FLT_MAX;
-                if (s.groups) {
-                    bmax = warp_max_b2<P>(b2);
-                    live &= ~__ballot_sync(0xffffffffu,
-                                           mine && group_beyond(sm.glb[wid][lane], sm.gwp[wid][lane], bmax));
-                }
+                float bmax = warp_max_b2<P>(b2);
+                live &= ~__ballot_sync(0xffffffffu, mine && group_beyond(sm.glb[wid][lane], sm.gwp[wid][lane], bmax));
                 if (!live) break;
-                unsigned pick = live;  // dense: index order
-                if (s.groups) {
-                    const bool cand = (live >> lane) & 1u;
-                    const unsigned key = cand ? sortable_key(sm.glb[wid][lane]) : 0xffffffffu;
-                    const unsigned kmin = __reduce_min_sync(0xffffffffu, key);
-                    pick = __ballot_sync(0xffffffffu, cand && key == kmin);
-                    if (!pick) break;  // cannot happen: kmin is a candidate's key
-                }
+                const bool cand = (live >> lane) & 1u;
+                const unsigned gkey = cand ? sortable_key(sm.glb[wid][lane]) : 0xffffffffu;
+                const unsigned gmin = __reduce_min_sync(0xffffffffu, gkey);
+                const unsigned pick = __ballot_sync(0xffffffffu, cand && gkey == gmin);
+                if (!pick) break;  // cannot happen: gmin is a candidate's key
                 const int gr = __ffs(pick) - 1;
                 live &= ~(1u << gr);
                 const int gbase = c * kChunk + gr * kGroup;
@@ -462,76 +559,45 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
                                     pack(cb.y, lb), gbase);
                     }
                 };
-                if (s.groups) {
-                    // Pruned: the seeds of the group whose own bound (lambda_i times the
-                    // squared distance from x_i to the warp's pixel box, plus wref - w_i)
-                    // is not above every pixel's second-best cost, scored in pairs
-                    // (l, l+1) (marked at the even bit l) by the exact update directly:
-                    // nearly every such pair changes some pixel's top-2.
-                    const int sl = gr * kGroup + lane;
-                    const bool real = sl < valid_in_chunk;
-                    float slb = FLT_MAX, swp = 0.f;
-                    if (real) {
-                        const float4 sb = sm.sbd[sl];
-                        swp = sm.swp[sl];
-                        const float xs[3] = {sb.x, sb.y, sb.z};
-                        float d2 = 0.f;
+                // Pruned: the seeds of the group whose own bound (lambda_i times the
+                // squared distance from x_i to the warp's pixel box, plus wref - w_i)
+                // is not above every pixel's second-best cost, scored in pairs
+                // (l, l+1) (marked at the even bit l) by the exact update directly:
+                // nearly every such pair changes some pixel's top-2.
+                const int sl = gr * kGroup + lane;
+                const bool real = sl < valid_in_chunk;
+                float slb = FLT_MAX, swp = 0.f;
+                if (real) {
+                    const float4 sb = sm.sbd[sl];
+                    swp = sm.swp[sl];
+                    const float xs[3] = {sb.x, sb.y, sb.z};
+                    float d2 = 0.f;
 #pragma unroll
-                        for (int a = 0; a < D; ++a) {
-                            const float lo = sm.wrel[wid][a], hi = sm.wrel[wid][3 + a];
-                            const float slack = 1e-6f * (fabsf(lo) + fabsf(hi) + 2.f * fabsf(xs[a]));
-                            const float t = fmaxf(fmaxf(xs[a] - hi, lo - xs[a]) - slack, 0.f);
-                            d2 = fmaf(t, t, d2);
-                        }
-                        slb = __fmul_rd(__fmul_rd(sb.w, d2), 1.f - 1e-5f) + swp;
+                    for (int a = 0; a < D; ++a) {
+                        const float lo = sm.wrel[wid][a], hi = sm.wrel[wid][3 + a];
+                        const float slack = 1e-6f * (fabsf(lo) + fabsf(hi) + 2.f * fabsf(xs[a]));
+                        const float t = fmaxf(fmaxf(xs[a] - hi, lo - xs[a]) - slack, 0.f);
+                        d2 = fmaf(t, t, d2);
                     }
-                    unsigned done = 0u;
-                    if (!(bmax < FLT_MAX)) {
-                        // first group of the tile: the pair holding the seed of smallest
-                        // bound goes first, so that the rest is tested against real costs
-                        const unsigned key = real ? sortable_key(slb) : 0xffffffffu;
-                        const unsigned kmin = __reduce_min_sync(0xffffffffu, key);
-                        const int j = (__ffs(__ballot_sync(0xffffffffu, key == kmin)) - 1) & ~1;
-                        update_pair(j);
-                        done = 1u << j;
-                        bmax = warp_max_b2<P>(b2);
-                    }
-                    const unsigned sv = __ballot_sync(0xffffffffu, real && !group_beyond(slb, swp, bmax));
-                    const unsigned pm = (sv | (sv >> 1)) & 0x55555555u & ~done;
-                    if (s.pairs_scored && lane == 0)
-                        atomicAdd(&sm.scored, (unsigned long long)(2 * __popc(pm | done)) *
-                                                  (unsigned long long)(32 * P));
-                    for (unsigned m = pm; m; m &= m - 1u) update_pair(__ffs(m) - 1);
-                    continue;
+                    slb = __fmul_rd(__fmul_rd(sb.w, d2), 1.f - 1e-5f) + swp;
                 }
+                unsigned done = 0u;
+                if (!(bmax < FLT_MAX)) {
+                    // first group of the tile: the pair holding the seed of smallest
+                    // bound goes first, so that the rest is tested against real costs
+                    const unsigned key = real ? sortable_key(slb) : 0xffffffffu;
+                    const unsigned kmin = __reduce_min_sync(0xffffffffu, key);
+                    const int j = (__ffs(__ballot_sync(0xffffffffu, key == kmin)) - 1) & ~1;
+                    update_pair(j);
+                    done = 1u << j;
+                    bmax = warp_max_b2<P>(b2);
+                }
+                const unsigned sv = __ballot_sync(0xffffffffu, real && !group_beyond(slb, swp, bmax));
+                const unsigned pm = (sv | (sv >> 1)) & 0x55555555u & ~done;
                 if (s.pairs_scored && lane == 0)
-                    atomicAdd(&sm.scored, (unsigned long long)min(kGroup, valid_in_chunk - gr * kGroup) *
+                    atomicAdd(&sm.scored, (unsigned long long)(2 * __popc(pm | done)) *
                                               (unsigned long long)(32 * P));
-                // dense: fast pass (smallest cost of this group per pixel, one 3-input
-                // min per two pairs), then the update pass only where it can matter
-                float gm[P];
-#pragma unroll
-                for (int p = 0; p < P; ++p) gm[p] = FLT_MAX;
-#pragma unroll 2
-                for (int l = 0; l < kGroup; l += 2) {
-                    float2 qa, qb, ba, bbb, aa2, ab2;
-                    seed_pair_coeffs<D>(sm.phi, gr * kGroup + l, f1, f2, qa, qb, ba, bbb, aa2, ab2);
-#pragma unroll
-                    for (int q = 0; q < P / 2; ++q) {
-                        const float2 ca = ffma2(ffma2(qa, y2[q], ba), y2[q], aa2);
-                        const float2 cb = ffma2(ffma2(qb, y2[q], bbb), y2[q], ab2);
-                        gm[2 * q] = fmin3(gm[2 * q], ca.x, cb.x);
-                        gm[2 * q + 1] = fmin3(gm[2 * q + 1], ca.y, cb.y);
-                    }
-                }
-                // a packed key differs from its cost by < 32 ulp: a group whose smallest
-                // cost exceeds b2 by the margin cannot change b1 or b2 and is skipped
-                bool need = false;
-#pragma unroll
-                for (int p = 0; p < P; ++p) need |= gm[p] < fmaf(fabsf(b2[p]), 0x1p-15f, b2[p]);
-                if (!__any_sync(0xffffffffu, need)) continue;
-#pragma unroll 2
-                for (int l = 0; l < kGroup; l += 2) update_pair(l);
+                for (unsigned m = pm; m; m &= m - 1u) update_pair(__ffs(m) - 1);
             }
         }
         __syncthreads();
@@ -542,9 +608,11 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
         for (int b = 0; b < 2; ++b)
             while (uses[b] < uses[2 + b] && mbar_wait_bounded(&sm.bar[b], uses[b] & 1u, &s.sc->status)) ++uses[b];
     }
-    // scan position of the best: its group base and the index bits of its key
+    // pruned: scan position of the best, its group base and the index bits of its key
+    if (s.groups) {
 #pragma unroll
-    for (int p = 0; p < P; ++p) GI[p] |= (int)(__float_as_uint(b1[p]) & 31u);
+        for (int p = 0; p < P; ++p) GI[p] |= (int)(__float_as_uint(b1[p]) & 31u);
+    }
     // scan position -> seed index
     if (s.perm && ok) {
 #pragma unroll
@@ -671,8 +739,8 @@ __device__ __forceinline__ bool score_tile(SharedLayout<D> &sm, const TileSrc &s
 }
 
 // Empty table and initialised chunk barriers; call once per CTA.
-template <int D>
-__device__ __forceinline__ void init_shared(SharedLayout<D> &sm) {
+template <int D, int NS>
+__device__ __forceinline__ void init_shared(SharedLayout<D, NS> &sm) {
     constexpr int K = moment_width(D);
     for (int t = threadIdx.x; t < kTable; t += blockDim.x) {
         sm.tkey[t] = -1;

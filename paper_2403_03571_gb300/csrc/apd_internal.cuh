@@ -124,6 +124,7 @@ constexpr unsigned kAttrFp32Score2 = 1u << 0, kAttrFp32Score3 = 1u << 1;
 constexpr unsigned kAttrTcScore = 1u << 3;     // + 1 bit per (dimension, operand kind): 4 bits
 constexpr unsigned kAttrTcScoreRec = 1u << 7;  // the recording variant: 4 bits
 constexpr unsigned kAttrPoints2 = 1u << 11, kAttrPoints3 = 1u << 12;
+constexpr unsigned kAttrFp32Small2 = 1u << 13, kAttrFp32Small3 = 1u << 14;
 
 // One evaluation of a weight solve (trial weights, scoring, rescoring, dual,
 // read-back of the device scalars) captured as a CUDA graph and replayed with
