@@ -12,7 +12,7 @@
 //                            one-instance path (Algorithm 1 fused with moments), then
 //   rescore   (persistent)   FP64 near-tie rescoring
 //   cells     (thread/cell)  the per-cell terms of eqs. (2.7)-(2.8) from the moments
-//   lbfgs     (CTA/instance) their sums, one transition of the L-BFGS / strong-Wolfe
+//   lbfgs     (2 CTAs/inst.) their sums, one transition of the L-BFGS / strong-Wolfe
 //                            state machine of Algorithm 2, the next trial point and its
 //                            weights in the seed records
 // The records' positions and matrices are made by one prep launch (CTA/instance) before
@@ -438,21 +438,44 @@ __global__ void __launch_bounds__(kCellThreads) batch_cells_kernel(const __grid_
 // zoom with safeguards) on f = -g~, two-loop recursion, curvature-pair skip,
 // best-iterate fallback, stop at the first evaluation with max rel err < eps.
 constexpr int kOwn = 8;  // seeds a thread keeps in registers
+// Exchange between the warps of an instance (see SolveCtx::gather).
+constexpr int kSolveBlocks = 2, kSolveWarps = kSolveThreads / 32;
+static_assert(kSolveWarps == 8, "the warps' values lie in eight lanes");
+struct SolveExchange {
+    unsigned long long buf[2][3 * kSolveWarps];
+    uint64_t bar[2];
+};
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// v into `to` of the cluster's block `rank`, its bytes counted at that block's barrier `bar`
+__device__ __forceinline__ void send_cluster(const void *to, unsigned long long v, const void *bar, int rank) {
+    uint32_t t, m;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(t) : "r"(smem_u32(to)), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(m) : "r"(smem_u32(bar)), "r"(rank));
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(t), "l"(v), "r"(m)
+                 : "memory");
+}
+
 struct SolveCtx {
     const BArgs &a;
     const BInst &I;
     BSolve &s;
-    double *sh;        // [16]
+    SolveExchange &ex;
+    DevScalars *sc;
+    int vt;            // thread of the instance, over the cluster's blocks
     int b, n, history;
     long long off;
     double *W, *Wt, *p, *gf, *gft, *Wbest, *Wout, *rho;
     unsigned turn;
+    int new_slot;
+    double new_rho;
 
     __device__ void copy(double *dst, const double *src) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+        for (int i = vt; i < n; i += kSolveThreads) dst[i] = src[i];
     }
     __device__ void set_trial(double t) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x) Wt[i] = W[i] + t * p[i];
+        for (int i = vt; i < n; i += kSolveThreads) Wt[i] = W[i] + t * p[i];
         s.cur_t = t;
         s.active = 1;
     }
@@ -462,20 +485,54 @@ struct SolveCtx {
         s.phase = PH_DONE;
         s.active = 0;
     }
-    // Deterministic block sum (block_sum's order: lanes by a butterfly, then the eight
-    // warps), one barrier: two buffers in turn.
-    __device__ double sum(double d) {
-        d = warp_sum(d);
-        double *buf = sh + 8 * (turn & 1);
+    // Each warp's value v into both blocks' buffer, N values a call; returns the value of
+    // warp (lane & 7).  A store into shared memory counts its bytes at the receiving block's
+    // barrier of the turn; a warp sends turn k + 1 after it has read turn k, so two buffers
+    // are enough.
+    template <int N>
+    __device__ void gather(unsigned long long (&v)[N]) {
+        const int lane = threadIdx.x & 31;
+        const unsigned k = turn & 1u, parity = (turn >> 1) & 1u;
         ++turn;
-        if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = d;
-        __syncthreads();
-        double r = buf[threadIdx.x & 7];
-        r += __shfl_xor_sync(0xffffffffu, r, 4);
-        r += __shfl_xor_sync(0xffffffffu, r, 2);
-        r += __shfl_xor_sync(0xffffffffu, r, 1);
-        return r;
+        if (threadIdx.x == 0) mbar_expect_tx(&ex.bar[k], N * kSolveWarps * 8);
+        if (lane < kSolveBlocks) {
+#pragma unroll
+            for (int e = 0; e < N; ++e)
+                send_cluster(&ex.buf[k][e * kSolveWarps + (vt >> 5)], v[e], &ex.bar[k], lane);
+        }
+        mbar_wait_bounded(&ex.bar[k], parity, &sc->status);
+#pragma unroll
+        for (int e = 0; e < N; ++e) v[e] = ex.buf[k][e * kSolveWarps + (lane & (kSolveWarps - 1))];
     }
+    // Deterministic sums (lanes by a butterfly, then the eight warps).
+    template <int N>
+    __device__ void sums(double (&d)[N]) {
+        unsigned long long v[N];
+#pragma unroll
+        for (int e = 0; e < N; ++e) v[e] = (unsigned long long)__double_as_longlong(warp_sum(d[e]));
+        gather<N>(v);
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            double q = __longlong_as_double((long long)v[e]);
+            q += __shfl_xor_sync(0xffffffffu, q, 4);
+            q += __shfl_xor_sync(0xffffffffu, q, 2);
+            q += __shfl_xor_sync(0xffffffffu, q, 1);
+            d[e] = q;
+        }
+    }
+    __device__ double sum(double d) {
+        double v[1] = {d};
+        sums<1>(v);
+        return v[0];
+    }
+    // Largest key over all warps.
+    __device__ unsigned long long max_key(unsigned long long k) {
+        unsigned long long v[1] = {warp_max_key(k)};
+        gather<1>(v);
+        return warp_max_key(v[0]);
+    }
+    // 1 / s.y of slot idx (the pair pushed in this launch is not read back)
+    __device__ double rho_of(int idx) const { return idx == new_slot ? new_rho : rho[idx]; }
     // p = -H gf (two-loop recursion, H0 = gamma I); returns <gf, p>.  Up to kOwn seeds a
     // thread keep p in registers, with the next pair's rows loaded ahead of the sums
     // (through memory a step took 5 us, 21 steps a direction); the roundings are written
@@ -485,7 +542,7 @@ struct SolveCtx {
     }
     __device__ double direction_own() {
         double al[kBHist], pr[kOwn], u[kOwn], v[kOwn];
-        const int t = threadIdx.x;
+        const int t = vt;
         const int hist = s.hist;
         auto row = [&](const double *base, int idx) { return base + (size_t)idx * a.total_n + off; };
         auto slot = [&](int k) { return (s.newest - k + kBHist) % kBHist; };
@@ -503,7 +560,7 @@ struct SolveCtx {
             for (int e = 0; e < kOwn; ++e)
                 if (t + e * kSolveThreads < n) d = __fma_rn(u[e], pr[e], d);
             if (k + 1 < hist) load(row(a.S, slot(k + 1)), u);
-            al[idx] = __dmul_rn(rho[idx], sum(d));
+            al[idx] = __dmul_rn(rho_of(idx), sum(d));
 #pragma unroll
             for (int e = 0; e < kOwn; ++e)
                 if (t + e * kSolveThreads < n) pr[e] = __fma_rn(-al[idx], v[e], pr[e]);
@@ -519,7 +576,7 @@ struct SolveCtx {
             for (int e = 0; e < kOwn; ++e)
                 if (t + e * kSolveThreads < n) d = __fma_rn(v[e], pr[e], d);
             if (k > 0) load(row(a.Y, slot(k - 1)), v);
-            const double c = __fma_rn(-rho[idx], sum(d), al[idx]);
+            const double c = __fma_rn(-rho_of(idx), sum(d), al[idx]);
 #pragma unroll
             for (int e = 0; e < kOwn; ++e)
                 if (t + e * kSolveThreads < n) pr[e] = __fma_rn(u[e], c, pr[e]);
@@ -537,28 +594,28 @@ struct SolveCtx {
     }
     __device__ double direction_any() {
         double al[kBHist];
-        for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = gf[i];
+        for (int i = vt; i < n; i += kSolveThreads) p[i] = gf[i];
         for (int k = 0; k < s.hist; ++k) {
             const int idx = (s.newest - k + kBHist) % kBHist;
             const double *sk = a.S + (size_t)idx * a.total_n + off;
             const double *yk = a.Y + (size_t)idx * a.total_n + off;
             double d = 0.0;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) d += sk[i] * p[i];
-            al[idx] = __dmul_rn(rho[idx], sum(d));
-            for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = __fma_rn(-al[idx], yk[i], p[i]);
+            for (int i = vt; i < n; i += kSolveThreads) d += sk[i] * p[i];
+            al[idx] = __dmul_rn(rho_of(idx), sum(d));
+            for (int i = vt; i < n; i += kSolveThreads) p[i] = __fma_rn(-al[idx], yk[i], p[i]);
         }
-        for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] *= s.gamma;
+        for (int i = vt; i < n; i += kSolveThreads) p[i] *= s.gamma;
         for (int k = s.hist - 1; k >= 0; --k) {
             const int idx = (s.newest - k + kBHist) % kBHist;
             const double *sk = a.S + (size_t)idx * a.total_n + off;
             const double *yk = a.Y + (size_t)idx * a.total_n + off;
             double d = 0.0;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) d += yk[i] * p[i];
-            const double c = __fma_rn(-rho[idx], sum(d), al[idx]);
-            for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = __fma_rn(sk[i], c, p[i]);
+            for (int i = vt; i < n; i += kSolveThreads) d += yk[i] * p[i];
+            const double c = __fma_rn(-rho_of(idx), sum(d), al[idx]);
+            for (int i = vt; i < n; i += kSolveThreads) p[i] = __fma_rn(sk[i], c, p[i]);
         }
         double d = 0.0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        for (int i = vt; i < n; i += kSolveThreads) {
             p[i] = -p[i];
             d += gf[i] * p[i];
         }
@@ -570,7 +627,7 @@ struct SolveCtx {
         double *sk = a.S + (size_t)slot * a.total_n + off;
         double *yk = a.Y + (size_t)slot * a.total_n + off;
         double sy = 0.0, yy = 0.0, ss = 0.0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        for (int i = vt; i < n; i += kSolveThreads) {
             const double si = Wt[i] - W[i];
             const double yi = gft[i] - gf[i];
             sk[i] = si;
@@ -579,11 +636,12 @@ struct SolveCtx {
             yy += yi * yi;
             ss += si * si;
         }
-        sy = sum(sy);
-        yy = sum(yy);
-        ss = sum(ss);
-        if (threadIdx.x == 0) rho[slot] = sy != 0.0 ? 1.0 / sy : 0.0;
-        __syncthreads();
+        double d[3] = {sy, yy, ss};
+        sums<3>(d);
+        sy = d[0], yy = d[1], ss = d[2];
+        new_slot = slot;
+        new_rho = sy != 0.0 ? 1.0 / sy : 0.0;
+        if (vt == 0) rho[slot] = new_rho;
         if (sy > 1e-12 * sqrt(ss * yy) && yy > 0.0) {
             s.newest = slot;
             s.hist = min(s.hist + 1, history);
@@ -593,18 +651,18 @@ struct SolveCtx {
     // The next evaluation's start: the trial weights in the scan-order and natural
     // records, the reference weight, the groups' weight gaps, cleared moments and queue.
     // Maxima by ordered keys (no FP64 comparisons).
-    __device__ void publish(DevScalars *sc, unsigned long long *skey) {
-        __syncthreads();  // Wt is written
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __device__ void publish() {
+        const int lane = vt & 31, wid = vt >> 5;
         unsigned long long wmax = 0ull;
         const int K = moment_width(I.g.dim);
         unsigned long long *mom = a.mom + I.seed_off * K;
-        for (int e = threadIdx.x; e < n * K; e += blockDim.x) mom[e] = 0ull;
+        for (int e = vt; e < n * K; e += kSolveThreads) mom[e] = 0ull;
         SeedRec *recs = a.recs + I.rec_off;
         SeedRec32 *r32 = a.recs32 + I.rec_off, *r32s = a.recs32s + I.rec_off;
         GroupBound *groups = a.groups + I.rec_off / 32;
         int bad = 0;
-        for (int p0 = wid * 32; p0 < n; p0 += kSolveThreads) {
+        unsigned long long mine = 0ull;  // of the lane's group among the first 32 of its warp
+        for (int p0 = wid * 32, it = 0; p0 < n; p0 += kSolveThreads, ++it) {
             const int q = p0 + lane;
             unsigned long long key = 0ull;
             if (q < n) {
@@ -622,16 +680,18 @@ struct SolveCtx {
             }
             const unsigned long long top = warp_max_key(key);
             if (lane == 0) groups[p0 >> 5].wmax = dkey_inv(top ? top : dkey(-DBL_MAX));
+            if (it == lane) mine = top;
             wmax = top > wmax ? top : wmax;
         }
         if (bad) atomicOr(&sc->status, ST_NONFINITE);
-        if (threadIdx.x == 0) *skey = 0ull;
-        __syncthreads();
-        if (lane == 0) atomicMax(skey, wmax);
-        __syncthreads();
-        const double wref = dkey_inv(*skey ? *skey : dkey(-DBL_MAX));
-        for (int g = threadIdx.x; g * 32 < n; g += blockDim.x) groups[g].wgap = __double2float_rd(wref - groups[g].wmax);
-        if (threadIdx.x == 0) {
+        const unsigned long long all = max_key(wmax);
+        const double wref = dkey_inv(all ? all : dkey(-DBL_MAX));
+        const int g0 = wid + lane * kSolveWarps;
+        if (g0 * 32 < n) groups[g0].wgap = __double2float_rd(wref - dkey_inv(mine ? mine : dkey(-DBL_MAX)));
+        if (lane == 0)  // further groups of the warp (its own lane 0 has written them)
+            for (int g = wid + 32 * kSolveWarps; g * 32 < n; g += kSolveWarps)
+                groups[g].wgap = __double2float_rd(wref - groups[g].wmax);
+        if (vt == 0) {
             sc->flag_count = 0u;
             sc->wref_key = dkey(wref);
             split_f32(wref, sc->wref_h, sc->wref_l);
@@ -641,19 +701,30 @@ struct SolveCtx {
 
 enum : int { NX_NONE = 0, NX_NEWDIR, NX_ACCEPT, NX_LSEND, NX_FAIL, NX_ZOOM, NX_GIVEUP };
 
-__global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid_constant__ BArgs a) {
-    __shared__ double sh[16];
-    __shared__ unsigned long long skey, sk_err, sk_min;
-    const int b = blockIdx.x;
+// Two blocks of four warps take an instance: an FP64 instruction occupies a warp's
+// scheduler for 64 clocks, so every warp has a scheduler of its own (eight warps on one SM
+// took turns: 82 us an evaluation of 48 instances, the largest with 1852 seeds and ten
+// pairs; so 65 us).  What is left is the chain of its 21 sums and scalar FP64 steps.
+__global__ void __launch_bounds__(kSolveThreads / kSolveBlocks) __cluster_dims__(kSolveBlocks, 1, 1)
+    batch_lbfgs_kernel(const __grid_constant__ BArgs a) {
+    __shared__ SolveExchange ex;
+    const int b = blockIdx.x / kSolveBlocks;
+    const int vt = threadIdx.x + (blockIdx.x % kSolveBlocks) * (kSolveThreads / kSolveBlocks);
     BSolve s = a.sol[b];
     if (!s.active) return;
+    if (threadIdx.x == 0) {
+        mbar_init(&ex.bar[0], 1);
+        mbar_init(&ex.bar[1], 1);
+        fence_mbar_init();
+    }
+    cluster_sync();
     const BInst &I = a.inst[b];
     const BParams prm = *a.prm;
     DevScalars *sc = a.scs + b;
     const long long off = I.seed_off;
-    SolveCtx c{a,          I,           s,           sh,          b,          I.n,  prm.history,
+    SolveCtx c{a,          I,           s,           ex,          sc,         vt,         b,          I.n,  prm.history,
                off,        a.W + off,   a.Wt + off,  a.p + off,   a.gf + off, a.gft + off,
-               a.Wbest + off, a.Wout + off, a.rho + (size_t)b * kBHist, 0u};
+               a.Wbest + off, a.Wout + off, a.rho + (size_t)b * kBHist, 0u,  -1,  0.0};
     const double c1 = 1e-4, c2 = 0.9;
     const int dim = I.g.dim;
 
@@ -663,13 +734,9 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
     double gval = 0.0, dot_gp = 0.0, err = 0.0, sum_v = 0.0, min_v = 0.0;
     if (s.phase != PH_EVAL_ONLY) {
         const bool with_p = in_line_search(s.phase), with_v = s.phase == PH_INIT || s.phase == PH_INIT_PRED;
-        if (threadIdx.x == 0) {
-            sk_err = 0ull;
-            sk_min = ~0ull;
-        }
         double gsum = 0.0, gp = 0.0, sv = 0.0;
         unsigned long long emax = 0ull, vmin = ~0ull;
-        for (int i = threadIdx.x; i < c.n; i += blockDim.x) {
+        for (int i = vt; i < c.n; i += kSolveThreads) {
             const double gr = -c.gft[i], wi = c.Wt[i], Q = a.Q[off + i];
             gsum = __dadd_rn(gsum, __fma_rn(gr, wi, __dmul_rn(I.g.cell, Q)));
             if (with_p) gp += -gr * c.p[i];
@@ -682,22 +749,17 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
                 vmin = k < vmin ? k : vmin;
             }
         }
-        __syncthreads();
-        emax = warp_max_key(emax);
-        vmin = ~warp_max_key(~vmin);
-        if ((threadIdx.x & 31) == 0) {
-            atomicMax(&sk_err, emax);
-            if (with_v) atomicMin(&sk_min, vmin);
-        }
-        gval = c.sum(gsum);
-        dot_gp = with_p ? c.sum(gp) : 0.0;
+        double d[2] = {gsum, gp};
+        c.sums<2>(d);
+        gval = d[0];
+        dot_gp = with_p ? d[1] : 0.0;
         sum_v = with_v ? c.sum(sv) : 0.0;
-        err = __longlong_as_double((long long)sk_err);
-        min_v = with_v ? dkey_inv(sk_min) : 0.0;
+        err = __longlong_as_double((long long)c.max_key(emax));
+        min_v = with_v ? dkey_inv(~c.max_key(~vmin)) : 0.0;
     }
     const double phi = -gval, dphi = dot_gp;
     s.rescored += sc->flag_count;
-    __syncthreads();
+    cluster_sync();  // both blocks have read the pass's status and counts
     int next = NX_NONE;
     double phi_acc = 0.0;
     if (s.phase == PH_EVAL_ONLY) {
@@ -708,7 +770,7 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
     } else if (bits) {
         s.evals += 1;
         c.finish(map_bits_dev(bits), c.Wbest);
-        if (threadIdx.x == 0) sc->status = 0;
+        if (vt == 0) sc->status = 0;
     } else {
         s.evals += 1;
         s.last_g = gval;
@@ -739,7 +801,7 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
             s.f_pred = phi;
             c.copy(c.W, c.Wt);
             c.copy(c.gf, c.gft);
-            for (int i = threadIdx.x; i < c.n; i += blockDim.x) c.Wt[i] = 0.0;
+            for (int i = vt; i < c.n; i += kSolveThreads) c.Wt[i] = 0.0;
             s.cur_t = -1.0;
             s.phase = PH_INIT_ZERO;
             s.active = 1;
@@ -905,9 +967,9 @@ __global__ void __launch_bounds__(kSolveThreads) batch_lbfgs_kernel(const __grid
         }
     }
     if (next != NX_NONE) c.finish(APD_NOT_CONVERGED, c.Wbest);  // guard exhausted (not expected)
-    __syncthreads();
-    if (s.active) c.publish(sc, &skey);
-    if (threadIdx.x == 0) {
+    cluster_sync();  // Wt is written
+    if (s.active) c.publish();
+    if (vt == 0) {
         a.sol[b] = s;
         if (s.active) atomicAdd(&a.sched->next_active, 1);
     }
@@ -1079,7 +1141,7 @@ int enqueue_iteration(apd_batch &bt, int vi, bool solve_steps, cudaStream_t st) 
         const unsigned cells = (unsigned)((bt.total_n + kCellThreads - 1) / kCellThreads);
         if (bt.dim == 3) batch_cells_kernel<3><<<cells, kCellThreads, 0, st>>>(a);
         else batch_cells_kernel<2><<<cells, kCellThreads, 0, st>>>(a);
-        batch_lbfgs_kernel<<<bt.count, kSolveThreads, 0, st>>>(a);
+        batch_lbfgs_kernel<<<bt.count * kSolveBlocks, kSolveThreads / kSolveBlocks, 0, st>>>(a);
         bt.launches += 2;
     }
     return cuda_rc(cudaGetLastError());
