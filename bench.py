@@ -68,8 +68,8 @@ def parse():
                     help="chosen form: the coarse solves of a Lloyd run continue one L-BFGS history (1) "
                          "or start afresh (0)")
     ap.add_argument("--incremental", type=int, default=1,
-                    help="incremental evaluations in weight solves: 1 on grids of at least 2^20 pixels "
-                         "(default), 2 on every grid, 0 every evaluation scores every pixel")
+                    help="incremental evaluations in weight solves: 2 records and re-decides on every grid; "
+                         "1 (default) and 0 score every pixel in every evaluation (full passes are faster)")
     ap.add_argument("--assign-res", type=int, default=0,
                     help="--mode assign: grid resolution per axis in place of the workload's")
     ap.add_argument("--assign-prune", action="store_true",
@@ -314,7 +314,8 @@ FLOPS_PER_PAIR = {3: 4.0 + 17.0 / 16.0, 2: 4.0 + 7.0 / 16.0}
 TC_FLOPS_PER_PAIR = 2 * 32
 COUNTERS_FILE = os.path.join(ROOT, "profiles", "ncu_counters.txt")
 SCORING_SOURCES = {"fp32": ("apd_assign_fp32.cu", "apd_fp32_tile.cuh"),
-                   "tc": ("apd_assign_tc.cu", "apd_tcgen05.cuh")}
+                   "tc": ("apd_assign_tc.cu", "apd_tcgen05.cuh"),
+                   "region": ("apd_assign_region.cu", "apd_region.cuh")}
 
 
 def kernel_source_hash(kind):
@@ -475,9 +476,11 @@ def roofline_block(form, dim, sms, workload):
     """Roofline of the scoring kernel (launch_ms: its mean device time per launch
     over the timed region, from the library's events around the kernel alone; the
     tensor-core form's candidate pre-pass runs before it and is not included).
+    Region form (pruning on, full passes): bound = the FP32 pipe; achieved = the
+    algorithmic flops (2F) of the evaluated pairs per second.
     FP32 form: bound = the FP32 pipe; achieved = executed FP32 flops of the
     evaluated pairs (the row-factored form, FLOPS_PER_PAIR each) per second.
-    Tensor-core form: bound = the tensor pipe; achieved = the contraction's flops
+    Tensor-core form (the dense sweep, recording passes): bound = the tensor pipe; achieved = the contraction's flops
     (2 x 32 per scored pair: split operands, K = 32) per second against the dense
     peak of the operand type.  Both report beside it the algorithmic rate (2F flops
     per evaluated pair), the dense-equivalent rate (all N x J pairs of Algorithm 1
@@ -504,7 +507,18 @@ def roofline_block(form, dim, sms, workload):
     def scaled(cnt, key):
         return int(round(cnt[key] * pairs_per_launch / cnt["pairs"])) if cnt else None
 
-    if form["precision"] == "fp32":
+    if form.get("region") and pruned:
+        peak = fp32_peak_tflops(sm_mhz, sms)
+        kern = "assign_region_kernel<%d>" % dim
+        cnt = ncu_counters(kern, workload, pruned, "region")
+        ach = sr * 2 * F / 1e12
+        out = {"bound": "alu", "kernel": kern, "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+               "frac": ach / peak, "traffic": scaled(cnt, "dram_bytes"),
+               "achieved_is": "algorithmic FP32 flops: 2F per evaluated pair (the candidate lists and "
+                              "the moments are not counted)",
+               "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 flops x {sm_mhz:.0f} MHz "
+                              f"(max SM clock from MEASURED_PEAKS.json, {peak_src})"}
+    elif form["precision"] == "fp32":
         peak = fp32_peak_tflops(sm_mhz, sms)
         kern = "assign_fp32_kernel<%d>" % dim
         cnt = ncu_counters(kern, workload, pruned, "fp32")
@@ -518,7 +532,7 @@ def roofline_block(form, dim, sms, workload):
     else:
         bf16 = float(peaks.get("bf16_tflops", 1900.0))
         peak = bf16 * (1.1 / 2.25) if form["precision"] == "tc_tf32" else bf16
-        # weight solves with incremental passes score with the recording variant
+        # weight solves with incremental passes on every grid score with the recording variant
         kern = "assign_tc_kernel<%d,%d%s>" % (dim, 0 if form["precision"] == "tc_tf32" else 1,
                                               ",1" if form.get("incremental") and pruned else "")
         cnt = ncu_counters(kern, workload, pruned, "tc")
@@ -572,7 +586,8 @@ def run_ours(args):
     forms["chosen"] = measure_form(args, ctx, args.precision, chosen_start=True)
     forms["chosen"]["precision"] = args.precision
     forms["chosen"]["pruned"] = bool(args.prune)
-    forms["chosen"]["incremental"] = bool(args.incremental)
+    forms["chosen"]["incremental"] = args.incremental > 1
+    forms["chosen"]["region"] = args.incremental < 2
     # the chosen form's final generators and its labels there (for the accuracy report)
     x_fin = (ctx["x_out"] if rounds > 0 else ctx["x0"]).clone()
     w_fin = ctx["w_out"].clone()
@@ -588,7 +603,8 @@ def run_ours(args):
     forms["chosen_alt"] = measure_form(args, ctx, alt, chosen_start=True)
     forms["chosen_alt"]["precision"] = alt
     forms["chosen_alt"]["pruned"] = bool(args.prune)
-    forms["chosen_alt"]["incremental"] = bool(args.incremental)
+    forms["chosen_alt"]["incremental"] = args.incremental > 1
+    forms["chosen_alt"]["region"] = args.incremental < 2
     forms["fp32"] = measure_form(args, ctx, "fp32")
     forms["fp32"]["precision"] = "fp32"
     if world > 1:

@@ -6,7 +6,7 @@
 // Two forms.  With region lists on the fine grid (apd_region.cuh: up to 16384 seeds,
 // r <= 16) mask_rows_kernel marks the boundary pixels and lists the fine regions they
 // reach, and the region scorer takes the marked pixels of those regions: 1000 seeds,
-// 128^3 refined by 2 (46 % of the fine voxels): 24.0 ms -> 0.47 ms for the whole call.
+// 128^3 refined by 2 (46 % of the fine voxels): 24.0 ms -> 0.30 ms for the whole call.
 // Otherwise:
 //
 // Mask.  One thread per coarse pixel compares its label with the 3^D
