@@ -1248,7 +1248,7 @@ int apd_points_moments(const apd_points *pts, const apd_seeds *seeds, double *mo
                        apd_workspace *ws, apd_stream_t stream) {
     APD_TRY(points_entry(pts, seeds, ws));
     if (!moments) return APD_ERR_ARG;
-    ws->w.kernel_launches += points_tiled(pts->count, seeds->n, ws->w) ? 6 : 3;
+    ws->w.kernel_launches += points_tiled(pts->count, seeds->n, ws->w) ? 6 : 2;
     return cuda_ok(launch_points_assign(pts->dim, pts->count, pts->y, pts->mass, seeds->n, seeds->x, seeds->A,
                                         seeds->w, moments, labels, ws->w, (cudaStream_t)stream));
 }
@@ -1262,7 +1262,7 @@ int apd_points_dual_value_grad(const apd_points *pts, const apd_seeds *seeds, co
     double *mom = reinterpret_cast<double *>(ws->w.moments);
     APD_TRY(cuda_ok(launch_points_assign(pts->dim, pts->count, pts->y, pts->mass, seeds->n, seeds->x, seeds->A,
                                          seeds->w, mom, nullptr, ws->w, st)));
-    ws->w.kernel_launches += points_tiled(pts->count, seeds->n, ws->w) ? 7 : 4;
+    ws->w.kernel_launches += points_tiled(pts->count, seeds->n, ws->w) ? 7 : 3;
     return cuda_ok(launch_points_dual(pts->dim, seeds->n, seeds->x, seeds->A, seeds->w, v, mom, ws->w, g_out, grad,
                                       max_rel_err, st));
 }

@@ -47,6 +47,7 @@ using namespace region;
 
 constexpr int kPtThreads = 256;
 constexpr int kMaxTiles = 1024;  // per axis
+constexpr int kPtManyPoints = 320;  // points per SM from which block sums pay
 constexpr size_t kPtShared = 200 * 1024;  // block sums of the moments
 
 // One tile: 2 max E of its list, the reference seed (natural index; -1: no list, the
@@ -604,10 +605,13 @@ cudaError_t launch_t(long long count, const double *y, const double *mass, int n
         points_lists_kernel<D><<<lb, kThreads, 0, st>>>(src, ws.pts_geo, heads, polys, pool);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        // block sums where n K doubles fit (one block of 1024 per SM) and a block gets
-        // several points per word it then adds to the global moments
+        // Block sums where n K doubles fit (one block of 1024 per SM) and a block gets
+        // several points per word it then adds to the global moments: those additions, by
+        // every block to the same n K words, cost 60 to 110 us whatever the count.
+        // MEASURED, us shared / global sums, 3D: n = 24, 20000 points 106 / 83, 80000 110 / 207;
+        // n = 80, 40000 81 / 82; n = 1000, 4 M (scoring alone) 275 / 610.
         const size_t smem = (size_t)n_mom * sizeof(double);
-        if (smem <= kPtShared && count >= 4ll * ws.sms * n) {
+        if (smem <= kPtShared && count >= (long long)std::max(kPtManyPoints, 4 * n) * ws.sms) {
             constexpr int T = 1024;
             constexpr unsigned bit = D == 3 ? kAttrPoints3 : kAttrPoints2;
             if (!(ws.attr_done & bit)) {
@@ -626,7 +630,11 @@ cudaError_t launch_t(long long count, const double *y, const double *mass, int n
         }
         return cudaGetLastError();
     }
+    // the seeds in their own order: no ranking (4 us of a 25 us call)
+    uint32_t *const codes = ws.codes;
+    ws.codes = nullptr;
     cudaError_t e = launch_seed_prep(none, n, x, A, w, ws, m64, n_mom, st);
+    ws.codes = codes;
     if (e != cudaSuccess) return e;
     const int blocks = (int)std::min<long long>(want_blocks, (long long)ws.sms * 8);
     points_assign_kernel<D><<<blocks, kPtThreads, 0, st>>>(count, y, mass, n, x, A, w, ws.recs32, ws.sc, mom, labels);
@@ -636,8 +644,13 @@ cudaError_t launch_t(long long count, const double *y, const double *mass, int n
 }  // namespace
 
 // The tiled form's six launches and lists against two passes over all seeds a point.
+// MEASURED, us direct / tiled: 2D n = 20, 20000 points 56 / 60, n = 30 66 / 64, n = 45 62 / 56,
+// n = 3000, 5000 points 438 / 57; 3D n = 8, 3000 points 50 / 54, n = 16, 5000 62 / 55 (direct
+// with the ranking it no longer makes); few seeds gain where the block sums do (n = 8,
+// 100000 points: 2D 338 / 167, 3D 492 / 173).
 bool points_tiled(long long count, int n, const Workspace &ws) {
-    return ws.groups && ws.pts_tiles && (n + kGroup - 1) / kGroup <= kMaxGroups && count >= 256 && n >= 8;
+    if (!ws.groups || !ws.pts_tiles || (n + kGroup - 1) / kGroup > kMaxGroups || count < 256) return false;
+    return n >= (ws.dim == 2 ? 40 : 12) || (n >= 8 && count >= (long long)kPtManyPoints * ws.sms);
 }
 
 cudaError_t launch_points_assign(int dim, long long count, const double *y, const double *mass, int n,

@@ -50,7 +50,8 @@ def _seeds(dim, n, seed, lo=0.0, hi=1.0, ws=0.3):
 
 
 @pytest.mark.parametrize("dim,n,count", [(2, 8, 255), (2, 8, 256), (3, 9, 257), (3, 40, 1000), (2, 700, 40001),
-                                         (3, 500, 30011), (3, 33, 3), (2, 3000, 5000)])
+                                         (3, 500, 30011), (3, 33, 3), (2, 3000, 5000), (2, 39, 300), (2, 40, 256),
+                                         (3, 11, 300), (3, 12, 256), (2, 8, 48639), (3, 8, 48640), (2, 13, 48641)])
 def test_counts(capi, dim, n, count):
     x, A, w = _seeds(dim, n, n)
     _check(capi, dim, np.random.default_rng(count).random((count, dim)), x, A, w)
