@@ -120,9 +120,10 @@ int apd_workspace_set_pruning(apd_workspace *ws, int32_t enable);
 
 /* Weight solves (Algorithm 2, and every solve inside the Lloyd, coarse-to-fine
  * and refining entry points) replay each evaluation after a solve's first from
- * a CUDA graph captured on first use: trial weights, scoring, rescoring,
- * moments, the dual of eqs. (2.7)-(2.8) and the read-back of its scalars, with
- * only the trial step changing between replays.  Results are the same with and
+ * a CUDA graph captured on first use: trial weights, scoring, moments, the dual
+ * of eqs. (2.7)-(2.8), which writes its scalars to pinned memory, and the
+ * L-BFGS pair of the trial, with only the trial step and the state of the
+ * history changing between replays.  Results are the same with and
  * without graphs; a sharded workspace never uses them.  enable = 0 switches
  * them off for this workspace (default on).  Returns APD_ERR_ARG for a null
  * workspace. */

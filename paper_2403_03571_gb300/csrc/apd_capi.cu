@@ -143,7 +143,7 @@ void destroy_graph(EvalGraph &e) {
 // the runtime tests' 3D alpha laws, the tensor-core form wins at ratios up to
 // 7.4 and loses 3.6x at 11.7).  The
 // conditioning comes from the seed preparation: read back once per preparation
-// (a stream synchronisation); passes that reuse the records reuse the value.
+// (the host waits for that copy alone); passes that reuse the records reuse the value.
 constexpr double kTcMaxCond = 10.0;
 bool use_tensor_cores(const GridDev &g, apd_precision prec, Workspace &ws, bool weights_only) {
     if (prec == APD_FP32 || tc_tile_count(g) > ws.tc_tile_cap) return false;
@@ -754,8 +754,9 @@ struct Solver {
 
     // L-BFGS iterations from the evaluated point ws.W (gradient ws.gf, f0 = f(ws.W)).
     // The direction, the trial point and its evaluation are queued back to back
-    // and read once; a pair pushed after an accepted step is taken or dropped by
-    // the device (its curvature test) and the host learns which at that read.
+    // and read once, the pair of the trial pushed behind it; the pair of an accepted step
+    // is taken or dropped by the device (its curvature test) and the host learns which at
+    // the next read.
     int iterate(double f0, double *out, bool &converged) {
         PushState ps{};
         ps.newest = kHistCap - 1;

@@ -126,8 +126,8 @@ constexpr unsigned kAttrTcScoreRec = 1u << 7;  // the recording variant: 4 bits
 constexpr unsigned kAttrPoints2 = 1u << 11, kAttrPoints3 = 1u << 12;
 constexpr unsigned kAttrFp32Small2 = 1u << 13, kAttrFp32Small3 = 1u << 14;
 
-// One evaluation of a weight solve (trial weights, scoring, rescoring, dual,
-// read-back of the device scalars) captured as a CUDA graph and replayed with
+// One evaluation of a weight solve (trial weights, scoring, dual, and a trial's
+// L-BFGS push) captured as a CUDA graph and replayed with
 // a new trial step t.  The key holds every argument the captured launches take.
 struct EvalGraph {
     std::vector<unsigned char> key;
