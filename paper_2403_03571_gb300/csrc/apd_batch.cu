@@ -353,9 +353,12 @@ __global__ void __launch_bounds__(region::kThreads, 4) batch_region_kernel(const
         const unsigned rest = local / (unsigned)I.tiles_x;
         const int by = (int)(rest % (unsigned)I.tiles_y), bz = (int)(rest / (unsigned)I.tiles_y);
         __syncthreads();
+        DevScalars *const sc = cur.sc;
         region::score_region<D>(sm, cur, bx, by, bz);
         __syncthreads();
-        if (threadIdx.x == 0 && sm.queued) atomicAdd(&cur.sc->flag_count, sm.queued);
+        // `cur` is not read below this barrier: the other warps are already writing the next
+        // item's into it (sm.queued is reset by this thread alone)
+        if (threadIdx.x == 0 && sm.queued) atomicAdd(&sc->flag_count, sm.queued);
     }
 }
 
