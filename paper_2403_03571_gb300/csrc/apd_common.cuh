@@ -5,6 +5,7 @@
 
 #include <float.h>
 
+#include "apd_eig.cuh"
 #include "apd_internal.cuh"
 
 namespace apd {
@@ -47,69 +48,6 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     }
     __syncthreads();
     return sh[32];
-}
-
-// Lower bound of the smallest eigenvalue of a symmetric positive-definite 2x2 or 3x3
-// matrix (FP64), close to it.  2x2: from the characteristic quadratic.  3x3: Newton's
-// method on the characteristic polynomial f from the left of the smallest root, where
-// f is negative, increasing and concave: every iterate stays left of the root, so any
-// number of steps gives a lower bound (steps taken 1e-6 short cover their FP32
-// quotient).  Starts: c0 / c1 (at least a third of the root) and mean - 2 spread.
-// The FP64 pipe issues a warp instruction every 64 clocks, so the trigonometric
-// solution (acos, cos) took 36 us per 1000 seeds against 5 us for this form.
-template <int D>
-__device__ __forceinline__ double lambda_min_sym(const double (&s)[D][D]) {
-    if (D == 2) {
-        const double m = 0.5 * (s[0][0] + s[1][1]);
-        const double h = 0.5 * (s[0][0] - s[1][1]);
-        const double r = sqrt(h * h + s[0][1] * s[0][1]);
-        // m - r computed as det / (m + r) to avoid cancellation
-        const double det = s[0][0] * s[1][1] - s[0][1] * s[0][1];
-        return (det / (m + r)) * (1.0 - 1e-9);
-    } else {
-        const double c2 = s[0][0] + s[1][1] + s[2][2];
-        const double m01 = s[0][0] * s[1][1] - s[0][1] * s[0][1], m02 = s[0][0] * s[2][2] - s[0][2] * s[0][2],
-                     m12 = s[1][1] * s[2][2] - s[1][2] * s[1][2];
-        const double c1 = m01 + m02 + m12;
-        const double c0 = s[0][0] * m12 - s[0][1] * (s[0][1] * s[2][2] - s[1][2] * s[0][2]) +
-                          s[0][2] * (s[0][1] * s[1][2] - s[1][1] * s[0][2]);
-        // mean - 2 sqrt(p2 / 6), p2 = ||S - mean I||^2 = ||S||^2 - c2^2 / 3 = 2 (c2^2 / 3 - c1)
-        const float q = (float)c2 / 3.f;
-        const float p2 = fmaxf((float)(c2 * c2 * (1.0 / 3.0) - c1), 0.f) * (2.f / 6.f);
-        const float iso = q - 2.f * sqrtf(p2) - 1e-5f * q;
-        const float start = fmaxf(((float)c0 / (float)c1) * (1.f - 1e-5f), iso);
-        double x = fmax((double)start, 0.0);
-        float df = 1.f;
-#pragma unroll 1
-        for (int it = 0; it < 6; ++it) {
-            const double f = ((x - c2) * x + c1) * x - c0;
-            df = (float)((3.0 * x - 2.0 * c2) * x + c1);
-            const float ff = (float)f;
-            if (!(df > 0.f) || !(ff < 0.f)) break;
-            x += (double)((-ff / df) * (1.f - 1e-6f));
-        }
-        // the rounding of f near the root: at most 1e-14 c2^3, divided by the slope
-        const float c = (float)c2;
-        const float slack = 1e-14f * c * c * c / fmaxf(df, 1e-30f);
-        return fmax(fmax(x * (1.0 - 1e-9) - (double)slack, (double)iso), 0.0);
-    }
-}
-
-// Upper bound of the largest eigenvalue: 2x2 m + r; 3x3 mean + 2 spread (the Frobenius
-// norm, which the caller also takes, is the other bound).
-template <int D>
-__device__ __forceinline__ double lambda_max_sym(const double (&s)[D][D]) {
-    if (D == 2) {
-        const double m = 0.5 * (s[0][0] + s[1][1]);
-        const double h = 0.5 * (s[0][0] - s[1][1]);
-        return (m + sqrt(h * h + s[0][1] * s[0][1])) * (1.0 + 1e-9);
-    } else {
-        const double p1 = s[0][1] * s[0][1] + s[0][2] * s[0][2] + s[1][2] * s[1][2];
-        const double q = (s[0][0] + s[1][1] + s[2][2]) * (1.0 / 3.0);
-        const double a0 = s[0][0] - q, a1 = s[1][1] - q, a2 = s[2][2] - q;
-        const float p2 = (float)(a0 * a0 + a1 * a1 + a2 * a2 + 2.0 * p1);
-        return q * (1.0 + 1e-9) + (double)(2.f * sqrtf(p2 * (1.f / 6.f)) * (1.f + 1e-6f));
-    }
 }
 
 __device__ __forceinline__ void split_f32(double v, float &hi, float &lo) {
@@ -181,8 +119,10 @@ __device__ __forceinline__ void build_seed(const int i, const int n, const doubl
 #pragma unroll
         for (int b = 0; b < D; ++b) f2 += s[a][b] * s[a][b];
     frob = sqrt(f2);
-    lam = spd ? lambda_min_sym<D>(s) : 0.0;
-    const double lmax = spd ? fmin(lambda_max_sym<D>(s), sqrt(f2) * (1.0 + 1e-12)) : 0.0;
+    double lmax = 0.0;
+    if (spd) eigen_bounds<D>(s, lam, lmax);
+    else lam = 0.0;
+    lmax = fmin(lmax, sqrt(f2) * (1.0 + 1e-12));
     if (!finite) bad = ST_NONFINITE;
     else if (!spd) bad = ST_NOT_SPD;
     if (!finite) {
