@@ -546,6 +546,7 @@ struct Solver {
         rescored += h.flag_count;
         if (h.status) {
             const int rc = map_bits(h.status);
+            cudaStreamSynchronize(st);
             cudaMemset(&ws.sc->status, 0, sizeof(int));
             return rc;
         }
@@ -833,10 +834,10 @@ struct Solver {
     }
 };
 
-int solve_impl(const GridDev &g, const apd_grid *grid, int n, const double *x, const double *A,
-               const double *w0, const double *v, double *w_out, const apd_solve_opts &o,
-               apd_solve_info &info, Workspace &ws, cudaStream_t st, bool need_moments_at_out,
-               bool judged = false, int *used = nullptr) {
+int solve_run(const GridDev &g, const apd_grid *grid, int n, const double *x, const double *A,
+              const double *w0, const double *v, double *w_out, const apd_solve_opts &o,
+              apd_solve_info &info, Workspace &ws, cudaStream_t st, bool need_moments_at_out,
+              bool judged, int *used) {
     Solver s(ws);
     s.g = g;
     s.n = n;
@@ -876,6 +877,22 @@ int solve_impl(const GridDev &g, const apd_grid *grid, int n, const double *x, c
     const double vmin = ws.sc_host->min_v;
     if (g.cell > o.eps * vmin / std::pow(2.0, g.dim)) return APD_WARN_TOL_INFEASIBLE;
     return APD_OK;
+}
+
+// A solve that ends in an error leaves nothing queued either: the host has read the last
+// evaluation's scalars while kernels behind them (the gradient's stores, the trial's push)
+// still used the workspace, and an evaluation cut short may have its number on the device
+// only.
+int solve_impl(const GridDev &g, const apd_grid *grid, int n, const double *x, const double *A,
+               const double *w0, const double *v, double *w_out, const apd_solve_opts &o,
+               apd_solve_info &info, Workspace &ws, cudaStream_t st, bool need_moments_at_out,
+               bool judged = false, int *used = nullptr) {
+    const int rc = solve_run(g, grid, n, x, A, w0, v, w_out, o, info, ws, st, need_moments_at_out, judged, used);
+    if (rc < 0) {
+        cudaStreamSynchronize(st);
+        ws.sc_seq = ws.sc_host->seq;
+    }
+    return rc;
 }
 
 }  // namespace
