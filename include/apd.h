@@ -113,9 +113,11 @@ void apd_workspace_destroy(apd_workspace *ws);
  * offset; a = the seed of least cost at the tile's centre) is positive.  That
  * leaves a few seeds per tile, too few for a tensor-core contraction.  Pixels whose
  * two smallest values are within the rounding bound are settled in FP64.  Labels
- * and moments are the same as without pruning.  Above 16384 seeds the FP32 kernel
- * skips whole 32-seed groups instead.  Applies to every later scoring call on the
- * workspace. */
+ * and moments are the same as without pruning.  Above 16384 seeds, and above 4096
+ * on fewer than 2.5 pixels a seed, the FP32 kernel skips whole 32-seed groups
+ * instead, and the tensor-core kernel (if asked for, and the seeds' conditioning
+ * allows) scores per-tile candidate lists.  Applies to every later scoring call on
+ * the workspace. */
 int apd_workspace_set_pruning(apd_workspace *ws, int32_t enable);
 
 /* Weight solves (Algorithm 2, and every solve inside the Lloyd, coarse-to-fine

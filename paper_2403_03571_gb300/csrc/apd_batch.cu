@@ -333,6 +333,7 @@ template <int D>
 __global__ void __launch_bounds__(region::kThreads, 4) batch_region_kernel(const __grid_constant__ BArgs a) {
     __shared__ region::Shared<D> sm;
     __shared__ region::Src cur;
+    extern __shared__ uint16_t tiles[];
     region::init_shared<D>(sm);
     const unsigned total = a.sched->total_items;
     const int n_act = a.sched->n_active;
@@ -354,7 +355,7 @@ __global__ void __launch_bounds__(region::kThreads, 4) batch_region_kernel(const
         const int by = (int)(rest % (unsigned)I.tiles_y), bz = (int)(rest / (unsigned)I.tiles_y);
         __syncthreads();
         DevScalars *const sc = cur.sc;
-        region::score_region<D>(sm, cur, bx, by, bz);
+        region::score_region<D>(sm, tiles, cur, bx, by, bz);
         __syncthreads();
         // `cur` is not read below this barrier: the other warps are already writing the next
         // item's into it (sm.queued is reset by this thread alone)
@@ -1041,6 +1042,7 @@ struct apd_batch {
     region::Src *d_srcs = nullptr;
     int sms = 152;
     bool can_region = false;           // every instance suits the region form
+    int tile_cap = 0;                  // its longest tile list
     void *blocks[40] = {};
     int nblocks = 0;
     cudaStream_t cap = nullptr;
@@ -1103,7 +1105,14 @@ int use_variant(apd_batch &bt, int vi, cudaStream_t st) {
     if (vi == kRegionVariant) {
         long long regions = 0;
         for (const BInst &I : t) regions += I.ntiles;
-        bt.grid_blocks = (int)std::min<long long>(regions, 4ll * bt.sms);
+        bt.grid_blocks = (int)std::min<long long>(regions, (long long)region::blocks_per_sm(bt.tile_cap) * bt.sms);
+        const int dense = (int)region::tile_bytes(region::kTileCapMax);
+        if (bt.tile_cap > region::kTileCap) {
+            if (bt.dim == 3)
+                BTRY(cuda_rc(cudaFuncSetAttribute(batch_region_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, dense)));
+            else
+                BTRY(cuda_rc(cudaFuncSetAttribute(batch_region_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dense)));
+        }
         return APD_OK;
     }
     const Variant &V = variants(bt.dim)[vi];
@@ -1131,8 +1140,9 @@ int enqueue_iteration(apd_batch &bt, int vi, bool solve_steps, cudaStream_t st) 
     batch_schedule_kernel<<<1, 1024, bt.smem_sched, st>>>(a);
     bt.launches += 2;
     if (vi == kRegionVariant) {
-        if (bt.dim == 3) batch_region_kernel<3><<<bt.grid_blocks, region::kThreads, 0, st>>>(a);
-        else batch_region_kernel<2><<<bt.grid_blocks, region::kThreads, 0, st>>>(a);
+        const size_t tiles = region::tile_bytes(bt.tile_cap);
+        if (bt.dim == 3) batch_region_kernel<3><<<bt.grid_blocks, region::kThreads, tiles, st>>>(a);
+        else batch_region_kernel<2><<<bt.grid_blocks, region::kThreads, tiles, st>>>(a);
     } else {
         BTRY(cuda_rc(variants(bt.dim)[vi].launch(a, bt.grid_blocks, bt.smem_assign, st)));
         if (bt.dim == 3) batch_rescore_kernel<3><<<bt.rescore_blocks, 256, bt.smem_sched + 4, st>>>(a);
@@ -1331,7 +1341,25 @@ int apd_batch_create(apd_batch **out, int32_t dim, int32_t count, const apd_grid
     alloc((void **)&a.err, N * sizeof(double));
     alloc((void **)&bt->d_srcs, count * sizeof(region::Src));
     a.srcs = bt->d_srcs;
+    int sms = 0;
+    if (ok && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device) != cudaSuccess) ok = false;
+    bt->rescore_blocks = std::max(1, sms) * kRescoreBlocksPerSM;
+    bt->sms = std::max(1, sms);
     bt->can_region = true;
+    {   // the tiles' lists: one length for the batch, by all regions, the most seeds and the smallest cells
+        int rd[3], most = 1;
+        region_dims(dim, rd);
+        long long regions = 0, cell = 1ll << 40;
+        for (int b = 0; b < count; ++b) {
+            const GridDev &g = bt->grids[b];
+            long long r = 1;
+            for (int k = 0; k < dim; ++k) r *= (g.res[k] + rd[k] - 1) / rd[k];
+            regions += r;
+            most = std::max(most, bt->n[b]);
+            cell = std::min(cell, g.J / bt->n[b]);
+        }
+        bt->tile_cap = region::tile_cap(regions, cell * most, most, bt->sms);
+    }
     if (ok) {
         std::vector<int32_t> inst_of(N);
         std::vector<region::Src> srcs(count);
@@ -1345,6 +1373,7 @@ int apd_batch_create(apd_batch **out, int32_t dim, int32_t count, const apd_grid
             src.gf = make_gridf(g);
             src.n = nb;
             src.n_groups = (nb + kGroup - 1) / kGroup;
+            src.tile_cap = bt->tile_cap;
             src.recs = a.recs32s + bt->rec_off[b];
             src.perm = (nb + kChunk - 1) / kChunk * kChunk <= kBSortMax ? a.perm + bt->rec_off[b] : nullptr;
             src.groups = a.groups + bt->rec_off[b] / 32;
@@ -1382,10 +1411,6 @@ int apd_batch_create(apd_batch **out, int32_t dim, int32_t count, const apd_grid
     if (ok && cudaFuncSetAttribute(dim == 3 ? (const void *)batch_rescore_kernel<3> : (const void *)batch_rescore_kernel<2>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bt->smem_sched + 4) != cudaSuccess)
         ok = false;
-    int sms = 0;
-    if (ok && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device) != cudaSuccess) ok = false;
-    bt->rescore_blocks = std::max(1, sms) * kRescoreBlocksPerSM;
-    bt->sms = std::max(1, sms);
     if (ok && tile >= 0) {
         bt->variant = tile;
         if (use_variant(*bt, tile, nullptr) != APD_OK) ok = false;

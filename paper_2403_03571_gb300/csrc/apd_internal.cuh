@@ -125,6 +125,7 @@ constexpr unsigned kAttrTcScore = 1u << 3;     // + 1 bit per (dimension, operan
 constexpr unsigned kAttrTcScoreRec = 1u << 7;  // the recording variant: 4 bits
 constexpr unsigned kAttrPoints2 = 1u << 11, kAttrPoints3 = 1u << 12;
 constexpr unsigned kAttrFp32Small2 = 1u << 13, kAttrFp32Small3 = 1u << 14;
+constexpr unsigned kAttrRegion2 = 1u << 15, kAttrRegion3 = 1u << 16, kAttrMasked2 = 1u << 17, kAttrMasked3 = 1u << 18;
 
 // One evaluation of a weight solve (trial weights, scoring, dual, and a trial's
 // L-BFGS push) captured as a CUDA graph and replayed with

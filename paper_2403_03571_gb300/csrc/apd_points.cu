@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 4)
             const int n_src = scan ? s.n_groups : (int)((total + 31u) / 32u);
             auto source = [&](int c) -> int {
                 const int e = c * 32 + lane;
-                if (scan) return e < s.n ? e : -1;
+                if (scan) return (sm.mask[c] >> lane) & 1u ? e : -1;
                 return e < (int)total ? (int)sm.list[e] : -1;
             };
             unsigned best = 0xffffffffu;

@@ -16,9 +16,11 @@
 //   * Region (16^3 voxels / 64^2 pixels, one block): the 32-seed groups' cost lower
 //     bounds, one group per lane; the seed a of least cost at the centre among the
 //     warps' nearest groups; the seeds of the groups that can beat a's largest cost
-//     are tested against a and listed in shared memory.
+//     are tested against a and listed in shared memory (past 1024: as a bit per seed).
 //   * Tile (8^3 / 32 x 16, one warp): the same test over the tile against the listed
-//     seed of least cost at the tile's centre.
+//     seed of least cost at the tile's centre.  Up to 48 polynomials stay in shared
+//     memory; of a longer list the positions stay, and its polynomials are formed again
+//     32 at a time (see tile_cap).
 // Measured (1000 seeds, 256^3, solve-sized weights): 108 us, 62.8 M warp
 // instructions (region lists 33 %, tile lists 23 %, pixels 27 %, moments 17 %) at half
 // of the issue slots; the tensor-core scorer with separate bounds took 456 us after a
@@ -60,13 +62,30 @@ namespace region {
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
-constexpr int kListCap = 1024;  // listed seeds of a region; beyond it the tiles scan the groups
+constexpr int kListCap = 1024;  // listed seeds of a region; beyond it the tiles take the groups that hold any
 constexpr int kBuf = 48;        // polynomials a warp keeps at a time
 constexpr int kFast = 8;        // polynomials of a tile whose labels fit the byte masks
 constexpr int kTilePix = 512;
 constexpr float kCoef = 64.f * 5.9604644775390625e-8f;
 constexpr float kEta = 5.9604644775390625e-8f;
 constexpr int kMaxGroups = kSortMax / kGroup;  // 512: two groups per lane and warp
+
+// Seeds of a tile's list kept by their scan position, in dynamic shared memory (16 bytes a
+// seed for a block): what does not fit the polynomials' buffer is formed again from there,
+// a list beyond it from the region's.  512 leave the caches their room; where the regions
+// are fewer than the SMs hold, or cells are so small that lists are long, a block gets more.
+// MEASURED, us per call, lists formed again from the region's only / from the tile's: 3D
+// n = 10000 on 96^3 1326 / 324, n = 3000 on 60^3 441 / 217; 2D n = 5000 on 300^2 601 / 240.
+constexpr int kTileCap = 512, kTileCapMax = 12032;
+inline int tile_cap(long long regions, long long pixels, int n, int sms) {
+    const int cap = regions <= sms ? kTileCapMax
+                    : regions <= 2ll * sms ? 4864
+                    : regions <= 3ll * sms || pixels < 128ll * n ? 2560 : kTileCap;
+    const int all = (n + 31) / 32 * 32;
+    return all < cap ? all : cap;
+}
+inline size_t tile_bytes(int cap) { return (size_t)kWarps * cap * sizeof(uint16_t); }
+inline int blocks_per_sm(int cap) { return cap <= 1472 ? 4 : cap <= 2560 ? 3 : cap <= 4864 ? 2 : 1; }
 
 template <int D>
 struct Geom;
@@ -88,6 +107,7 @@ struct Src {
     GridDev g;
     GridF gf;
     int n, n_groups;
+    int tile_cap;              // seeds a tile keeps by position
     const SeedRec32 *recs;     // scan order
     const int32_t *perm;       // scan position -> seed index (null: identity)
     const GroupBound *groups;  // bounds of the scan-order groups
@@ -114,6 +134,7 @@ struct Shared {
     float4 poly[kWarps][kBuf][3];
     float4 ref[kWarps][5];             // the warp's best seed (region), then its tile's reference
     uint16_t list[kListCap];           // scan positions
+    unsigned mask[kMaxGroups];         // a group's listed seeds
     uint16_t queue[kWarps][kTilePix];  // the tile's near ties: pixel of the tile
     unsigned lut[256];  // row mask -> count | sum x << 8 | sum x^2 << 16
     unsigned key[kWarps];
@@ -459,7 +480,10 @@ __device__ __forceinline__ unsigned region_list(Shared<D> &sm, const Src &s, con
         for (int t = 0; t < 2; ++t) {
             if (s.n_groups <= t * kThreads) break;
             const int grp = wid + kWarps * (lane + 32 * t);
-            if (grp < s.n_groups) glb[t] = group_lower<D>(s.groups[grp], alo, ahi);
+            if (grp < s.n_groups) {
+                glb[t] = group_lower<D>(s.groups[grp], alo, ahi);
+                sm.mask[grp] = 0u;
+            }
         }
     }
     // each warp's group of least bound, and in it the seed of least cost at the centre
@@ -534,7 +558,10 @@ __device__ __forceinline__ unsigned region_list(Shared<D> &sm, const Src &s, con
             const unsigned km = __ballot_sync(full, keep);
             if (km) {
                 unsigned at = 0u;
-                if (lane == 0) at = atomicAdd(&sm.count, (unsigned)__popc(km));
+                if (lane == 0) {
+                    sm.mask[wid + kWarps * (gl + 32 * t)] = km;
+                    at = atomicAdd(&sm.count, (unsigned)__popc(km));
+                }
                 at = __shfl_sync(full, at, 0) + (unsigned)__popc(km & ((1u << lane) - 1u));
                 if (keep && at < (unsigned)kListCap) sm.list[at] = (uint16_t)p;
             }
@@ -544,13 +571,101 @@ __device__ __forceinline__ unsigned region_list(Shared<D> &sm, const Src &s, con
     return sm.count;
 }
 
-// Scores region (bx, by, bz); `s` is the same in every thread.  The caller puts a
-// barrier between the previous region and the next.
+// The seeds that region_list has listed, in chunks of a warp.
+template <int D>
+struct Listed {
+    unsigned total;
+    bool scan;  // too many for the list: chunk c is what is listed of group c
+    int chunks;
+    __device__ __forceinline__ Listed(const Src &s, unsigned total_)
+        : total(total_), scan(total_ > (unsigned)kListCap), chunks(scan ? s.n_groups : (int)((total_ + 31u) / 32u)) {}
+    __device__ __forceinline__ bool none(const Shared<D> &sm, int c) const { return scan && sm.mask[c] == 0u; }
+    // scan position of this lane's candidate of chunk c (-1: none)
+    __device__ __forceinline__ int at(const Shared<D> &sm, int c) const {
+        const int lane = threadIdx.x & 31, e = c * 32 + lane;
+        if (scan) return (sm.mask[c] >> lane) & 1u ? e : -1;
+        return e < (int)total ? (int)sm.list[e] : -1;
+    }
+};
+
+// The warp's tile's offset from the region's centre and half-widths (rounded up).
+template <int D>
+__device__ __forceinline__ void tile_box(const GridDev &g, const int (&tc)[3], float (&toff)[3], float (&tr)[3]) {
+    using G = Geom<D>;
+    const int tdim[3] = {G::TX, G::TY, G::TZ}, rdim[3] = {G::RX, G::RY, G::RZ};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        toff[a] = a < D ? (float)(tc[a] * tdim[a] + tdim[a] / 2 - rdim[a] / 2) * g.h32[a] : 0.f;
+        tr[a] = a < D ? __fmul_ru(__fmul_ru(0.5f * (float)(tdim[a] - 1), g.h32[a]), 1.f + 0x1p-22f) : 0.f;
+    }
+}
+template <int D>
+__device__ __forceinline__ void warp_tile(int wid, int (&tc)[3]) {
+    using G = Geom<D>;
+    tc[0] = wid % (G::RX / G::TX);
+    tc[1] = (wid / (G::RX / G::TX)) % (G::RY / G::TY);
+    tc[2] = wid / ((G::RX / G::TX) * (G::RY / G::TY));
+}
+
+// The polynomial of seed p as entry `at` of the warp's buffer.
+template <int D>
+__device__ __forceinline__ void put_poly(float4 (*buf)[3], int at, const Src &s, int p, const Diff<D> &F) {
+    constexpr int NP = Geom<D>::NP;
+    const int id = s.perm ? s.perm[p] : p;
+    buf[at][0] = make_float4(F.d0, F.g[0], F.g[1], D == 3 ? F.g[D - 1] : 0.f);
+    if (D == 3) {
+        buf[at][1] = make_float4(F.a[0], 2.f * F.a[1], 2.f * F.a[2], F.a[NP - 3]);
+        buf[at][2] = make_float4(2.f * F.a[NP - 2], F.a[NP - 1], __int_as_float(id), 0.f);
+    } else {
+        buf[at][1] = make_float4(F.a[0], 2.f * F.a[1], F.a[2], __int_as_float(id));
+    }
+}
+
+// A tile whose polynomials do not fit the warp's buffer: piece c of them formed again,
+// from the tile's list where it is complete (`listed` seeds), else from the region's.
+// Returns their number.  Out of line: few tiles come here, and inlined in four places it
+// cost the others registers (256^3, 1000 seeds: 108 us -> 115 us).
+template <int D>
+__device__ __noinline__ int refill(Shared<D> &sm, const Src &s, const uint16_t *tile, const int bx, const int by,
+                                   const int bz, const int c, const int listed, const int best_pos) {
+    using G = Geom<D>;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int k[3] = {bx * G::RX + G::RX / 2, by * G::RY + G::RY / 2, bz * G::RZ + G::RZ / 2};
+    float ch[3] = {0.f, 0.f, 0.f}, cl[3] = {0.f, 0.f, 0.f}, toff[3], tr[3];
+#pragma unroll
+    for (int a = 0; a < D; ++a) axis_point(s.gf, a, k[a], ch[a], cl[a]);
+    int tc[3];
+    warp_tile<D>(wid, tc);
+    tile_box<D>(s.g, tc, toff, tr);
+    Local<D> R, L;
+    int id;
+    load_local<D>(sm.ref[wid], R, id);
+    const bool kept = listed <= s.tile_cap;
+    int p;
+    if (kept) p = 32 * c + lane < listed ? (int)tile[32 * c + lane] : -1;
+    else p = Listed<D>(s, sm.count).at(sm, c);
+    __syncwarp();
+    bool keep = false;
+    Diff<D> F;
+    if (p >= 0 && p != best_pos) {
+        local_terms<D>(s.recs[p], ch, cl, toff, tr, s.gf, L);
+        difference<D>(L, R, F);
+        keep = kept || can_win<D>(F, tr);
+    }
+    const unsigned km = __ballot_sync(0xffffffffu, keep);
+    if (keep) put_poly<D>(sm.poly[wid], __popc(km & ((1u << lane) - 1u)), s, p, F);
+    __syncwarp();
+    return __popc(km);
+}
+
+// Scores region (bx, by, bz); `s` is the same in every thread; `tiles`: kWarps lists of
+// tile_cap positions in shared memory.  The caller puts a barrier between the previous
+// region and the next.
 template <int D, bool MASKED = false>
-__device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const int bx, const int by, const int bz) {
+__device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, const Src &s, const int bx, const int by,
+                                             const int bz) {
     using G = Geom<D>;
     constexpr int K = moment_width(D);
-    constexpr int NP = G::NP;
     const GridDev &g = s.g;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const unsigned full = 0xffffffffu;
@@ -562,10 +677,10 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
     float4(&ref)[5] = sm.ref[wid];
 
     // the warp's tile
-    const int tc[3] = {wid % (G::RX / G::TX), (wid / (G::RX / G::TX)) % (G::RY / G::TY),
-                       wid / ((G::RX / G::TX) * (G::RY / G::TY))};
-    int kb[3], lo3[3], cnt[3];
-    float toff[3] = {0.f, 0.f, 0.f}, tr[3] = {0.f, 0.f, 0.f};
+    int tc[3], kb[3], lo3[3], cnt[3];
+    float toff[3], tr[3];
+    warp_tile<D>(wid, tc);
+    tile_box<D>(g, tc, toff, tr);
     bool empty = false, whole = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -574,8 +689,6 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
         if (a < D) {
             hi = min(hi, a == D - 1 ? win_hi(g) : g.res[a]);
             if (a == D - 1) lo = max(lo, win_lo(g));
-            toff[a] = (float)(tc[a] * tdim[a] + tdim[a] / 2 - rdim[a] / 2) * g.h32[a];
-            tr[a] = __fmul_ru(__fmul_ru(0.5f * (float)(tdim[a] - 1), g.h32[a]), 1.f + 0x1p-22f);
         }
         lo3[a] = lo;
         cnt[a] = hi - lo;
@@ -642,13 +755,8 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
     }
     float r0h, r0l;
     const unsigned total = region_list<D>(sm, s, ch, cl, rr, r0h, r0l);
-    const bool scan = total > (unsigned)kListCap;  // too many: the tiles take every group
-    const int n_src = scan ? s.n_groups : (int)((total + 31u) / 32u);
-    auto source = [&](int c) -> int {  // scan position of candidate `lane` of chunk c (-1: none)
-        const int e = c * 32 + lane;
-        if (scan) return e < n ? e : -1;
-        return e < (int)total ? (int)sm.list[e] : -1;
-    };
+    const Listed<D> src(s, total);
+    const int n_src = src.chunks;
 
     if (empty) return;
     const WordMap wm = word_map<D>();
@@ -659,7 +767,8 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
     Local<D> L;  // of the last chunk (the only one of most lists)
     int pos = -1;
     for (int c = 0; c < n_src; ++c) {
-        pos = source(c);
+        if (src.none(sm, c)) continue;
+        pos = src.at(sm, c);
         unsigned ck = 0xffffffffu;
         if (pos >= 0) {
             local_terms<D>(s.recs[pos], ch, cl, toff, tr, s.gf, L);
@@ -687,8 +796,11 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
     int m = 0;          // in the buffer
     int listed = 0;     // in all chunks
     float4(*buf)[3] = sm.poly[wid];
-    auto build = [&](int c) {
-        const int p = n_src == 1 ? pos : source(c);
+    uint16_t *const tile = tiles + wid * s.tile_cap;
+    bool one = true;  // every polynomial is in the buffer
+    for (int c = 0; c < n_src; ++c) {
+        if (src.none(sm, c)) continue;
+        const int p = n_src == 1 ? pos : src.at(sm, c);
         bool keep = false;
         Diff<D> F;
         if (p >= 0 && p != best_pos) {
@@ -697,43 +809,25 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, const Src &s, const 
             keep = can_win<D>(F, tr);
         }
         const unsigned km = __ballot_sync(full, keep);
-        const int at = m + __popc(km & ((1u << lane) - 1u));
+        const int before = __popc(km & ((1u << lane) - 1u));
         const int add = __popc(km);
-        const bool fits = m + add <= kBuf;
+        one = one && m + add <= kBuf;
         if (keep) {
             Emax = fmaxf(Emax, F.E);
-            if (fits) {
-                const int id = s.perm ? s.perm[p] : p;
-                buf[at][0] = make_float4(F.d0, F.g[0], F.g[1], D == 3 ? F.g[D - 1] : 0.f);
-                if (D == 3) {
-                    buf[at][1] = make_float4(F.a[0], 2.f * F.a[1], 2.f * F.a[2], F.a[NP - 3]);
-                    buf[at][2] = make_float4(2.f * F.a[NP - 2], F.a[NP - 1], __int_as_float(id), 0.f);
-                } else {
-                    buf[at][1] = make_float4(F.a[0], 2.f * F.a[1], F.a[2], __int_as_float(id));
-                }
-            }
+            if (one) put_poly<D>(buf, m + before, s, p, F);
+            if (n_src > 1 && listed + before < s.tile_cap) tile[listed + before] = (uint16_t)p;
         }
-        if (fits) m += add;
-        return fits ? add : -add - 1;
-    };
-    bool one = true;  // every polynomial is in the buffer
-    for (int c = 0; c < n_src; ++c) {
-        const int add = build(c);
-        listed += add >= 0 ? add : -add - 1;
-        one = one && add >= 0;
+        if (one) m += add;
+        listed += add;
     }
     Emax = __uint_as_float(__reduce_max_sync(full, __float_as_uint(Emax)));
     __syncwarp();
     if (lane == 0) atomicAdd(&sm.pairs, (unsigned)(listed + 1));
     // every polynomial of the tile in turn, f(k) on buffer entry k; called by the whole warp
     auto each = [&](auto f) {
-        for (int c = 0; c < (one ? 1 : n_src); ++c) {
-            if (!one) {
-                __syncwarp();
-                m = 0;
-                build(c);
-                __syncwarp();
-            }
+        const int pieces = one ? 1 : listed <= s.tile_cap ? (listed + 31) / 32 : n_src;
+        for (int c = 0; c < pieces; ++c) {
+            if (!one) m = refill<D>(sm, s, tile, bx, by, bz, c, listed, best_pos);
             for (int k = 0; k < m; ++k) f(k);
         }
     };
