@@ -979,8 +979,8 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
         // point sets: about 32 tiles a seed, room for eight polynomials a tile
         w.pts_bytes = (size_t)std::min<long long>(32ll * std::max(max_n, 64), 1ll << 17) * (16 + 8 * 48);
         alloc((void **)&w.pts_tiles, w.pts_bytes);
-        alloc((void **)&w.pts_geo, sizeof(PtsGeo));
-        if (ok && cudaMemset(w.pts_geo, 0, sizeof(PtsGeo)) != cudaSuccess) ok = false;
+        alloc((void **)&w.pts_geo, 2 * sizeof(PtsGeo));
+        if (ok && cudaMemset(w.pts_geo, 0, 2 * sizeof(PtsGeo)) != cudaSuccess) ok = false;
     }
     alloc((void **)&w.grad, (size_t)max_n * sizeof(double));
     alloc((void **)&w.W, (size_t)max_n * sizeof(double));

@@ -8,8 +8,9 @@
 // (apd_region.cuh: the difference of two costs over the tile's box), stored as
 // polynomials; a thread per point finds its tile, evaluates the few polynomials there
 // and settles near ties in FP64 itself.  The points need no order.
-//   points_box_kernel    the box and the tiling, on the device (high words of the
-//                        coordinates: 20 bits are enough for a box)
+//   points_box_kernel    the boxes and the tilings, on the device (high words of the
+//                        coordinates: 20 bits are enough for a box): one tiling, or a fine
+//                        one around the seeds and a coarse one of the whole box
 //   points_lists_kernel  a block per 2 x 2 (x 2) tiles, eight warps listing, a warp
 //                        per tile storing
 //   points_score_kernel  labels and moments
@@ -98,78 +99,10 @@ __device__ __forceinline__ void split_trunc(double v, float &hi, float &lo) {
     lo = __uint_as_float(__float_as_uint(r * scale) | sign);
 }
 
-// The points' box from the high words of their coordinates, then (last block) the
-// tiling: about `want` tiles of near-cubic shape.
+// About `want` tiles of near-cubic shape over the box lo .. lo + ext.
 template <int D>
-__global__ void __launch_bounds__(kPtThreads)
-    points_box_kernel(const long long count, const double *__restrict__ y, const long long want,
-                      unsigned *__restrict__ part, PtsGeo *__restrict__ geo) {
-    __shared__ unsigned smn[D], smx[D];
-    __shared__ bool last;
-    if (threadIdx.x < D) {
-        smn[threadIdx.x] = 0xffffffffu;
-        smx[threadIdx.x] = 0u;
-    }
-    __syncthreads();
-    unsigned mn[D], mx[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        mn[a] = 0xffffffffu;
-        mx[a] = 0u;
-    }
-    const uint2 *y2 = reinterpret_cast<const uint2 *>(y);
-#pragma unroll 4
-    for (long long j = (long long)blockIdx.x * kPtThreads + threadIdx.x; j < count; j += (long long)gridDim.x * kPtThreads)
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            const unsigned h = y2[j * D + a].y;
-            if ((h & 0x7ff00000u) == 0x7ff00000u) continue;  // not finite
-            const unsigned k = h ^ ((h >> 31) ? 0xffffffffu : 0x80000000u);
-            mn[a] = min(mn[a], k);
-            mx[a] = max(mx[a], k);
-        }
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        mn[a] = __reduce_min_sync(0xffffffffu, mn[a]);
-        mx[a] = __reduce_max_sync(0xffffffffu, mx[a]);
-        if ((threadIdx.x & 31) == 0) {
-            atomicMin(&smn[a], mn[a]);
-            atomicMax(&smx[a], mx[a]);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            part[(size_t)blockIdx.x * 6 + a] = smn[a];
-            part[(size_t)blockIdx.x * 6 + 3 + a] = smx[a];
-        }
-        __threadfence();
-        last = atomicAdd(&geo->done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
-    __threadfence();
-    float lo[3] = {0.f, 0.f, 0.f}, ext[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        unsigned m = 0xffffffffu, x = 0u;
-        for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) {
-            m = min(m, *(volatile unsigned *)&part[(size_t)b * 6 + a]);
-            x = max(x, *(volatile unsigned *)&part[(size_t)b * 6 + 3 + a]);
-        }
-        m = __reduce_min_sync(0xffffffffu, m);
-        x = __reduce_max_sync(0xffffffffu, x);
-        // outward: the dropped low words all zeros or all ones
-        const unsigned hm = (m >> 31) ? m ^ 0x80000000u : ~m, hx = (x >> 31) ? x ^ 0x80000000u : ~x;
-        const double dl = __longlong_as_double((long long)(((unsigned long long)hm << 32) | ((hm >> 31) ? 0xffffffffull : 0ull)));
-        const double dh = __longlong_as_double((long long)(((unsigned long long)hx << 32) | ((hx >> 31) ? 0ull : 0xffffffffull)));
-        const bool some = m <= x;
-        lo[a] = some ? __double2float_rd(dl) : 0.f;
-        ext[a] = some ? __fsub_ru(__double2float_ru(dh), lo[a]) : 1.f;
-    }
-    if (threadIdx.x != 0) return;
-    float big = 1e-30f;
+__device__ void make_tiling(const float (&lo)[3], const float (&box)[3], const long long want, PtsGeo *geo) {
+    float ext[3] = {box[0], box[1], box[2]}, big = 1e-30f;
 #pragma unroll
     for (int a = 0; a < D; ++a) big = fmaxf(big, ext[a]);
     float vol = 1.f;
@@ -210,6 +143,115 @@ __global__ void __launch_bounds__(kPtThreads)
         geo->r[a] = h * (1.f + 0x1p-9f);
         geo->ext[a] = ext[a];
     }
+}
+
+// The points' and the seeds' boxes from the high words of their coordinates, then (last
+// block) the tilings.  geo[0] tiles the points' box with all `want` tiles, unless that box
+// is more than four times the seeds' neighbourhood on an axis (an outlier among the points,
+// or seeds in one place): uniform tiles would then be as large as many cells, their lists
+// all seeds and their gaps beyond any difference.  geo[0] then tiles that neighbourhood (half
+// the seeds' extent more on every side) with three quarters of the tiles and geo[1] the
+// whole box with the rest.  MEASURED, us per call, one tiling / two (direct form): 1000
+// seeds, 10^6 points in 3D, one of them at 1000 box lengths 60756 / 332 (3691), at 10
+// 2199 / 333 (3689); 5000 seeds, 3000 points 14538 / 596 (969).
+template <int D>
+__global__ void __launch_bounds__(kPtThreads)
+    points_box_kernel(const long long count, const double *__restrict__ y, const int n, const double *__restrict__ x,
+                      const int point_blocks, const long long want, unsigned *__restrict__ part,
+                      PtsGeo *__restrict__ geo) {
+    __shared__ unsigned smn[D], smx[D];
+    __shared__ bool last;
+    if (threadIdx.x < D) {
+        smn[threadIdx.x] = 0xffffffffu;
+        smx[threadIdx.x] = 0u;
+    }
+    __syncthreads();
+    unsigned mn[D], mx[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        mn[a] = 0xffffffffu;
+        mx[a] = 0u;
+    }
+    // the blocks behind the points' take the seeds
+    const bool seeds = (int)blockIdx.x >= point_blocks;
+    const uint2 *v2 = reinterpret_cast<const uint2 *>(seeds ? x : y);
+    const long long m = seeds ? n : count;
+    const int blk = (int)blockIdx.x - (seeds ? point_blocks : 0), nblk = seeds ? (int)gridDim.x - point_blocks : point_blocks;
+#pragma unroll 4
+    for (long long j = (long long)blk * kPtThreads + threadIdx.x; j < m; j += (long long)nblk * kPtThreads)
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const unsigned h = v2[j * D + a].y;
+            if ((h & 0x7ff00000u) == 0x7ff00000u) continue;  // not finite
+            const unsigned k = h ^ ((h >> 31) ? 0xffffffffu : 0x80000000u);
+            mn[a] = min(mn[a], k);
+            mx[a] = max(mx[a], k);
+        }
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        mn[a] = __reduce_min_sync(0xffffffffu, mn[a]);
+        mx[a] = __reduce_max_sync(0xffffffffu, mx[a]);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&smn[a], mn[a]);
+            atomicMax(&smx[a], mx[a]);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            part[(size_t)blockIdx.x * 6 + a] = smn[a];
+            part[(size_t)blockIdx.x * 6 + 3 + a] = smx[a];
+        }
+        __threadfence();
+        last = atomicAdd(&geo->done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    float lo[2][3] = {}, hi[2][3] = {};  // points, seeds
+    bool some[2] = {true, true};
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            unsigned m = 0xffffffffu, v = 0u;
+            for (int b = (q ? point_blocks : 0) + (int)threadIdx.x; b < (q ? (int)gridDim.x : point_blocks); b += 32) {
+                m = min(m, __ldcg(&part[(size_t)b * 6 + a]));
+                v = max(v, __ldcg(&part[(size_t)b * 6 + 3 + a]));
+            }
+            m = __reduce_min_sync(0xffffffffu, m);
+            v = __reduce_max_sync(0xffffffffu, v);
+            // outward: the dropped low words all zeros or all ones
+            const unsigned hm = (m >> 31) ? m ^ 0x80000000u : ~m, hx = (v >> 31) ? v ^ 0x80000000u : ~v;
+            const double dl = __longlong_as_double((long long)(((unsigned long long)hm << 32) | ((hm >> 31) ? 0xffffffffull : 0ull)));
+            const double dh = __longlong_as_double((long long)(((unsigned long long)hx << 32) | ((hx >> 31) ? 0ull : 0xffffffffull)));
+            const bool any = m <= v;
+            some[q] = some[q] && any;
+            lo[q][a] = any ? __double2float_rd(dl) : 0.f;
+            hi[q][a] = any ? __double2float_ru(dh) : 1.f;
+        }
+    if (threadIdx.x != 0) return;
+    float ext[3] = {0.f, 0.f, 0.f}, near_lo[3] = {0.f, 0.f, 0.f}, near_ext[3] = {0.f, 0.f, 0.f}, margin = 0.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) margin = fmaxf(margin, 0.5f * (hi[1][a] - lo[1][a]));
+    bool wide = false, meet = some[0] && some[1];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        ext[a] = __fsub_ru(hi[0][a], lo[0][a]);
+        near_lo[a] = fmaxf(lo[0][a], lo[1][a] - margin);
+        near_ext[a] = __fsub_ru(fminf(hi[0][a], hi[1][a] + margin), near_lo[a]);
+        wide = wide || ext[a] > 4.f * near_ext[a];
+        meet = meet && near_ext[a] >= 0.f;
+    }
+    const bool two = wide && meet && want >= 8;
+    if (two) {
+        make_tiling<D>(near_lo, near_ext, want - want / 4, geo);
+        make_tiling<D>(lo[0], ext, want / 4, geo + 1);
+    } else {
+        make_tiling<D>(lo[0], ext, want, geo);
+        geo[1].n_regions = 0;
+    }
     geo->pool = 0u;
     geo->done = 0u;
 }
@@ -217,8 +259,8 @@ __global__ void __launch_bounds__(kPtThreads)
 // Candidate lists of the tiles, stored.
 template <int D>
 __global__ void __launch_bounds__(kThreads, 4)
-    points_lists_kernel(const __grid_constant__ Src src, PtsGeo *__restrict__ geo, TileHead *__restrict__ heads,
-                        float4 *__restrict__ polys, const unsigned pool_cap) {
+    points_lists_kernel(const __grid_constant__ Src src, PtsGeo *__restrict__ geo, TileHead *__restrict__ all_heads,
+                        const int second, const int first_blocks, float4 *__restrict__ polys, const unsigned pool_cap) {
     using G = Geom<D>;
     constexpr int NP = G::NP;
     constexpr int PV = D == 3 ? 3 : 2;  // float4s of a polynomial
@@ -226,22 +268,27 @@ __global__ void __launch_bounds__(kThreads, 4)
     __shared__ Src s;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const unsigned full = 0xffffffffu;
+    const bool other = (int)blockIdx.x >= first_blocks;  // the blocks of the second tiling
+    const PtsGeo *const ge = geo + (other ? 1 : 0);
+    TileHead *const heads = all_heads + (other ? second : 0);
+    const int nr = ge->n_regions;
+    if (nr == 0) return;
     for (int i = tid; i < (int)(sizeof(Src) / 4); i += kThreads)
         reinterpret_cast<int *>(&s)[i] = reinterpret_cast<const int *>(&src)[i];
+    const int stride = other ? (int)gridDim.x - first_blocks : first_blocks;
     __syncthreads();
-    if (tid == 0) s.gf = geo->gf;
+    if (tid == 0) s.gf = ge->gf;
     __syncthreads();
-    const int nr = geo->n_regions;
     const float hh[3] = {s.gf.hh[0], s.gf.hh[1], s.gf.hh[2]};
     float tr[3], rr[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        tr[a] = a < D ? geo->r[a] : 0.f;
+        tr[a] = a < D ? ge->r[a] : 0.f;
         rr[a] = a < D ? hh[a] + tr[a] : 0.f;
     }
-    for (int reg = (int)blockIdx.x; reg < nr; reg += (int)gridDim.x) {
-        const int q = reg / geo->regions[0];
-        const int rb[3] = {reg % geo->regions[0], D == 3 ? q % geo->regions[1] : q, D == 3 ? q / geo->regions[1] : 0};
+    for (int reg = (int)blockIdx.x - (other ? first_blocks : 0); reg < nr; reg += stride) {
+        const int q = reg / ge->regions[0];
+        const int rb[3] = {reg % ge->regions[0], D == 3 ? q % ge->regions[1] : q, D == 3 ? q / ge->regions[1] : 0};
         float ch[3] = {0.f, 0.f, 0.f}, cl[3] = {0.f, 0.f, 0.f};
 #pragma unroll
         for (int a = 0; a < D; ++a) axis_point(s.gf, a, 4 * rb[a] + 2, ch[a], cl[a]);
@@ -255,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, 4)
         for (int a = 0; a < 3; ++a) {
             ti[a] = a < D ? 2 * rb[a] + tc[a] : 0;
             if (a < D) toff[a] = tc[a] ? hh[a] : -hh[a];
-            real = real && ti[a] < geo->t[a];
+            real = real && ti[a] < ge->t[a];
         }
         if (real) {
             const bool scan = total > (unsigned)kListCap;
@@ -316,7 +363,7 @@ __global__ void __launch_bounds__(kThreads, 4)
                 h.ref = fits ? ref_id : -1;
                 h.first = first;
                 h.count = count;
-                heads[(size_t)ti[0] + (size_t)geo->t[0] * ((size_t)ti[1] + (size_t)geo->t[1] * (size_t)ti[2])] = h;
+                heads[(size_t)ti[0] + (size_t)ge->t[0] * ((size_t)ti[1] + (size_t)ge->t[1] * (size_t)ti[2])] = h;
             }
             if (fits && count) {
                 unsigned at = first;
@@ -354,14 +401,14 @@ __global__ void __launch_bounds__(T)
     points_score_kernel(const long long count, const double *__restrict__ y, const double *__restrict__ mass,
                         const int n, const double *__restrict__ x, const double *__restrict__ A,
                         const double *__restrict__ w, const SeedRec32 *__restrict__ r32, const PtsGeo *__restrict__ geo,
-                        const TileHead *__restrict__ heads, const float4 *__restrict__ polys,
+                        const TileHead *__restrict__ heads, const int second, const float4 *__restrict__ polys,
                         DevScalars *__restrict__ sc, double *__restrict__ mom, int32_t *__restrict__ labels) {
     constexpr int PV = D == 3 ? 3 : 2;
     constexpr int K = moment_width(D);
-    __shared__ PtsGeo ge;
+    __shared__ PtsGeo tilings[2];
     extern __shared__ double acc[];
-    for (int i = threadIdx.x; i < (int)(sizeof(PtsGeo) / 4); i += T)
-        reinterpret_cast<int *>(&ge)[i] = reinterpret_cast<const int *>(geo)[i];
+    for (int i = threadIdx.x; i < (int)(2 * sizeof(PtsGeo) / 4); i += T)
+        reinterpret_cast<int *>(tilings)[i] = reinterpret_cast<const int *>(geo)[i];
     if (SHARED)
         for (int i = threadIdx.x; i < n * K; i += T) acc[i] = 0.0;
     __syncthreads();
@@ -374,18 +421,30 @@ __global__ void __launch_bounds__(T)
         double yy[D];
         float yh[3] = {0.f, 0.f, 0.f}, yl[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
         size_t tile = 0;
-        bool inside = active;
 #pragma unroll
         for (int a = D - 1; a >= 0; --a) {
             yy[a] = active ? y[j * D + a] : 0.0;
             split_trunc(yy[a], yh[a], yl[a]);
-            const float d = (yh[a] - ge.gf.loh[a]) + yl[a];
-            const int t = min(max((int)(d * ge.inv[a]), 0), ge.t[a] - 1);
-            float ch, cl;
-            axis_point(ge.gf, a, 2 * t + 1, ch, cl);
-            e[a] = (yh[a] - ch) + (yl[a] - cl);
-            inside = inside && fabsf(e[a]) <= ge.r[a];  // false for a NaN
-            tile = tile * (size_t)ge.t[a] + (size_t)t;
+        }
+        auto locate = [&](const PtsGeo &ge) -> bool {  // the point's tile and its offset from the centre
+            bool in = active;
+            tile = 0;
+#pragma unroll
+            for (int a = D - 1; a >= 0; --a) {
+                const float d = (yh[a] - ge.gf.loh[a]) + yl[a];
+                const int t = min(max((int)(d * ge.inv[a]), 0), ge.t[a] - 1);
+                float ch, cl;
+                axis_point(ge.gf, a, 2 * t + 1, ch, cl);
+                e[a] = (yh[a] - ch) + (yl[a] - cl);
+                in = in && fabsf(e[a]) <= ge.r[a];  // false for a NaN
+                tile = tile * (size_t)ge.t[a] + (size_t)t;
+            }
+            return in;
+        };
+        bool inside = locate(tilings[0]);
+        if (!inside && tilings[1].n_regions) {
+            inside = locate(tilings[1]);
+            tile += (size_t)second;
         }
         const double mj = active ? mass[j] : 0.0;
         TileHead h{0.f, -1, 0u, 0u};
@@ -581,9 +640,11 @@ cudaError_t launch_t(long long count, const double *y, const double *mass, int n
         // about 32 tiles a seed, no more than one per two points or the store holds
         const long long cap = (long long)(ws.pts_bytes / (sizeof(TileHead) + 8 * 48));
         const long long tiles = std::max<long long>(1, std::min<long long>(std::min<long long>(32ll * n, count / 2), cap));
+        const int second = (int)(tiles - tiles / 4);  // first tile of the second tiling
+        const int sblocks = std::min((n + kPtThreads - 1) / kPtThreads, 64);
         // the blocks' boxes (24 bytes each) go where the tiles' headers follow
-        points_box_kernel<D><<<blocks, kPtThreads, 0, st>>>(count, y, tiles, reinterpret_cast<unsigned *>(ws.pts_tiles),
-                                                            ws.pts_geo);
+        points_box_kernel<D><<<blocks + sblocks, kPtThreads, 0, st>>>(
+            count, y, n, x, blocks, tiles, reinterpret_cast<unsigned *>(ws.pts_tiles), ws.pts_geo);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         e = launch_seed_prep(none, n, x, A, w, ws, m64, n_mom, st, ws.pts_geo);
@@ -602,7 +663,8 @@ cudaError_t launch_t(long long count, const double *y, const double *mass, int n
         const size_t rest = ws.pts_bytes - ((size_t)tiles * sizeof(TileHead) + 255) / 256 * 256;
         const unsigned pool = (unsigned)std::min<size_t>(rest / ((D == 3 ? 3 : 2) * sizeof(float4)), 0x7fffffffu);
         const int lb = (int)std::min<long long>(4ll * ws.sms, tiles);
-        points_lists_kernel<D><<<lb, kThreads, 0, st>>>(src, ws.pts_geo, heads, polys, pool);
+        const int lb2 = (int)std::min<long long>(ws.sms, std::max<long long>(1, tiles / 32));  // most calls need none
+        points_lists_kernel<D><<<lb + lb2, kThreads, 0, st>>>(src, ws.pts_geo, heads, second, lb, polys, pool);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         // Block sums where n K doubles fit (one block of 1024 per SM) and a block gets
@@ -622,11 +684,11 @@ cudaError_t launch_t(long long count, const double *y, const double *mass, int n
             }
             const int per_sm = smem <= kPtShared / 2 ? 2 : 1;
             points_score_kernel<D, true, T><<<per_sm * ws.sms, T, smem, st>>>(
-                count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, polys, ws.sc, mom, labels);
+                count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, second, polys, ws.sc, mom, labels);
         } else {
             const int sb = (int)std::min<long long>(want_blocks, (long long)ws.sms * 8);
             points_score_kernel<D, false, kPtThreads><<<sb, kPtThreads, 0, st>>>(
-                count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, polys, ws.sc, mom, labels);
+                count, y, mass, n, x, A, w, ws.recs32, ws.pts_geo, heads, second, polys, ws.sc, mom, labels);
         }
         return cudaGetLastError();
     }
