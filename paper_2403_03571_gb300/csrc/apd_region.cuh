@@ -40,14 +40,17 @@
 // tile or region of one cell adds its sums in closed form.
 //
 // Rounding.  With u = 2^-24, p_b = |d_b| + r_b + 2^-24 (|x_b| + |y|_max,b) and
-// S = sum_bc |A_bc| p_b p_c, the position differences (FP32 pairs) err by at most
-// 5 u p_b, so q, G and the pixel terms of one seed by at most 17 u S (A's own
-// rounding 1, the differences 10, the dot products 6); forming D0, G and dA adds
-// 3 u (S_i + S_a + |dw| + ...), the row coefficients, the two FMAs and the pixel
-// offsets 19 u (S_i + S_a): 39 u in all.  kCoef = 64 is used for both the list test
-// and the certificate.  A pixel is labelled when its two smallest values are more
-// than 2 max_i E_i apart, E_i = 64 u (S_i + S_a + W), W = |dw| + 2^-24 (|w_i| +
-// |w_a|); every other pixel is settled
+// S = sum_bc |A_bc| p_b p_c: a difference d is two FP32 subtractions of pairs (one
+// rounding of c - x, one of the sum) and the tile's offset o (two roundings) added, so it
+// errs by at most 3 u |d| + 4 u |o|, and a pixel's own offset by 2 u r.  |o| <= 8/7 r in
+// 3D, 3.2 r on the second axis in 2D (tiles 24 h from the centre, r = 7.5 h): 6.6 u p and
+// 14.8 u p.  The cost of one seed then errs by at most 21 u S in 3D (A's own rounding 1,
+// the differences 2 x 6.6, the dot products 6), 35 u S in 2D (1, 2 x 14.8, 4); forming D0,
+// G and dA adds 3 u (S_i + S_a + |dw| + ...), the row coefficients and the two FMAs 9 u,
+// in 2D 5 u, of the same: 33 u (3D) and 43 u (2D) in all, and the list test's sums no more
+// than the pixels'.  kCoef = 64 is used for both the list test and the certificate.  A
+// pixel is labelled when its two smallest values are more than 2 max_i E_i apart,
+// E_i = 64 u (S_i + S_a + W), W = |dw| + 2^-24 (|w_i| + |w_a|); every other pixel is settled
 // by its warp in FP64 with the reference arithmetic over the seeds within the gap, a
 // lane per pixel: no rescoring launch follows.
 #pragma once
@@ -138,7 +141,6 @@ struct Shared {
     uint16_t queue[kWarps][kTilePix];  // the tile's near ties: pixel of the tile
     unsigned lut[256];  // row mask -> count | sum x << 8 | sum x^2 << 16
     unsigned key[kWarps];
-    int pos[kWarps];
     unsigned count;     // listed seeds
     unsigned pairs;
     unsigned queued;    // pixels settled in FP64
@@ -508,7 +510,6 @@ __device__ __forceinline__ unsigned region_list(Shared<D> &sm, const Src &s, con
         const int who = __ffs(__ballot_sync(full, ck == cm)) - 1;
         if (lane == who) {
             sm.key[wid] = cm;
-            sm.pos[wid] = have ? p : 0;
             if (have) {
                 float v = L.q + 1e-5f * (L.S + fabsf(wn)) + 1e-30f;
 #pragma unroll
