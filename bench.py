@@ -229,7 +229,7 @@ def run_reference(args, evals_per_apd):
         "n_gpus": args.gpus, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": 1000.0 * t_eval, "step": "one complete FP64 evaluation of the dual",
         "higher_is_better": True, "scaling": "strong", "vs_baseline": None, "dtype": "f64",
-        "data": "synthetic", "config": config_dict(args.workload, inst, rounds, args.precision),
+        "data": "synthetic", "config": config_dict(args.workload, inst, rounds, "f64"),
         "pair_evals_per_s": pairs / t_eval, "evaluation_s": t_eval, "evals_per_apd": evals_per_apd,
         "cpu_baseline": {"value": val, "unit": "APD/s", "cores": cores, "kind": "oracle", "sample": sample},
         "e2e": {"value": val, "unit": "APD/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0},
@@ -285,7 +285,16 @@ PRECISION_TEXT = {
     "fp32": "fp32 CUDA-core scoring, fp64 near-tie rescoring",
     "tc_tf32": "tcgen05 TF32 scoring (FP32 accumulate), FP32 candidate rescoring, fp64 near-tie rescoring",
     "tc_bf16": "tcgen05 BF16 scoring (FP32 accumulate), FP32 candidate rescoring, fp64 near-tie rescoring",
+    "region": "fp32 CUDA-core scoring of candidate lists (cost differences), fp64 near-tie settling",
+    "f64": "fp64 costs on the host cores",
 }
+
+
+def scoring_form(args, precision=None):
+    """The arithmetic that a chosen form runs: pruned full passes score candidate lists in
+    FP32 whatever precision is asked for; the tensor cores take dense and recording passes."""
+    precision = precision or args.precision
+    return "region" if args.prune and (args.incremental < 2 or precision == "fp32") else precision
 
 
 def config_dict(workload, inst, rounds, precision="fp32"):
@@ -587,7 +596,7 @@ def run_ours(args):
     forms["chosen"]["precision"] = args.precision
     forms["chosen"]["pruned"] = bool(args.prune)
     forms["chosen"]["incremental"] = args.incremental > 1
-    forms["chosen"]["region"] = args.incremental < 2
+    forms["chosen"]["region"] = scoring_form(args) == "region"
     # the chosen form's final generators and its labels there (for the accuracy report)
     x_fin = (ctx["x_out"] if rounds > 0 else ctx["x0"]).clone()
     w_fin = ctx["w_out"].clone()
@@ -604,7 +613,7 @@ def run_ours(args):
     forms["chosen_alt"]["precision"] = alt
     forms["chosen_alt"]["pruned"] = bool(args.prune)
     forms["chosen_alt"]["incremental"] = args.incremental > 1
-    forms["chosen_alt"]["region"] = args.incremental < 2
+    forms["chosen_alt"]["region"] = scoring_form(args, alt) == "region"
     forms["fp32"] = measure_form(args, ctx, "fp32")
     forms["fp32"]["precision"] = "fp32"
     if world > 1:
@@ -632,9 +641,9 @@ def run_ours(args):
         "higher_is_better": True,
         "scaling": "strong",
         "vs_baseline": None,
-        "dtype": {"tc_tf32": "tf32/f32/f64", "tc_bf16": "bf16/f32/f64"}.get(args.precision, "f32/f64"),
+        "dtype": {"tc_tf32": "tf32/f32/f64", "tc_bf16": "bf16/f32/f64"}.get(scoring_form(args), "f32/f64"),
         "data": "synthetic",
-        "config": config_dict(args.workload, inst, rounds, args.precision)
+        "config": config_dict(args.workload, inst, rounds, scoring_form(args))
         | {"parallelism": (f"one diagram over {world} ranks: slabs of the last grid axis, int64 allreduce "
                            "of the per-cell moments per evaluation (NCCL)") if world > 1 else "one GPU"},
         "pair_evals_per_s": chosen["pair_evals_per_s"],
@@ -654,9 +663,7 @@ def run_ours(args):
                           "prediction judged against W = 0"
                           + ("; the coarse solves continue one L-BFGS history across the rounds"
                              if args.carry_history else "")
-                          + f"; {args.precision} scoring"
-                          + (" with seed pruning (tensor cores: per-tile candidate lists; FP32: group and "
-                             "per-seed bounds)" if args.prune else ""))
+                          + f"; {PRECISION_TEXT[scoring_form(args)]}")
     out["coarse_evaluations_per_apd"] = chosen["coarse_evaluations_per_apd"]
     out["warm_start_network"] = chosen["warm_start_network"]
     if not args.no_configs and world == 1:
