@@ -960,7 +960,13 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
     alloc((void **)&w.flag_gi, (size_t)max_j * sizeof(int32_t));
     alloc((void **)&w.pairs_scored, sizeof(unsigned long long));
     alloc((void **)&w.groups, (size_t)(w.n_pad_max / 32) * sizeof(GroupBound));
-    alloc((void **)&w.sc, sizeof(DevScalars));
+    // the device's scalars, the points' tilings and the push's state, cleared together
+    const size_t geo_at = (sizeof(DevScalars) + 255) / 256 * 256;
+    const size_t push_at = geo_at + (2 * sizeof(PtsGeo) + 255) / 256 * 256, scalars = push_at + sizeof(PushState);
+    alloc((void **)&w.sc, scalars);
+    if (ok && cudaMemset(w.sc, 0, scalars) != cudaSuccess) ok = false;
+    w.pts_geo = reinterpret_cast<PtsGeo *>(reinterpret_cast<uint8_t *>(w.sc) + geo_at);
+    w.push_state = reinterpret_cast<PushState *>(reinterpret_cast<uint8_t *>(w.sc) + push_at);
     // tensor-core tiles hold 512 pixels; 2x slack covers ragged grids (thinner grids
     // are scored by the FP32 kernel)
     w.tc_tile_cap = max_j / 256 + 1024;
@@ -969,19 +975,21 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
     alloc((void **)&w.tc_meta, (size_t)w.tc_tile_cap * sizeof(int4));
     alloc((void **)&w.tc_texcl, (size_t)w.tc_tile_cap * sizeof(float));
     alloc((void **)&w.tc_list, (size_t)w.tc_tile_cap * tc_list_cap() * sizeof(int));
-    alloc((void **)&w.tc_bops, (size_t)w.tc_tile_cap * tc_bops_bytes_per_tile());
+    // the stored operands of a tensor-core pass; a point set's tiles take the same memory
+    // (about 32 tiles a seed, room for eight polynomials a tile): either call writes what
+    // it reads
+    size_t bops = (size_t)w.tc_tile_cap * tc_bops_bytes_per_tile();
+    if (w.n_pad_max <= kSortMax) {
+        w.pts_bytes = (size_t)std::min<long long>(32ll * std::max(max_n, 64), 1ll << 17) * (16 + 8 * 48);
+        bops = std::max(bops, w.pts_bytes);
+    }
+    alloc((void **)&w.tc_bops, bops);
+    if (w.pts_bytes) w.pts_tiles = reinterpret_cast<uint8_t *>(w.tc_bops);
     alloc((void **)&w.tc_axis, (size_t)3 * w.tc_tile_cap * sizeof(float4));
     // super-tiles: at most one per tile
     w.part_rows = (int)nb;
     // one row per warp of an evaluation's first kernel (part_rows: the blocks the sums are made in)
     alloc((void **)&w.part, std::max(nb, (size_t)w.n_pad_max / 32) * kPartStride * sizeof(double));
-    if (w.n_pad_max <= kSortMax) {
-        // point sets: about 32 tiles a seed, room for eight polynomials a tile
-        w.pts_bytes = (size_t)std::min<long long>(32ll * std::max(max_n, 64), 1ll << 17) * (16 + 8 * 48);
-        alloc((void **)&w.pts_tiles, w.pts_bytes);
-        alloc((void **)&w.pts_geo, 2 * sizeof(PtsGeo));
-        if (ok && cudaMemset(w.pts_geo, 0, 2 * sizeof(PtsGeo)) != cudaSuccess) ok = false;
-    }
     alloc((void **)&w.grad, (size_t)max_n * sizeof(double));
     alloc((void **)&w.W, (size_t)max_n * sizeof(double));
     alloc((void **)&w.Wt, (size_t)max_n * sizeof(double));
@@ -995,7 +1003,6 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
     w.lb_rows = w.sms;
     alloc((void **)&w.lb_part, (size_t)w.lb_rows * kLbfgsDots * sizeof(double));
     alloc((void **)&w.lb_coef, sizeof(LbfgsCoef));
-    alloc((void **)&w.push_state, sizeof(PushState));
     alloc((void **)&w.rho, kHistCap * sizeof(double));
     alloc((void **)&w.X, (size_t)max_n * dim * sizeof(double));
     alloc((void **)&w.vbuf, (size_t)max_n * sizeof(double));
@@ -1003,7 +1010,6 @@ int apd_workspace_create(apd_workspace **out, int32_t dim, int32_t max_n, int64_
     alloc((void **)&w.wpred, (size_t)max_n * sizeof(double));
     if (ok && cudaMallocHost((void **)&w.sc_host, sizeof(DevScalars)) != cudaSuccess) ok = false;
     if (ok) std::memset(w.sc_host, 0, sizeof(DevScalars));
-    if (ok && cudaMemset(w.sc, 0, sizeof(DevScalars)) != cudaSuccess) ok = false;
     if (ok && cudaMemset(w.pairs_scored, 0, sizeof(unsigned long long)) != cudaSuccess) ok = false;
     if (ok && cudaMemset(w.recs, 0, (size_t)w.n_pad_max * sizeof(SeedRec)) != cudaSuccess) ok = false;
     if (ok && cudaDeviceSynchronize() != cudaSuccess) ok = false;
@@ -1023,8 +1029,8 @@ void apd_workspace_destroy(apd_workspace *ws) {
     if (w.cap_stream) cudaStreamDestroy(w.cap_stream);
     if (w.cond_ev) cudaEventDestroy(w.cond_ev);
     void *ptrs[] = {w.recs, w.recs32, w.recs_tmp, w.codes, w.scodes, w.perm, w.recs32s, w.tc_centre, w.tc_start, w.tc_meta, w.tc_texcl, w.tc_list, w.tc_bops, w.tc_axis, w.moments, w.flags, w.flag_gi, w.pairs_scored, w.groups, w.sc, w.part, w.grad, w.W, w.Wt, w.p, w.gf, w.gft,
-                    w.Wbest, w.S, w.Y, w.gram, w.lb_part, w.lb_coef, w.push_state, w.rho, w.X, w.vbuf, w.wfeat, w.wpred,
-                    w.S2, w.Y2, w.gram2, w.rho2, w.inc_labels, w.inc_gap, w.inc_rec, w.inc_hist, w.inc_drift, w.inc_mom0, w.inc_w0, w.inc_aux, w.pts_tiles, w.pts_geo};
+                    w.Wbest, w.S, w.Y, w.gram, w.lb_part, w.lb_coef, w.rho, w.X, w.vbuf, w.wfeat, w.wpred,
+                    w.S2, w.Y2, w.gram2, w.rho2, w.inc_labels, w.inc_gap, w.inc_rec, w.inc_hist, w.inc_drift, w.inc_mom0, w.inc_w0, w.inc_aux};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (w.sc_host) cudaFreeHost(w.sc_host);

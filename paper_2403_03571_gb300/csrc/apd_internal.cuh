@@ -189,7 +189,7 @@ struct Workspace {
     DevScalars *sc_host = nullptr;      // pinned host mirror, written by a solver evaluation's last kernel
     unsigned int sc_seq = 0;            // number of the last evaluation the host has read
     PtsGeo *pts_geo = nullptr;          // [2] tilings of the last point set (n_regions 0: no second)
-    uint8_t *pts_tiles = nullptr;       // its tiles' headers, then their polynomials (pts_bytes)
+    uint8_t *pts_tiles = nullptr;       // its tiles' headers, then their polynomials (pts_bytes; in tc_bops)
     size_t pts_bytes = 0;
     double *part = nullptr;             // [part_rows][kPartStride] per-block partials (dual, trial weights)
     int part_rows = 0;
