@@ -13,7 +13,7 @@ using namespace region;
 // Four blocks per SM (64 registers, some spills) were a little faster than three, and those
 // than two without spills (256^3, 1000 seeds: the whole call 195, 197 and 207 us with the
 // preparation it had then): the lists' two barriers and the dependent loads want more warps
-// more than they want registers.  The kernel itself takes 101 us there.
+// more than they want registers.  The kernel itself takes 99 us there.
 template <int D>
 __global__ void __launch_bounds__(kThreads, 4)
     assign_region_kernel(const __grid_constant__ Src src, const int nx, const int ny, const int toff) {
@@ -115,8 +115,8 @@ bool region_lists(const GridDev &g, int n, const Workspace &ws) {
 // kernel (or the tensor-core lists): a tile's list is then longer than its pixels.
 // MEASURED, us per call, regions / FP32 kernel: 2D n = 5000 on 100^2 1469 / 1335, n = 12000
 // on 128^2 2148 / 1650; 3D n = 8300 on 20 x 17 x 16 3363 / 2324, n = 9000 on 28^3 1741 / 1434;
-// and above the line 3D n = 5000 on 32^3 863 / 1067, n = 16000 on 48^3 1379 / 1860, with fewer
-// seeds 2D n = 3000 on 80^2 808 / 1286.
+// and above the line 3D n = 5000 on 32^3 933 / 1056, n = 16000 on 48^3 1442 / 1892, with fewer
+// seeds 2D n = 3000 on 80^2 768 / 1301.
 bool region_form(const GridDev &g, int n, const Workspace &ws) {
     const bool crowded = n > 4096 && 2 * g.J < 5ll * n;
     return ws.prune && !crowded && region_lists(g, n, ws);

@@ -78,7 +78,7 @@ constexpr int kMaxGroups = kSortMax / kGroup;  // 512: two groups per lane and w
 // a list beyond it from the region's.  512 leave the caches their room; where the regions
 // are fewer than the SMs hold, or cells are so small that lists are long, a block gets more.
 // MEASURED, us per call, lists formed again from the region's only / from the tile's: 3D
-// n = 10000 on 96^3 1326 / 324, n = 3000 on 60^3 441 / 217; 2D n = 5000 on 300^2 601 / 240.
+// n = 10000 on 96^3 1326 / 347, n = 3000 on 60^3 441 / 223; 2D n = 5000 on 300^2 601 / 245.
 constexpr int kTileCap = 512, kTileCapMax = 12032;
 inline int tile_cap(long long regions, long long pixels, int n, int sms) {
     const int cap = regions <= sms ? kTileCapMax
@@ -137,7 +137,7 @@ struct Shared {
     float4 poly[kWarps][kBuf][3];
     float4 ref[kWarps][5];             // the warp's best seed (region), then its tile's reference
     uint16_t list[kListCap];           // scan positions
-    unsigned mask[kMaxGroups];         // a group's listed seeds
+    unsigned mask[kMaxGroups];         // a group's listed seeds (where there are more than kListCap)
     uint16_t queue[kWarps][kTilePix];  // the tile's near ties: pixel of the tile
     unsigned lut[256];  // row mask -> count | sum x << 8 | sum x^2 << 16
     unsigned key[kWarps];
@@ -453,6 +453,37 @@ __device__ __forceinline__ float group_lower(const GroupBound &gb, const float (
     return __fadd_rd(__fmul_rd(__fmul_rd(gb.lam, d2), 1.f - 1e-5f), gb.wgap);
 }
 
+struct Box {
+    float ch[3], cl[3], rr[3];
+};
+
+// Where the list is too short: the same test of every seed against the region's reference,
+// a bit per seed.  Out of line, and its work done twice, since few regions come here.
+template <int D>
+__device__ __noinline__ void mask_groups(Shared<D> &sm, const Src &s, const Box b) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned full = 0xffffffffu;
+    const float zero3[3] = {0.f, 0.f, 0.f};
+    const unsigned k = lane < kWarps ? sm.key[lane] : 0xffffffffu;
+    const unsigned km = __reduce_min_sync(full, k);
+    Local<D> R;
+    int a0;
+    load_local<D>(sm.ref[__ffs(__ballot_sync(full, lane < kWarps && k == km)) - 1], R, a0);
+    for (int grp = wid; grp < s.n_groups; grp += kWarps) {
+        const int p = grp * 32 + lane;
+        bool keep = false;
+        if (p < s.n) {
+            Local<D> L;
+            Diff<D> F;
+            local_terms<D>(s.recs[p], b.ch, b.cl, zero3, b.rr, s.gf, L);
+            difference<D>(L, R, F);
+            keep = p == a0 || can_win<D>(F, b.rr);
+        }
+        const unsigned bits = __ballot_sync(full, keep);
+        if (lane == 0) sm.mask[grp] = bits;
+    }
+}
+
 // The seeds that can be the argmin somewhere in the box of half-widths rr around ch + cl,
 // listed in sm.list by the whole block (two barriers; none follows the last entry's
 // write but the second).  Returns their number, which may exceed kListCap (the list is
@@ -482,10 +513,7 @@ __device__ __forceinline__ unsigned region_list(Shared<D> &sm, const Src &s, con
         for (int t = 0; t < 2; ++t) {
             if (s.n_groups <= t * kThreads) break;
             const int grp = wid + kWarps * (lane + 32 * t);
-            if (grp < s.n_groups) {
-                glb[t] = group_lower<D>(s.groups[grp], alo, ahi);
-                sm.mask[grp] = 0u;
-            }
+            if (grp < s.n_groups) glb[t] = group_lower<D>(s.groups[grp], alo, ahi);
         }
     }
     // each warp's group of least bound, and in it the seed of least cost at the centre
@@ -559,17 +587,19 @@ __device__ __forceinline__ unsigned region_list(Shared<D> &sm, const Src &s, con
             const unsigned km = __ballot_sync(full, keep);
             if (km) {
                 unsigned at = 0u;
-                if (lane == 0) {
-                    sm.mask[wid + kWarps * (gl + 32 * t)] = km;
-                    at = atomicAdd(&sm.count, (unsigned)__popc(km));
-                }
+                if (lane == 0) at = atomicAdd(&sm.count, (unsigned)__popc(km));
                 at = __shfl_sync(full, at, 0) + (unsigned)__popc(km & ((1u << lane) - 1u));
                 if (keep && at < (unsigned)kListCap) sm.list[at] = (uint16_t)p;
             }
         }
     }
     __syncthreads();
-    return sm.count;
+    const unsigned total = sm.count;
+    if (total > (unsigned)kListCap) {
+        mask_groups<D>(sm, s, Box{{ch[0], ch[1], ch[2]}, {cl[0], cl[1], cl[2]}, {rr[0], rr[1], rr[2]}});
+        __syncthreads();
+    }
+    return total;
 }
 
 // The seeds that region_list has listed, in chunks of a warp.
@@ -624,10 +654,9 @@ __device__ __forceinline__ void put_poly(float4 (*buf)[3], int at, const Src &s,
 
 // A tile whose polynomials do not fit the warp's buffer: piece c of them formed again,
 // from the tile's list where it is complete (`listed` seeds), else from the region's.
-// Returns their number.  Out of line: few tiles come here, and inlined in four places it
-// cost the others registers (256^3, 1000 seeds: 108 us -> 115 us).
+// Returns their number.
 template <int D>
-__device__ __noinline__ int refill(Shared<D> &sm, const Src &s, const uint16_t *tile, const int bx, const int by,
+__device__ __forceinline__ int refill(Shared<D> &sm, const Src &s, const uint16_t *tile, const int bx, const int by,
                                    const int bz, const int c, const int listed, const int best_pos) {
     using G = Geom<D>;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -659,187 +688,60 @@ __device__ __noinline__ int refill(Shared<D> &sm, const Src &s, const uint16_t *
     return __popc(km);
 }
 
-// Scores region (bx, by, bz); `s` is the same in every thread; `tiles`: kWarps lists of
-// tile_cap positions in shared memory.  The caller puts a barrier between the previous
-// region and the next.
-template <int D, bool MASKED = false>
-__device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, const Src &s, const int bx, const int by,
-                                             const int bz) {
-    using G = Geom<D>;
-    constexpr int K = moment_width(D);
-    const GridDev &g = s.g;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const unsigned full = 0xffffffffu;
-    const float finf = __int_as_float(0x7f800000);
-    const int n = s.n;
-    const int tdim[3] = {G::TX, G::TY, G::TZ};
-    const int rdim[3] = {G::RX, G::RY, G::RZ};
-    const int rb[3] = {bx * G::RX, by * G::RY, bz * G::RZ};
-    float4(&ref)[5] = sm.ref[wid];
-
-    // the warp's tile
+// The warp's tile of region (bx, by, bz): its first pixel, the pixels of it that are scored.
+template <int D>
+struct TileWindow {
     int tc[3], kb[3], lo3[3], cnt[3];
-    float toff[3], tr[3];
-    warp_tile<D>(wid, tc);
-    tile_box<D>(g, tc, toff, tr);
-    bool empty = false, whole = true;
+    bool empty, whole;
+    __device__ __forceinline__ TileWindow(const GridDev &g, const int bx, const int by, const int bz)
+        : empty(false), whole(true) {
+        using G = Geom<D>;
+        const int tdim[3] = {G::TX, G::TY, G::TZ};
+        const int rb[3] = {bx * G::RX, by * G::RY, bz * G::RZ};
+        warp_tile<D>(threadIdx.x >> 5, tc);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        kb[a] = rb[a] + tc[a] * tdim[a];
-        int lo = kb[a], hi = kb[a] + tdim[a];
-        if (a < D) {
-            hi = min(hi, a == D - 1 ? win_hi(g) : g.res[a]);
-            if (a == D - 1) lo = max(lo, win_lo(g));
-        }
-        lo3[a] = lo;
-        cnt[a] = hi - lo;
-        empty = empty || cnt[a] <= 0;
-        whole = whole && cnt[a] == tdim[a];
-    }
-    const int x0 = D == 3 ? 0 : 8 * (lane & 3);  // the lane's first pixel and rows in the tile
-    const int y0 = D == 3 ? (lane & 7) : (lane >> 2), z0 = D == 3 ? (lane >> 3) : 0;
-    const int k0 = kb[0] + x0;
-    const int w0 = min(8, g.res[0] - k0);
-    const unsigned wmask = w0 >= 8 ? 0xffu : (w0 > 0 ? (1u << w0) - 1u : 0u);
-    // row r of the lane: the pixels scored
-    auto row_valid = [&](int r) -> unsigned {
-        const int k1 = kb[1] + (D == 3 ? y0 : y0 + 8 * r), kl = D == 3 ? kb[2] + z0 + 4 * r : k1;
-        return k1 < g.res[1] && kl >= win_lo(g) && kl < win_hi(g) ? wmask : 0u;
-    };
-    unsigned marked[2] = {0u, 0u};
-    if constexpr (MASKED) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const unsigned vm = row_valid(r);
-            if (!vm) continue;
-            const int k1 = kb[1] + (D == 3 ? y0 : y0 + 8 * r), k2 = D == 3 ? kb[2] + z0 + 4 * r : 0;
-            const uint8_t *row = s.mask + (size_t)s.cres[0] * ((size_t)(k1 / s.r) + (size_t)s.cres[1] * (size_t)(k2 / s.r));
-            int kx = k0 / s.r, next = (kx + 1) * s.r;
-            bool on = row[kx] != 0;
-#pragma unroll
-            for (int p = 0; p < 8; ++p) {
-                if (!((vm >> p) & 1u)) continue;
-                if (k0 + p == next) {
-                    on = row[++kx] != 0;
-                    next += s.r;
-                }
-                marked[r] |= on ? 1u << p : 0u;
+        for (int a = 0; a < 3; ++a) {
+            kb[a] = rb[a] + tc[a] * tdim[a];
+            int lo = kb[a], hi = kb[a] + tdim[a];
+            if (a < D) {
+                hi = min(hi, a == D - 1 ? win_hi(g) : g.res[a]);
+                if (a == D - 1) lo = max(lo, win_lo(g));
             }
+            lo3[a] = lo;
+            cnt[a] = hi - lo;
+            empty = empty || cnt[a] <= 0;
+            whole = whole && cnt[a] == tdim[a];
         }
-        whole = __all_sync(full, marked[0] == 0xffu && marked[1] == 0xffu);
-        empty = !__any_sync(full, (marked[0] | marked[1]) != 0u);
-        if (!__syncthreads_or(!empty)) return;  // no marked pixel in the region
     }
-    auto row_mask = [&](int r) -> unsigned { return MASKED ? marked[r] : row_valid(r); };
+};
 
-    // region centre (lane a: axis a) as an FP32 pair, half-widths rounded up
-    float ch[3] = {0.f, 0.f, 0.f}, cl[3] = {0.f, 0.f, 0.f};
-    {
-        float h = 0.f, l = 0.f;
-        if (lane < D) {
-            const int k = lane == 0 ? rb[0] + G::RX / 2 : (lane == 1 ? rb[1] + G::RY / 2 : rb[2] + G::RZ / 2);
-            axis_point(s.gf, lane, k, h, l);
-        }
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            ch[a] = __shfl_sync(full, h, a);
-            cl[a] = __shfl_sync(full, l, a);
-        }
+// A lane's two rows of eight pixels.
+template <int D>
+struct LaneRows {
+    int x0, y0, z0, k0, kb1, kb2;  // first pixel and rows in the tile, in the grid
+    unsigned wmask;
+    __device__ __forceinline__ LaneRows(const GridDev &g, const int (&kb)[3]) {
+        const int lane = threadIdx.x & 31;
+        x0 = D == 3 ? 0 : 8 * (lane & 3);
+        y0 = D == 3 ? (lane & 7) : (lane >> 2);
+        z0 = D == 3 ? (lane >> 3) : 0;
+        k0 = kb[0] + x0;
+        kb1 = kb[1];
+        kb2 = kb[2];
+        const int w0 = min(8, g.res[0] - k0);
+        wmask = w0 >= 8 ? 0xffu : (w0 > 0 ? (1u << w0) - 1u : 0u);
     }
-    float rr[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-        rr[a] = __fmul_ru(__fmul_ru(0.5f * (float)(rdim[a] - 1), g.h32[a]), 1.f + 0x1p-22f);
-    if (tid == 0) {
-        sm.pairs = 0u;
-        sm.queued = 0u;
+    __device__ __forceinline__ int k1(int r) const { return kb1 + (D == 3 ? y0 : y0 + 8 * r); }
+    __device__ __forceinline__ int k2(int r) const { return D == 3 ? kb2 + z0 + 4 * r : 0; }
+    // row r: the pixels scored
+    __device__ __forceinline__ unsigned valid(const GridDev &g, int r) const {
+        const int kl = D == 3 ? k2(r) : k1(r);
+        return k1(r) < g.res[1] && kl >= win_lo(g) && kl < win_hi(g) ? wmask : 0u;
     }
-    float r0h, r0l;
-    const unsigned total = region_list<D>(sm, s, ch, cl, rr, r0h, r0l);
-    const Listed<D> src(s, total);
-    const int n_src = src.chunks;
-
-    if (empty) return;
-    const WordMap wm = word_map<D>();
-
-    // the listed seed of least cost at the tile's centre
-    unsigned best = 0xffffffffu;
-    int best_pos = 0x7fffffff;
-    Local<D> L;  // of the last chunk (the only one of most lists)
-    int pos = -1;
-    for (int c = 0; c < n_src; ++c) {
-        if (src.none(sm, c)) continue;
-        pos = src.at(sm, c);
-        unsigned ck = 0xffffffffu;
-        if (pos >= 0) {
-            local_terms<D>(s.recs[pos], ch, cl, toff, tr, s.gf, L);
-            ck = min(okey(L.q - ((L.wh - r0h) + (L.wl - r0l))), 0xfffffffeu);
-        }
-        const unsigned cm = __reduce_min_sync(full, ck);
-        const int who = (int)__reduce_min_sync(full, ck == cm && pos >= 0 ? (unsigned)pos : 0x7fffffffu);
-        if (cm < best || (cm == best && who < best_pos)) {
-            best = cm;
-            best_pos = who;
-            if (pos == who && pos >= 0) store_local<D>(ref, L, s.perm ? s.perm[pos] : pos);
-        }
-    }
-    if (best == 0xffffffffu) {  // cannot happen: the region lists a0
-        if (lane == 0) atomicOr(&s.sc->status, ST_BAD_LABEL);
-        return;
-    }
-    __syncwarp();
-    Local<D> R;
-    int ref_id;
-    load_local<D>(ref, R, ref_id);
-
-    // polynomials of the seeds that can win somewhere in the tile, compacted
-    float Emax = 0.f;
-    int m = 0;          // in the buffer
-    int listed = 0;     // in all chunks
-    float4(*buf)[3] = sm.poly[wid];
-    uint16_t *const tile = tiles + wid * s.tile_cap;
-    bool one = true;  // every polynomial is in the buffer
-    for (int c = 0; c < n_src; ++c) {
-        if (src.none(sm, c)) continue;
-        const int p = n_src == 1 ? pos : src.at(sm, c);
-        bool keep = false;
-        Diff<D> F;
-        if (p >= 0 && p != best_pos) {
-            if (n_src > 1) local_terms<D>(s.recs[p], ch, cl, toff, tr, s.gf, L);
-            difference<D>(L, R, F);
-            keep = can_win<D>(F, tr);
-        }
-        const unsigned km = __ballot_sync(full, keep);
-        const int before = __popc(km & ((1u << lane) - 1u));
-        const int add = __popc(km);
-        one = one && m + add <= kBuf;
-        if (keep) {
-            Emax = fmaxf(Emax, F.E);
-            if (one) put_poly<D>(buf, m + before, s, p, F);
-            if (n_src > 1 && listed + before < s.tile_cap) tile[listed + before] = (uint16_t)p;
-        }
-        if (one) m += add;
-        listed += add;
-    }
-    Emax = __uint_as_float(__reduce_max_sync(full, __float_as_uint(Emax)));
-    __syncwarp();
-    if (lane == 0) atomicAdd(&sm.pairs, (unsigned)(listed + 1));
-    // every polynomial of the tile in turn, f(k) on buffer entry k; called by the whole warp
-    auto each = [&](auto f) {
-        const int pieces = one ? 1 : listed <= s.tile_cap ? (listed + 31) / 32 : n_src;
-        for (int c = 0; c < pieces; ++c) {
-            if (!one) m = refill<D>(sm, s, tile, bx, by, bz, c, listed, best_pos);
-            for (int k = 0; k < m; ++k) f(k);
-        }
-    };
-
-    const long long plane = (long long)g.res[0] * (long long)g.res[1];
-    auto row_id = [&](int r) -> long long {
-        const int k1 = kb[1] + (D == 3 ? y0 : y0 + 8 * r), k2 = D == 3 ? kb[2] + z0 + 4 * r : 0;
-        return (long long)k0 + (long long)g.res[0] * k1 + plane * k2;
-    };
-    auto put_labels = [&](int r, unsigned vm, const unsigned (&lab)[8]) {
-        int32_t *q = s.labels + row_id(r);
+    __device__ __forceinline__ void put_labels(const Src &s, int r, unsigned vm, const unsigned (&lab)[8]) const {
+        const GridDev &g = s.g;
+        const long long plane = (long long)g.res[0] * (long long)g.res[1];
+        int32_t *q = s.labels + ((long long)k0 + (long long)g.res[0] * k1(r) + plane * k2(r));
         if (vm == 0xffu && (reinterpret_cast<uintptr_t>(q) & 15) == 0) {
             reinterpret_cast<int4 *>(q)[0] = make_int4(lab[0], lab[1], lab[2], lab[3]);
             reinterpret_cast<int4 *>(q)[1] = make_int4(lab[4], lab[5], lab[6], lab[7]);
@@ -848,28 +750,28 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, con
             for (int p = 0; p < 8; ++p)
                 if ((vm >> p) & 1u) q[p] = (int)lab[p];
         }
-    };
-
-    if (listed == 0) {  // one cell
-        unsigned long long word;
-        if (MASKED && !whole) {
-            unsigned pk[5];
-            packed_sums<D>(sm.lut, marked, (unsigned)x0, (unsigned)y0, (unsigned)z0, pk);
-            word = packed_word<D>(wm, word_scale(wm, kb), pk);
-        } else {
-            word = box_word<D>(wm, word_scale(wm, lo3), cnt);
-        }
-        if (lane < K) atomicAdd(&s.gmom[(size_t)ref_id * K + lane], word);
-        if (s.labels) {
-            const unsigned id = (unsigned)ref_id;
-            const unsigned lab[8] = {id, id, id, id, id, id, id, id};
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-                if (const unsigned vm = row_mask(r)) put_labels(r, vm, lab);
-        }
-        return;
     }
+};
 
+// Labels and moments of the warp's tile from its polynomials less the reference's:
+// each(f) calls f(k) for every one, in buffer entry k; m of them with `fast`, else any
+// number.  Emax: the largest E of the list.
+template <int D, bool MASKED, class Each>
+__device__ __forceinline__ void score_pixels(Shared<D> &sm, const Src &s, const int (&kb)[3], const int (&cnt)[3],
+                                             const bool whole, const unsigned (&marked)[2], const int ref_id,
+                                             const float Emax, const bool fast, const int m, const Each each) {
+    using G = Geom<D>;
+    constexpr int K = moment_width(D);
+    const GridDev &g = s.g;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned full = 0xffffffffu;
+    const float finf = __int_as_float(0x7f800000);
+    const int n = s.n;
+    const LaneRows<D> rows(g, kb);
+    const int x0 = rows.x0, y0 = rows.y0, z0 = rows.z0;
+    const float4(*buf)[3] = sm.poly[wid];
+    const WordMap wm = word_map<D>();
+    auto row_mask = [&](int r) -> unsigned { return MASKED ? marked[r] : rows.valid(g, r); };
     // ---- pixels: lane owns two rows of eight ----
     float2 dx[4];
 #pragma unroll
@@ -878,7 +780,6 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, con
                             ((float)(x0 + 2 * q + 1 - G::TX / 2) + 0.5f) * g.h32[0]);
     const float gap = 2.f * Emax;
     const WordScale ws = word_scale(wm, kb);
-    const bool fast = one && m <= kFast;
     // the costs of buffer entry k on the row (f1, f2), less the reference's; its seed
     auto row_values = [&](int k, float f1, float f2, float (&v)[8]) -> unsigned {
         const float4 v0 = buf[k][0], v1 = buf[k][1];
@@ -969,7 +870,7 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, con
 #pragma unroll
                     for (int p = 0; p < 8; ++p) lab[p] = (mk >> p) & 1u ? id : lab[p];
                 }
-                put_labels(r, vm, lab);
+                rows.put_labels(s, r, vm, lab);
             }
             enqueue(r, qm);
             const unsigned ok = vm & ~qm;
@@ -1027,7 +928,7 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, con
                 if (!(b2[p] - b1[p] > gap)) qm |= 1u << p;
             const unsigned vm = row_mask(r);
             qm &= vm;
-            if (s.labels && vm) put_labels(r, vm, lab[r]);
+            if (s.labels && vm) rows.put_labels(s, r, vm, lab[r]);
             enqueue(r, qm);
             const unsigned ok = vm & ~qm;
 #pragma unroll
@@ -1123,7 +1024,7 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, con
                 atomicOr(&s.sc->status, ST_BAD_LABEL);
             } else {
                 if (s.labels)
-                    s.labels[(long long)kp[0] + (long long)g.res[0] * kp[1] + (D == 3 ? plane * kp[2] : 0ll)] = ib;
+                    s.labels[(long long)kp[0] + (long long)g.res[0] * kp[1] + (D == 3 ? (long long)g.res[0] * (long long)g.res[1] * kp[2] : 0ll)] = ib;
                 unsigned long long u[3], *o = s.gmom + (size_t)ib * K;
 #pragma unroll
                 for (int a = 0; a < D; ++a) u[a] = 2ull * (unsigned long long)kp[a] + 1ull;
@@ -1138,6 +1039,197 @@ __device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, con
             }
         }
     }
+}
+
+// A tile whose polynomials do not fit the warp's buffer: they are formed again for every
+// pass over them (refill).  Out of line, with what it needs formed again too: beside the
+// other tiles' code the passes cost those registers and a tenth of their instructions (a
+// batch of 48 2D diagrams: 71.3 M warp instructions an evaluation, so 65.8 M; spills 512 /
+// 1108 bytes, so 144 / 352 in 3D).
+template <int D, bool MASKED>
+__device__ __noinline__ void score_pixels_refilled(Shared<D> &sm, const Src &s, const uint16_t *tile, const int bx,
+                                                   const int by, const int bz, const unsigned marked0,
+                                                   const unsigned marked1, const int listed, const int best_pos,
+                                                   const float Emax) {
+    const unsigned full = 0xffffffffu;
+    const TileWindow<D> t(s.g, bx, by, bz);
+    const unsigned marked[2] = {marked0, marked1};
+    const bool whole = MASKED ? __all_sync(full, marked0 == 0xffu && marked1 == 0xffu) : t.whole;
+    const int ref_id = __float_as_int(sm.ref[threadIdx.x >> 5][1].w);  // see store_local
+    const int pieces = listed <= s.tile_cap ? (listed + 31) / 32 : Listed<D>(s, sm.count).chunks;
+    score_pixels<D, MASKED>(sm, s, t.kb, t.cnt, whole, marked, ref_id, Emax, false, 0, [&](auto f) {
+        for (int c = 0; c < pieces; ++c) {
+            const int m = refill<D>(sm, s, tile, bx, by, bz, c, listed, best_pos);
+            for (int k = 0; k < m; ++k) f(k);
+        }
+    });
+}
+
+// Scores region (bx, by, bz); `s` is the same in every thread; `tiles`: kWarps lists of
+// tile_cap positions in shared memory.  The caller puts a barrier between the previous
+// region and the next.
+template <int D, bool MASKED = false>
+__device__ __forceinline__ void score_region(Shared<D> &sm, uint16_t *tiles, const Src &s, const int bx, const int by,
+                                             const int bz) {
+    using G = Geom<D>;
+    constexpr int K = moment_width(D);
+    const GridDev &g = s.g;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned full = 0xffffffffu;
+    const int rdim[3] = {G::RX, G::RY, G::RZ};
+    const int rb[3] = {bx * G::RX, by * G::RY, bz * G::RZ};
+    float4(&ref)[5] = sm.ref[wid];
+
+    const TileWindow<D> win(g, bx, by, bz);
+    const int (&kb)[3] = win.kb;
+    float toff[3], tr[3];
+    tile_box<D>(g, win.tc, toff, tr);
+    bool empty = win.empty, whole = win.whole;
+    const LaneRows<D> rows(g, kb);
+    unsigned marked[2] = {0u, 0u};
+    if constexpr (MASKED) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const unsigned vm = rows.valid(g, r);
+            if (!vm) continue;
+            const int k0 = rows.k0, k1 = rows.k1(r), k2 = rows.k2(r);
+            const uint8_t *row = s.mask + (size_t)s.cres[0] * ((size_t)(k1 / s.r) + (size_t)s.cres[1] * (size_t)(k2 / s.r));
+            int kx = k0 / s.r, next = (kx + 1) * s.r;
+            bool on = row[kx] != 0;
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                if (!((vm >> p) & 1u)) continue;
+                if (k0 + p == next) {
+                    on = row[++kx] != 0;
+                    next += s.r;
+                }
+                marked[r] |= on ? 1u << p : 0u;
+            }
+        }
+        whole = __all_sync(full, marked[0] == 0xffu && marked[1] == 0xffu);
+        empty = !__any_sync(full, (marked[0] | marked[1]) != 0u);
+        if (!__syncthreads_or(!empty)) return;  // no marked pixel in the region
+    }
+
+    // region centre (lane a: axis a) as an FP32 pair, half-widths rounded up
+    float ch[3] = {0.f, 0.f, 0.f}, cl[3] = {0.f, 0.f, 0.f};
+    {
+        float h = 0.f, l = 0.f;
+        if (lane < D) {
+            const int k = lane == 0 ? rb[0] + G::RX / 2 : (lane == 1 ? rb[1] + G::RY / 2 : rb[2] + G::RZ / 2);
+            axis_point(s.gf, lane, k, h, l);
+        }
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            ch[a] = __shfl_sync(full, h, a);
+            cl[a] = __shfl_sync(full, l, a);
+        }
+    }
+    float rr[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+        rr[a] = __fmul_ru(__fmul_ru(0.5f * (float)(rdim[a] - 1), g.h32[a]), 1.f + 0x1p-22f);
+    if (tid == 0) {
+        sm.pairs = 0u;
+        sm.queued = 0u;
+    }
+    float r0h, r0l;
+    const unsigned total = region_list<D>(sm, s, ch, cl, rr, r0h, r0l);
+    const Listed<D> src(s, total);
+    const int n_src = src.chunks;
+
+    if (empty) return;
+
+    // the listed seed of least cost at the tile's centre
+    unsigned best = 0xffffffffu;
+    int best_pos = 0x7fffffff;
+    Local<D> L;  // of the last chunk (the only one of most lists)
+    int pos = -1;
+    for (int c = 0; c < n_src; ++c) {
+        if (src.none(sm, c)) continue;
+        pos = src.at(sm, c);
+        unsigned ck = 0xffffffffu;
+        if (pos >= 0) {
+            local_terms<D>(s.recs[pos], ch, cl, toff, tr, s.gf, L);
+            ck = min(okey(L.q - ((L.wh - r0h) + (L.wl - r0l))), 0xfffffffeu);
+        }
+        const unsigned cm = __reduce_min_sync(full, ck);
+        const int who = (int)__reduce_min_sync(full, ck == cm && pos >= 0 ? (unsigned)pos : 0x7fffffffu);
+        if (cm < best || (cm == best && who < best_pos)) {
+            best = cm;
+            best_pos = who;
+            if (pos == who && pos >= 0) store_local<D>(ref, L, s.perm ? s.perm[pos] : pos);
+        }
+    }
+    if (best == 0xffffffffu) {  // cannot happen: the region lists a0
+        if (lane == 0) atomicOr(&s.sc->status, ST_BAD_LABEL);
+        return;
+    }
+    __syncwarp();
+    Local<D> R;
+    int ref_id;
+    load_local<D>(ref, R, ref_id);
+
+    // polynomials of the seeds that can win somewhere in the tile, compacted
+    float Emax = 0.f;
+    int m = 0;          // in the buffer
+    int listed = 0;     // in all chunks
+    float4(*buf)[3] = sm.poly[wid];
+    uint16_t *const tile = tiles + wid * s.tile_cap;
+    bool one = true;  // every polynomial is in the buffer
+    for (int c = 0; c < n_src; ++c) {
+        if (src.none(sm, c)) continue;
+        const int p = n_src == 1 ? pos : src.at(sm, c);
+        bool keep = false;
+        Diff<D> F;
+        if (p >= 0 && p != best_pos) {
+            if (n_src > 1) local_terms<D>(s.recs[p], ch, cl, toff, tr, s.gf, L);
+            difference<D>(L, R, F);
+            keep = can_win<D>(F, tr);
+        }
+        const unsigned km = __ballot_sync(full, keep);
+        const int before = __popc(km & ((1u << lane) - 1u));
+        const int add = __popc(km);
+        one = one && m + add <= kBuf;
+        if (keep) {
+            Emax = fmaxf(Emax, F.E);
+            if (one) put_poly<D>(buf, m + before, s, p, F);
+            if (total > (unsigned)kBuf && listed + before < s.tile_cap) tile[listed + before] = (uint16_t)p;
+        }
+        if (one) m += add;
+        listed += add;
+    }
+    Emax = __uint_as_float(__reduce_max_sync(full, __float_as_uint(Emax)));
+    __syncwarp();
+    if (lane == 0) atomicAdd(&sm.pairs, (unsigned)(listed + 1));
+    if (listed == 0) {  // one cell
+        const WordMap wm = word_map<D>();
+        unsigned long long word;
+        if (MASKED && !whole) {
+            unsigned pk[5];
+            packed_sums<D>(sm.lut, marked, (unsigned)rows.x0, (unsigned)rows.y0, (unsigned)rows.z0, pk);
+            word = packed_word<D>(wm, word_scale(wm, kb), pk);
+        } else {
+            word = box_word<D>(wm, word_scale(wm, win.lo3), win.cnt);
+        }
+        if (lane < K) atomicAdd(&s.gmom[(size_t)ref_id * K + lane], word);
+        if (s.labels) {
+            const unsigned id = (unsigned)ref_id;
+            const unsigned lab[8] = {id, id, id, id, id, id, id, id};
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (const unsigned vm = MASKED ? marked[r] : rows.valid(g, r)) rows.put_labels(s, r, vm, lab);
+        }
+        return;
+    }
+
+    if (!one) {
+        score_pixels_refilled<D, MASKED>(sm, s, tile, bx, by, bz, marked[0], marked[1], listed, best_pos, Emax);
+        return;
+    }
+    score_pixels<D, MASKED>(sm, s, kb, win.cnt, whole, marked, ref_id, Emax, m <= kFast, m, [&](auto f) {
+        for (int k = 0; k < m; ++k) f(k);
+    });
 }
 
 }  // namespace region
