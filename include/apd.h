@@ -147,7 +147,7 @@ int apd_workspace_set_graphs(apd_workspace *ws, int32_t enable);
  * max D - min D.  Labels and moments are the same as with full passes.
  * enable: 0 every pass a full one; 1 (default) incremental passes where they
  * cost less than full ones, which is nowhere since full passes score from
- * difference lists (256^3 x 1000 seeds: 108 us, against 116 us for a re-decision
+ * difference lists (256^3 x 1000 seeds: 99 us, against 116 us for a re-decision
  * and 667 us for a recording); 2 incremental passes on every grid.
  * Returns APD_ERR_ARG for a null workspace or another enable value. */
 int apd_workspace_set_incremental(apd_workspace *ws, int32_t enable);

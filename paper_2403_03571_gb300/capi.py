@@ -307,8 +307,9 @@ class Workspace:
         _check(load().apd_workspace_set_graphs(self.handle, int(bool(enable))), "apd_workspace_set_graphs")
 
     def set_incremental(self, mode=1):
-        """Incremental evaluations in weight solves: 0 (or False) off, 1 (or True,
-        the default) on grids of at least 2^20 pixels, 2 on every grid."""
+        """Incremental evaluations in weight solves: 2 records and re-decides on every
+        grid; 0 (or False) and 1 (or True, the default) score every pixel in every
+        evaluation, which is faster."""
         _check(load().apd_workspace_set_incremental(self.handle, int(mode)),
                "apd_workspace_set_incremental")
 

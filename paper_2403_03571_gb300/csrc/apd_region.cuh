@@ -21,11 +21,11 @@
 //     seed of least cost at the tile's centre.  Up to 48 polynomials stay in shared
 //     memory; of a longer list the positions stay, and its polynomials are formed again
 //     32 at a time (see tile_cap).
-// Measured (1000 seeds, 256^3, solve-sized weights): 108 us, 62.8 M warp
+// Measured (1000 seeds, 256^3, solve-sized weights): 99 us, 61.0 M warp
 // instructions (region lists 33 %, tile lists 23 %, pixels 27 %, moments 17 %) at half
 // of the issue slots; the tensor-core scorer with separate bounds took 456 us after a
 // 92 us list pre-pass, and 14 us of rescoring followed.  10^4 seeds, 200^3, axis
-// ratios up to 3.3 (the alpha = 0.7 law): 6.2 ms -> 0.94 ms, since the bound E is local
+// ratios up to 3.3 (the alpha = 0.7 law): 6.2 ms -> 0.79 ms, since the bound E is local
 // (the FP32 kernel's grows with the largest condition number of all seeds).
 // Scoring.  What is left is a handful of polynomials D_i(e) per tile (a itself is 0
 // everywhere): a lane owns two rows of eight pixels, the two row coefficients cost
